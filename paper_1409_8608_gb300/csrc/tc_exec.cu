@@ -29,6 +29,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "tc_internal.h"
@@ -68,6 +69,7 @@ struct TileDesc {
     int init, alpha_one;
     int a_m_fast, b_n_fast;  // load mapping: M (N) contiguous in memory
     int64_t tile0;           // batched form: the problem's first tile in the list
+    int64_t shape;           // tile shape (simt_rows)
 };
 
 struct GatherDesc {
@@ -223,25 +225,69 @@ __global__ void __launch_bounds__(256) coop_reduce_kernel(const PhaseDesc d) {
 }
 
 // ---------------------------------------------------------------- gemm / SIMT GETT
-// One CTA computes a BM x BN tile of one task's C slice; K runs over the
-// linearised contracted space in chunks of BK staged through shared memory.
-template <typename T, int BM, int BN, int BK, int TM, int TN>
-__device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid) {
-    constexpr int TX = BN / TN, TY = BM / TM, NT = TX * TY;
-    // A thread owns rows ty*V + r + g*TY*V (r < V, g < TM/V) and likewise
-    // columns: with V = 4 for FP32 each group is one 16-byte shared-memory
-    // read, so a K step issues TM/4 + TN/4 loads for TM*TN FMAs instead of
-    // TM + TN; FP64 (V = 1) is bound by the DFMA rate either way.
-    constexpr int V = (sizeof(T) == 4 && TM % 4 == 0 && TN % 4 == 0) ? 4 : 1;
-    auto row_of = [](int ty_, int i) { return (i / V) * (TY * V) + ty_ * V + i % V; };
-    auto col_of = [](int tx_, int j) { return (j / V) * (TX * V) + tx_ * V + j % V; };
+// x = q * y + r for non-negative x, y > 0, in 32 bits when both fit (a
+// 64-bit division is a long dependent sequence on every tile's first path)
+__device__ __forceinline__ int64_t divmod_pos(int64_t x, int64_t y, int64_t &r) {
+    if (((x | y) >> 31) == 0) {
+        const uint32_t q = (uint32_t)x / (uint32_t)y;
+        r = x - (int64_t)q * y;
+        return q;
+    }
+    const int64_t q = x / y;
+    r = x - q * y;
+    return q;
+}
+
+__device__ __forceinline__ uint64_t pack_f2(float lo, float hi) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+
+__device__ __forceinline__ void unpack_f2(uint64_t v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+
+// two independent FP32 fused multiply-adds in one instruction (each rounded
+// as fmaf rounds)
+__device__ __forceinline__ void fma_f2(uint64_t &c, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+
+template <typename T, int BM, int BN, int BK>
+struct TileSmem {
     // two stage buffers; rows padded by 4 elements so that the K-contiguous
     // store mapping below spreads a warp over all 32 banks
-    constexpr int PAD = 4;
-    __shared__ __align__(16) T As[2][BK][BM + PAD];
-    __shared__ __align__(16) T Bs[2][BK][BN + PAD];
-    __shared__ int64_t offAm[BM], offCm[BM], offBn[BN], offCn[BN];
-    __shared__ int64_t kA[2][BK], kB[2][BK];
+    static constexpr int PAD = 4;
+    T As[2][BK][BM + PAD];
+    T Bs[2][BK][BN + PAD];
+    int64_t offAm[BM], offCm[BM], offBn[BN], offCn[BN];
+    int64_t kA[2][BK], kB[2][BK];
+};
+
+// One CTA computes a BM x BN tile of one task's C slice; K runs over the
+// linearised contracted space in stages of BK through shared memory.  Each
+// thread keeps the memory offsets of the rows it copies in registers, so a
+// stage's copies read only its K offsets from shared memory (with both read
+// per element the offset tables took as many shared-memory cycles as the
+// operands: 68 % of the pipe at 37 % of the FMA rate on FP32).  With that,
+// paired FP32 multiply-adds and C stored by column runs, FP32 512^3 iaj,jbic
+// i=j=16 went from 2.35 to 1.83 ms and the n = 256 gemm nest from 0.287 to
+// 0.213 ms; FP64 512^3 from 56.76 to 55.06 ms (the DFMA rate).
+template <typename T, int BM, int BN, int BK, int TM, int TN>
+__device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid, TileSmem<T, BM, BN, BK> &sm) {
+    // rows across the lanes (TX), so that a warp's stores of one column of C
+    // cover a contiguous run of its first index
+    constexpr int TX = BM / TM, TY = BN / TN, NT = TX * TY;
+    // FP32: a thread owns V consecutive rows per group, V = 2 or 4 (one 8- or
+    // 16-byte shared-memory read per group; its rows multiply in pairs with
+    // fma.rn.f32x2, which halves the issue slots of the FMAs), and likewise
+    // columns; FP64 (V = 1) is bound by the DFMA rate either way
+    constexpr bool F32 = sizeof(T) == 4;
+    constexpr int V = F32 ? (TM % 4 == 0 && TN % 4 == 0 ? 4 : 2) : 1;
+    static_assert(TM % V == 0 && TN % V == 0, "groups of V");
+    auto row_of = [](int tx_, int i) { return (i / V) * (TX * V) + tx_ * V + i % V; };
+    auto col_of = [](int ty_, int j) { return (j / V) * (TY * V) + ty_ * V + j % V; };
     const T *__restrict__ A = (const T *)d.A;
     const T *__restrict__ B = (const T *)d.B;
     T *__restrict__ C = (T *)d.C;
@@ -249,14 +295,13 @@ __device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid) {
     const int tid = threadIdx.x;
     const int tx = tid % TX, ty = tid / TX;
 
-    const int64_t tm = bid % d.tiles_m;
-    bid /= d.tiles_m;
-    const int64_t tn = bid % d.tiles_n;
-    int64_t task = bid / d.tiles_n;
+    int64_t tm, tn;
+    bid = divmod_pos(bid, d.tiles_m, tm);
+    int64_t task = divmod_pos(bid, d.tiles_n, tn);
     int64_t tA = 0, tB = 0, tC = 0;
     for (int m = d.task.n - 1; m >= 0; --m) {
-        int64_t x = task % d.task.ext[m];
-        task /= d.task.ext[m];
+        int64_t x;
+        task = divmod_pos(task, d.task.ext[m], x);
         tA += x * d.task.sA[m];
         tB += x * d.task.sB[m];
         tC += x * d.task.sC[m];
@@ -268,14 +313,14 @@ __device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid) {
             oa = tA;
             oc = tC;
             for (int m = 0; m < d.m.n; ++m) {
-                int64_t x = mm % d.m.ext[m];
-                mm /= d.m.ext[m];
+                int64_t x;
+                mm = divmod_pos(mm, d.m.ext[m], x);
                 oa += x * d.m.sA[m];
                 oc += x * d.m.sC[m];
             }
         }
-        offAm[i] = oa;
-        offCm[i] = oc;
+        sm.offAm[i] = oa;
+        sm.offCm[i] = oc;
     }
     for (int j = tid; j < BN; j += NT) {
         int64_t nn = tn * BN + j;
@@ -284,247 +329,311 @@ __device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid) {
             ob = tB;
             oc = 0;
             for (int m = 0; m < d.n.n; ++m) {
-                int64_t x = nn % d.n.ext[m];
-                nn /= d.n.ext[m];
+                int64_t x;
+                nn = divmod_pos(nn, d.n.ext[m], x);
                 ob += x * d.n.sB[m];
                 oc += x * d.n.sC[m];
             }
         }
-        offBn[j] = ob;
-        offCn[j] = oc;
+        sm.offBn[j] = ob;
+        sm.offCn[j] = oc;
     }
-    __syncthreads();
-
-    T acc[TM][TN];
-#pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const int64_t om = offCm[row_of(ty, i)];
-#pragma unroll
-        for (int j = 0; j < TN; ++j) {
-            const int64_t on = offCn[col_of(tx, j)];
-            T v = T(0);
-            if (d.init != 2 && om >= 0 && on >= 0) {
-                v = C[om + on];
-                if (d.init == 1) v = beta * v;
-            }
-            acc[i][j] = v;
-        }
-    }
-
-    // K offsets of a stage into table buffer b (threads kk < BK); the K
-    // position's digits in 32-bit arithmetic when K fits (a 64-bit division
-    // is a long dependent sequence, and the other warps wait for these
-    // tables at the stage's barrier)
+    // K offsets of a stage into table buffer b (threads kk < BK)
     auto k_tables = [&](int64_t k0, int b) {
-        for (int kk = tid; kk < BK; kk += NT) {
-            int64_t k = k0 + kk;
+        if (tid < BK) {
+            int64_t k = k0 + tid;
             int64_t oa = -1, ob = -1;
             if (k < d.K) {
                 oa = 0;
                 ob = 0;
-                if (d.K < (int64_t(1) << 31)) {
-                    uint32_t k32 = (uint32_t)k;
-                    for (int m = d.red.n - 1; m >= 0; --m) {
-                        const uint32_t e = (uint32_t)d.red.ext[m];
-                        const int64_t x = (int64_t)(k32 % e);
-                        k32 /= e;
-                        oa += x * d.red.sA[m];
-                        ob += x * d.red.sB[m];
-                    }
-                } else {
-                    for (int m = d.red.n - 1; m >= 0; --m) {
-                        int64_t x = k % d.red.ext[m];
-                        k /= d.red.ext[m];
-                        oa += x * d.red.sA[m];
-                        ob += x * d.red.sB[m];
-                    }
+                for (int m = d.red.n - 1; m >= 0; --m) {
+                    int64_t x;
+                    k = divmod_pos(k, d.red.ext[m], x);
+                    oa += x * d.red.sA[m];
+                    ob += x * d.red.sB[m];
                 }
             }
-            kA[b][kk] = oa;
-            kB[b][kk] = ob;
+            sm.kA[b][tid] = oa;
+            sm.kB[b][tid] = ob;
         }
     };
-    // Element e of a stage's R x BK operand tile: with M (N) contiguous in
-    // memory, consecutive threads take consecutive rows; otherwise groups
-    // of 8 threads take 8 consecutive K positions of one row (32-byte runs
-    // in memory; with the padded rows a warp's stores hit 32 distinct banks).
-    static_assert(BK % 8 == 0, "K stage is a multiple of 8");
-    auto place = [](int e, bool rfast, int R, int &r, int &kk) {
-        if (rfast) {
-            r = e % R;
-            kk = e / R;
-        } else {
-            r = (e / 8) % R;
-            kk = (e / (8 * R)) * 8 + e % 8;
-        }
-    };
-    // a stage's A and B elements of this thread, into registers
-    constexpr int LA = BM * BK / NT, LB = BN * BK / NT;
-    static_assert(LA * NT == BM * BK && LB * NT == BN * BK, "even split");
-    T ra[LA], rb[LB];
-    auto load_stage = [&](int b) {
+    static_assert(NT >= BK, "one thread per K offset");
+    k_tables(0, 0);
+    if (BK < d.K) k_tables(BK, 1);
+    __syncthreads();
+
+    // accumulators: FP32 row pairs (2i, 2i + 1), FP64 one by one
+    constexpr int NACC = F32 ? TM / 2 : TM;
+    using Acc = typename std::conditional<F32, uint64_t, double>::type;
+    Acc acc[NACC][TN];
+    if (d.init == 2) {
 #pragma unroll
-        for (int l = 0; l < LA; ++l) {
-            int i, kk;
-            place(tid + l * NT, d.a_m_fast, BM, i, kk);
-            const int64_t om = offAm[i], ok = kA[b][kk];
+        for (int i = 0; i < NACC; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; ++j) acc[i][j] = Acc(0);
+    } else {
+        auto start = [&](int i, int j) {
+            const int64_t om = sm.offCm[row_of(tx, i)], on = sm.offCn[col_of(ty, j)];
             T v = T(0);
-            if (om >= 0 && ok >= 0) {
-                v = A[om + ok];
-                if (!d.alpha_one) v = alpha * v;
+            if (om >= 0 && on >= 0) {
+                v = C[om + on];
+                if (d.init == 1) v = beta * v;
             }
-            ra[l] = v;
-        }
+            return v;
+        };
 #pragma unroll
-        for (int l = 0; l < LB; ++l) {
-            int j, kk;
-            place(tid + l * NT, d.b_n_fast, BN, j, kk);
-            const int64_t on = offBn[j], ok = kB[b][kk];
-            rb[l] = (on >= 0 && ok >= 0) ? B[on + ok] : T(0);
+        for (int i = 0; i < NACC; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; ++j) {
+                if constexpr (F32) acc[i][j] = pack_f2(start(2 * i, j), start(2 * i + 1, j));
+                else acc[i][j] = start(i, j);
+            }
+    }
+
+    // Elements of a stage's R x BK operand tile that a thread copies: with
+    // M (N) contiguous in memory (rfast), consecutive threads take
+    // consecutive rows and a thread always the same row; otherwise groups of
+    // 8 threads take 8 consecutive K positions of one row (32-byte runs in
+    // memory; with the padded rows a warp's stores hit 32 distinct banks)
+    // and a thread meets at most R / (NT / 8) rows.
+    static_assert(BK % 8 == 0 && NT % BM == 0 && NT % BN == 0, "copy mapping");
+    constexpr int QA = BM > NT / 8 ? BM / (NT / 8) : 1, QB = BN > NT / 8 ? BN / (NT / 8) : 1;
+    constexpr int LA = BM * BK / NT, LB = BN * BK / NT;
+    static_assert(LA * NT == BM * BK && LB * NT == BN * BK && LA % QA == 0 && LB % QB == 0, "even split");
+    const bool fa = d.a_m_fast != 0, fb = d.b_n_fast != 0;
+    const int rA0 = fa ? tid % BM : (tid / 8) % BM, rB0 = fb ? tid % BN : (tid / 8) % BN;
+    const int kA0 = fa ? tid / BM : (tid / (8 * BM)) * 8 + tid % 8;
+    const int kB0 = fb ? tid / BN : (tid / (8 * BN)) * 8 + tid % 8;
+    int64_t roA[QA], roB[QB];
+#pragma unroll
+    for (int q = 0; q < QA; ++q) roA[q] = sm.offAm[fa ? rA0 : (rA0 + q * (NT / 8)) % BM];
+#pragma unroll
+    for (int q = 0; q < QB; ++q) roB[q] = sm.offBn[fb ? rB0 : (rB0 + q * (NT / 8)) % BN];
+    // element l of the thread: row slot, row and K position
+    auto at = [](bool fast, int R, int Q, int l, int r0, int k0, int &q, int &r, int &kk) {
+        if (fast) {
+            q = 0;
+            r = r0;
+            kk = k0 + l * (NT / R);
+        } else {
+            q = l % Q;
+            r = r0 + q * (NT / 8);
+            // R < NT / 8: the NT threads cover NT / (8R) octets of K per step
+            kk = k0 + (l / Q) * (R < NT / 8 ? NT / R : 8);
         }
     };
-    auto store_stage = [&](int sb) {
-#pragma unroll
-        for (int l = 0; l < LA; ++l) {
-            int i, kk;
-            place(tid + l * NT, d.a_m_fast, BM, i, kk);
-            As[sb][kk][i] = ra[l];
-        }
-#pragma unroll
-        for (int l = 0; l < LB; ++l) {
-            int j, kk;
-            place(tid + l * NT, d.b_n_fast, BN, j, kk);
-            Bs[sb][kk][j] = rb[l];
-        }
-    };
-    // FP32 with alpha = 1: the stage's elements go straight to shared memory
-    // with 4-byte asynchronous copies (zero-filled past the extents), so no
-    // register holds them and no second pass stores them; the same values
-    // land in the same places as through load_stage + store_stage
-    const bool async_copy = sizeof(T) == 4 && d.alpha_one;
-    auto async_stage = [&](int b) {
-        auto cp4 = [](void *dst, const void *src, bool valid) {
+    // with alpha = 1 the elements go straight to shared memory with
+    // asynchronous copies (zero-filled past the extents); otherwise through
+    // registers, A scaled by alpha on the way: the same values land in the
+    // same places
+    const bool async_copy = d.alpha_one;
+    auto cp = [](void *dst, const void *src, bool valid) {
+        if constexpr (F32)
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
                              (uint32_t)__cvta_generic_to_shared(dst)),
                          "l"(src), "r"(valid ? 4 : 0)
                          : "memory");
+        else
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
+                             (uint32_t)__cvta_generic_to_shared(dst)),
+                         "l"(src), "r"(valid ? 8 : 0)
+                         : "memory");
+    };
+    auto async_stage = [&](int b) {
+        auto side = [&](auto fast, auto rows, auto Lc, auto Qc, const T *base, const int64_t *ro, const int64_t *kt, int r0,
+                        int k0, T *dst, int pitch) {
+#pragma unroll
+            for (int l = 0; l < decltype(Lc)::value; ++l) {
+                int q, r, kk;
+                at(decltype(fast)::value, decltype(rows)::value, decltype(Qc)::value, l, r0, k0, q, r, kk);
+                const int64_t om = ro[q], ok = kt[kk];
+                const bool v = om >= 0 && ok >= 0;
+                cp(dst + kk * pitch + r, v ? base + om + ok : base, v);
+            }
         };
-#pragma unroll
-        for (int l = 0; l < LA; ++l) {
-            int i, kk;
-            place(tid + l * NT, d.a_m_fast, BM, i, kk);
-            const int64_t om = offAm[i], ok = kA[b][kk];
-            const bool v = om >= 0 && ok >= 0;
-            cp4(&As[b][kk][i], v ? A + om + ok : A, v);
-        }
-#pragma unroll
-        for (int l = 0; l < LB; ++l) {
-            int j, kk;
-            place(tid + l * NT, d.b_n_fast, BN, j, kk);
-            const int64_t on = offBn[j], ok = kB[b][kk];
-            const bool v = on >= 0 && ok >= 0;
-            cp4(&Bs[b][kk][j], v ? B + on + ok : B, v);
-        }
+        using Yes = std::true_type;
+        using No = std::false_type;
+        if (fa) side(Yes{}, std::integral_constant<int, BM>{}, std::integral_constant<int, LA>{}, std::integral_constant<int, QA>{}, A, roA, sm.kA[b], rA0, kA0, &sm.As[b][0][0], BM + sm.PAD);
+        else side(No{}, std::integral_constant<int, BM>{}, std::integral_constant<int, LA>{}, std::integral_constant<int, QA>{}, A, roA, sm.kA[b], rA0, kA0, &sm.As[b][0][0], BM + sm.PAD);
+        if (fb) side(Yes{}, std::integral_constant<int, BN>{}, std::integral_constant<int, LB>{}, std::integral_constant<int, QB>{}, B, roB, sm.kB[b], rB0, kB0, &sm.Bs[b][0][0], BN + sm.PAD);
+        else side(No{}, std::integral_constant<int, BN>{}, std::integral_constant<int, LB>{}, std::integral_constant<int, QB>{}, B, roB, sm.kB[b], rB0, kB0, &sm.Bs[b][0][0], BN + sm.PAD);
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     auto async_wait = []() { asm volatile("cp.async.wait_all;" ::: "memory"); };
+    auto plain_stage = [&](int b) {  // alpha != 1
+        for (int e = tid; e < BM * BK; e += NT) {
+            const int r = fa ? e % BM : (e / 8) % BM, kk = fa ? e / BM : (e / (8 * BM)) * 8 + e % 8;
+            const int64_t om = sm.offAm[r], ok = sm.kA[b][kk];
+            sm.As[b][kk][r] = om >= 0 && ok >= 0 ? alpha * A[om + ok] : T(0);
+        }
+        for (int e = tid; e < BN * BK; e += NT) {
+            const int r = fb ? e % BN : (e / 8) % BN, kk = fb ? e / BN : (e / (8 * BN)) * 8 + e % 8;
+            const int64_t on = sm.offBn[r], ok = sm.kB[b][kk];
+            sm.Bs[b][kk][r] = on >= 0 && ok >= 0 ? B[on + ok] : T(0);
+        }
+    };
+    auto step = [&](int sb, int kk) {
+        if constexpr (F32) {
+            uint64_t a[TM / 2], b[TN];
+#pragma unroll
+            for (int g = 0; g < TM / V; ++g) {
+                if constexpr (V == 4) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&sm.As[sb][kk][row_of(tx, V * g)]);
+                    a[2 * g] = v.x;
+                    a[2 * g + 1] = v.y;
+                } else {
+                    a[g] = *reinterpret_cast<const unsigned long long *>(&sm.As[sb][kk][row_of(tx, V * g)]);
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < TN / V; ++g) {
+                if constexpr (V == 4) {
+                    const float4 v = *reinterpret_cast<const float4 *>(&sm.Bs[sb][kk][col_of(ty, V * g)]);
+                    b[4 * g] = pack_f2(v.x, v.x);
+                    b[4 * g + 1] = pack_f2(v.y, v.y);
+                    b[4 * g + 2] = pack_f2(v.z, v.z);
+                    b[4 * g + 3] = pack_f2(v.w, v.w);
+                } else {
+                    const float2 v = *reinterpret_cast<const float2 *>(&sm.Bs[sb][kk][col_of(ty, V * g)]);
+                    b[2 * g] = pack_f2(v.x, v.x);
+                    b[2 * g + 1] = pack_f2(v.y, v.y);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < TM / 2; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) fma_f2(acc[i][j], a[i], b[j]);
+        } else {
+            T a[TM], b[TN];
+#pragma unroll
+            for (int i = 0; i < TM; ++i) a[i] = sm.As[sb][kk][row_of(tx, i)];
+#pragma unroll
+            for (int j = 0; j < TN; ++j) b[j] = sm.Bs[sb][kk][col_of(ty, j)];
+#pragma unroll
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+                for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        }
+    };
     // Stage s sits in buffer s & 1 (shared memory and K tables alike).
-    // While stage s is multiplied, stage s + 1's global loads are in flight
-    // and then stored to the other buffer, whose last reader (stage s - 1)
-    // finished before the barrier that ended the previous iteration; one
-    // barrier per stage.  Stage s + 2's K tables go to buffer s & 1 right
-    // after stage s + 1's loads have read theirs (buffer s & 1 was last read
-    // by stage s's loads, before that barrier), so that their integer work
-    // overlaps the multiplications instead of delaying the barrier.
-    k_tables(0, 0);
-    __syncthreads();
+    // While stage s is multiplied, stage s + 1's copies are in flight into
+    // the other buffer, whose last reader (stage s - 1) finished before the
+    // barrier that ended the previous iteration; one barrier per stage.
+    // Stage s + 2's K tables go to buffer s & 1 right after stage s + 1's
+    // copies have read theirs (buffer s & 1 was last read by stage s's
+    // copies, before that barrier), so that their integer work overlaps the
+    // multiplications.  The last stage stops at K (its padding would cost
+    // whole multiplications: K = 8 spent as much as K = 16).
     if (async_copy) {
         async_stage(0);
         async_wait();
     } else {
-        load_stage(0);
-        store_stage(0);
+        plain_stage(0);
     }
-    if (BK < d.K) k_tables(BK, 1);
     __syncthreads();
     int sb = 0;
     for (int64_t k0 = 0; k0 < d.K; k0 += BK, sb ^= 1) {
         const bool more = k0 + BK < d.K;
-        if (more) {
-            if (async_copy) async_stage(sb ^ 1);
-            else load_stage(sb ^ 1);
-        }
+        if (more && async_copy) async_stage(sb ^ 1);
         if (k0 + 2 * BK < d.K) k_tables(k0 + 2 * BK, sb);
+        if (k0 + BK <= d.K) {
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            T a[TM], b[TN];
-            if constexpr (V == 4) {
-#pragma unroll
-                for (int g = 0; g < TM / 4; ++g) {
-                    const float4 v = *reinterpret_cast<const float4 *>(&As[sb][kk][row_of(ty, 4 * g)]);
-                    a[4 * g] = v.x;
-                    a[4 * g + 1] = v.y;
-                    a[4 * g + 2] = v.z;
-                    a[4 * g + 3] = v.w;
-                }
-#pragma unroll
-                for (int g = 0; g < TN / 4; ++g) {
-                    const float4 v = *reinterpret_cast<const float4 *>(&Bs[sb][kk][col_of(tx, 4 * g)]);
-                    b[4 * g] = v.x;
-                    b[4 * g + 1] = v.y;
-                    b[4 * g + 2] = v.z;
-                    b[4 * g + 3] = v.w;
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < TM; ++i) a[i] = As[sb][kk][row_of(ty, i)];
-#pragma unroll
-                for (int j = 0; j < TN; ++j) b[j] = Bs[sb][kk][col_of(tx, j)];
-            }
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] = fma_t<T>(a[i], b[j], acc[i][j]);
+            for (int kk = 0; kk < BK; ++kk) step(sb, kk);
+        } else {
+            const int klen = (int)(d.K - k0);
+#pragma unroll 1
+            for (int kk = 0; kk < klen; ++kk) step(sb, kk);
         }
         if (more) {
             if (async_copy) async_wait();
-            else store_stage(sb ^ 1);
+            else plain_stage(sb ^ 1);
         }
         __syncthreads();
     }
 
 #pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const int64_t om = offCm[row_of(ty, i)];
+    for (int g = 0; g < TM / V; ++g) {
+        int64_t om[V];
+#pragma unroll
+        for (int v = 0; v < V; ++v) om[v] = sm.offCm[row_of(tx, V * g + v)];
+        const bool run = V > 1 && om[0] >= 0 && om[V - 1] == om[0] + V - 1;
 #pragma unroll
         for (int j = 0; j < TN; ++j) {
-            const int64_t on = offCn[col_of(tx, j)];
-            if (om >= 0 && on >= 0) C[om + on] = acc[i][j];
+            const int64_t on = sm.offCn[col_of(ty, j)];
+            if (on < 0) continue;
+            T x[V];
+            if constexpr (F32) {
+#pragma unroll
+                for (int v = 0; v < V; v += 2) unpack_f2(acc[(V * g + v) / 2][j], x[v], x[v + 1]);
+            } else {
+                x[0] = acc[g][j];
+            }
+            T *p = C + om[0] + on;
+            // the group's rows are one aligned run of C: one store
+            if (run && ((uintptr_t)p % (V * sizeof(T))) == 0) {
+                if constexpr (V == 4) *reinterpret_cast<float4 *>(p) = make_float4(x[0], x[1], x[2], x[3]);
+                else if constexpr (V == 2) *reinterpret_cast<float2 *>(p) = make_float2(x[0], x[1]);
+            } else {
+#pragma unroll
+                for (int v = 0; v < V; ++v)
+                    if (om[v] >= 0) C[om[v] + on] = x[v];
+            }
         }
     }
 }
 
-template <typename T, int BM, int BN, int BK, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN)) tile_kernel(const TileDesc d) {
-    tile_body<T, BM, BN, BK, TM, TN>(d, blockIdx.x);
+// Tile shapes.  The largest keeps the least traffic per multiplication; the
+// smaller ones spread small results over the SMs: with the FP64 rate at two
+// multiply-adds per SM and clock a 64 x 64 tile of K = 3920 holds one SM for
+// 4 ms, and nothing is lost per multiplication down to 16 x 16 (64^3 i = 8:
+// 25.9 us with 64 tiles of 64 x 64 and K padded to 16, 10.3 us with 1024
+// tiles of 16 x 16 stopping at K; a burst of 24 mixed requests 6.03 -> 2.02
+// ms, 5.0 of it one FP64 tile).  The tile does not change any output's chain.
+constexpr int kSimtShapes = 3;
+constexpr int simt_rows(bool f64, int shape) { return (f64 ? 64 : 128) >> shape; }
+
+// The largest shape whose tiles give each SM at least two (FP32, two
+// blocks resident) or eight (FP64), else the smallest.
+int simt_shape(bool f64, int64_t M, int64_t N, int64_t tasks);
+
+template <typename T, int SHAPE>
+struct TileOf {
+    static constexpr bool F64 = sizeof(T) == 8;
+    static constexpr int B = simt_rows(F64, SHAPE);
+    static constexpr int TT = B / 16;  // 16 x 16 threads
+    using Smem = TileSmem<T, B, B, 16>;
+    static __device__ __forceinline__ void run(const TileDesc &d, int64_t bid, void *buf) {
+        tile_body<T, B, B, 16, TT, TT>(d, bid, *reinterpret_cast<Smem *>(buf));
+    }
+};
+
+template <typename T, int SHAPE>
+__global__ void __launch_bounds__(256, 2) tile_kernel(const TileDesc d) {
+    __shared__ __align__(16) unsigned char buf[sizeof(typename TileOf<T, SHAPE>::Smem)];
+    TileOf<T, SHAPE>::run(d, blockIdx.x, buf);
 }
 
 // Batched form of the SIMT GETT (no paper counterpart): CTA t computes tile
 // t of the flattened tile list of many problems, each with its own
-// descriptor (modes, strides, operands); the descriptor of the tile's
-// problem is copied to shared memory first.  A problem's tiles compute
-// exactly as tile_kernel computes them, whatever else is in the batch.
-template <typename T, int BM, int BN, int BK, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
+// descriptor (modes, strides, operands, tile shape); the descriptor of the
+// tile's problem is copied to shared memory first.  A problem's tiles
+// compute exactly as tile_kernel computes them, whatever else is in the
+// batch.
+template <typename T>
+__global__ void __launch_bounds__(256, 2)
 tile_batch_kernel(const TileDesc *__restrict__ descs, const int32_t *__restrict__ tile_prob) {
     __shared__ __align__(16) TileDesc sd;
+    __shared__ __align__(16) unsigned char buf[sizeof(typename TileOf<T, 0>::Smem)];
     static_assert(sizeof(TileDesc) % 8 == 0, "descriptor in 8-byte words");
     constexpr int kWords = sizeof(TileDesc) / 8;
     const int q = tile_prob[blockIdx.x];
     for (int w = threadIdx.x; w < kWords; w += blockDim.x)
         ((int64_t *)&sd)[w] = ((const int64_t *)(descs + q))[w];
     __syncthreads();
-    tile_body<T, BM, BN, BK, TM, TN>(sd, (int64_t)blockIdx.x - sd.tile0);
+    const int64_t bid = (int64_t)blockIdx.x - sd.tile0;
+    if (sd.shape == 0) TileOf<T, 0>::run(sd, bid, buf);
+    else if (sd.shape == 1) TileOf<T, 1>::run(sd, bid, buf);
+    else TileOf<T, 2>::run(sd, bid, buf);
 }
 
 // ---------------------------------------------------------------- copy
@@ -567,6 +676,22 @@ int device_sms() {
         if (sms <= 0) sms = 1;
     }
     return sms;
+}
+
+int simt_shape(bool f64, int64_t M, int64_t N, int64_t tasks) {
+    for (int s = 0; s + 1 < kSimtShapes; ++s) {
+        const int64_t b = simt_rows(f64, s);
+        if (((M + b - 1) / b) * ((N + b - 1) / b) * tasks >= (int64_t)device_sms() * (f64 ? 8 : 2)) return s;
+    }
+    return kSimtShapes - 1;
+}
+
+// one launch over the first `tiles` tiles of d's shape
+template <typename T>
+void launch_tiles(const TileDesc &d, int64_t tiles, cudaStream_t st) {
+    if (d.shape == 0) tile_kernel<T, 0><<<(unsigned)tiles, 256, 0, st>>>(d);
+    else if (d.shape == 1) tile_kernel<T, 1><<<(unsigned)tiles, 256, 0, st>>>(d);
+    else tile_kernel<T, 2><<<(unsigned)tiles, 256, 0, st>>>(d);
 }
 
 int64_t grid_for(int64_t total, int per_block) {
@@ -739,6 +864,7 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
         td.alpha = alpha;
         td.beta = beta;
         td.alpha_one = alpha_one;
+        td.shape = simt_shape(sizeof(T) == 8, td.M, td.N, ntasks);
         // map threads along whichever of M / K is contiguous in memory
         int64_t kinA = td.red.n ? td.red.sA[td.red.n - 1] : 0;
         int64_t kinB = td.red.n ? td.red.sB[td.red.n - 1] : 0;
@@ -849,19 +975,10 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
             td.B = Beff;
             td.C = Cptr;
             td.init = init;
-            if constexpr (sizeof(T) == 8) {
-                constexpr int BM = 64, BN = 64;
-                td.tiles_m = (td.M + BM - 1) / BM;
-                td.tiles_n = (td.N + BN - 1) / BN;
-                int64_t grid = cut(td.tiles_m * td.tiles_n * ntasks);
-                tile_kernel<T, 64, 64, 16, 4, 4><<<(unsigned)grid, 256, 0, st>>>(td);
-            } else {
-                constexpr int BM = 128, BN = 128;
-                td.tiles_m = (td.M + BM - 1) / BM;
-                td.tiles_n = (td.N + BN - 1) / BN;
-                int64_t grid = cut(td.tiles_m * td.tiles_n * ntasks);
-                tile_kernel<T, 128, 128, 16, 8, 8><<<(unsigned)grid, 256, 0, st>>>(td);
-            }
+            const int64_t b = simt_rows(sizeof(T) == 8, (int)td.shape);
+            td.tiles_m = (td.M + b - 1) / b;
+            td.tiles_n = (td.N + b - 1) / b;
+            launch_tiles<T>(td, cut(td.tiles_m * td.tiles_n * ntasks), st);
         } else {
             PhaseDesc q = pd;
             q.A = Aeff;
@@ -921,8 +1038,7 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
 // of A, N = free indices of B, K = contracted indices.
 // The SIMT GETT's descriptor: M = free indices of A, N = free indices of B
 // (each sorted by their C stride), K = contracted indices with the one
-// contiguous in A (or else in B) innermost; tiles of 64 x 64 (FP64) or
-// 128 x 128 (FP32).
+// contiguous in A (or else in B) innermost; the tile shape by simt_shape.
 template <typename T>
 void describe_gett_simt(const Plan &p, T alpha, const T *A, const T *B, T beta, T *C, TileDesc &td) {
     std::memset(&td, 0, sizeof(td));
@@ -965,7 +1081,10 @@ void describe_gett_simt(const Plan &p, T alpha, const T *A, const T *B, T beta, 
     int64_t kinB = td.red.n ? td.red.sB[td.red.n - 1] : 0;
     td.a_m_fast = td.m.n ? (td.m.sA[0] <= kinA || kinA == 0) : 0;
     td.b_n_fast = td.n.n ? (td.n.sB[0] <= kinB || kinB == 0) : 0;
-    const int64_t bm = sizeof(T) == 8 ? 64 : 128;
+    int64_t tasks = 1;
+    for (int id : p.batch) tasks *= p.ext[id];
+    td.shape = simt_shape(sizeof(T) == 8, td.M, td.N, tasks);
+    const int64_t bm = simt_rows(sizeof(T) == 8, (int)td.shape);
     td.tiles_m = (td.M + bm - 1) / bm;
     td.tiles_n = (td.N + bm - 1) / bm;
 }
@@ -986,10 +1105,7 @@ tc_status run_gett_simt(Plan &p, T alpha, const T *A, const T *B, T beta, T *C,
     };
     const int64_t tiles = td.tiles_m * td.tiles_n * task_count(td);
     if (tiles > 0x7fffffff) return fail(TC_ERROR_INVALID_EXTENT, "too many tiles for one launch");
-    if constexpr (sizeof(T) == 8)
-        tile_kernel<T, 64, 64, 16, 4, 4><<<(unsigned)cut(tiles), 256, 0, st>>>(td);
-    else
-        tile_kernel<T, 128, 128, 16, 8, 8><<<(unsigned)cut(tiles), 256, 0, st>>>(td);
+    launch_tiles<T>(td, cut(tiles), st);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? TC_SUCCESS
                             : fail(TC_ERROR_CUDA, std::string("GETT tile_kernel launch (") +
@@ -1018,11 +1134,9 @@ tc_status simt_launch_batch(tc_dtype dt, const void *ddescs, const int32_t *dtil
     if (ntiles > 0x7fffffff) return fail(TC_ERROR_INVALID_ARGUMENT, "batch has too many tiles");
     cudaStream_t st = (cudaStream_t)stream;
     if (dt == TC_F64)
-        tile_batch_kernel<double, 64, 64, 16, 4, 4>
-            <<<(unsigned)ntiles, 256, 0, st>>>((const TileDesc *)ddescs, dtile_prob);
+        tile_batch_kernel<double><<<(unsigned)ntiles, 256, 0, st>>>((const TileDesc *)ddescs, dtile_prob);
     else
-        tile_batch_kernel<float, 128, 128, 16, 8, 8>
-            <<<(unsigned)ntiles, 256, 0, st>>>((const TileDesc *)ddescs, dtile_prob);
+        tile_batch_kernel<float><<<(unsigned)ntiles, 256, 0, st>>>((const TileDesc *)ddescs, dtile_prob);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? TC_SUCCESS : fail(TC_ERROR_CUDA, cudaGetErrorString(e));
 }
@@ -1033,8 +1147,10 @@ int64_t nest_phase_items(const Plan &p, const Algorithm &alg, bool *tiled) {
     for (int id : L.task_ids) ntasks *= p.ext[id];
     if (alg.kernel == TC_KERNEL_GEMM) {
         *tiled = true;
-        const int64_t bm = p.dtype == TC_F64 ? 64 : 128;
-        return ((p.ext[L.out_ids[0]] + bm - 1) / bm) * ((p.ext[L.out_ids[1]] + bm - 1) / bm) * ntasks;
+        const int64_t M = p.ext[L.out_ids[0]], N = p.ext[L.out_ids[1]];
+        const bool f64 = p.dtype == TC_F64, simt = f64 || p.dtype == TC_F32;
+        const int64_t bm = simt ? simt_rows(f64, simt_shape(f64, M, N, ntasks)) : 128;
+        return ((M + bm - 1) / bm) * ((N + bm - 1) / bm) * ntasks;
     }
     *tiled = false;
     int64_t nout = 1;
@@ -1047,8 +1163,11 @@ int64_t gett_items(const Plan &p) {
     for (int id : p.freeA) M *= p.ext[id];
     for (int id : p.freeB) N *= p.ext[id];
     for (int id : p.batch) H *= p.ext[id];
-    if (p.dtype == TC_F64) return ((M + 63) / 64) * ((N + 63) / 64) * H;
-    if (p.dtype == TC_F32) return ((M + 127) / 128) * ((N + 127) / 128) * H;
+    if (p.dtype == TC_F64 || p.dtype == TC_F32) {
+        const bool f64 = p.dtype == TC_F64;
+        const int64_t b = simt_rows(f64, simt_shape(f64, M, N, H));
+        return ((M + b - 1) / b) * ((N + b - 1) / b) * H;
+    }
     const int64_t bn = p.gett_bn ? p.gett_bn : (N >= 256 ? 256 : 128);
     return ((M + 127) / 128) * ((N + bn - 1) / bn) * H;
 }
