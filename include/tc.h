@@ -252,26 +252,26 @@ tc_status tc_plan_set_gett_tma(tc_plan plan, int32_t enable);
  * when it has at most 1/8 of the larger one's elements and its images fit
  * in 64 MiB; 2: the smaller input (FP32 inputs) whenever its images fit in
  * 64 MiB; 3: both inputs whenever their images fit in 2 GiB (else none),
- * each stage's two images then reach shared memory as two 1-D bulk copies
- * and no input is staged by TMA.  Other values give
+ * the GETT then streams the images alone (in CTA pairs and tile widths of
+ * its own choice).  Other values give
  * TC_ERROR_INVALID_ARGUMENT.  The workspace is allocated by the first
  * execute that needs it (tc_algorithm_workspace(plan, 0) bounds it).  The
  * K order, and so the rounding of the sums, depends on whether an input is
  * pre-converted but not on which (modes 1-3 with a pre-converted input give
  * the same bits) nor on tc_plan_set_gett_tma.  With pre-conversion an
- * execute launches two kernels (pre-pass, GETT), three with both inputs. */
+ * execute launches two kernels (pre-pass, GETT). */
 tc_status tc_plan_set_gett_pack(tc_plan plan, int32_t mode);
 
 /* Tensor-core GETT, FP32-input kinds (TC_BF16X3, TC_TF32): CTA pairs.
  * With 1, and where the launch allows it (256-column tiles, no
  * compensated accumulation, more than 128 rows of M, every input staged by
- * TMA or pre-converted; or, for TC_BF16X3 with both inputs pre-converted
- * (tc_plan_set_gett_pack), any layout with more than 128 rows of M, on
- * 256-column tiles or compensated 128-column ones), clusters of two CTAs
+ * TMA or the smaller one pre-converted), clusters of two CTAs
  * share each MMA (tcgen05.mma.cta_group::2, M = 256): each CTA stages and
  * converts (or copies) its 128 rows of A and half of the tile's rows of B,
  * so a CTA moves half the B bytes per MMA; 0 (default) keeps one CTA per
- * tile.  Results are the same bits either way.  Other values give
+ * tile.  With both inputs pre-converted (tc_plan_set_gett_pack), any dtype,
+ * 0 leaves the choice to the size and 1 asks for pairs wherever M has more
+ * than 128 rows.  Results are the same bits either way.  Other values give
  * TC_ERROR_INVALID_ARGUMENT. */
 tc_status tc_plan_set_gett_pair(tc_plan plan, int32_t enable);
 

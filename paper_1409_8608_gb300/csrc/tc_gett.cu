@@ -50,23 +50,14 @@
 #include <type_traits>
 #include <vector>
 
+#include "tc_gett.cuh"
 #include "tc_internal.h"
-#include "tc_tcgen05.cuh"
 
 namespace tc {
 
 namespace {
 
 using namespace dev;
-
-enum GettKind { GK_BF16X3 = 0, GK_BF16 = 1, GK_F16 = 2, GK_TF32 = 3, GK_TF32X3 = 4, GK_E4M3 = 5 };
-
-// MMA on TF32 words (kind::tf32, 4-byte operand elements)
-__host__ __device__ constexpr bool tf32_kind(int k) { return k == GK_TF32 || k == GK_TF32X3; }
-// FP32 inputs, converted (or split) by the converter warps
-__host__ __device__ constexpr bool float_input(int k) {
-    return k == GK_BF16X3 || k == GK_TF32 || k == GK_TF32X3 || k == GK_E4M3;
-}
 
 constexpr int kBM = 128;                  // accumulator rows = TMEM lanes
 constexpr int kBK = 32;                   // K elements per stage, global-load path
@@ -88,18 +79,8 @@ constexpr int kTmaWarp = kMmaWarp + 1;                // warp 13
 constexpr int kThreads = (kTmaWarp + 1) * 32;
 constexpr int kTmaRank = 5;
 
-struct GettDesc {
-    int nm, nn, nk;                       // number of M / N / K modes
-    int64_t m_ext[kMaxModes], m_sA[kMaxModes], m_sC[kMaxModes];
-    int64_t n_ext[kMaxModes], n_sB[kMaxModes], n_sC[kMaxModes];
-    int n_chain;                          // C offset of column n is n * n_sC[0]
-    int64_t k_ext[kMaxModes], k_sA[kMaxModes], k_sB[kMaxModes];  // outermost first
-    int64_t M, N, K;
+struct GettDesc : GettModes {
     int64_t tiles_m, tiles_n;
-    // batch (Hadamard) indices, in A, B and C: the tile list runs over
-    // batch values outermost, then N tiles, then M tiles (batch_offsets)
-    int nb;
-    int64_t b_ext[kMaxModes], b_sA[kMaxModes], b_sB[kMaxModes], b_sC[kMaxModes];
     const void *A;
     const void *B;
     float *C;
@@ -135,194 +116,19 @@ struct GettDesc {
     int64_t tile0;
     int64_t tile_begin;  // first tile of this launch (batched form; else 0)
     int one_stage;       // batched form: every problem's K fits one stage
-    // pre-converted input (0 none, 1 A, 2 B, 3 both): its stage images,
-    // laid out [row tile][K stage][slice][core-matrix image] as the
-    // converters would write them to shared memory (3: A's at pk_base, B's
-    // at pkb_base)
+    // pre-converted input (0 none, 1 A, 2 B): its stage images, laid out
+    // [row tile][K stage][slice][core-matrix image] as the converters would
+    // write them to shared memory
     int pk;
     const char *pk_base;
     int64_t pk_tile_bytes;  // one row tile's images (every K stage)
-    const char *pkb_base;
-    int64_t pkb_tile_bytes;
 };
 
 // number of batch values of a descriptor (1 without batch indices)
-inline int64_t batch_count(const GettDesc &d) {
+inline int64_t batch_count(const GettModes &d) {
     int64_t h = 1;
     for (int m = 0; m < d.nb; ++m) h *= d.b_ext[m];
     return h;
-}
-
-// Named barrier over one warp role that also ORs a predicate across it.
-template <int ID, int COUNT>
-__device__ __forceinline__ bool role_sync_or(bool pred) {
-    uint32_t out;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "barrier.cta.red.or.pred q, %2, %3, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(out)
-        : "r"((uint32_t)pred), "n"(ID), "n"(COUNT)
-        : "memory");
-    return out != 0;
-}
-
-// ---- CTA pairs (cta_group::2): two CTAs of a cluster of two share each MMA.
-// The pair's MMA is M = 256: each CTA holds 128 rows of A and half of the
-// B tile in its own shared memory (at the same offsets), and each CTA's
-// tensor memory receives its 128 rows of the accumulator.  One thread of
-// the even CTA issues the MMAs; its commits arrive on both CTAs' barriers.
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-// Every thread of both CTAs: release this CTA's prior writes, acquire the
-// peer's.
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// The shared::cluster address of the same shared-memory offset in CTA `rank`.
-__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-
-// Arrival on an mbarrier of another CTA of the cluster (release at cluster
-// scope: this thread's prior shared-memory writes are visible to a thread
-// that acquires the barrier's phase).
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait_cl(uint64_t *bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
-// Bounded wait that acquires at cluster scope (barriers other CTAs of the
-// pair arrive on); false when the limit expired.
-__device__ __forceinline__ bool mbar_wait_cl(uint64_t *bar, uint32_t parity) {
-    if (mbar_try_wait_cl(bar, parity)) return true;
-    const uint64_t t0 = globaltimer();
-    while (!mbar_try_wait_cl(bar, parity)) {
-        if (globaltimer() - t0 > kWaitLimitNs) return false;
-    }
-    return true;
-}
-
-// One warp of each CTA of the pair allocates collectively; the address is
-// the same in both CTAs.
-__device__ __forceinline__ void tmem_alloc2(uint32_t *dst_smem, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
-                 "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tmem_dealloc2(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-
-// Commit of the pair's MMAs issued so far by this thread: arrives once on
-// the barrier at this shared-memory offset in every CTA of `mask`.
-__device__ __forceinline__ void mma_commit2(uint64_t *bar, uint16_t mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            smem_u32(bar)),
-        "h"(mask)
-        : "memory");
-}
-
-template <int KIND, bool PAIR = false>
-__device__ __forceinline__ void mma_issue(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
-    if constexpr (PAIR && tf32_kind(KIND)) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
-    } else if constexpr (PAIR) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
-    } else if constexpr (tf32_kind(KIND)) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
-    } else if constexpr (KIND == GK_E4M3) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
-    } else {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "setp.ne.u32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
-    }
-}
-
-// 64 consecutive columns of this warp's 32 lanes with one wait: the load
-// latency is paid once per 64 columns instead of once per 32.
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, uint32_t (&r)[64]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x64.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%64];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
-        : "r"(taddr)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// Two 32-column loads (the split accumulators) and their FP32 sum: both
-// loads and the wait in one statement, so no use of the registers can be
-// scheduled before the wait.
-__device__ __forceinline__ void tmem_ld32_sum(uint32_t ta, uint32_t tb, uint32_t (&r)[32]) {
-    uint32_t a[32], b[32];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%64];\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,"
-        "%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%65];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]),
-          "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15]),
-          "=r"(a[16]), "=r"(a[17]), "=r"(a[18]), "=r"(a[19]), "=r"(a[20]), "=r"(a[21]), "=r"(a[22]), "=r"(a[23]),
-          "=r"(a[24]), "=r"(a[25]), "=r"(a[26]), "=r"(a[27]), "=r"(a[28]), "=r"(a[29]), "=r"(a[30]), "=r"(a[31]),
-          "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7]),
-          "=r"(b[8]), "=r"(b[9]), "=r"(b[10]), "=r"(b[11]), "=r"(b[12]), "=r"(b[13]), "=r"(b[14]), "=r"(b[15]),
-          "=r"(b[16]), "=r"(b[17]), "=r"(b[18]), "=r"(b[19]), "=r"(b[20]), "=r"(b[21]), "=r"(b[22]), "=r"(b[23]),
-          "=r"(b[24]), "=r"(b[25]), "=r"(b[26]), "=r"(b[27]), "=r"(b[28]), "=r"(b[29]), "=r"(b[30]), "=r"(b[31])
-        : "r"(ta), "r"(tb)
-        : "memory");
-#pragma unroll
-    for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(__fadd_rn(__uint_as_float(a[j]), __uint_as_float(b[j])));
 }
 
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
@@ -347,30 +153,7 @@ __device__ __forceinline__ void tmem_st32_zero(uint32_t taddr) {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ uint32_t f32_to_tf32(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return r;
-}
-
-
 // ------------------------------------------------------------------ layout
-template <int KIND, int BK>
-struct KindTraits {
-    static constexpr int kElemBytes = tf32_kind(KIND) ? 4 : (KIND == GK_E4M3 ? 1 : 2);  // smem operand element
-    static constexpr int kSlices = KIND == GK_BF16X3 ? 3 : (KIND == GK_TF32X3 ? 2 : 1);
-    static constexpr int kChunk = 16 / kElemBytes;              // K elements per 16-byte row
-    static constexpr int kKc = BK / kChunk;                     // core matrices along K per stage
-    static constexpr int kKsteps = BK * kElemBytes / 32;        // MMA instructions along K per stage
-    // instruction-descriptor operand format: kind::tf32 TF32 = 2; kind::f16
-    // F16 = 0, BF16 = 1; kind::f8f6f4 E4M3 = 0
-    static constexpr uint32_t kFmt = tf32_kind(KIND) ? 2u : ((KIND == GK_F16 || KIND == GK_E4M3) ? 0u : 1u);
-    using In = typename std::conditional<KIND == GK_BF16, __nv_bfloat16,
-                                         typename std::conditional<KIND == GK_F16, __half, float>::type>::type;
-    static constexpr int kInBytes = sizeof(In);
-    static constexpr int kVec = 16 / kInBytes;                  // input elements per 16-byte load
-};
-
 // STAGES: depth of the operand ring (converted tiles the MMA reads);
 // SSTG: depth of the TMA staging ring (0 = no TMA staging).  The staging
 // ring is the deeper one: it covers the load latency.
@@ -402,76 +185,6 @@ struct SmemPlan {
     static constexpr int kBars = (2 * STAGES + 4 * kSstg + 5) * 8 + 16;
     static constexpr int kTotal = kOpBytes + kStgBytes + kKTab + kRowTab + kColTab + kRecs * 64 + kRecs * 16 + kBars;
 };
-
-// x = q * y + r for non-negative x, y > 0: 32-bit division when both fit
-// (a 64-bit division is a long dependent instruction sequence, and these
-// sit on the per-tile critical path of every role)
-__device__ __forceinline__ int64_t divmod(int64_t x, int64_t y, int64_t &r) {
-    if (((x | y) >> 31) == 0) {
-        const uint32_t q = (uint32_t)x / (uint32_t)y;
-        r = x - (int64_t)q * y;
-        return q;
-    }
-    const int64_t q = x / y;
-    r = x - q * y;
-    return q;
-}
-
-__device__ __forceinline__ void decode(int64_t x, int n, const int64_t *ext, const int64_t *s1,
-                                       const int64_t *s2, int64_t &o1, int64_t &o2) {
-    // first mode fastest
-    for (int m = 0; m < n; ++m) {
-        int64_t v;
-        x = divmod(x, ext[m], v);
-        o1 += v * s1[m];
-        o2 += v * s2[m];
-    }
-}
-
-// Converts N (4 or 8) FP32 values into the 16-bit slices or TF32 words
-// and stores them at dst (one slice after another, slice_stride apart).
-// qs: E4M3 only, the operand's inverse scale (a power of two).
-template <int KIND, int N>
-__device__ __forceinline__ void store_converted(const float (&x)[N], char *dst, int slice_stride, float qs = 1.0f) {
-    if constexpr (KIND == GK_BF16X3) {
-        uint32_t w0[N / 2], w1[N / 2], w2[N / 2];
-#pragma unroll
-        for (int e = 0; e < N; e += 2) split3x2(x[e], x[e + 1], w0[e / 2], w1[e / 2], w2[e / 2]);
-        if constexpr (N == 8) {
-            *(uint4 *)(dst) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
-            *(uint4 *)(dst + slice_stride) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
-            *(uint4 *)(dst + 2 * slice_stride) = make_uint4(w2[0], w2[1], w2[2], w2[3]);
-        } else {
-            *(uint2 *)(dst) = make_uint2(w0[0], w0[1]);
-            *(uint2 *)(dst + slice_stride) = make_uint2(w1[0], w1[1]);
-            *(uint2 *)(dst + 2 * slice_stride) = make_uint2(w2[0], w2[1]);
-        }
-    } else if constexpr (KIND == GK_TF32X3) {  // N == 4: x = hi + lo (+ at most 2^-22 |x|)
-        uint32_t h[4], l[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            h[e] = f32_to_tf32(x[e]);
-            l[e] = f32_to_tf32(x[e] - __uint_as_float(h[e]));  // the difference is exact
-        }
-        *(uint4 *)(dst) = make_uint4(h[0], h[1], h[2], h[3]);
-        *(uint4 *)(dst + slice_stride) = make_uint4(l[0], l[1], l[2], l[3]);
-    } else if constexpr (KIND == GK_E4M3) {  // N == 4 or 16: x * qs rounded to E4M3, saturating
-        (void)slice_stride;
-        uint32_t w[N / 4];
-#pragma unroll
-        for (int e = 0; e < N; e += 4) {
-            const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(x[e] * qs, x[e + 1] * qs), __NV_SATFINITE, __NV_E4M3);
-            const uint32_t hi =
-                __nv_cvt_float2_to_fp8x2(make_float2(x[e + 2] * qs, x[e + 3] * qs), __NV_SATFINITE, __NV_E4M3);
-            w[e / 4] = lo | (hi << 16);
-        }
-        if constexpr (N == 16) *(uint4 *)(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-        else *(uint32_t *)(dst) = w[0];
-    } else {  // TF32: N == 4
-        *(uint4 *)(dst) = make_uint4(f32_to_tf32(x[0]), f32_to_tf32(x[1]), f32_to_tf32(x[2]),
-                                     f32_to_tf32(x[3]));
-    }
-}
 
 // Global-load path: one operand's share of a stage (ROWS rows x BK K
 // elements), loads first (all in flight), then conversion and stores.
@@ -695,8 +408,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB) {
     using T = KindTraits<KIND, BK>;
     using SP = SmemPlan<KIND, BN, STAGES, BK, SSTG, BATCH, PAIR>;
-    // (pairs with the compensated form: both inputs pre-converted only)
-    static_assert(!(PAIR && BATCH), "CTA pairs: not in the batched form");
+    static_assert(!(PAIR && (BATCH || COMP)), "CTA pairs: not in the batched or the compensated form");
     constexpr bool TMA = SP::TMA;
     constexpr int SS = SP::kSstg;
     constexpr int BNL = SP::kBNL;  // B rows this CTA stages and converts
@@ -776,9 +488,8 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
         // or the four of one group when the groups take turns
         const uint32_t conv_warps = grouped ? kProducerThreads / 32 / kConvGroups : kProducerThreads / 32;
         for (int s = 0; s < STAGES; ++s) {
-            // pairs: both CTAs' converters arrive on rank 0's barrier; with
-            // both inputs pre-converted the copying lane arms it alone
-            mbar_init(&full[s], d.pk == 3 ? (PAIR && crank == 0 ? 2u : 1u) : conv_warps * (PAIR ? 2 : 1));
+            // pairs: both CTAs' converters arrive on rank 0's barrier
+            mbar_init(&full[s], conv_warps * (PAIR ? 2 : 1));
             mbar_init(&empty[s], 1);
         }
         // a staging slot is free again once every stage of its box is converted
@@ -975,7 +686,7 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
                 }
             }
         }
-        for (int64_t tile = d.tile_begin + blockIdx.x; tile < d.num_tiles && !stop && !grouped && !PAIR && d.pk != 3;
+        for (int64_t tile = d.tile_begin + blockIdx.x; tile < d.num_tiles && !stop && !grouped && !PAIR;
              tile += gridDim.x, ++it) {
             const GettDesc &P = tile_desc<BATCH>(d, tile);
             int64_t boA, boB, boC;
@@ -1093,47 +804,7 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
         }
     } else if (warp == kTmaWarp) {
         // ---------------------------------------------------------- TMA issue
-        if (!BATCH && d.pk == 3) {
-            // both inputs pre-converted: one lane copies each stage's two
-            // images (contiguous runs of the workspace) straight into the
-            // operand ring with 1-D bulk copies; the converters stay idle.
-            // Pairs: each CTA copies its 128 rows of A and its half of the
-            // tile's B rows into its own ring (images of 128-row and
-            // BN/2-row tiles, two per pair tile)
-            if (lane == 0) {
-                asm volatile("griddepcontrol.wait;" ::: "memory");  // the pre-pass grids are complete
-                constexpr uint32_t kImgA = (uint32_t)(T::kSlices * SP::kATile);
-                constexpr uint32_t kImgB = (uint32_t)(T::kSlices * SP::kBTile);
-                int64_t g = 0;
-                bool stop = false;
-                for (int64_t tile = d.tile_begin + slot0; tile < d.num_tiles && !stop; tile += nslots) {
-                    int64_t mt;
-                    const int64_t nt = divmod(tile, d.tiles_m, mt);
-                    const char *ia = d.pk_base + (PAIR ? 2 * mt + crank : mt) * d.pk_tile_bytes;
-                    const char *ib = d.pkb_base + (PAIR ? 2 * nt + crank : nt) * d.pkb_tile_bytes;
-                    for (int kt = 0; kt < nkt; ++kt, ++g) {
-                        const int s = (int)(g % STAGES);
-                        if (*abort_flag ||
-                            (g >= STAGES && !mbar_wait(&empty[s], (uint32_t)(((g / STAGES) - 1) & 1)))) {
-                            stop = true;
-                            break;
-                        }
-                        char *stage = ops + s * SP::kStage;
-                        mbar_arrive_expect_tx(&full[s], kImgA + kImgB);
-                        bulk_load(stage, ia + kt * (int64_t)kImgA, kImgA, &full[s]);
-                        bulk_load(stage + kImgA, ib + kt * (int64_t)kImgB, kImgB, &full[s]);
-                    }
-                }
-                if (stop) {
-                    *abort_flag = 1;
-                    atomicExch(d.status, (int)TC_ERROR_TIMEOUT);
-                    // the copies still in flight land before the CTA may
-                    // exit: each slot's last issue completes its phase
-                    for (int64_t q = g > STAGES ? g - STAGES : 0; q < g; ++q)
-                        mbar_wait(&full[q % STAGES], (uint32_t)((q / STAGES) & 1));
-                }
-            }
-        } else if (TMA && any_tma && lane == 0) {
+        if (TMA && any_tma && lane == 0) {
             int64_t g = 0;
             bool stop = false;
             // box coordinates of a tile's rows, and of one of its K stages
@@ -1297,26 +968,6 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
             if constexpr (PAIR) mma_commit2(drain, (uint16_t)1);
             else mma_commit(drain);
             mbar_wait(drain, 0);
-        } else if (PAIR && !BATCH && d.pk == 3 && lane == 0) {
-            // both inputs pre-converted, second CTA of a pair: its copies
-            // complete on its own stage barriers; this lane passes each
-            // completed stage on to the issuer's barrier in the first CTA
-            int64_t g = 0;
-            bool stop = false;
-            for (int64_t tile = d.tile_begin + slot0; tile < d.num_tiles && !stop; tile += nslots) {
-                for (int kt = 0; kt < nkt; ++kt, ++g) {
-                    const int s = (int)(g % STAGES);
-                    if (*abort_flag || !mbar_wait(&full[s], (uint32_t)((g / STAGES) & 1))) {
-                        stop = true;
-                        break;
-                    }
-                    mbar_arrive_remote(mapa_shared(smem_u32(&full[s]), 0u));
-                }
-            }
-            if (stop) {
-                *abort_flag = 1;
-                atomicExch(d.status, (int)TC_ERROR_TIMEOUT);
-            }
         }
         __syncwarp();
     } else {
@@ -1521,10 +1172,6 @@ __global__ void __launch_bounds__(128) pack_kernel(const GettDesc d, int op, int
     // and aligned
     const bool whole = d.nk > 0 && d.k_ext[d.nk - 1] % CH == 0;
     const int64_t s_in = d.nk > 0 ? ks[d.nk - 1] : 0;
-    // E4M3: the input divided by its scale (a power of two, written by the
-    // scale kernel earlier in the stream)
-    float qs = 1.0f;
-    if constexpr (KIND == GK_E4M3) qs = 1.0f / d.qscale[op];
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < total; c += (int64_t)gridDim.x * blockDim.x) {
         // rows fastest, then K chunks, K stages, row tiles (divmod: 32-bit
         // divisions whenever the values fit)
@@ -1584,86 +1231,7 @@ __global__ void __launch_bounds__(128) pack_kernel(const GettDesc d, int op, int
         }
         char *dst = out + (rt * nkt + kt) * (int64_t)(T::kSlices * slice) + (kc * (rows / 8) + row / 8) * 128 +
                     (row % 8) * 16;
-        store_converted<KIND, CH>(x, dst, slice, qs);
-    }
-}
-
-// Pre-conversion of one 16-bit input (BF16 / FP16; op 0 = A, 1 = B) for the
-// both-inputs path: its stage images in the core-matrix layout, the values
-// as they are, zeros for rows past the extent and K positions past K.  One
-// thread per 16-byte core-matrix row (8 K positions of one row).
-__global__ void __launch_bounds__(128) pack16_kernel(const GettDesc d, int op, int rows, int bk, int64_t rtiles,
-                                                     char *out) {
-    constexpr int CH = 8;
-    const int kcn = bk / CH;
-    const int64_t nkt = (d.K + bk - 1) / bk;
-    const int64_t R = op == 0 ? d.M : d.N;
-    const int64_t total = rtiles * nkt * kcn * rows;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const uint16_t *__restrict__ src = (const uint16_t *)(op == 0 ? d.A : d.B);
-    const int nr = op == 0 ? d.nm : d.nn;
-    const int64_t *rext = op == 0 ? d.m_ext : d.n_ext;
-    const int64_t *rs = op == 0 ? d.m_sA : d.n_sB;
-    const int64_t *ks = op == 0 ? d.k_sA : d.k_sB;
-    const int64_t slice = (int64_t)rows * bk * 2;
-    const bool whole = d.nk > 0 && d.k_ext[d.nk - 1] % CH == 0;  // a chunk is one run of the innermost K mode
-    const int64_t s_in = d.nk > 0 ? ks[d.nk - 1] : 0;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < total; c += (int64_t)gridDim.x * blockDim.x) {
-        int64_t row, kc, kt;
-        int64_t q = divmod(c, rows, row);
-        q = divmod(q, kcn, kc);
-        const int64_t rt = divmod(q, nkt, kt);
-        int64_t r = rt * rows + row, ro = -1;
-        if (r < R) {
-            ro = 0;
-            for (int m = 0; m < nr; ++m) {
-                int64_t v;
-                r = divmod(r, rext[m], v);
-                ro += v * rs[m];
-            }
-        }
-        uint16_t x[CH];
-#pragma unroll
-        for (int e = 0; e < CH; ++e) x[e] = 0;
-        uint4 w = make_uint4(0u, 0u, 0u, 0u);
-        bool vec = false;
-        if (ro >= 0 && whole) {
-            int64_t k = kt * bk + kc * CH, ko = 0;
-            if (k < d.K) {
-                for (int m = d.nk - 1; m >= 0; --m) {
-                    int64_t v;
-                    k = divmod(k, d.k_ext[m], v);
-                    ko += v * ks[m];
-                }
-                const uint16_t *p = src + ro + ko;
-                if (s_in == 1 && ((uintptr_t)p & 15) == 0) {
-                    w = *reinterpret_cast<const uint4 *>(p);
-                    vec = true;
-                } else {
-#pragma unroll
-                    for (int e = 0; e < CH; ++e) x[e] = p[e * s_in];
-                }
-            }
-        } else if (ro >= 0) {
-#pragma unroll
-            for (int e = 0; e < CH; ++e) {
-                int64_t k = kt * bk + kc * CH + e;
-                if (k < d.K) {
-                    int64_t ko = 0;
-                    for (int m = d.nk - 1; m >= 0; --m) {  // innermost K mode fastest
-                        int64_t v;
-                        k = divmod(k, d.k_ext[m], v);
-                        ko += v * ks[m];
-                    }
-                    x[e] = src[ro + ko];
-                }
-            }
-        }
-        if (!vec)
-            w = make_uint4(x[0] | ((uint32_t)x[1] << 16), x[2] | ((uint32_t)x[3] << 16), x[4] | ((uint32_t)x[5] << 16),
-                           x[6] | ((uint32_t)x[7] << 16));
-        char *dst = out + (rt * nkt + kt) * slice + (kc * (rows / 8) + row / 8) * 128 + (row % 8) * 16;
-        *(uint4 *)dst = w;
+        store_converted<KIND, CH>(x, dst, slice);
     }
 }
 
@@ -1777,18 +1345,6 @@ tc_status launch_kind(GettDesc &d, int bn, bool tma, bool comp, bool pair, const
     d.tiles_n = (d.N + bn - 1) / bn;
     d.num_tiles = d.tiles_m * d.tiles_n * batch_count(d);
     if (d.tile_frac < 1.0) d.num_tiles = std::max<int64_t>(1, (int64_t)(d.num_tiles * d.tile_frac));
-    // CTA pairs with both inputs pre-converted (pair tiles of 256 x BN;
-    // per CTA 128 rows of A and BN/2 of B in each 32-position stage):
-    // split-BF16 256 x 256 (four stages) or compensated 256 x 128, whose
-    // two chunk accumulators and (hi, lo) take each CTA's 512 tensor-memory
-    // columns
-    if (pair && d.pk == 3) {
-        if constexpr (KIND == GK_BF16X3) {
-            if (comp) return launch_gett<KIND, 128, 5, kBK, 0, true, false, true>(d, ta, tb, st);
-            if (bn == 256) return launch_gett<KIND, 256, 4, kBK, 0, false, false, true>(d, ta, tb, st);
-        }
-        return fail(TC_ERROR_UNSUPPORTED_DTYPE, "no CTA-pair launch for this pre-converted form");
-    }
     // CTA pairs (tiles of 256 x 256): four operand stages of 128 + 128
     // rows and three staging slots of two-stage boxes
     if constexpr (KIND == GK_BF16X3 || KIND == GK_TF32) {
@@ -2040,14 +1596,12 @@ int pack_choice(const Plan &p, int64_t &bound) {
     // both inputs: on request (3), and by default for the compensated form
     // (whose 128-column tiles would otherwise convert each input once per
     // tile of the other) and wherever both M and N reach kPackBothMinMN (each
-    // input would be converted or re-laid out at least four times); A's
-    // rows round up to a 128-row tile, B's to a 256-row one, K to a
-    // 32-position stage, plus the alignment of B's images
+    // input would be converted or re-laid out at least four times)
     int64_t comp_k = 0;
     if (p.dtype == TC_BF16X3 || p.dtype == TC_TF32X3) comp_k = p.comp_chunk < 0 ? kCompChunkK : p.comp_chunk;
     const bool comp = comp_k > 0 && K > comp_k;
     if (p.gett_pack == 3 || (p.gett_pack == 1 && (comp || (M >= kPackBothMinMN && N >= kPackBothMinMN)))) {
-        const int64_t b2 = (M + N + 512) * (K + kBK - 1) * image_bytes(p.dtype) + 256;
+        const int64_t b2 = packed_bytes(p.dtype, M, N, K);
         if (b2 <= kPackBothMaxBytes) {
             bound = b2;
             return 3;
@@ -2086,7 +1640,7 @@ void gett_release(Plan &) {}
 // The GETT's modes: M = free indices of A and N = free indices of B, each
 // sorted by their C stride; the K order as below.  pk: the pre-converted
 // input (0 none, 1 A, 2 B).
-tc_status describe_modes(const Plan &p, int pk, GettDesc &d) {
+tc_status describe_modes(const Plan &p, int pk, GettModes &d) {
     auto by_c_stride = [&](std::vector<int> ids) {
         std::stable_sort(ids.begin(), ids.end(), [&](int x, int y) {
             return p.op[OP_C].stride_of(x) < p.op[OP_C].stride_of(y);
@@ -2188,6 +1742,44 @@ tc_status describe_modes(const Plan &p, int pk, GettDesc &d) {
 }
 
 
+// E4M3: the inputs' power-of-two scales into the plan's buffer, enqueued
+// before the kernels that read them (stream order).
+static tc_status e4m3_scales(Plan &p, const void *A, const void *B, cudaStream_t st, const float **out) {
+    if (!p.qbuf) {
+        cudaError_t e = cudaMalloc(&p.qbuf, 16);
+        if (e != cudaSuccess) {
+            p.qbuf = nullptr;
+            return fail(TC_ERROR_OUT_OF_MEMORY, cudaGetErrorString(e));
+        }
+    }
+    unsigned *mx = (unsigned *)p.qbuf;
+    float *scale = (float *)((char *)p.qbuf + 8);
+    cudaMemsetAsync(mx, 0, 8, st);
+    for (int o = 0; o < 2; ++o) {
+        const Layout &L = p.op[o == 0 ? OP_A : OP_B];
+        AbsmaxDesc a;
+        std::memset(&a, 0, sizeof(a));
+        int64_t total = 1, span = 1;
+        for (int m = 0; m < L.n; ++m) {
+            a.ext[m] = p.ext[L.idx[m]];
+            a.stride[m] = L.stride[m];
+            total *= a.ext[m];
+            span += (a.ext[m] - 1) * a.stride[m];
+        }
+        a.n = span == total ? 0 : L.n;
+        a.total = total;
+        a.src = (const float *)(o == 0 ? A : B);
+        a.out = mx + o;
+        const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 152 * 8));
+        absmax_kernel<<<(unsigned)grid, 256, 0, st>>>(a);
+    }
+    e4m3_scale_kernel<<<1, 32, 0, st>>>(mx, scale);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
+    *out = scale;
+    return TC_SUCCESS;
+}
+
 tc_status exec_gett(Plan &p, const void *alpha, const void *A, const void *B, const void *beta,
                     void *C, void *stream, const Probe *probe) {
     if (p.dtype == TC_F64 || p.dtype == TC_F32) return exec_gett_simt(p, alpha, A, B, beta, C, stream, probe);
@@ -2211,6 +1803,20 @@ tc_status exec_gett(Plan &p, const void *alpha, const void *A, const void *B, co
     if (p.dtype == TC_BF16X3 || p.dtype == TC_TF32X3) comp_k = p.comp_chunk < 0 ? kCompChunkK : p.comp_chunk;
     const bool comp = comp_k > 0 && d.K > comp_k;
     if (comp) bn = 128;
+    // split accumulators: split-BF16 without the compensated form; by
+    // default only past 64 contracted positions (6K/16 > 24 accumulations
+    // into one FP32 accumulator), where the roundings of the single
+    // accumulator reach the 1e-6 level
+    constexpr int64_t kSplitMinK = 65;
+    const bool want_split = p.gett_split > 0 || (p.gett_split < 0 && d.K >= kSplitMinK);
+    d.split = ((p.dtype == TC_BF16X3 || p.dtype == TC_TF32X3) && !comp && want_split) ? 1 : 0;
+    cudaStream_t st = (cudaStream_t)stream;
+    if (p.dtype == TC_E4M3) {
+        s = e4m3_scales(p, A, B, st, &d.qscale);
+        if (s != TC_SUCCESS) return s;
+    }
+    if (pk == 3)
+        return exec_packed(p, alpha, A, B, beta, C, stream, probe ? probe->fraction : 1.0, comp_k, d.split != 0, d.qscale);
     // TMA staging for each operand TMA can describe (tiles of 128 x bn, or
     // in a CTA pair 128 rows of A and bn / 2 rows of B per CTA)
     CUtensorMap tmA, tmB;
@@ -2257,8 +1863,7 @@ tc_status exec_gett(Plan &p, const void *alpha, const void *A, const void *B, co
     // batch indices: the global-load path (the TMA warp and the
     // pre-converted images walk M and N tiles only)
     // (E4M3: the global-load path only)
-    // (both inputs pre-converted: no input is staged)
-    if (p.gett_tma && pk != 3 && p.dtype != TC_E4M3 && d.nb == 0 && d.K < (int64_t(1) << 31)) {  // 32-bit K positions in the TMA warp
+    if (p.gett_tma && p.dtype != TC_E4M3 && d.nb == 0 && d.K < (int64_t(1) << 31)) {  // 32-bit K positions in the TMA warp
         if (p.gett_pair && (p.dtype == TC_BF16X3 || p.dtype == TC_TF32) && !comp && bn == 256 && d.M > kBM) {
             GettDesc dp = d;
             CUtensorMap pa, pb;
@@ -2274,11 +1879,6 @@ tc_status exec_gett(Plan &p, const void *alpha, const void *A, const void *B, co
         }
         if (!pair) tma = plan_tma(d, tmA, tmB, bn);
     }
-    // CTA pairs with both inputs pre-converted: no staging, so every
-    // layout qualifies (more than one 128-row tile; split-BF16 on 256-wide
-    // tiles or compensated)
-    if (pk == 3 && p.gett_pair && d.M > kBM && d.nb == 0 && p.dtype == TC_BF16X3 && (comp || bn == 256))
-        pair = true;
     if (comp) d.chunk_stages = (int)(comp_k / (tma ? kBKT : kBK));
     // global-load mappings (used by operands without TMA staging)
     auto pick = [&](const void *base, int rows, int nrow, const int64_t *rext, const int64_t *rs,
@@ -2300,88 +1900,7 @@ tc_status exec_gett(Plan &p, const void *alpha, const void *A, const void *B, co
     d.status = p.dev_status;
     d.tiles_m = pair ? (d.M + 2 * kBM - 1) / (2 * kBM) : (d.M + kBM - 1) / kBM;
     d.tile_frac = probe ? probe->fraction : 1.0;
-    // split accumulators: split-BF16 without the compensated form; by
-    // default only past 64 contracted positions (6K/16 > 24 accumulations
-    // into one FP32 accumulator), where the roundings of the single
-    // accumulator reach the 1e-6 level
-    constexpr int64_t kSplitMinK = 65;
-    const bool want_split = p.gett_split > 0 || (p.gett_split < 0 && d.K >= kSplitMinK);
-    d.split = ((p.dtype == TC_BF16X3 || p.dtype == TC_TF32X3) && !comp && want_split) ? 1 : 0;
-    cudaStream_t st = (cudaStream_t)stream;
-    if (p.dtype == TC_E4M3) {
-        // the inputs' scales, written before the pre-passes and the GETT read
-        // them (stream order)
-        if (!p.qbuf) {
-            cudaError_t e = cudaMalloc(&p.qbuf, 16);
-            if (e != cudaSuccess) {
-                p.qbuf = nullptr;
-                return fail(TC_ERROR_OUT_OF_MEMORY, cudaGetErrorString(e));
-            }
-        }
-        unsigned *mx = (unsigned *)p.qbuf;
-        float *scale = (float *)((char *)p.qbuf + 8);
-        cudaMemsetAsync(mx, 0, 8, st);
-        for (int o = 0; o < 2; ++o) {
-            const Layout &L = p.op[o == 0 ? OP_A : OP_B];
-            AbsmaxDesc a;
-            std::memset(&a, 0, sizeof(a));
-            int64_t total = 1, span = 1;
-            for (int m = 0; m < L.n; ++m) {
-                a.ext[m] = p.ext[L.idx[m]];
-                a.stride[m] = L.stride[m];
-                total *= a.ext[m];
-                span += (a.ext[m] - 1) * a.stride[m];
-            }
-            a.n = span == total ? 0 : L.n;
-            a.total = total;
-            a.src = (const float *)(o == 0 ? A : B);
-            a.out = mx + o;
-            const int64_t grid = std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 152 * 8));
-            absmax_kernel<<<(unsigned)grid, 256, 0, st>>>(a);
-        }
-        e4m3_scale_kernel<<<1, 32, 0, st>>>(mx, scale);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
-        d.qscale = scale;
-    }
-    if (pk == 3) {
-        // both inputs' stage images (128-row tiles of A, bn-row tiles of B,
-        // 32-position K stages), A's first, then B's on a 256-byte boundary;
-        // the GETT copies each stage's two images with 1-D bulk copies.
-        // Pairs: B in bn/2-row tiles, both inputs in an even number of row
-        // tiles (two per pair tile; rows past the extent are zeros)
-        const int64_t nktp = (d.K + kBK - 1) / kBK;
-        const int brows = pair ? bn / 2 : bn;
-        const int64_t stA = (int64_t)kBM * kBK * image_bytes(p.dtype), stB = (int64_t)brows * kBK * image_bytes(p.dtype);
-        const int64_t rtA = pair ? 2 * ((d.M + 2 * kBM - 1) / (2 * kBM)) : (d.M + kBM - 1) / kBM;
-        const int64_t rtB = pair ? 2 * ((d.N + bn - 1) / bn) : (d.N + bn - 1) / bn;
-        const int64_t offB = (rtA * nktp * stA + 255) / 256 * 256;
-        // offB + rtB * nktp * stB <= pk_bound (rows round up by less than
-        // 128 and bn <= 256, K by less than 32)
-        s = ensure_device_resources(p, (size_t)pk_bound);
-        if (s != TC_SUCCESS) return s;
-        d.pk = 3;
-        d.pk_base = (const char *)p.workspace;
-        d.pk_tile_bytes = nktp * stA;
-        d.pkb_base = (const char *)p.workspace + offB;
-        d.pkb_tile_bytes = nktp * stB;
-        for (int o = 0; o < 2; ++o) {
-            const int rows = o == 0 ? kBM : brows;
-            const int64_t rt = o == 0 ? rtA : rtB;
-            const int64_t bytes = rt * nktp * (o == 0 ? stA : stB);
-            const int64_t chunks =
-                bytes / 16 / (p.dtype == TC_TF32X3 ? 2 : (p.dtype == TC_BF16X3 ? 3 : 1));  // 16-byte rows of slice 0
-            const unsigned grid = (unsigned)std::min<int64_t>((chunks + 127) / 128, 152 * 16);
-            char *out = (char *)p.workspace + (o == 0 ? 0 : offB);
-            if (p.dtype == TC_BF16 || p.dtype == TC_F16) pack16_kernel<<<grid, 128, 0, st>>>(d, o, rows, kBK, rt, out);
-            else if (p.dtype == TC_E4M3) pack_kernel<GK_E4M3><<<grid, 128, 0, st>>>(d, o, rows, kBK, rt, out);
-            else if (p.dtype == TC_TF32) pack_kernel<GK_TF32><<<grid, 128, 0, st>>>(d, o, rows, kBK, rt, out);
-            else if (p.dtype == TC_TF32X3) pack_kernel<GK_TF32X3><<<grid, 128, 0, st>>>(d, o, rows, kBK, rt, out);
-            else pack_kernel<GK_BF16X3><<<grid, 128, 0, st>>>(d, o, rows, kBK, rt, out);
-        }
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
-    } else if (pk) {
+    if (pk) {
         // the smaller input's stage images, for the stage depth the launch
         // uses; pairs read them as two images per pair tile (an even count)
         const int bkp = tma ? kBKT : kBK;

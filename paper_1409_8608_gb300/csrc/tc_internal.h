@@ -120,6 +120,33 @@ size_t gett_workspace_bytes(const Plan &p);
 void gett_release(Plan &p);
 tc_status ensure_device_resources(Plan &p, size_t workspace_bytes);
 
+// The tensor-core GETT's modes: M = free indices of A and N = free indices of
+// B (first mode fastest), K = contracted indices (outermost first), batch
+// indices.
+struct GettModes {
+    int nm, nn, nk;                       // number of M / N / K modes
+    int64_t m_ext[kMaxModes], m_sA[kMaxModes], m_sC[kMaxModes];
+    int64_t n_ext[kMaxModes], n_sB[kMaxModes], n_sC[kMaxModes];
+    int n_chain;                          // C offset of column n is n * n_sC[0]
+    int64_t k_ext[kMaxModes], k_sA[kMaxModes], k_sB[kMaxModes];  // outermost first
+    int64_t M, N, K;
+    // batch (Hadamard) indices, in A, B and C: the tile list runs over
+    // batch values outermost, then N tiles, then M tiles
+    int nb;
+    int64_t b_ext[kMaxModes], b_sA[kMaxModes], b_sB[kMaxModes], b_sC[kMaxModes];
+};
+
+// Fills the modes; pk: an input (or both) is read pre-converted, so the K
+// order follows the larger input alone (tc_gett.cu).
+tc_status describe_modes(const Plan &p, int pk, GettModes &d);
+
+// The tensor-core GETT with both inputs pre-converted (tc_packed.cu): the
+// bytes of their images, and one execute.  comp_k > 0: compensated over
+// chunks of comp_k; qscale: E4M3's input scales.
+int64_t packed_bytes(tc_dtype dt, int64_t M, int64_t N, int64_t K);
+tc_status exec_packed(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
+                      void *stream, double fraction, int64_t comp_k, bool split, const float *qscale);
+
 // One phase of a gemm loop nest on the tensor cores (tensor dtypes): the
 // kernel's free index of A (m: sA, sC) and of B (n: sB, sC), its K modes
 // (the in-task contracted loops outermost first, the kernel's contracted

@@ -386,7 +386,7 @@ tc_status tc_autotune(tc_plan plan, const void *A, const void *B, void *C, void 
         const int bn = c["gett_tile"], tm = c["gett_tma"];
         const int pair = c.count("gett_pair") ? c["gett_pair"] : 0, pack = c.count("gett_pack") ? c["gett_pack"] : 1;
         if ((bn == 0 || bn == 128 || bn == 256) && (tm == 0 || tm == 1) && (pair == 0 || pair == 1) &&
-            pack >= 0 && pack <= 2) {
+            pack >= 0 && pack <= 3) {
             p.gett_bn = bn;
             p.gett_tma = tm;
             p.gett_pair = pair;

@@ -58,6 +58,32 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity,
     return true;
 }
 
+// The same wait beside a role that may have given up: also false once
+// *abort_flag is set (looked at only while the barrier is not complete).
+__device__ __forceinline__ bool mbar_wait_or(uint64_t *bar, uint32_t parity, volatile int *abort_flag) {
+    if (mbar_try_wait(bar, parity)) return true;
+    const uint64_t t0 = globaltimer();
+    while (!mbar_try_wait(bar, parity)) {
+        if (*abort_flag || globaltimer() - t0 > kWaitLimitNs) return false;
+    }
+    return true;
+}
+
+// One lane of the (converged) warp.  tcgen05.mma takes its descriptors and
+// addresses from uniform registers: code that a whole warp runs with the
+// issue under this predicate keeps them there, while a branch on the lane
+// number makes the compiler move every operand there first, instruction by
+// instruction (170 clocks per MMA on the pre-converted GETT).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
     asm volatile(
         "{\n\t.reg .b64 st;\n\t"
