@@ -435,7 +435,8 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
     uint32_t *tmem_slot = (uint32_t *)(drain + 1);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    // (warp-uniform, so that the TMA and MMA warps' operands are)
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
     const int nkt = (int)((d.K + BK - 1) / BK);
     constexpr uint32_t kTmemCols = COMP ? 4 * BN : 2 * BN;
     static_assert(kTmemCols <= 512, "tensor memory columns");
@@ -522,7 +523,7 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
     if (warp >= kEpiWarps && warp < kMmaWarp) {
         // ---------------------------------------------------------- converters
@@ -804,7 +805,8 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
         }
     } else if (warp == kTmaWarp) {
         // ---------------------------------------------------------- TMA issue
-        if (TMA && any_tma && lane == 0) {
+        // (the whole warp runs the loops; one elected lane issues)
+        if (TMA && any_tma) {
             int64_t g = 0;
             bool stop = false;
             // box coordinates of a tile's rows, and of one of its K stages
@@ -859,19 +861,23 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
                 tile_rc(tile, rc);
                 for (int kt = 0; kt < nkt; kt += spb, ++g) {
                     const int s = (int)(g % NSL);
-                    if (g >= NSL && (*abort_flag || !mbar_wait(&sempty[s], (uint32_t)(((g / NSL) - 1) & 1)))) {
+                    int32_t c[2][kTmaRank];
+                    stage_c(rc, kt, c);
+                    if (g >= NSL && !__all_sync(0xffffffffu, mbar_wait_or(&sempty[s], (uint32_t)(((g / NSL) - 1) & 1),
+                                                                          abort_flag))) {
                         stop = true;
                         break;
                     }
-                    int32_t c[2][kTmaRank];
-                    stage_c(rc, kt, c);
                     char *box = stg + s * (boxA + boxB);
-                    mbar_arrive_expect_tx(&sfull[s], d.tma_bytes);
-                    if (d.tma[0]) tma_load_5d(box, &tmA, &sfull[s], c[0]);
-                    if (d.tma[1]) tma_load_5d(box + boxA, &tmB, &sfull[s], c[1]);
+                    if (elect_one()) {
+                        mbar_arrive_expect_tx(&sfull[s], d.tma_bytes);
+                        if (d.tma[0]) tma_load_5d(box, &tmA, &sfull[s], c[0]);
+                        if (d.tma[1]) tma_load_5d(box + boxA, &tmB, &sfull[s], c[1]);
+                    }
+                    __syncwarp();
                 }
             }
-            if (stop) {
+            if (stop && lane == 0) {
                 *abort_flag = 1;
                 atomicExch(d.status, (int)TC_ERROR_TIMEOUT);
             }
@@ -881,7 +887,8 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
         // ---------------------------------------------------------- MMA issuer
         // (pairs: rank 0 issues for both CTAs; the other MMA warp only
         // takes part in the tensor-memory allocation)
-        if (lane == 0 && crank == 0) {
+        // The whole warp runs the loops and waits; one elected lane issues
+        if (crank == 0) {
             constexpr uint32_t kM = PAIR ? 2 * kBM : kBM;
             constexpr uint32_t idesc = (1u << 4) | (T::kFmt << 7) | (T::kFmt << 10) |
                                        ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
@@ -930,7 +937,7 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
                 const int cstg_t = BATCH ? nkt_t : cstg, nch_t = BATCH ? 1 : nch;
                 for (int c = 0; c < nch_t && !stop; ++c, ++u) {
                     const int buf = (int)(u % nbuf);
-                    if (u >= nbuf && !bwait(&tempty[buf], (uint32_t)(((u / nbuf) - 1) & 1))) {
+                    if (u >= nbuf && !__all_sync(0xffffffffu, bwait(&tempty[buf], (uint32_t)(((u / nbuf) - 1) & 1)))) {
                         stop = true;
                         break;
                     }
@@ -940,13 +947,14 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
                     const int kt_end = min(nkt_t, (c + 1) * cstg_t);
                     for (int kt = c * cstg_t; kt < kt_end; ++kt, ++g) {
                         const int s = (int)(g % STAGES);
-                        if (*abort_flag || !bwait(&full[s], (uint32_t)((g / STAGES) & 1))) {
+                        if (!__all_sync(0xffffffffu, !*abort_flag && bwait(&full[s], (uint32_t)((g / STAGES) & 1)))) {
                             stop = true;
                             break;
                         }
                         tc_fence_after();
                         const uint64_t so = (uint64_t)((s * SP::kStage) >> 4);
                         const bool first = kt == c * cstg_t;
+                        if (elect_one()) {
                         if constexpr (KIND == GK_BF16X3) {
                             if (nprod == 6) issue_stage(std::integral_constant<int, 6>{}, ad0 + so, bd0 + so, dt, first);
                             else if (nprod == 3) issue_stage(std::integral_constant<int, 3>{}, ad0 + so, bd0 + so, dt, first);
@@ -956,17 +964,22 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
                                         first);
                         }
                         commit(&empty[s]);
+                        if (kt + 1 == kt_end) commit(&tfull[buf]);  // arrives when this unit's MMAs are done
+                        }
+                        __syncwarp();
                     }
-                    commit(&tfull[buf]);  // arrives when this unit's MMAs are done
                 }
             }
-            if (stop) {
+            if (stop && lane == 0) {
                 *abort_flag = 1;
                 atomicExch(d.status, (int)TC_ERROR_TIMEOUT);
             }
             // nothing issued may still run when the tensor memory is freed
-            if constexpr (PAIR) mma_commit2(drain, (uint16_t)1);
-            else mma_commit(drain);
+            if (elect_one()) {
+                if constexpr (PAIR) mma_commit2(drain, (uint16_t)1);
+                else mma_commit(drain);
+            }
+            __syncwarp();
             mbar_wait(drain, 0);
         }
         __syncwarp();
