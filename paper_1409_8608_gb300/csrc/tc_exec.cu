@@ -422,11 +422,8 @@ __device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid, TileSm
             kk = k0 + (l / Q) * (R < NT / 8 ? NT / R : 8);
         }
     };
-    // with alpha = 1 the elements go straight to shared memory with
-    // asynchronous copies (zero-filled past the extents); otherwise through
-    // registers, A scaled by alpha on the way: the same values land in the
-    // same places
-    const bool async_copy = d.alpha_one;
+    // the elements go straight to shared memory with asynchronous copies
+    // (zero-filled past the extents)
     auto cp = [](void *dst, const void *src, bool valid) {
         if constexpr (F32)
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
@@ -457,19 +454,17 @@ __device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid, TileSm
         else side(No{}, std::integral_constant<int, BM>{}, std::integral_constant<int, LA>{}, std::integral_constant<int, QA>{}, A, roA, sm.kA[b], rA0, kA0, &sm.As[b][0][0], BM + sm.PAD);
         if (fb) side(Yes{}, std::integral_constant<int, BN>{}, std::integral_constant<int, LB>{}, std::integral_constant<int, QB>{}, B, roB, sm.kB[b], rB0, kB0, &sm.Bs[b][0][0], BN + sm.PAD);
         else side(No{}, std::integral_constant<int, BN>{}, std::integral_constant<int, LB>{}, std::integral_constant<int, QB>{}, B, roB, sm.kB[b], rB0, kB0, &sm.Bs[b][0][0], BN + sm.PAD);
-        asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    auto async_wait = []() { asm volatile("cp.async.wait_all;" ::: "memory"); };
-    auto plain_stage = [&](int b) {  // alpha != 1
-        for (int e = tid; e < BM * BK; e += NT) {
-            const int r = fa ? e % BM : (e / 8) % BM, kk = fa ? e / BM : (e / (8 * BM)) * 8 + e % 8;
-            const int64_t om = sm.offAm[r], ok = sm.kA[b][kk];
-            sm.As[b][kk][r] = om >= 0 && ok >= 0 ? alpha * A[om + ok] : T(0);
-        }
-        for (int e = tid; e < BN * BK; e += NT) {
-            const int r = fb ? e % BN : (e / 8) % BN, kk = fb ? e / BN : (e / (8 * BN)) * 8 + e % 8;
-            const int64_t on = sm.offBn[r], ok = sm.kB[b][kk];
-            sm.Bs[b][kk][r] = on >= 0 && ok >= 0 ? B[on + ok] : T(0);
+    // the stage's copies have landed; with alpha != 1 each thread scales the
+    // elements of A that it copied itself
+    auto land_stage = [&](int b) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if (d.alpha_one) return;
+#pragma unroll
+        for (int l = 0; l < LA; ++l) {
+            int q, r, kk;
+            at(fa, BM, QA, l, rA0, kA0, q, r, kk);
+            sm.As[b][kk][r] = alpha * sm.As[b][kk][r];
         }
     };
     auto step = [&](int sb, int kk) {
@@ -524,17 +519,13 @@ __device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid, TileSm
     // copies, before that barrier), so that their integer work overlaps the
     // multiplications.  The last stage stops at K (its padding would cost
     // whole multiplications: K = 8 spent as much as K = 16).
-    if (async_copy) {
-        async_stage(0);
-        async_wait();
-    } else {
-        plain_stage(0);
-    }
+    async_stage(0);
+    land_stage(0);
     __syncthreads();
     int sb = 0;
     for (int64_t k0 = 0; k0 < d.K; k0 += BK, sb ^= 1) {
         const bool more = k0 + BK < d.K;
-        if (more && async_copy) async_stage(sb ^ 1);
+        if (more) async_stage(sb ^ 1);
         if (k0 + 2 * BK < d.K) k_tables(k0 + 2 * BK, sb);
         if (k0 + BK <= d.K) {
 #pragma unroll
@@ -544,10 +535,7 @@ __device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid, TileSm
 #pragma unroll 1
             for (int kk = 0; kk < klen; ++kk) step(sb, kk);
         }
-        if (more) {
-            if (async_copy) async_wait();
-            else plain_stage(sb ^ 1);
-        }
+        if (more) land_stage(sb ^ 1);
         __syncthreads();
     }
 
@@ -634,6 +622,23 @@ tile_batch_kernel(const TileDesc *__restrict__ descs, const int32_t *__restrict_
     if (sd.shape == 0) TileOf<T, 0>::run(sd, bid, buf);
     else if (sd.shape == 1) TileOf<T, 1>::run(sd, bid, buf);
     else TileOf<T, 2>::run(sd, bid, buf);
+}
+
+// Tiles of a device list: item m + tiles_m * n stands for sub_m x sub_n tiles
+// of the largest shape.
+template <typename T>
+__global__ void __launch_bounds__(256, 2) tile_list_kernel(const TileDesc d, const int64_t *__restrict__ list,
+                                                           int64_t tiles_m, int sub_m, int sub_n) {
+    __shared__ __align__(16) unsigned char buf[sizeof(typename TileOf<T, 0>::Smem)];
+    const int64_t count = list[0] * sub_m * sub_n;
+    for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
+        const int64_t item = list[1 + q / (sub_m * sub_n)];
+        const int sub = (int)(q % (sub_m * sub_n));
+        const int64_t tm = item % tiles_m * sub_m + sub % sub_m, tn = item / tiles_m * sub_n + sub / sub_m;
+        if (tm >= d.tiles_m || tn >= d.tiles_n) continue;
+        __syncthreads();  // the last tile's tables have been read
+        TileOf<T, 0>::run(d, tm + d.tiles_m * tn, buf);
+    }
 }
 
 // ---------------------------------------------------------------- copy
@@ -1114,6 +1119,24 @@ tc_status run_gett_simt(Plan &p, T alpha, const T *A, const T *B, T beta, T *C,
 }
 
 }  // namespace
+
+tc_status simt_run_list(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
+                        const int64_t *list, int64_t tiles_m, int rows, int cols, void *stream) {
+    TileDesc td;
+    cudaStream_t st = (cudaStream_t)stream;
+    const bool f64 = p.dtype == TC_F64;
+    const int b = simt_rows(f64, 0);
+    if (f64) describe_gett_simt<double>(p, *(const double *)alpha, (const double *)A, (const double *)B, *(const double *)beta, (double *)C, td);
+    else describe_gett_simt<float>(p, *(const float *)alpha, (const float *)A, (const float *)B, *(const float *)beta, (float *)C, td);
+    td.shape = 0;
+    td.tiles_m = (td.M + b - 1) / b;
+    td.tiles_n = (td.N + b - 1) / b;
+    const unsigned grid = (unsigned)device_sms() * (f64 ? 4 : 2);
+    if (f64) tile_list_kernel<double><<<grid, 256, 0, st>>>(td, list, tiles_m, rows / b, cols / b);
+    else tile_list_kernel<float><<<grid, 256, 0, st>>>(td, list, tiles_m, rows / b, cols / b);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? TC_SUCCESS : fail(TC_ERROR_CUDA, cudaGetErrorString(e));
+}
 
 size_t simt_desc_bytes() { return sizeof(TileDesc); }
 
