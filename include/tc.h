@@ -159,8 +159,9 @@ tc_status tc_plan_select(tc_plan plan, int32_t alg_id);
 tc_status tc_plan_selected(tc_plan plan, int32_t *alg_id);
 
 /* Bytes of device workspace the algorithm needs (copy buffers; for GETT,
- * id 0, the pre-converted input of tc_plan_set_gett_pack, else 0).  The
- * plan allocates it on the first tc_execute of that algorithm and keeps it
+ * id 0, the pre-converted input of tc_plan_set_gett_pack, else 0; a large
+ * TC_F64 / TC_F32 GETT needs none but uses scratch when it can have it, see
+ * tc_execute).  The plan allocates it on the first tc_execute of that algorithm and keeps it
  * until tc_plan_destroy; call tc_execute once before capturing a CUDA
  * graph.  The workspace serves one execute at a time, so tc_execute
  * refuses a second stream while the plan's last execute is in flight
@@ -174,7 +175,19 @@ tc_status tc_algorithm_workspace(tc_plan plan, int32_t alg_id, size_t *bytes);
  * TC_ERROR_INVALID_ARGUMENT is returned: concurrent executes of one plan
  * would share its workspace.  Executes on the same stream queue behind one
  * another as usual.  While `stream` is capturing a CUDA graph the check is
- * skipped and nothing is recorded. */
+ * skipped and nothing is recorded.
+ *
+ * TC_F64 and TC_F32 with GETT selected: where the size makes it the faster
+ * form (K from 32 to 2^20, TC_F32 to 4096; no batch indices), the tensor
+ * cores compute the contraction from exact 8-bit digits of the inputs, FP64
+ * from 62 and FP32 from 30 bits below the largest magnitude of a row of A
+ * and a column of B, rounded once: at least as close to the exact result as
+ * a chain of K fused multiply-adds.  Parts of C whose rows or columns hold
+ * too many small entries for that, infinities, NaN or extreme exponents run
+ * as such chains, like smaller sizes.  The images of the digits take up to
+ * 64 MiB for B and 256 MiB for A, allocated by the first execute outside a
+ * stream capture and kept; when that fails, or inside a capture before, the
+ * chains run instead. */
 tc_status tc_execute(tc_plan plan, const void *alpha, const void *A,
                      const void *B, const void *beta, void *C, void *stream);
 

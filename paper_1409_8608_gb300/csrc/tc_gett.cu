@@ -1795,7 +1795,16 @@ static tc_status e4m3_scales(Plan &p, const void *A, const void *B, cudaStream_t
 
 tc_status exec_gett(Plan &p, const void *alpha, const void *A, const void *B, const void *beta,
                     void *C, void *stream, const Probe *probe) {
-    if (p.dtype == TC_F64 || p.dtype == TC_F32) return exec_gett_simt(p, alpha, A, B, beta, C, stream, probe);
+    if (p.dtype == TC_F64 || p.dtype == TC_F32) {
+        bool done = false;
+        const tc_status sd = exec_digits(p, alpha, A, B, beta, C, stream, probe ? probe->fraction : 1.0, &done);
+        if (sd != TC_SUCCESS) return sd;
+        if (done) {
+            p.last_stream = stream;
+            return TC_SUCCESS;
+        }
+        return exec_gett_simt(p, alpha, A, B, beta, C, stream, probe);
+    }
     tc_status s = ensure_device_resources(p, 0);
     if (s != TC_SUCCESS) return s;
     p.last_stream = stream;

@@ -17,7 +17,9 @@
 namespace tc {
 namespace dev {
 
-enum GettKind { GK_BF16X3 = 0, GK_BF16 = 1, GK_F16 = 2, GK_TF32 = 3, GK_TF32X3 = 4, GK_E4M3 = 5 };
+// (GK_D64, GK_D32: FP64 and FP32 inputs as exact BF16 digits, tc_packed.cu)
+enum GettKind { GK_BF16X3 = 0, GK_BF16 = 1, GK_F16 = 2, GK_TF32 = 3, GK_TF32X3 = 4, GK_E4M3 = 5, GK_D64 = 6, GK_D32 = 7 };
+__host__ __device__ constexpr bool digit_kind(int k) { return k == GK_D64 || k == GK_D32; }
 
 // MMA on TF32 words (kind::tf32, 4-byte operand elements)
 __host__ __device__ constexpr bool tf32_kind(int k) { return k == GK_TF32 || k == GK_TF32X3; }
@@ -198,6 +200,28 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         : "memory");
 }
 
+// Four columns of each of eight accumulators `stride` columns apart, one wait:
+// r[4 n + j] is column j of accumulator n.
+__device__ __forceinline__ void tmem_ld8x4(uint32_t t, uint32_t stride, uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%32];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%33];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%34];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12,%13,%14,%15}, [%35];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%16,%17,%18,%19}, [%36];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%20,%21,%22,%23}, [%37];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%24,%25,%26,%27}, [%38];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%28,%29,%30,%31}, [%39];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(t), "r"(t + stride), "r"(t + 2 * stride), "r"(t + 3 * stride), "r"(t + 4 * stride), "r"(t + 5 * stride),
+          "r"(t + 6 * stride), "r"(t + 7 * stride)
+        : "memory");
+}
+
 // Two 32-column loads (the split accumulators) and their FP32 sum: both
 // loads and the wait in one statement, so no use of the registers can be
 // scheduled before the wait.
@@ -236,7 +260,7 @@ __device__ __forceinline__ uint32_t f32_to_tf32(float x) {
 template <int KIND, int BK>
 struct KindTraits {
     static constexpr int kElemBytes = tf32_kind(KIND) ? 4 : (KIND == GK_E4M3 ? 1 : 2);  // smem operand element
-    static constexpr int kSlices = KIND == GK_BF16X3 ? 3 : (KIND == GK_TF32X3 ? 2 : 1);
+    static constexpr int kSlices = KIND == GK_BF16X3 ? 3 : (KIND == GK_TF32X3 ? 2 : (KIND == GK_D64 ? 8 : (KIND == GK_D32 ? 4 : 1)));
     static constexpr int kChunk = 16 / kElemBytes;              // K elements per 16-byte row
     static constexpr int kKc = BK / kChunk;                     // core matrices along K per stage
     static constexpr int kKsteps = BK * kElemBytes / 32;        // MMA instructions along K per stage
@@ -244,7 +268,8 @@ struct KindTraits {
     // F16 = 0, BF16 = 1; kind::f8f6f4 E4M3 = 0
     static constexpr uint32_t kFmt = tf32_kind(KIND) ? 2u : ((KIND == GK_F16 || KIND == GK_E4M3) ? 0u : 1u);
     using In = typename std::conditional<KIND == GK_BF16, __nv_bfloat16,
-                                         typename std::conditional<KIND == GK_F16, __half, float>::type>::type;
+                                         typename std::conditional<KIND == GK_F16, __half,
+                                                                   typename std::conditional<KIND == GK_D64, double, float>::type>::type>::type;
     static constexpr int kInBytes = sizeof(In);
     static constexpr int kVec = 16 / kInBytes;                  // input elements per 16-byte load
 };

@@ -76,6 +76,8 @@ struct Plan {
     void *host_dev[3] = {nullptr, nullptr, nullptr};  // tc_execute_host: device copies of A, B, C
     size_t host_dev_bytes[3] = {0, 0, 0};
     void *gett_state = nullptr;     // owned by the GETT executor
+    void *digit_ws = nullptr;       // TC_F64 / TC_F32: digit images of a large GETT (tc_packed.cu)
+    size_t digit_bytes = 0;
     void *qbuf = nullptr;           // TC_E4M3: the inputs' maxima and scales (16 bytes)
     void *flush_buf = nullptr;      // predictor: remote regions / L2 flush
     size_t flush_bytes = 0;
@@ -146,6 +148,15 @@ tc_status describe_modes(const Plan &p, int pk, GettModes &d);
 int64_t packed_bytes(tc_dtype dt, int64_t M, int64_t N, int64_t K);
 tc_status exec_packed(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
                       void *stream, double fraction, int64_t comp_k, bool split, const float *qscale);
+
+// A large FP64 / FP32 GETT as exact digits on the tensor cores (tc_packed.cu);
+// *done = false, with nothing enqueued, where the SIMT tiles are to run.
+tc_status exec_digits(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C, void *stream,
+                      double fraction, bool *done);
+// The SIMT GETT over the tiles of a device list (list[0] of them, each
+// m + tiles_m * n of tiles of rows x cols, whole SIMT tiles).
+tc_status simt_run_list(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
+                        const int64_t *list, int64_t tiles_m, int rows, int cols, void *stream);
 
 // One phase of a gemm loop nest on the tensor cores (tensor dtypes): the
 // kernel's free index of A (m: sA, sC) and of B (n: sB, sC), its K modes

@@ -31,6 +31,41 @@
 // number the same tiles took 178 and 918 us (elect_one).  The compensated
 // sums' (hi, lo) in registers leave the tensor memory to two accumulators.
 //
+// FP64 and FP32 (GK_D64, GK_D32): digits.  The FP64 unit runs two
+// multiply-adds per SM and clock (1.26 TFLOP/s), so a large FP64 or FP32 GETT
+// is computed from integers on the tensor cores (the digit splitting of
+// Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix
+// multiplication by using fast routines of matrix multiplication", 2012):
+//   * a row of A (column of B) is scaled by the power of two 2^e just above
+//     its largest magnitude and cut into S balanced base-256 digits d_s,
+//     |d| <= 128 (64 for s = 0), x = 2^e sum_s d_s 2^(-6-8s), S = 8 (FP64) or
+//     4 (FP32): 62 or 30 bits below 2^e, exact as BF16 values;
+//   * FP64: the products d_s d_t with s + t = l < 8 add up in accumulator l.
+//     A sum over 128 K positions stays within 2^24 in magnitude, so every
+//     FP32 accumulation is exact, in any order; the epilogue adds the levels
+//     as 64-bit integers (0-3 and 4-7 apart) and rounds the total once;
+//   * FP32: level 0 has its own accumulator, exact up to K = 4096, levels 1
+//     to 3 (weights 2^-8 and less) share a second one; the two are added and
+//     rounded once.
+// What is left out is at most 2^-59 (FP64) or 2^-28 (FP32) of 2^(eA + eB) per
+// term: the products of level S and past it, and the bits under the last
+// digit.  That is small against |A||B| only where the row and the column
+// hold enough large entries, so the pre-pass counts per row the entries
+// below 2^(e-5) (FP64) or 2^(e-3) (FP32): where those of a row of A and of a
+// column of B are together at most K / 2, at least K / 2 terms of the sum
+// are at least 2^(eA+eB-10) (2^-6), and the error left out is at most
+// 2^-48 |A||B| (2^-21), under the K 2^-53 (K 2^-24) of a chain of fused
+// multiply-adds for K >= 32; on uniform entries only the last rounding is
+// left.  Tiles where that does not hold (wide ranges or many zeros along K,
+// infinities, NaN, exponents near the ends) go to a list, and the SIMT tiles
+// compute them.  B is taken in panels whose images stay in L2.
+// abc=iaj,jbic 512^3 i=j=16: FP64 56.7 -> 3.28 ms (18 panels: pre-pass 23 us,
+// GETT 160 us each; the shared-memory port takes 1760 of its clocks per 16 K
+// positions, draining the levels, which nothing overlaps, most of the rest),
+// FP32 2.35 -> 0.62 ms (9 panels: 21 and 45 us).  Error against 80-bit and
+// longer sums on uniform entries: below that of the chains (FP32 3.2e-8
+// against 2.9e-7 of the result's 2-norm).
+//
 // Every wait on an mbarrier is bounded; on expiry the kernel records
 // TC_ERROR_TIMEOUT, stops issuing, drains, frees its tensor memory, returns.
 #include <cuda.h>
@@ -64,7 +99,7 @@ constexpr int kMapRow = 512;               // bytes per row of an image tensor m
 // K positions per stage: about 32-48 KB of images per CTA
 template <int KIND>
 __host__ __device__ constexpr int stage_k() {
-    return KIND == GK_TF32X3 ? 16 : ((KIND == GK_BF16 || KIND == GK_F16 || KIND == GK_E4M3) ? 64 : 32);
+    return KIND == GK_TF32X3 || KIND == GK_D64 ? 16 : ((KIND == GK_BF16 || KIND == GK_F16 || KIND == GK_E4M3) ? 64 : 32);
 }
 template <int KIND>
 using Traits = KindTraits<KIND, stage_k<KIND>()>;
@@ -83,6 +118,14 @@ struct PackedDesc : GettModes {
     int nprod, split;
     int *status;
     const float *qscale;        // E4M3: the inputs' scales
+    // digits: first column of the panel (N then counts the panel's), scalars
+    // in FP64, per row the exponent field of its largest magnitude, per
+    // image row tile the most small entries of a row, and the tiles left to
+    // SIMT (list[0]: how many)
+    int64_t n_begin;
+    double alpha64, beta64;
+    int *exps[2], *small[2];
+    int64_t *list;
 };
 
 // One input's share of the pre-pass.
@@ -191,6 +234,198 @@ __global__ void __launch_bounds__(kPackThreads) pack_images_kernel(const __grid_
     }
 }
 
+// ---- digits
+template <int KIND>
+struct Digits {
+    static constexpr bool F64 = KIND == GK_D64;
+    using In = typename std::conditional<F64, double, float>::type;
+    static constexpr int kLarge = 4;                  // FP64, large: exponent field at least the row's minus this
+    static constexpr int kLow = F64 ? 623 : 77, kHigh = F64 ? 1423 : 177;  // exponent fields taken
+    static constexpr int kChunkK = F64 ? 128 : 1 << 12;  // K positions per accumulation
+    static constexpr int kBn = F64 ? 64 : 128;        // columns per tile: 8 levels, or two double-buffered accumulators
+    static constexpr int64_t kMaxK = F64 ? 1 << 20 : 1 << 12;  // the summed levels stay below 2^62; level 0 exact
+};
+constexpr int kRowBad = 1 << 29;
+constexpr int kDigitK = 256;  // K positions a block holds at a time
+
+// One input as digit images: a block takes 32 rows; K positions stay in
+// registers between the search for the largest magnitudes and the digits (a
+// longer K is read twice, the second time mostly from L2).
+template <int KIND>
+__global__ void __launch_bounds__(kPackThreads, Digits<KIND>::F64 ? 2 : 4) pack_digits_kernel(const __grid_constant__ PackedDesc d,
+                                                                   const PackJob ja, const PackJob jb) {
+    using D = Digits<KIND>;
+    using T = Traits<KIND>;
+    using In = typename D::In;
+    constexpr int BK = stage_k<KIND>(), S = T::kSlices, P = kPackRows + 1;
+    extern __shared__ __align__(16) unsigned char dsm[];
+    In *tile = (In *)dsm;  // [kDigitK][P]
+    __shared__ int64_t koff[kDigitK], roff[kPackRows];
+    __shared__ unsigned emax[kPackRows];
+    __shared__ int nlarge[kPackRows];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const bool second = blockIdx.x >= ja.blocks;
+    const PackJob &J = second ? jb : ja;
+    const int64_t r0 = (second ? (int64_t)blockIdx.x - ja.blocks : (int64_t)blockIdx.x) * kPackRows;
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    const In *__restrict__ src = (const In *)(J.op == 0 ? d.A : d.B);
+    if (tid < kPackRows) {
+        int64_t r = r0 + tid, o = -1, u = 0;
+        if (r < (J.op == 0 ? d.M : d.N)) {
+            o = 0;
+            if (J.op == 0) decode(r, d.nm, d.m_ext, d.m_sA, d.m_sC, o, u);
+            else decode(r + d.n_begin, d.nn, d.n_ext, d.n_sB, d.n_sC, o, u);
+        }
+        roff[tid] = o;
+        emax[tid] = 0;
+        nlarge[tid] = 0;
+    }
+    constexpr int NL = kDigitK * kPackRows / kPackThreads, KJ = kDigitK / 32;
+    In x[NL];
+    auto load = [&](int64_t k0) {  // (a barrier on both sides of the offset table)
+        __syncthreads();
+        static_assert(kDigitK == kPackThreads, "one thread per K offset");
+        int64_t k = k0 + tid, o = -1, u = 0;
+        if (k < d.K) {
+            o = 0;
+            const int64_t *ks = J.op == 0 ? d.k_sA : d.k_sB;
+            for (int m = d.nk - 1; m >= 0; --m) {
+                k = divmod(k, d.k_ext[m], u);
+                o += u * ks[m];
+            }
+        }
+        koff[tid] = o;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+            const int64_t ro = roff[J.rfast ? lane : warp * 4 + j / KJ];
+            const int64_t ko = koff[J.rfast ? warp + 8 * j : lane + 32 * (j % KJ)];
+            x[j] = ro >= 0 && ko >= 0 ? __ldg(src + ro + ko) : In(0);
+        }
+    };
+    // largest magnitude: the high word of |x| (for FP64 with a bit for a
+    // nonzero low word), ordered as integers
+    auto mag = [](In v) -> unsigned {
+        if constexpr (D::F64) {
+            const unsigned long long b = __double_as_longlong(v);
+            return ((unsigned)(b >> 32) & 0x7fffffffu) | ((unsigned)b != 0 ? 1u : 0u);
+        } else {
+            return __float_as_uint(v) & 0x7fffffffu;
+        }
+    };
+    unsigned mx[4] = {0, 0, 0, 0};
+    for (int64_t k0 = 0; k0 < d.K; k0 += kDigitK) {
+        load(k0);
+#pragma unroll
+        for (int j = 0; j < NL; ++j) mx[(j / KJ) & 3] = max(mx[(j / KJ) & 3], mag(x[j]));
+    }
+    if (J.rfast) {
+        atomicMax(&emax[lane], max(max(mx[0], mx[1]), max(mx[2], mx[3])));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const unsigned m = __reduce_max_sync(0xffffffffu, mx[i]);
+            if (lane == 0) emax[warp * 4 + i] = m;
+        }
+    }
+    __syncthreads();
+    const unsigned top = emax[lane];
+    const int E = (int)(top >> (D::F64 ? 20 : 23));
+    const int64_t R = r0 + lane;
+    int64_t rr;
+    const int64_t rt = divmod(R, J.rows, rr);
+    const int slice = J.rows * BK * 2;
+    char *out = J.out + rt * d.ktiles * (int64_t)(S * slice) + (rr / 8) * 128 + (rr % 8) * 16;
+    int large = 0;
+    // FP32: 2^-e (rows whose exponent is not taken get zeros)
+    const float down = D::F64 || E < D::kLow || E > D::kHigh ? 0.0f : __uint_as_float((unsigned)(253 - E) << 23);
+    const bool once = d.K <= kDigitK;
+    for (int64_t k0 = 0; k0 < (int64_t)d.ktiles * BK; k0 += kDigitK) {
+        if (!once) load(k0);
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+            if (J.rfast) tile[(warp + 8 * j) * P + lane] = x[j];
+            else tile[(lane + 32 * (j % KJ)) * P + warp * 4 + j / KJ] = x[j];
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int c = warp; c < kDigitK / 8; c += kPackThreads / 32) {  // chunks of 8 K positions
+            const int64_t k = k0 + c * 8;
+            if (R >= J.total_rows || k >= (int64_t)d.ktiles * BK) break;
+            char *dst = out + (k / BK) * (int64_t)(S * slice) + (int)((k % BK) / 8) * (J.rows / 8) * 128;
+            if constexpr (D::F64) {
+                unsigned long long y[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const unsigned long long b = __double_as_longlong(tile[(c * 8 + e) * P + lane]);
+                    const unsigned long long frac = b & ((1ull << 52) - 1);
+                    const int ex = (int)(b >> 52) & 2047;
+                    const unsigned long long m = ex ? frac | (1ull << 52) : frac;
+                    const int sh = E - (ex ? ex : 1);
+                    large += m != 0 && sh <= D::kLarge;
+                    // x 2^-e 2^62 = m 2^(9 - sh), rounded where bits fall
+                    // under the last digit
+                    unsigned long long w;
+                    if (sh <= 9) w = m << (9 - sh);
+                    else w = sh <= 62 ? (m + (1ull << (sh - 10))) >> (sh - 9) : 0ull;
+                    if (b >> 63) w = 0ull - w;
+                    y[e] = w + 0x8080808080808080ull;  // bytes: digit + 128
+                }
+#pragma unroll
+                for (int s = 0; s < S; ++s) {
+                    // 2^23 + byte as FP32 less 2^23 + 128: the digit, whose
+                    // upper half is its BF16 value
+                    constexpr unsigned kMagic = 0x4B000000u;
+                    const int byte = S - 1 - s;
+                    unsigned q[4];
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) {
+                        float f[2];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const unsigned word = (unsigned)(y[e + h] >> (byte >= 4 ? 32 : 0));
+                            f[h] = __uint_as_float(__byte_perm(word, kMagic, 0x7440 | (byte & 3))) - 8388736.0f;
+                        }
+                        q[e / 2] = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632);
+                    }
+                    *(uint4 *)(dst + (int64_t)s * slice) = make_uint4(q[0], q[1], q[2], q[3]);
+                }
+            } else {
+                // z = x 2^-e, |z| < 1: rounding to a multiple of 2^(-6-8s) by
+                // adding 1.5 2^(17-8s) leaves d_s 2^(-6-8s), a BF16 value
+                float z[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    z[e] = tile[(c * 8 + e) * P + lane] * down;
+                    large += fabsf(z[e]) >= 0.125f;
+                }
+#pragma unroll
+                for (int s = 0; s < S; ++s) {
+                    const float add = __uint_as_float(((unsigned)(127 + 17 - 8 * s) << 23) | 0x400000u);
+                    unsigned q[4];
+#pragma unroll
+                    for (int e = 0; e < 8; e += 2) {
+                        const float w0 = __fsub_rn(__fadd_rn(z[e], add), add), w1 = __fsub_rn(__fadd_rn(z[e + 1], add), add);
+                        z[e] = __fsub_rn(z[e], w0);
+                        z[e + 1] = __fsub_rn(z[e + 1], w1);
+                        q[e / 2] = __byte_perm(__float_as_uint(w0), __float_as_uint(w1), 0x7632);
+                    }
+                    *(uint4 *)(dst + (int64_t)s * slice) = make_uint4(q[0], q[1], q[2], q[3]);
+                }
+            }
+        }
+    }
+    atomicAdd(&nlarge[lane], large);
+    __syncthreads();
+    if (tid < kPackRows && R < J.total_rows) {  // warp 0: lane = row
+        int few = (int)min(d.K, (int64_t)kRowBad) - nlarge[lane];
+        if (top == 0) few = 0;  // a row of zeros (or past the extent): exact
+        else if (E < D::kLow || E > D::kHigh) few = kRowBad;
+        d.exps[J.op][R] = top == 0 ? D::kLow : E;
+        if (few > 0) atomicMax(&d.small[J.op][(J.op == 0 ? 0 : d.n_begin / J.rows) + rt], few);
+    }
+}
+
 // A box of an image map into shared memory, counted on the barrier at
 // shared::cluster address `bar` (a pair: the first CTA's).
 template <bool PAIR>
@@ -247,6 +482,35 @@ __device__ __forceinline__ void store_row(const uint32_t (&r)[32], float *__rest
     }
 }
 
+// (hi 2^24 + lo) 2^s rounded to nearest even; the result is a normal number.
+__device__ __forceinline__ double fixed_to_double(int64_t hi, int64_t lo, int s) {
+    // the 96-bit sum as (h, l), l the lowest 32 bits, unsigned
+    const uint64_t low32 = ((uint64_t)(hi & 0xff) << 24) + (uint32_t)lo;
+    int64_t h = (hi >> 8) + (lo >> 32) + (int64_t)(low32 >> 32);
+    uint32_t l = (uint32_t)low32;
+    const uint64_t sign = (uint64_t)h & 0x8000000000000000ull;
+    if (h < 0) {
+        h = l ? ~h : -h;
+        l = 0u - l;
+    }
+    if (((uint64_t)h | l) == 0) return 0.0;
+    // left-aligned: 64 bits and a sticky bit
+    uint64_t top;
+    uint32_t rest = 0;
+    const int z = h ? __clzll(h) : 64 + __clz((int)l);  // leading zeros of the 96 bits
+    if (z < 32) {
+        top = z ? ((uint64_t)h << z) | (l >> (32 - z)) : (uint64_t)h;
+        rest = l << z;
+    } else {
+        top = (((uint64_t)(uint32_t)h << 32) | l) << (z - 32);
+    }
+    uint64_t m = top >> 11;  // 53 bits, the leading one at bit 52
+    const uint32_t low = (uint32_t)top & 0x7ffu;
+    m += low > 0x400u || (low == 0x400u && (rest != 0 || (m & 1)));
+    const int field = 95 - z + s + 1023;
+    return __longlong_as_double((int64_t)(sign | (((uint64_t)(field - 1) << 52) + m)));
+}
+
 // COMP: compensated accumulation -- units of d.chunk K stages, double-buffered
 // in tensor memory, each folded by TwoSum into a (hi, lo) pair that the
 // epilogue threads hold in registers (64 columns each: bn <= 128).  Otherwise
@@ -261,6 +525,8 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
     extern __shared__ __align__(128) char ring[];
     __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], tfull[2], tempty[2], drain;
     __shared__ int64_t cN[2][kMaxBn];
+    constexpr bool DIG = digit_kind(KIND);
+    __shared__ int cE[DIG ? 2 : 1][DIG ? 128 : 1];  // digits: exponent fields of the tile's columns
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_word;
     volatile int *abort_flag = &abort_word;
@@ -277,8 +543,8 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
         *abort_flag = 1;
         atomicExch(d.status, (int)TC_ERROR_TIMEOUT);
     };
-    const bool split = !COMP && d.split != 0;
-    const int nbuf = split && d.bn > 128 ? 1 : 2;
+    const bool split = KIND == GK_D32 || (!COMP && d.split != 0);
+    const int nbuf = KIND == GK_D64 || (split && d.bn > 128) ? 1 : 2;
     const uint32_t small_off = split ? (d.bn > 128 ? 256u : 128u) : 0u;  // the smaller products' accumulator
     if (threadIdx.x == 0) {
         for (int s = 0; s < d.stages; ++s) {
@@ -309,6 +575,17 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
     // complete from here on
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const uint32_t stage_bytes = d.img_a + d.img_b;
+    // digits: a tile with too many small entries is left to SIMT
+    auto skip = [&](int64_t mt, int64_t nt) -> bool {
+        if constexpr (!DIG) return false;
+        const int64_t na = mt * kCtas, nb = d.n_begin / d.brows + nt * kCtas;
+        int a = d.small[0][na], b = d.small[1][nb];
+        if constexpr (PAIR) {
+            a = max(a, d.small[0][na + 1]);
+            b = max(b, d.small[1][nb + 1]);
+        }
+        return 2 * ((int64_t)a + b) > d.K;
+    };
 
     if (warp == kCopyWarp) {
         // --------------------------------------------------------- copies
@@ -319,6 +596,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
         for (int64_t tile = slot0; tile < d.num_tiles && !stop; tile += nslots) {
             int64_t mt;
             const int64_t nt = divmod(tile, d.tiles_m, mt);
+            if (skip(mt, nt)) continue;
             int32_t ra = (int32_t)((mt * kCtas + crank) * d.ktiles) * rows_a;
             int32_t rb = (int32_t)((nt * kCtas + crank) * d.ktiles) * rows_b;
             for (int kt = 0; kt < d.ktiles; ++kt, ra += rows_a, rb += rows_b) {
@@ -379,6 +657,23 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                     }
                 }
             };
+            // digits: product d_s d_t into accumulator s + t (FP64), or into the
+            // second one unless s = t = 0 (FP32)
+            auto issue_digits = [&](uint64_t as, uint64_t bs, uint32_t dt, bool first, int nks) {
+                constexpr int S = T::kSlices;
+#pragma unroll
+                for (int ks = 0; ks < T::kKsteps; ++ks) {
+                    if (ks >= nks) break;
+#pragma unroll
+                    for (int s = 0; s < S; ++s)
+#pragma unroll
+                        for (int t = 0; t < S - s; ++t)
+                            mma_issue<KIND, PAIR>(dt + (uint32_t)(KIND == GK_D64 ? (s + t) * 64 : (s + t ? 128 : 0)),
+                                                  as + (uint64_t)((s * sliceA + ks * 2 * lboA) >> 4),
+                                                  bs + (uint64_t)((t * sliceB + ks * 2 * lboB) >> 4), idesc,
+                                                  !(first && ks == 0 && s == 0 && (KIND == GK_D64 || t < 2)));
+                }
+            };
             auto commit = [&](uint64_t *bar) {
                 if constexpr (PAIR) mma_commit2(bar, (uint16_t)3);  // both CTAs' barriers
                 else mma_commit(bar);
@@ -388,6 +683,11 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
             uint32_t ph = 0, aph = 1;  // parities: stage filled; accumulator drained (free at first)
             bool stop = false;
             for (int64_t tile = slot0; tile < d.num_tiles && !stop; tile += nslots) {
+                if constexpr (DIG) {
+                    int64_t mt;
+                    const int64_t nt = divmod(tile, d.tiles_m, mt);
+                    if (skip(mt, nt)) continue;
+                }
                 int64_t left = d.K;  // K positions from this stage on
                 for (int c = 0; c < nch && !stop; ++c) {
                     if (!__all_sync(0xffffffffu, bwait(&tempty[buf], aph))) {
@@ -409,7 +709,9 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                         // K steps of the stage that hold K positions
                         const int nks = left >= BK ? T::kKsteps : (int)((left * T::kElemBytes + 31) / 32);
                         if (elect_one()) {
-                            if constexpr (KIND == GK_BF16X3) {
+                            if constexpr (DIG) {
+                                issue_digits(as, bs, dt, first, nks);
+                            } else if constexpr (KIND == GK_BF16X3) {
                                 if (d.nprod == 6) issue_stage(std::integral_constant<int, 6>{}, as, bs, dt, first, nks);
                                 else if (d.nprod == 3) issue_stage(std::integral_constant<int, 3>{}, as, bs, dt, first, nks);
                                 else issue_stage(std::integral_constant<int, 9>{}, as, bs, dt, first, nks);
@@ -446,13 +748,22 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
         const int nch = (d.ktiles + d.chunk - 1) / d.chunk;
         int it = 0, buf = 0;
         uint32_t aph = 0;  // parity: accumulator filled
+        int64_t dhi[32], dlo[32];  // FP64 digits: levels 0-3 (units of 2^-36) and 4-7 (2^-60), 32 columns
+        const bool plain = d.init == 2 && d.alpha64 == 1.0;
         constexpr int G = COMP ? 2 : 1;
         float hi[G][32], lo[G][32];
         for (int64_t tile = slot0; tile < d.num_tiles; tile += nslots, ++it) {
             int64_t mt, rem, ignored = 0;
             const int64_t nt = divmod(tile, d.tiles_m, mt);
-            const int64_t n0 = nt * d.bn, mm = (mt * kCtas + crank) * kRows + row;
-            const int nval = (int)min((int64_t)d.bn, d.N - n0);
+            if (skip(mt, nt)) {
+                if (et == 0 && crank == 0) {
+                    const unsigned long long at = atomicAdd((unsigned long long *)d.list, 1ull);
+                    d.list[1 + at] = mt + d.tiles_m * (d.n_begin / d.bn + nt);
+                }
+                continue;
+            }
+            const int64_t n0 = d.n_begin + nt * d.bn, mm = (mt * kCtas + crank) * kRows + row;
+            const int nval = (int)min((int64_t)d.bn, d.N - nt * d.bn);
             // one stride across the tile's columns where C has one
             int64_t lin = 0, on0 = 0, om = -1;
             int64_t *cn = cN[it & 1];
@@ -472,6 +783,11 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
             if (mm < d.M) {
                 om = 0;
                 decode(mm, d.nm, d.m_ext, d.m_sA, d.m_sC, ignored, om);
+            }
+            int rowE = 0;
+            if constexpr (DIG) {
+                rowE = d.exps[0][mm];  // (padded rows have one too)
+                if (et < d.bn) cE[it & 1][et] = d.exps[1][nt * d.bn + et];
             }
             if (role_sync_or<2, kEpiThreads>(*abort_flag)) break;
             bool aborted = false;
@@ -518,12 +834,52 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                         }
                     }
                 }
-                if constexpr (!COMP) {
+                if constexpr (KIND == GK_D64) {
+                    if (c == 0) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) dhi[j] = dlo[j] = 0;
+                    }
+                    // integers from integral FP32 values without conversion
+                    // instructions (which run at a few lanes per clock):
+                    // adding 1.5 2^23 leaves |v| <= 2^22 in the low bits, a
+                    // larger v goes in two halves, v = 256 h + l
+                    constexpr float kAdd = 12582912.0f;
+                    constexpr unsigned kAddBits = 0x4B400000u;
+                    auto small_int = [&](float v) -> int { return (int)(__float_as_uint(__fadd_rn(v, kAdd)) - kAddBits); };
+                    auto big_int = [&](float v) -> int {
+                        const float h = __fmaf_rn(v, 0.00390625f, kAdd), l = __fmaf_rn(__fsub_rn(h, kAdd), -256.0f, v);
+                        return (int)(__float_as_uint(h) * 256u + __float_as_uint(__fadd_rn(l, kAdd)) - kAddBits * 257u);
+                    };
+#pragma unroll
+                    for (int g4 = 0; g4 < 8; ++g4) {  // four columns of every level at a time
+                        uint32_t r[32];
+                        tmem_ld8x4(tmem + lane_off + (uint32_t)(half * 32 + g4 * 4), 64, r);
+                        auto lev = [&](int n, int j) { return __uint_as_float(r[n * 4 + j]); };
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            // levels 0 to 2: |i| <= 2^22; level 7 joins level
+                            // 6 rounded (to at most half its unit)
+                            const int i01 = small_int(lev(0, j)) * 256 + small_int(lev(1, j));
+                            const int i23 = small_int(lev(2, j)) * 256 + big_int(lev(3, j));
+                            dhi[g4 * 4 + j] += (int64_t)i01 * 65536 + i23;
+                            dlo[g4 * 4 + j] += (int64_t)big_int(lev(4, j)) * 65536 + (int64_t)big_int(lev(5, j)) * 256 +
+                                               big_int(__fmaf_rn(lev(7, j), 0.00390625f, lev(6, j)));
+                        }
+                    }
+                }
+                if constexpr (!COMP && KIND != GK_D64) {
 #pragma unroll 1
                     for (int c0 = half * 32; c0 < d.bn; c0 += 64) {
                         uint32_t r[32];
                         if (split) tmem_ld32_sum(acc + (uint32_t)c0, acc + small_off + (uint32_t)c0, r);
                         else tmem_ld32(acc + (uint32_t)c0, r);
+                        if constexpr (KIND == GK_D32) {  // powers of two: 2^eA of the row, 2^eB of each column
+                            const int *ce = cE[it & 1] + c0;
+                            const float up = __uint_as_float((unsigned)(rowE + 1) << 23);
+#pragma unroll
+                            for (int j = 0; j < 32; ++j)
+                                r[j] = __float_as_uint(__uint_as_float(r[j]) * up * __uint_as_float((unsigned)(ce[j] + 1) << 23));
+                        }
                         store_row(r, C, om, c0, lin, on0, nval, cn, alpha, d.beta, d.init);
                     }
                 }
@@ -536,6 +892,22 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                 if (++buf == nbuf) buf = 0, aph ^= 1u;
             }
             if (aborted) continue;
+            if constexpr (KIND == GK_D64) {
+                // (the next tile accumulates meanwhile)
+                const int *ce = cE[it & 1];
+                if (om >= 0) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) {
+                        const int cc = half * 32 + j;
+                        if (cc >= nval) break;
+                        double *q = (double *)d.C + om + (lin != 0 ? on0 + (int64_t)cc * lin : cn[cc]);
+                        double v = fixed_to_double(dhi[j], dlo[j], rowE + ce[cc] - 2104);
+                        // (FP64 instructions cost 16 clocks a warp)
+                        if (plain) *q = v;
+                        else *q = d.init == 2 ? d.alpha64 * v : fma(d.alpha64, v, d.beta64 * *q);
+                    }
+                }
+            }
             if constexpr (COMP) {
                 // (the next tile's first chunk accumulates meanwhile)
 #pragma unroll
@@ -721,7 +1093,190 @@ tc_status run_packed(Plan &p, PackedDesc &d, bool comp, int64_t comp_k, double f
     return t.pair ? launch_gett<KIND, false, true>(d, ta, tb, st) : launch_gett<KIND, false, false>(d, ta, tb, st);
 }
 
+// ---- digits, host side
+constexpr int64_t kDigitPanelBytes = int64_t(64) << 20;  // images of one panel of B: half of L2
+constexpr int64_t kDigitMaxABytes = int64_t(256) << 20;
+constexpr int64_t kDigitMinK = 32;       // where the bound of the digits meets the chain's
+constexpr int64_t kDigitMaxTiles = int64_t(1) << 22;
+
+struct DigitPlan {
+    bool pair;
+    int64_t tiles_m, tiles_n, panel_tiles;  // panel_tiles: columns of tiles per panel of B
+    int64_t rows_a, image_a, image_b;       // padded rows of A; bytes of A's images and of a panel's
+    int64_t off_b, off_exp_a, off_exp_b, off_small_a, off_small_b, off_list, zero_bytes, bytes;
+};
+
+// The digit form of an M x N x K product, or false where SIMT is the faster
+// estimate or the form does not apply.  Clocks per 16 K positions as
+// choose_tile counts them (the shared-memory port), plus what draining the
+// levels of a unit costs; SIMT at its measured rates.
+template <int KIND>
+bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
+    using D = Digits<KIND>;
+    using T = Traits<KIND>;
+    constexpr int BK = stage_k<KIND>(), S = T::kSlices;
+    if (K < kDigitMinK || K > D::kMaxK) return false;
+    const int64_t Kp = (K + BK - 1) / BK * BK;
+    double best = -1;
+    for (int pair = 1; pair >= 0; --pair) {
+        const int64_t rows = pair ? 2 * kRows : kRows, slots = pair ? sm_count() / 2 : sm_count();
+        if (slots < 1) continue;
+        DigitPlan q;
+        q.pair = pair != 0;
+        q.tiles_m = (M + rows - 1) / rows;
+        q.tiles_n = (N + D::kBn - 1) / D::kBn;
+        if (q.tiles_n > kDigitMaxTiles / q.tiles_m) continue;
+        q.rows_a = q.tiles_m * rows;
+        q.image_a = q.rows_a * Kp * S * 2;
+        if (q.image_a > kDigitMaxABytes) continue;
+        // panels that fill whole waves
+        int64_t pt = std::max<int64_t>(1, kDigitPanelBytes / (Kp * S * 2 * D::kBn));
+        if (pt < q.tiles_n && pt * q.tiles_m > slots) pt = std::max<int64_t>(1, pt * q.tiles_m / slots * slots / q.tiles_m);
+        q.panel_tiles = std::min(pt, q.tiles_n);
+        q.image_b = q.panel_tiles * D::kBn * Kp * S * 2;
+        const int64_t panels = (q.tiles_n + q.panel_tiles - 1) / q.panel_tiles;
+        const int brows = pair ? D::kBn / 2 : D::kBn, nprod = S * (S + 1) / 2;
+        const double port = ((4096.0 + 32.0 * brows) * nprod + 32.0 * (kRows + brows) * S) / 128.0;
+        const double tile = (Kp / 16) * std::max(D::kBn / 2.0 * nprod, port) +
+                            (D::F64 ? (K + D::kChunkK - 1) / D::kChunkK * 6000.0 : 0.0) + 3000.0;
+        const int64_t waves = (panels - 1) * ((q.panel_tiles * q.tiles_m + slots - 1) / slots) +
+                              ((q.tiles_n - (panels - 1) * q.panel_tiles) * q.tiles_m + slots - 1) / slots;
+        const double pack = (double)(q.rows_a + q.tiles_n * D::kBn) * Kp * (sizeof(typename D::In) + S * 2) / 3e12;
+        const double sec = waves * tile / 1.9e9 + pack + 12e-6 + panels * 6e-6;
+        if (best < 0 || sec < best) {
+            best = sec;
+            P = q;
+        }
+    }
+    if (best < 0) return false;
+    const double simt = 2.0 * (double)M * (double)N * (double)K / (D::F64 ? 1.24e12 : 37e12);
+    if (best > 0.8 * simt) return false;
+    auto up = [](int64_t x) { return (x + 511) / 512 * 512; };
+    P.off_b = P.image_a;
+    P.off_exp_a = P.off_b + P.image_b;
+    P.off_exp_b = P.off_exp_a + up(P.rows_a * 4);
+    // zeroed before each execute: the row tiles' counts and the list's length
+    P.off_small_a = P.off_exp_b + up(P.panel_tiles * D::kBn * 4);
+    P.off_small_b = P.off_small_a + up(P.rows_a / kRows * 4);
+    P.off_list = P.off_small_b + up(P.tiles_n * 2 * 4);
+    P.zero_bytes = P.off_list + 8 - P.off_small_a;
+    P.bytes = P.off_list + up((P.tiles_m * P.tiles_n + 1) * 8);
+    return true;
+}
+
+template <int KIND>
+tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta, double fraction, cudaStream_t st,
+                     bool *done) {
+    using D = Digits<KIND>;
+    using T = Traits<KIND>;
+    constexpr int BK = stage_k<KIND>();
+    DigitPlan P;
+    if (!plan_digits<KIND>(d.M, d.N, d.K, P)) return TC_SUCCESS;
+    if (p.digit_bytes < (size_t)P.bytes) {
+        // taken once, by the first execute outside a capture; without it the
+        // SIMT tiles run
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return TC_SUCCESS;
+        }
+        if (p.digit_ws) cudaFree(p.digit_ws);
+        p.digit_ws = nullptr;
+        p.digit_bytes = 0;
+        if (cudaMalloc(&p.digit_ws, (size_t)P.bytes) != cudaSuccess) {
+            cudaGetLastError();
+            p.digit_ws = nullptr;
+            return TC_SUCCESS;
+        }
+        p.digit_bytes = (size_t)P.bytes;
+    }
+    tc_status s = ensure_device_resources(p, 0);
+    if (s != TC_SUCCESS) return s;
+    char *ws = (char *)p.digit_ws;
+    if constexpr (D::F64) {
+        d.alpha64 = *(const double *)alpha;
+        d.beta64 = *(const double *)beta;
+        d.init = d.beta64 == 0.0 ? 2 : 1;
+    } else {
+        d.alpha = *(const float *)alpha;
+        d.beta = *(const float *)beta;
+        d.init = d.beta == 0.0f ? 2 : 1;
+    }
+    int64_t tiles_n = P.tiles_n;
+    const int64_t N = fraction < 1.0 ? std::min<int64_t>(d.N, std::max<int64_t>(D::kBn, (int64_t)(d.N * fraction))) : d.N;
+    tiles_n = (N + D::kBn - 1) / D::kBn;
+    d.status = p.dev_status;
+    d.bn = D::kBn;
+    d.brows = P.pair ? D::kBn / 2 : D::kBn;
+    d.tiles_m = P.tiles_m;
+    d.ktiles = (int)((d.K + BK - 1) / BK);
+    d.chunk = std::min(d.ktiles, D::kChunkK / BK);
+    d.img_a = (uint32_t)(T::kSlices * kRows * BK * 2);
+    d.img_b = (uint32_t)(T::kSlices * d.brows * BK * 2);
+    d.stages = std::min<int>(kMaxStages, kRingBytes / (int)(d.img_a + d.img_b));
+    d.exps[0] = (int *)(ws + P.off_exp_a);
+    d.exps[1] = (int *)(ws + P.off_exp_b);
+    d.small[0] = (int *)(ws + P.off_small_a);
+    d.small[1] = (int *)(ws + P.off_small_b);
+    d.list = (int64_t *)(ws + P.off_list);
+    CUtensorMap ta, tb;
+    s = image_map(ta, ws, P.image_a, d.img_a);
+    if (s == TC_SUCCESS) s = image_map(tb, ws + P.off_b, P.image_b, d.img_b);
+    if (s != TC_SUCCESS) return s;
+    constexpr int kPackSmem = kDigitK * (kPackRows + 1) * (int)sizeof(typename D::In);
+    static bool configured = false;
+    if (!configured) {
+        const cudaError_t ea = cudaFuncSetAttribute(pack_digits_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPackSmem);
+        if (ea != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(ea));
+        configured = true;
+    }
+    cudaError_t e = cudaMemsetAsync(ws + P.off_small_a, 0, (size_t)P.zero_bytes, st);
+    if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
+    for (int64_t t0 = 0; t0 < tiles_n; t0 += P.panel_tiles) {
+        d.n_begin = t0 * D::kBn;
+        d.tiles_n = std::min(P.panel_tiles, tiles_n - t0);
+        d.N = std::min<int64_t>(N - d.n_begin, d.tiles_n * D::kBn);
+        d.num_tiles = d.tiles_m * d.tiles_n;
+        PackJob ja = {}, jb = {};
+        ja.op = 0;
+        ja.rows = kRows;
+        ja.total_rows = P.rows_a;
+        ja.rfast = d.nm > 0 && d.m_sA[0] < d.k_sA[d.nk - 1];
+        ja.out = ws;
+        ja.blocks = t0 == 0 ? (ja.total_rows + kPackRows - 1) / kPackRows : 0;  // A's with the first panel
+        jb.op = 1;
+        jb.rows = d.brows;
+        jb.total_rows = d.tiles_n * D::kBn;
+        jb.rfast = d.nn > 0 && d.n_sB[0] < d.k_sB[d.nk - 1];
+        jb.out = ws + P.off_b;
+        jb.blocks = (jb.total_rows + kPackRows - 1) / kPackRows;
+        pack_digits_kernel<KIND><<<(unsigned)(ja.blocks + jb.blocks), kPackThreads, kPackSmem, st>>>(d, ja, jb);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
+        s = P.pair ? launch_gett<KIND, false, true>(d, ta, tb, st) : launch_gett<KIND, false, false>(d, ta, tb, st);
+        if (s != TC_SUCCESS) return s;
+    }
+    s = simt_run_list(p, alpha, d.A, d.B, beta, d.C, d.list, P.tiles_m, P.pair ? 2 * kRows : kRows, D::kBn, st);
+    if (s == TC_SUCCESS) *done = true;
+    return s;
+}
+
 }  // namespace
+
+tc_status exec_digits(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C, void *stream,
+                      double fraction, bool *done) {
+    *done = false;
+    if (!p.batch.empty() || p.contracted.empty()) return TC_SUCCESS;
+    PackedDesc d;
+    std::memset(&d, 0, sizeof(d));
+    tc_status s = describe_modes(p, 3, d);
+    if (s != TC_SUCCESS) return s;
+    d.A = A;
+    d.B = B;
+    d.C = C;
+    if (p.dtype == TC_F64) return run_digits<GK_D64>(p, d, alpha, beta, fraction, (cudaStream_t)stream, done);
+    return run_digits<GK_D32>(p, d, alpha, beta, fraction, (cudaStream_t)stream, done);
+}
 
 int64_t packed_bytes(tc_dtype dt, int64_t M, int64_t N, int64_t K) {
     int img = 6, bk = stage_k<GK_BF16X3>();

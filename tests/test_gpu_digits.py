@@ -1,0 +1,129 @@
+"""Large FP64 / FP32 GETTs as exact digits on the tensor cores: exact on
+integers, within the stated bound of |A||B| on uniform entries (and closer
+than one rounding per term), rows and columns at the edges of tiles and of
+panels, and the tiles that the digits may not compute -- wide ranges and
+zeros along K, infinities and NaN, exponents near the ends -- left to the
+SIMT tiles bit for bit."""
+import numpy as np
+import pytest
+
+from paper_1409_8608_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+NP = {"f64": np.float64, "f32": np.float32}
+U = {"f64": 2.0 ** -53, "f32": 2.0 ** -24}
+# M, N, K large enough for the digits to be the faster estimate
+SIZES = {"f64": [(300, 4000, 257), (129, 9001, 130)], "f32": [(700, 16001, 301), (513, 30000, 256)]}
+
+
+@pytest.fixture(scope="module")
+def tcmod():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+    __graft_entry__.build_library()
+    from paper_1409_8608_gb300 import tc
+    tc.load()
+    return tc
+
+
+def execute(tc, dtype, A, B, C0=None, alpha=1.0, beta=0.0, spec="ab=ai,ib"):
+    """A (M, K) and B (K, N) as the spec's dense operands; returns C (M, N)
+    and the same product by SIMT (a plan whose strides give B a batch index
+    of extent 1, which only the SIMT tiles take)."""
+    M, K = A.shape
+    N = B.shape[1]
+    lay = {"ab=ai,ib": (A.T, B.T), "ab=ia,bi": (A, B)}[spec]  # reversed modes, C order
+    dA, dB = (torch.from_numpy(np.ascontiguousarray(x)).cuda().reshape(-1) for x in lay)
+    out = []
+    for s, ext in ((spec, {"a": M, "b": N, "i": K}),
+                   (spec.replace("=", "h=").replace(",", "h,") + "h", {"a": M, "b": N, "i": K, "h": 1})):
+        plan = tc.Plan(s, [ext[c] for c in synth.index_order(s)], dtype=dtype)
+        dC = torch.full((N, M), float("nan"), dtype=dA.dtype, device="cuda:0") if C0 is None else \
+            torch.from_numpy(np.ascontiguousarray(C0.T)).cuda()
+        plan.execute(dA, dB, dC, alpha=alpha, beta=beta)
+        torch.cuda.synchronize()
+        plan.device_status()
+        plan.close()
+        out.append(dC.cpu().numpy().T)
+    return out
+
+
+@pytest.mark.parametrize("spec", ["ab=ai,ib", "ab=ia,bi"])
+@pytest.mark.parametrize("dtype,size", [(d, s) for d in SIZES for s in SIZES[d]])
+def test_exact_on_integers(tcmod, dtype, size, spec):
+    M, N, K = size
+    rng = np.random.default_rng(5)
+    top = 2 ** 22 if dtype == "f64" else 100  # sums below 2^53 and 2^24
+    A, B = rng.integers(-top, top + 1, (M, K)), rng.integers(-top, top + 1, (K, N))
+    A[3] = 0  # a row of zeros
+    want = (torch.from_numpy(A).double().cuda() @ torch.from_numpy(B).double().cuda()).cpu().numpy()
+    got, simt = execute(tcmod, dtype, A.astype(NP[dtype]), B.astype(NP[dtype]), spec=spec)
+    assert np.array_equal(got, want) and np.array_equal(simt, want)
+    C0 = rng.integers(-50, 50, (M, N)).astype(NP[dtype])
+    got, _ = execute(tcmod, dtype, A.astype(NP[dtype]), B.astype(NP[dtype]), C0, 0.5, -2.0, spec=spec)
+    assert np.array_equal(got, (0.5 * want - 2.0 * C0).astype(NP[dtype]))
+
+
+@pytest.mark.parametrize("dtype,size", [(d, s) for d in SIZES for s in SIZES[d]])
+def test_error_on_uniform(tcmod, dtype, size):
+    M, N, K = size
+    rng = np.random.default_rng(6)
+    A, B = (rng.uniform(-1, 1, s).astype(NP[dtype]) for s in ((M, K), (K, N)))
+    got, simt = execute(tcmod, dtype, A, B)
+    i, j = rng.integers(0, M, 2000), rng.integers(0, N, 2000)
+    terms = A[i].astype(np.longdouble) * B[:, j].T.astype(np.longdouble)
+    want, scale = terms.sum(1), np.abs(terms).sum(1)
+    err = np.abs(got[i, j] - want)
+    # rounded once: half a unit in the last place, and the digits left out
+    # (2^-59 or 2^-28 of at most |x|, |y| < 1 per term; FP32 also the rounding
+    # of the 9 K / 16 additions of levels 1 to 3 at 2^-7 of the sum's size)
+    left = K * 2.0 ** -59 if dtype == "f64" else K * 2.0 ** -28 + 9 * K / 16 * 2.0 ** -24 * 2.0 ** -6 * K ** 0.5
+    assert np.all(err <= U[dtype] * np.abs(want) * 1.01 + left), float(np.max(err / scale))
+    # and no further off than the chain of fused multiply-adds
+    assert np.linalg.norm(err) <= np.linalg.norm(simt[i, j] - want)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_extreme_digits(tcmod, dtype):
+    # every digit at its end: the level sums reach their bound
+    M, N, K = SIZES[dtype][0]
+    x = np.nextafter(NP[dtype](1), NP[dtype](0))
+    for a, b in ((x, x), (-x, x), (x, NP[dtype](0.50390625)), (NP[dtype](-0.50196), x)):
+        A, B = np.full((M, K), a, NP[dtype]), np.full((K, N), b, NP[dtype])
+        got, _ = execute(tcmod, dtype, A, B)
+        want = np.longdouble(a) * np.longdouble(b) * K
+        left = K * 2.0 ** (-59 if dtype == "f64" else -28)
+        if dtype == "f32":
+            # the 9 K / 16 additions of levels 1 to 3, whose sum is at most
+            # K 2^-6, each truncated to 24 bits
+            left += 9 * K / 16 * 2.0 ** -23 * K * 2.0 ** -6
+        assert np.all(np.abs(got - want) <= U[dtype] * abs(want) * 1.01 + left)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_left_to_simt(tcmod, dtype):
+    M, N, K = SIZES[dtype][0]
+    rng = np.random.default_rng(7)
+    A, B = (rng.uniform(0.5, 1, s).astype(NP[dtype]) for s in ((M, K), (K, N)))
+    tiny, huge = (1e-310, 1e300) if dtype == "f64" else (1e-42, 1e37)
+    A[5, 1], A[6, 2] = np.inf, np.nan
+    B[3, 70] = -np.inf
+    A[7] = tiny
+    A[8, :] = huge
+    A[280, : K // 2 + 9] = 0              # mostly zeros along K
+    A[281] *= NP[dtype](2.0) ** -np.arange(K, dtype=NP[dtype])  # wide range along K
+    B[:, N - 1] = 0
+    B[0, N - 1] = 1
+    got, simt = execute(tcmod, dtype, A, B)
+    bad = np.zeros((M, N), bool)
+    bad[[5, 6, 7, 8, 280, 281]] = True
+    bad[:, [70, N - 1]] = True
+    assert np.array_equal(got[bad], simt[bad], equal_nan=True)
+    i, j = np.nonzero(~bad)
+    pick = rng.integers(0, len(i), 2000)
+    i, j = i[pick], j[pick]
+    want = (A[i].astype(np.longdouble) * B[:, j].T.astype(np.longdouble)).sum(1)
+    assert np.all(np.abs(got[i, j] - want) <= K * U[dtype] * np.abs(want))
