@@ -1470,9 +1470,10 @@ bool encoder() {
 // TMA cannot describe it (the operand then takes the global-load path).
 // nrow/row_ext/row_s: the operand's row modes (M for A, N for B), first
 // mode fastest; K modes as in the descriptor (outermost first).
+// map == nullptr: only whether it can be described.
 bool plan_tma_operand(const Plan &p, int opnd, const void *base, int in_bytes, int rows, int nrow,
                       const int64_t *row_ext, const int64_t *row_s, int nk, const int64_t *k_ext,
-                      const int64_t *k_s, GettDesc &d, CUtensorMap &map, int kpb) {
+                      const int64_t *k_s, GettDesc &d, CUtensorMap *map, int kpb) {
     const int o = opnd == OP_A ? 0 : 1;
     if (((uintptr_t)base & 15) != 0 || nrow < 1) return false;
     if (row_ext[0] % rows != 0) return false;  // tiles must be boxes of the first row mode
@@ -1558,6 +1559,7 @@ bool plan_tma_operand(const Plan &p, int opnd, const void *base, int in_bytes, i
     if (d.srow[o] % 4 != 0 || in_bytes != 4) v4 = false;
     d.sk_vec4[o] = v4 ? 1 : 0;
     if (K < kpb || K % kpb != 0) return false;  // every box covers kpb valid K positions
+    if (!map) return true;
     // encode (rank 5: unused dimensions have extent 1)
     if (!encoder()) return false;
     cuuint64_t gdim[kTmaRank], gstride[kTmaRank - 1];
@@ -1575,7 +1577,7 @@ bool plan_tma_operand(const Plan &p, int opnd, const void *base, int in_bytes, i
     CUtensorMapDataType dt = in_bytes == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                            : (p.dtype == TC_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                                                 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
-    CUresult r = g_encode(&map, dt, kTmaRank, const_cast<void *>(base), gdim, gstride, box, estr,
+    CUresult r = g_encode(map, dt, kTmaRank, const_cast<void *>(base), gdim, gstride, box, estr,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return false;
@@ -1793,6 +1795,30 @@ static tc_status e4m3_scales(Plan &p, const void *A, const void *B, cudaStream_t
     return TC_SUCCESS;
 }
 
+// Automatic pre-conversion beyond pack_choice: both inputs as images in
+// optional scratch.  Measured (us, images / the inputs as they are, split-
+// BF16, TF32, BF16): K = 256 512 x 512^2 386 / 426, 257 / 356, 211 / 740 and
+// up to 11 x faster where few tiles have a long K (256^2, K = 4096, 23 / 393);
+// K = 143 301 x 19691 25 / 45, 21 / 42, 19 / 35; K = 64 300 x 200000 (ragged)
+// 91 / 120, 83 / 134, 77 / 95 but 512 x 512^2 181 / 151, 154 / 136, 145 / 153;
+// K = 16 512 x 512^2 147 / 115, 143 / 112, 142 / 110, K = 25 81 x 18190 10 /
+// 12, 12 / 12, 12 / 10.  So: from K = 128 always, from K = 48 unless TMA
+// stages both inputs of a large result, below only the split forms of a small
+// result.  (d, pk: the modes and the choice without this.)
+static bool images_win(const Plan &p, const GettModes &d, int pk) {
+    if (p.gett_pack != 1 || d.nb != 0 || d.K > (int64_t(1) << 24)) return false;
+    if (d.K >= 128) return true;
+    if (d.K < 48) return (p.dtype == TC_BF16X3 || p.dtype == TC_TF32X3) && d.M * d.N <= (int64_t(1) << 22);
+    if (p.dtype == TC_E4M3 || d.M * d.N < (int64_t(1) << 24)) return true;
+    const int in_bytes = (p.dtype == TC_BF16 || p.dtype == TC_F16) ? 2 : 4;
+    GettDesc t;
+    std::memset(&t, 0, sizeof(t));
+    return !((pk == 1 || plan_tma_operand(p, OP_A, nullptr, in_bytes, kBM, d.nm, d.m_ext, d.m_sA, d.nk, d.k_ext, d.k_sA, t,
+                                          nullptr, kBKT)) &&
+             (pk == 2 || plan_tma_operand(p, OP_B, nullptr, in_bytes, 256, d.nn, d.n_ext, d.n_sB, d.nk, d.k_ext, d.k_sB, t,
+                                          nullptr, kBKT)));
+}
+
 tc_status exec_gett(Plan &p, const void *alpha, const void *A, const void *B, const void *beta,
                     void *C, void *stream, const Probe *probe) {
     if (p.dtype == TC_F64 || p.dtype == TC_F32) {
@@ -1838,7 +1864,13 @@ tc_status exec_gett(Plan &p, const void *alpha, const void *A, const void *B, co
         if (s != TC_SUCCESS) return s;
     }
     if (pk == 3)
-        return exec_packed(p, alpha, A, B, beta, C, stream, probe ? probe->fraction : 1.0, comp_k, d.split != 0, d.qscale);
+        return exec_packed(p, alpha, A, B, beta, C, stream, probe ? probe->fraction : 1.0, comp_k, d.split != 0, d.qscale,
+                           nullptr);
+    if (images_win(p, d, pk)) {
+        bool done = false;
+        s = exec_packed(p, alpha, A, B, beta, C, stream, probe ? probe->fraction : 1.0, comp_k, d.split != 0, d.qscale, &done);
+        if (s != TC_SUCCESS || done) return s;
+    }
     // TMA staging for each operand TMA can describe (tiles of 128 x bn, or
     // in a CTA pair 128 rows of A and bn / 2 rows of B per CTA)
     CUtensorMap tmA, tmB;
@@ -1848,9 +1880,9 @@ tc_status exec_gett(Plan &p, const void *alpha, const void *A, const void *B, co
     d.spb = 1;
     auto plan_tma = [&](GettDesc &dd, CUtensorMap &ma, CUtensorMap &mb, int brows) -> bool {
         dd.tma[0] = pk != 1 && plan_tma_operand(p, OP_A, A, in_bytes, kBM, dd.nm, dd.m_ext, dd.m_sA, dd.nk, dd.k_ext,
-                                                dd.k_sA, dd, ma, kBKT);
+                                                dd.k_sA, dd, &ma, kBKT);
         dd.tma[1] = pk != 2 && plan_tma_operand(p, OP_B, B, in_bytes, brows, dd.nn, dd.n_ext, dd.n_sB, dd.nk,
-                                                dd.k_ext, dd.k_sB, dd, mb, kBKT);
+                                                dd.k_ext, dd.k_sB, dd, &mb, kBKT);
         bool any = dd.tma[0] || dd.tma[1];
         // boxes of two stages where the K modes allow them for at least as
         // many operands: each TMA box costs a fixed few hundred cycles on top
@@ -1861,9 +1893,9 @@ tc_status exec_gett(Plan &p, const void *alpha, const void *A, const void *B, co
             std::memset(&a2, 0, sizeof(a2));
             std::memset(&b2, 0, sizeof(b2));
             const bool ta = pk != 1 && plan_tma_operand(p, OP_A, A, in_bytes, kBM, dd.nm, dd.m_ext, dd.m_sA, dd.nk,
-                                                        dd.k_ext, dd.k_sA, d2, a2, kBoxK);
+                                                        dd.k_ext, dd.k_sA, d2, &a2, kBoxK);
             const bool tb = pk != 2 && plan_tma_operand(p, OP_B, B, in_bytes, brows, dd.nn, dd.n_ext, dd.n_sB, dd.nk,
-                                                        dd.k_ext, dd.k_sB, d2, b2, kBoxK);
+                                                        dd.k_ext, dd.k_sB, d2, &b2, kBoxK);
             if ((ta || tb) && (int)ta + (int)tb >= (int)(bool)dd.tma[0] + (int)(bool)dd.tma[1]) {
                 dd = d2;
                 dd.tma[0] = ta;

@@ -76,8 +76,8 @@ struct Plan {
     void *host_dev[3] = {nullptr, nullptr, nullptr};  // tc_execute_host: device copies of A, B, C
     size_t host_dev_bytes[3] = {0, 0, 0};
     void *gett_state = nullptr;     // owned by the GETT executor
-    void *digit_ws = nullptr;       // TC_F64 / TC_F32: digit images of a large GETT (tc_packed.cu)
-    size_t digit_bytes = 0;
+    void *scratch = nullptr;        // GETT: images that an execute can do without (tc_packed.cu)
+    size_t scratch_bytes = 0;
     void *qbuf = nullptr;           // TC_E4M3: the inputs' maxima and scales (16 bytes)
     void *flush_buf = nullptr;      // predictor: remote regions / L2 flush
     size_t flush_bytes = 0;
@@ -144,10 +144,12 @@ tc_status describe_modes(const Plan &p, int pk, GettModes &d);
 
 // The tensor-core GETT with both inputs pre-converted (tc_packed.cu): the
 // bytes of their images, and one execute.  comp_k > 0: compensated over
-// chunks of comp_k; qscale: E4M3's input scales.
+// chunks of comp_k; qscale: E4M3's input scales.  With done the images go to
+// optional scratch instead of the workspace, and *done = false, with nothing
+// enqueued, where that is not to be had.
 int64_t packed_bytes(tc_dtype dt, int64_t M, int64_t N, int64_t K);
 tc_status exec_packed(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
-                      void *stream, double fraction, int64_t comp_k, bool split, const float *qscale);
+                      void *stream, double fraction, int64_t comp_k, bool split, const float *qscale, bool *done);
 
 // A large FP64 / FP32 GETT as exact digits on the tensor cores (tc_packed.cu);
 // *done = false, with nothing enqueued, where the SIMT tiles are to run.

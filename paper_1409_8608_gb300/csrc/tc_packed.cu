@@ -118,11 +118,10 @@ struct PackedDesc : GettModes {
     int nprod, split;
     int *status;
     const float *qscale;        // E4M3: the inputs' scales
-    // digits: first column of the panel (N then counts the panel's), scalars
-    // in FP64, per row the exponent field of its largest magnitude, per
+    int64_t n_begin;            // first column of the panel (N then counts the panel's)
+    // digits: scalars in FP64, per row the exponent field of its largest magnitude, per
     // image row tile the most small entries of a row, and the tiles left to
     // SIMT (list[0]: how many)
-    int64_t n_begin;
     double alpha64, beta64;
     int *exps[2], *small[2];
     int64_t *list;
@@ -177,7 +176,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_images_kernel(const __grid_
         if (r < (J.op == 0 ? d.M : d.N)) {
             o = 0;
             if (J.op == 0) decode(r, d.nm, d.m_ext, d.m_sA, d.m_sC, o, u);
-            else decode(r, d.nn, d.n_ext, d.n_sB, d.n_sC, o, u);
+            else decode(r + d.n_begin, d.nn, d.n_ext, d.n_sB, d.n_sC, o, u);
         }
         roff[tid - kPackK] = o;
     }
@@ -1038,64 +1037,111 @@ tc_status launch_gett(const PackedDesc &d, const CUtensorMap &ta, const CUtensor
     return e == cudaSuccess ? TC_SUCCESS : fail(TC_ERROR_CUDA, cudaGetErrorString(e));
 }
 
+constexpr int64_t kPanelBytes = int64_t(64) << 20;       // images of one panel of B: half of L2
+constexpr int64_t kScratchMaxABytes = int64_t(256) << 20;
+
+// Scratch that an execute can do without: taken once, outside a capture, and
+// kept.  False: not to be had, the caller runs the form without it.
+bool optional_scratch(Plan &p, int64_t bytes, cudaStream_t st) {
+    if (p.scratch_bytes >= (size_t)bytes) return true;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    if (p.scratch) cudaFree(p.scratch);
+    p.scratch = nullptr;
+    p.scratch_bytes = 0;
+    if (cudaMalloc(&p.scratch, (size_t)bytes) != cudaSuccess) {
+        cudaGetLastError();
+        p.scratch = nullptr;
+        return false;
+    }
+    p.scratch_bytes = (size_t)bytes;
+    return true;
+}
+
+// Tiles of B per panel: whole waves where B takes several panels.
+int64_t panel_tiles_for(int64_t tiles_n, int64_t tiles_m, int64_t tile_bytes, int64_t slots) {
+    int64_t pt = std::max<int64_t>(1, kPanelBytes / tile_bytes);
+    if (pt < tiles_n && pt * tiles_m > slots) pt = std::max<int64_t>(1, pt * tiles_m / slots * slots / tiles_m);
+    return std::min(pt, tiles_n);
+}
+
+// done == nullptr: the images in the plan's workspace, B as a whole.  Else in
+// optional scratch, B in panels; *done tells whether it ran.
 template <int KIND>
-tc_status run_packed(Plan &p, PackedDesc &d, bool comp, int64_t comp_k, double fraction, cudaStream_t st) {
+tc_status run_packed(Plan &p, PackedDesc &d, bool comp, int64_t comp_k, double fraction, cudaStream_t st, bool *done) {
     using T = Traits<KIND>;
     constexpr int BK = stage_k<KIND>();
     const int nprod = KIND == GK_BF16X3 ? d.nprod : (KIND == GK_TF32X3 ? 3 : 1);
     int max_bn = comp ? 128 : (p.gett_bn == 128 ? 128 : kMaxBn);
-    Tile t = choose_tile(d.M, d.N, (double)((d.K * T::kElemBytes + 31) / 32), nprod, T::kSlices, max_bn, d.split != 0);
+    d.ktiles = (int)((d.K + BK - 1) / BK);
+    const int64_t col_bytes = (int64_t)d.ktiles * BK * T::kSlices * T::kElemBytes;
+    const int64_t panel_n = done ? std::min(d.N, std::max<int64_t>(kMaxBn, kPanelBytes / col_bytes)) : d.N;
+    Tile t = choose_tile(d.M, panel_n, (double)((d.K * T::kElemBytes + 31) / 32), nprod, T::kSlices, max_bn, d.split != 0);
     if (p.gett_pair && d.M > kRows) t.pair = true;
-    if (fraction < 1.0) d.N = std::min<int64_t>(d.N, std::max<int64_t>(t.bn, (int64_t)(d.N * fraction)));
+    const int64_t N = fraction < 1.0 ? std::min<int64_t>(d.N, std::max<int64_t>(t.bn, (int64_t)(d.N * fraction))) : d.N;
     d.bn = t.bn;
     d.brows = t.pair ? t.bn / 2 : t.bn;
     const int64_t rows = t.pair ? 2 * kRows : kRows;
     d.tiles_m = (d.M + rows - 1) / rows;
-    d.tiles_n = (d.N + d.bn - 1) / d.bn;
-    d.num_tiles = d.tiles_m * d.tiles_n;
-    d.ktiles = (int)((d.K + BK - 1) / BK);
     d.chunk = comp ? (int)(comp_k / BK) : d.ktiles;
     d.img_a = (uint32_t)(T::kSlices * kRows * BK * T::kElemBytes);
     d.img_b = (uint32_t)(T::kSlices * d.brows * BK * T::kElemBytes);
     d.stages = std::min<int>(kMaxStages, kRingBytes / (int)(d.img_a + d.img_b));
+    const int64_t tiles_n = (N + d.bn - 1) / d.bn;
+    const int64_t panel = done ? panel_tiles_for((d.N + d.bn - 1) / d.bn, d.tiles_m, d.bn * col_bytes, sm_count() / (t.pair ? 2 : 1))
+                               : tiles_n;
+    const int64_t bytes_a = d.tiles_m * rows * col_bytes, bytes_b = panel * d.bn * col_bytes;
+    tc_status s = ensure_device_resources(p, done ? 0 : (size_t)packed_bytes(p.dtype, d.M, N, d.K));
+    if (s != TC_SUCCESS) return s;
+    if (done && (bytes_a > kScratchMaxABytes || !optional_scratch(p, bytes_a + bytes_b, st))) return TC_SUCCESS;
+    d.status = p.dev_status;
     PackJob ja = {}, jb = {};
     ja.op = 0;
     ja.rows = kRows;
     ja.total_rows = d.tiles_m * rows;
+    ja.out = (char *)(done ? p.scratch : p.workspace);
     jb.op = 1;
     jb.rows = d.brows;
-    jb.total_rows = d.tiles_n * d.bn;
-    const int64_t bytes_a = ja.total_rows / ja.rows * d.ktiles * (int64_t)d.img_a;
-    const int64_t bytes_b = jb.total_rows / jb.rows * d.ktiles * (int64_t)d.img_b;
-    tc_status s = ensure_device_resources(p, (size_t)packed_bytes(p.dtype, d.M, d.N, d.K));
-    if (s != TC_SUCCESS) return s;
-    d.status = p.dev_status;
-    ja.out = (char *)p.workspace;
     jb.out = ja.out + bytes_a;
     // lanes along whichever of the first row mode and the innermost K mode
     // has the smaller stride
     ja.rfast = d.nm > 0 && (d.nk == 0 || d.m_sA[0] < d.k_sA[d.nk - 1]);
     jb.rfast = d.nn > 0 && (d.nk == 0 || d.n_sB[0] < d.k_sB[d.nk - 1]);
     const int64_t kblocks = ((int64_t)d.ktiles * BK + kPackK - 1) / kPackK;
-    ja.blocks = (ja.total_rows + kPackRows - 1) / kPackRows * kblocks;
-    jb.blocks = (jb.total_rows + kPackRows - 1) / kPackRows * kblocks;
-    if (ja.blocks + jb.blocks > 0x7fffffff) return fail(TC_ERROR_INVALID_EXTENT, "too many blocks for the pre-pass");
     CUtensorMap ta, tb;
     s = image_map(ta, ja.out, bytes_a, d.img_a);
     if (s == TC_SUCCESS) s = image_map(tb, jb.out, bytes_b, d.img_b);
     if (s != TC_SUCCESS) return s;
-    pack_images_kernel<KIND><<<(unsigned)(ja.blocks + jb.blocks), kPackThreads, 0, st>>>(d, ja, jb);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
-    if constexpr (KIND == GK_BF16X3 || KIND == GK_TF32X3) {
-        if (comp) return t.pair ? launch_gett<KIND, true, true>(d, ta, tb, st) : launch_gett<KIND, true, false>(d, ta, tb, st);
+    for (int64_t t0 = 0; t0 < tiles_n; t0 += panel) {
+        d.n_begin = t0 * d.bn;
+        d.tiles_n = std::min(panel, tiles_n - t0);
+        d.N = std::min(N - d.n_begin, d.tiles_n * d.bn);
+        d.num_tiles = d.tiles_m * d.tiles_n;
+        jb.total_rows = d.tiles_n * d.bn;
+        ja.blocks = t0 == 0 ? (ja.total_rows + kPackRows - 1) / kPackRows * kblocks : 0;  // A's with the first panel
+        jb.blocks = (jb.total_rows + kPackRows - 1) / kPackRows * kblocks;
+        if (ja.blocks + jb.blocks > 0x7fffffff) return fail(TC_ERROR_INVALID_EXTENT, "too many blocks for the pre-pass");
+        pack_images_kernel<KIND><<<(unsigned)(ja.blocks + jb.blocks), kPackThreads, 0, st>>>(d, ja, jb);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
+        bool launched = false;
+        if constexpr (KIND == GK_BF16X3 || KIND == GK_TF32X3) {
+            if (comp) {
+                s = t.pair ? launch_gett<KIND, true, true>(d, ta, tb, st) : launch_gett<KIND, true, false>(d, ta, tb, st);
+                launched = true;
+            }
+        }
+        if (!launched) s = t.pair ? launch_gett<KIND, false, true>(d, ta, tb, st) : launch_gett<KIND, false, false>(d, ta, tb, st);
+        if (s != TC_SUCCESS) return s;
     }
-    return t.pair ? launch_gett<KIND, false, true>(d, ta, tb, st) : launch_gett<KIND, false, false>(d, ta, tb, st);
+    if (done) *done = true;
+    return TC_SUCCESS;
 }
 
 // ---- digits, host side
-constexpr int64_t kDigitPanelBytes = int64_t(64) << 20;  // images of one panel of B: half of L2
-constexpr int64_t kDigitMaxABytes = int64_t(256) << 20;
 constexpr int64_t kDigitMinK = 32;       // where the bound of the digits meets the chain's
 constexpr int64_t kDigitMaxTiles = int64_t(1) << 22;
 
@@ -1128,11 +1174,8 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
         if (q.tiles_n > kDigitMaxTiles / q.tiles_m) continue;
         q.rows_a = q.tiles_m * rows;
         q.image_a = q.rows_a * Kp * S * 2;
-        if (q.image_a > kDigitMaxABytes) continue;
-        // panels that fill whole waves
-        int64_t pt = std::max<int64_t>(1, kDigitPanelBytes / (Kp * S * 2 * D::kBn));
-        if (pt < q.tiles_n && pt * q.tiles_m > slots) pt = std::max<int64_t>(1, pt * q.tiles_m / slots * slots / q.tiles_m);
-        q.panel_tiles = std::min(pt, q.tiles_n);
+        if (q.image_a > kScratchMaxABytes) continue;
+        q.panel_tiles = panel_tiles_for(q.tiles_n, q.tiles_m, Kp * S * 2 * D::kBn, slots);
         q.image_b = q.panel_tiles * D::kBn * Kp * S * 2;
         const int64_t panels = (q.tiles_n + q.panel_tiles - 1) / q.panel_tiles;
         const int brows = pair ? D::kBn / 2 : D::kBn, nprod = S * (S + 1) / 2;
@@ -1172,27 +1215,10 @@ tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta
     constexpr int BK = stage_k<KIND>();
     DigitPlan P;
     if (!plan_digits<KIND>(d.M, d.N, d.K, P)) return TC_SUCCESS;
-    if (p.digit_bytes < (size_t)P.bytes) {
-        // taken once, by the first execute outside a capture; without it the
-        // SIMT tiles run
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            return TC_SUCCESS;
-        }
-        if (p.digit_ws) cudaFree(p.digit_ws);
-        p.digit_ws = nullptr;
-        p.digit_bytes = 0;
-        if (cudaMalloc(&p.digit_ws, (size_t)P.bytes) != cudaSuccess) {
-            cudaGetLastError();
-            p.digit_ws = nullptr;
-            return TC_SUCCESS;
-        }
-        p.digit_bytes = (size_t)P.bytes;
-    }
+    if (!optional_scratch(p, P.bytes, st)) return TC_SUCCESS;  // the SIMT tiles run
     tc_status s = ensure_device_resources(p, 0);
     if (s != TC_SUCCESS) return s;
-    char *ws = (char *)p.digit_ws;
+    char *ws = (char *)p.scratch;
     if constexpr (D::F64) {
         d.alpha64 = *(const double *)alpha;
         d.beta64 = *(const double *)beta;
@@ -1293,7 +1319,8 @@ int64_t packed_bytes(tc_dtype dt, int64_t M, int64_t N, int64_t K) {
 }
 
 tc_status exec_packed(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C, void *stream,
-                      double fraction, int64_t comp_k, bool split, const float *qscale) {
+                      double fraction, int64_t comp_k, bool split, const float *qscale, bool *done) {
+    if (done) *done = false;
     PackedDesc d;
     std::memset(&d, 0, sizeof(d));
     tc_status s = describe_modes(p, 3, d);
@@ -1310,12 +1337,12 @@ tc_status exec_packed(Plan &p, const void *alpha, const void *A, const void *B, 
     const bool comp = comp_k > 0 && d.K > comp_k;
     cudaStream_t st = (cudaStream_t)stream;
     switch (p.dtype) {
-    case TC_BF16X3: return run_packed<GK_BF16X3>(p, d, comp, comp_k, fraction, st);
-    case TC_BF16: return run_packed<GK_BF16>(p, d, false, 0, fraction, st);
-    case TC_F16: return run_packed<GK_F16>(p, d, false, 0, fraction, st);
-    case TC_TF32: return run_packed<GK_TF32>(p, d, false, 0, fraction, st);
-    case TC_TF32X3: return run_packed<GK_TF32X3>(p, d, comp, comp_k, fraction, st);
-    case TC_E4M3: return run_packed<GK_E4M3>(p, d, false, 0, fraction, st);
+    case TC_BF16X3: return run_packed<GK_BF16X3>(p, d, comp, comp_k, fraction, st, done);
+    case TC_BF16: return run_packed<GK_BF16>(p, d, false, 0, fraction, st, done);
+    case TC_F16: return run_packed<GK_F16>(p, d, false, 0, fraction, st, done);
+    case TC_TF32: return run_packed<GK_TF32>(p, d, false, 0, fraction, st, done);
+    case TC_TF32X3: return run_packed<GK_TF32X3>(p, d, comp, comp_k, fraction, st, done);
+    case TC_E4M3: return run_packed<GK_E4M3>(p, d, false, 0, fraction, st, done);
     default: return fail(TC_ERROR_UNSUPPORTED_DTYPE, "dtype has no pre-converted GETT");
     }
 }

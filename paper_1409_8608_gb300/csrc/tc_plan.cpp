@@ -347,7 +347,7 @@ tc_status tc_plan_destroy(tc_plan plan) {
         if (p.dev_status) cudaFree(p.dev_status);
         if (p.flush_buf) cudaFree(p.flush_buf);
         if (p.qbuf) cudaFree(p.qbuf);
-        if (p.digit_ws) cudaFree(p.digit_ws);
+        if (p.scratch) cudaFree(p.scratch);
         if (p.busy_event) cudaEventDestroy((cudaEvent_t)p.busy_event);
         for (void *d : p.host_dev)
             if (d) cudaFree(d);
