@@ -589,11 +589,24 @@ struct TileOf {
     static constexpr bool F64 = sizeof(T) == 8;
     static constexpr int B = simt_rows(F64, SHAPE);
     static constexpr int TT = B / 16;  // 16 x 16 threads
-    using Smem = TileSmem<T, B, B, 16>;
+    // FP32: the smaller tiles take longer stages, whose barriers and copies
+    // would otherwise cost more than their multiplications (32 x 128 with K =
+    // 5704: 356 stages of 16)
+    static constexpr int BK = F64 ? 16 : 16 << SHAPE;
+    using Smem = TileSmem<T, B, B, BK>;
     static __device__ __forceinline__ void run(const TileDesc &d, int64_t bid, void *buf) {
-        tile_body<T, B, B, 16, TT, TT>(d, bid, *reinterpret_cast<Smem *>(buf));
+        tile_body<T, B, B, BK, TT, TT>(d, bid, *reinterpret_cast<Smem *>(buf));
     }
 };
+
+// shared memory that holds any shape's
+template <typename T>
+__host__ __device__ constexpr size_t tile_smem() {
+    size_t m = sizeof(typename TileOf<T, 0>::Smem);
+    if (sizeof(typename TileOf<T, 1>::Smem) > m) m = sizeof(typename TileOf<T, 1>::Smem);
+    if (sizeof(typename TileOf<T, 2>::Smem) > m) m = sizeof(typename TileOf<T, 2>::Smem);
+    return m;
+}
 
 template <typename T, int SHAPE>
 __global__ void __launch_bounds__(256, 2) tile_kernel(const TileDesc d) {
@@ -610,8 +623,10 @@ __global__ void __launch_bounds__(256, 2) tile_kernel(const TileDesc d) {
 template <typename T>
 __global__ void __launch_bounds__(256, 2)
 tile_batch_kernel(const TileDesc *__restrict__ descs, const int32_t *__restrict__ tile_prob) {
+    constexpr size_t kBytes = tile_smem<T>();
     __shared__ __align__(16) TileDesc sd;
-    __shared__ __align__(16) unsigned char buf[sizeof(typename TileOf<T, 0>::Smem)];
+    __shared__ __align__(16) unsigned char buf[kBytes];
+    static_assert(kBytes >= sizeof(typename TileOf<T, 1>::Smem) && kBytes >= sizeof(typename TileOf<T, 2>::Smem), "every shape fits");
     static_assert(sizeof(TileDesc) % 8 == 0, "descriptor in 8-byte words");
     constexpr int kWords = sizeof(TileDesc) / 8;
     const int q = tile_prob[blockIdx.x];

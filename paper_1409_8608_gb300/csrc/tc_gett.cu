@@ -1808,7 +1808,7 @@ static tc_status e4m3_scales(Plan &p, const void *A, const void *B, cudaStream_t
 static bool images_win(const Plan &p, const GettModes &d, int pk) {
     if (p.gett_pack != 1 || d.nb != 0 || d.K > (int64_t(1) << 24)) return false;
     if (d.K >= 128) return true;
-    if (d.K < 48) return (p.dtype == TC_BF16X3 || p.dtype == TC_TF32X3) && d.M * d.N <= (int64_t(1) << 22);
+    if (d.K < 48) return (p.dtype == TC_BF16X3 || p.dtype == TC_TF32X3) && d.M * d.N <= (int64_t(1) << 21);
     if (p.dtype == TC_E4M3 || d.M * d.N < (int64_t(1) << 24)) return true;
     const int in_bytes = (p.dtype == TC_BF16 || p.dtype == TC_F16) ? 2 : 4;
     GettDesc t;

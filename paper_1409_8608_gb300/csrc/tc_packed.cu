@@ -238,7 +238,6 @@ template <int KIND>
 struct Digits {
     static constexpr bool F64 = KIND == GK_D64;
     using In = typename std::conditional<F64, double, float>::type;
-    static constexpr int kLarge = 4;                  // FP64, large: exponent field at least the row's minus this
     static constexpr int kLow = F64 ? 623 : 77, kHigh = F64 ? 1423 : 177;  // exponent fields taken
     static constexpr int kChunkK = F64 ? 128 : 1 << 12;  // K positions per accumulation
     static constexpr int kBn = F64 ? 64 : 128;        // columns per tile: 8 levels, or two double-buffered accumulators
@@ -353,6 +352,7 @@ __global__ void __launch_bounds__(kPackThreads, Digits<KIND>::F64 ? 2 : 4) pack_
             if (R >= J.total_rows || k >= (int64_t)d.ktiles * BK) break;
             char *dst = out + (k / BK) * (int64_t)(S * slice) + (int)((k % BK) / 8) * (J.rows / 8) * 128;
             if constexpr (D::F64) {
+                constexpr int kLarge = 4;  // large: exponent field at least the row's minus this
                 unsigned long long y[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(kPackThreads, Digits<KIND>::F64 ? 2 : 4) pack_
                     const int ex = (int)(b >> 52) & 2047;
                     const unsigned long long m = ex ? frac | (1ull << 52) : frac;
                     const int sh = E - (ex ? ex : 1);
-                    large += m != 0 && sh <= D::kLarge;
+                    large += m != 0 && sh <= kLarge;
                     // x 2^-e 2^62 = m 2^(9 - sh), rounded where bits fall
                     // under the last digit
                     unsigned long long w;
@@ -443,12 +443,53 @@ __device__ __forceinline__ void image_load(void *dst, const CUtensorMap *map, ui
             : "memory");
 }
 
-// Stores 32 accumulator columns c0.. of this thread's row (C offset om, -1:
-// none): the columns at on0 + j*lin when lin != 0, else through the table cn
-// (-1 past N).  Old values are read eight at a time ahead of the stores.
-__device__ __forceinline__ void store_row(const uint32_t (&r)[32], float *__restrict__ C, int64_t om, int c0,
-                                          int64_t lin, int64_t on0, int nval, const int64_t *cn, float alpha,
+// This thread's row of W accumulator columns c0.. (C offset om, -1: none): the
+// columns at on0 + j*lin when lin != 0, else through the table cn.
+template <int W>
+__device__ __forceinline__ void load_old(float (&old)[W], const float *__restrict__ C, int64_t om, int c0, int64_t lin,
+                                         int64_t on0, int nval, const int64_t *cn) {
+    if (om < 0) return;
+    if (lin != 0 && c0 + W <= nval) {
+        const float *p = C + om + on0 + (int64_t)c0 * lin;
+#pragma unroll
+        for (int j = 0; j < W; ++j) old[j] = p[j * lin];
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < W; ++j)
+        if (c0 + j < nval) old[j] = C[om + (lin != 0 ? on0 + (int64_t)(c0 + j) * lin : cn[c0 + j])];
+}
+
+template <int W>
+__device__ __forceinline__ void store_row(const uint32_t (&r)[W], const float (&old)[W], float *__restrict__ C, int64_t om,
+                                          int c0, int64_t lin, int64_t on0, int nval, const int64_t *cn, float alpha,
                                           float beta, int init) {
+    if (om < 0) return;
+    if (lin != 0 && c0 + W <= nval) {  // (no test per column: the common case)
+        float *p = C + om + on0 + (int64_t)c0 * lin;
+        if (init == 2) {
+#pragma unroll
+            for (int j = 0; j < W; ++j) p[j * lin] = alpha * __uint_as_float(r[j]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < W; ++j) p[j * lin] = fmaf(beta, old[j], alpha * __uint_as_float(r[j]));
+        }
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < W; ++j) {
+        if (c0 + j >= nval) continue;
+        float v = alpha * __uint_as_float(r[j]);
+        if (init == 1) v = fmaf(beta, old[j], v);
+        C[om + (lin != 0 ? on0 + (int64_t)(c0 + j) * lin : cn[c0 + j])] = v;
+    }
+}
+
+// store_row with few registers: old values read eight at a time ahead of the
+// stores.
+__device__ __forceinline__ void store_row_low(const uint32_t (&r)[32], float *__restrict__ C, int64_t om, int c0,
+                                              int64_t lin, int64_t on0, int nval, const int64_t *cn, float alpha,
+                                              float beta, int init) {
     if (om < 0) return;
     float *p = C + om + on0 + (int64_t)c0 * lin;
     if (lin != 0 && init == 2) {
@@ -514,7 +555,7 @@ __device__ __forceinline__ double fixed_to_double(int64_t hi, int64_t lo, int s)
 // in tensor memory, each folded by TwoSum into a (hi, lo) pair that the
 // epilogue threads hold in registers (64 columns each: bn <= 128).  Otherwise
 // one unit per tile: one accumulator, or with d.split two (the (0,0) products
-// apart); double-buffered where they take at most 256 columns.
+// apart; bn <= 128), double-buffered.
 template <int KIND, bool COMP, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
 packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__ CUtensorMap tmA,
@@ -543,8 +584,8 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
         atomicExch(d.status, (int)TC_ERROR_TIMEOUT);
     };
     const bool split = KIND == GK_D32 || (!COMP && d.split != 0);
-    const int nbuf = KIND == GK_D64 || (split && d.bn > 128) ? 1 : 2;
-    const uint32_t small_off = split ? (d.bn > 128 ? 256u : 128u) : 0u;  // the smaller products' accumulator
+    const int nbuf = KIND == GK_D64 ? 1 : 2;
+    const uint32_t small_off = split ? 128u : 0u;  // the smaller products' accumulator (bn <= 128)
     if (threadIdx.x == 0) {
         for (int s = 0; s < d.stages; ++s) {
             mbar_init(&full[s], 1);   // the issuing CTA's copy lane arms it for every CTA's bytes
@@ -790,6 +831,12 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
             }
             if (role_sync_or<2, kEpiThreads>(*abort_flag)) break;
             bool aborted = false;
+            // the old values of the first columns are on their way before
+            // the accumulator is waited for, later ones before the stores
+            // ahead of them (a column at a time each cost a memory latency:
+            // 46 us for 24 MB of C; the compensated form has no registers for it)
+            float old[32];
+            if (!COMP && KIND != GK_D64 && d.init == 1) load_old(old, C, om, half * 32, lin, on0, nval, cn);
             for (int c = 0; c < nch; ++c) {
                 bool ok = bwait(&tfull[buf], aph);
                 ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld needs the whole warp
@@ -866,7 +913,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                         }
                     }
                 }
-                if constexpr (!COMP && KIND != GK_D64) {
+                if constexpr (KIND != GK_D64 && !COMP) {
 #pragma unroll 1
                     for (int c0 = half * 32; c0 < d.bn; c0 += 64) {
                         uint32_t r[32];
@@ -879,7 +926,8 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                             for (int j = 0; j < 32; ++j)
                                 r[j] = __float_as_uint(__uint_as_float(r[j]) * up * __uint_as_float((unsigned)(ce[j] + 1) << 23));
                         }
-                        store_row(r, C, om, c0, lin, on0, nval, cn, alpha, d.beta, d.init);
+                        store_row(r, old, C, om, c0, lin, on0, nval, cn, alpha, d.beta, d.init);
+                        if (d.init == 1 && c0 + 64 < d.bn) load_old(old, C, om, c0 + 64, lin, on0, nval, cn);
                     }
                 }
                 tc_fence_before();
@@ -891,6 +939,18 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                 if (++buf == nbuf) buf = 0, aph ^= 1u;
             }
             if (aborted) continue;
+            if constexpr (COMP) {
+                // (the next tile's first chunk accumulates meanwhile)
+#pragma unroll
+                for (int gi = 0; gi < 2; ++gi) {
+                    const int c0 = half * 32 + gi * 64;
+                    if (c0 >= d.bn) break;
+                    uint32_t r[32];
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(hi[gi][j]);
+                    store_row_low(r, C, om, c0, lin, on0, nval, cn, alpha, d.beta, d.init);
+                }
+            }
             if constexpr (KIND == GK_D64) {
                 // (the next tile accumulates meanwhile)
                 const int *ce = cE[it & 1];
@@ -905,18 +965,6 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                         if (plain) *q = v;
                         else *q = d.init == 2 ? d.alpha64 * v : fma(d.alpha64, v, d.beta64 * *q);
                     }
-                }
-            }
-            if constexpr (COMP) {
-                // (the next tile's first chunk accumulates meanwhile)
-#pragma unroll
-                for (int gi = 0; gi < 2; ++gi) {
-                    const int c0 = half * 32 + gi * 64;
-                    if (c0 >= d.bn) break;
-                    uint32_t r[32];
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(hi[gi][j]);
-                    store_row(r, C, om, c0, lin, on0, nval, cn, alpha, d.beta, d.init);
                 }
             }
         }
@@ -980,7 +1028,7 @@ struct Tile {
 // bn / 2 clocks of the tensor pipe, or what the shared-memory port needs for
 // its operands and its share of the copies; 2500 clocks per tile for filling
 // the pipeline and draining the last accumulator.
-Tile choose_tile(int64_t M, int64_t N, double ksteps, int nprod, int slices, int max_bn, bool single_buffer_past_128) {
+Tile choose_tile(int64_t M, int64_t N, double ksteps, int nprod, int slices, int max_bn) {
     Tile best{false, 128};
     double best_cost = -1;
     for (int pair = 1; pair >= 0; --pair) {
@@ -989,8 +1037,7 @@ Tile choose_tile(int64_t M, int64_t N, double ksteps, int nprod, int slices, int
         for (int bn = max_bn; bn >= 32; bn -= 16) {
             const int brows = pair ? bn / 2 : bn;
             const double port = ((4096.0 + 32.0 * brows) * nprod + 32.0 * (kRows + brows) * slices) / 128.0;
-            const double tile = ksteps * std::max(bn / 2.0 * nprod, port) + 2500.0 +
-                                (single_buffer_past_128 && bn > 128 ? 10.0 * bn : 0.0);
+            const double tile = ksteps * std::max(bn / 2.0 * nprod, port) + 2500.0;
             const int64_t tiles = ((M + rows - 1) / rows) * ((N + bn - 1) / bn);
             const double cost = (double)((tiles + slots - 1) / slots) * tile;
             if (best_cost < 0 || cost < best_cost) {
@@ -1037,7 +1084,13 @@ tc_status launch_gett(const PackedDesc &d, const CUtensorMap &ta, const CUtensor
     return e == cudaSuccess ? TC_SUCCESS : fail(TC_ERROR_CUDA, cudaGetErrorString(e));
 }
 
-constexpr int64_t kPanelBytes = int64_t(64) << 20;       // images of one panel of B: half of L2
+// Images of one panel of B.  The digit forms read each panel several times
+// their own time: half of L2.  The others spend less time per byte, and more
+// launches cost more than reading the images from HBM (split-BF16 512^3
+// iaj,jbic: 7 panels of 64 MiB 122 us of pre-pass and 290 us of GETT, one of
+// 402 MB 102 and 257 us).
+constexpr int64_t kDigitPanelBytes = int64_t(64) << 20;
+constexpr int64_t kPanelBytes = int64_t(512) << 20;
 constexpr int64_t kScratchMaxABytes = int64_t(256) << 20;
 
 // Scratch that an execute can do without: taken once, outside a capture, and
@@ -1062,8 +1115,8 @@ bool optional_scratch(Plan &p, int64_t bytes, cudaStream_t st) {
 }
 
 // Tiles of B per panel: whole waves where B takes several panels.
-int64_t panel_tiles_for(int64_t tiles_n, int64_t tiles_m, int64_t tile_bytes, int64_t slots) {
-    int64_t pt = std::max<int64_t>(1, kPanelBytes / tile_bytes);
+int64_t panel_tiles_for(int64_t panel_bytes, int64_t tiles_n, int64_t tiles_m, int64_t tile_bytes, int64_t slots) {
+    int64_t pt = std::max<int64_t>(1, panel_bytes / tile_bytes);
     if (pt < tiles_n && pt * tiles_m > slots) pt = std::max<int64_t>(1, pt * tiles_m / slots * slots / tiles_m);
     return std::min(pt, tiles_n);
 }
@@ -1075,11 +1128,13 @@ tc_status run_packed(Plan &p, PackedDesc &d, bool comp, int64_t comp_k, double f
     using T = Traits<KIND>;
     constexpr int BK = stage_k<KIND>();
     const int nprod = KIND == GK_BF16X3 ? d.nprod : (KIND == GK_TF32X3 ? 3 : 1);
-    int max_bn = comp ? 128 : (p.gett_bn == 128 ? 128 : kMaxBn);
+    // (split accumulators: 128 columns leave room for two pairs of them, 257
+    // against 289 us on 512^3 iaj,jbic)
+    const int max_bn = comp || d.split || p.gett_bn == 128 ? 128 : kMaxBn;
     d.ktiles = (int)((d.K + BK - 1) / BK);
     const int64_t col_bytes = (int64_t)d.ktiles * BK * T::kSlices * T::kElemBytes;
     const int64_t panel_n = done ? std::min(d.N, std::max<int64_t>(kMaxBn, kPanelBytes / col_bytes)) : d.N;
-    Tile t = choose_tile(d.M, panel_n, (double)((d.K * T::kElemBytes + 31) / 32), nprod, T::kSlices, max_bn, d.split != 0);
+    Tile t = choose_tile(d.M, panel_n, (double)((d.K * T::kElemBytes + 31) / 32), nprod, T::kSlices, max_bn);
     if (p.gett_pair && d.M > kRows) t.pair = true;
     const int64_t N = fraction < 1.0 ? std::min<int64_t>(d.N, std::max<int64_t>(t.bn, (int64_t)(d.N * fraction))) : d.N;
     d.bn = t.bn;
@@ -1091,7 +1146,7 @@ tc_status run_packed(Plan &p, PackedDesc &d, bool comp, int64_t comp_k, double f
     d.img_b = (uint32_t)(T::kSlices * d.brows * BK * T::kElemBytes);
     d.stages = std::min<int>(kMaxStages, kRingBytes / (int)(d.img_a + d.img_b));
     const int64_t tiles_n = (N + d.bn - 1) / d.bn;
-    const int64_t panel = done ? panel_tiles_for((d.N + d.bn - 1) / d.bn, d.tiles_m, d.bn * col_bytes, sm_count() / (t.pair ? 2 : 1))
+    const int64_t panel = done ? panel_tiles_for(kPanelBytes, (d.N + d.bn - 1) / d.bn, d.tiles_m, d.bn * col_bytes, sm_count() / (t.pair ? 2 : 1))
                                : tiles_n;
     const int64_t bytes_a = d.tiles_m * rows * col_bytes, bytes_b = panel * d.bn * col_bytes;
     tc_status s = ensure_device_resources(p, done ? 0 : (size_t)packed_bytes(p.dtype, d.M, N, d.K));
@@ -1175,7 +1230,7 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
         q.rows_a = q.tiles_m * rows;
         q.image_a = q.rows_a * Kp * S * 2;
         if (q.image_a > kScratchMaxABytes) continue;
-        q.panel_tiles = panel_tiles_for(q.tiles_n, q.tiles_m, Kp * S * 2 * D::kBn, slots);
+        q.panel_tiles = panel_tiles_for(kDigitPanelBytes, q.tiles_n, q.tiles_m, Kp * S * 2 * D::kBn, slots);
         q.image_b = q.panel_tiles * D::kBn * Kp * S * 2;
         const int64_t panels = (q.tiles_n + q.panel_tiles - 1) / q.panel_tiles;
         const int brows = pair ? D::kBn / 2 : D::kBn, nprod = S * (S + 1) / 2;
