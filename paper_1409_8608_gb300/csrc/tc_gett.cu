@@ -1800,7 +1800,7 @@ static tc_status e4m3_scales(Plan &p, const void *A, const void *B, cudaStream_t
 // BF16, TF32, BF16): K = 256 512 x 512^2 386 / 426, 257 / 356, 211 / 740 and
 // up to 11 x faster where few tiles have a long K (256^2, K = 4096, 23 / 393);
 // K = 143 301 x 19691 25 / 45, 21 / 42, 19 / 35; K = 64 300 x 200000 (ragged)
-// 91 / 120, 83 / 134, 77 / 95 but 512 x 512^2 181 / 151, 154 / 136, 145 / 153;
+// 91 / 120, 83 / 134, 77 / 95, but 512 x 512^2 181 / 151, 154 / 136, 145 / 153;
 // K = 16 512 x 512^2 147 / 115, 143 / 112, 142 / 110, K = 25 81 x 18190 10 /
 // 12, 12 / 12, 12 / 10.  So: from K = 128 always, from K = 48 unless TMA
 // stages both inputs of a large result, below only the split forms of a small

@@ -17,8 +17,8 @@
 //                    cp.async.bulk.tensor into a ring (both CTAs of a pair
 //                    count their bytes on the issuing CTA's barrier);
 //   MMA warp 8       one lane issues the stage's slice products;
-//   epilogue warps 0-7  drain the accumulators (two warps per 32 lanes,
-//                    alternate groups of 32 columns) and store C.
+//   epilogue warps 0-7  drain the accumulators and store C (two groups of
+//                    four, alternate tiles or alternate 32 columns).
 // Why pairs and these widths: an MMA of N columns takes N / 2 clocks and reads
 // 4 KB of A and 32 bytes per row of B held here through the shared-memory
 // port (128 bytes per clock), next to the copies' writes.  A lone CTA on
@@ -90,7 +90,6 @@ constexpr int kRingBytes = 192 * 1024;     // operand ring
 constexpr int kMaxStages = 8;
 constexpr int kMaxBn = 256;
 constexpr int kEpiWarps = 8;
-constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kMmaWarp = kEpiWarps, kCopyWarp = kEpiWarps + 1;
 constexpr int kThreads = (kCopyWarp + 1) * 32;
 constexpr uint32_t kTmemCols = 512;
@@ -564,9 +563,16 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
     constexpr int BK = stage_k<KIND>();
     extern __shared__ __align__(128) char ring[];
     __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages], tfull[2], tempty[2], drain;
-    __shared__ int64_t cN[2][kMaxBn];
+    // The epilogue: two groups of four warps take alternate tiles, each its
+    // own accumulator, so that one tile's index arithmetic, waits and memory
+    // latencies overlap the other's stores; where a tile needs every register
+    // (compensated) or all of the tensor memory (FP64 digits), the groups
+    // share a tile, alternate 32 columns each.
+    constexpr bool kAlt = !COMP && KIND != GK_D64;
+    constexpr int kGroupWarps = kAlt ? kEpiWarps / 2 : kEpiWarps;
+    __shared__ int64_t cN[kAlt ? 4 : 2][kMaxBn];
     constexpr bool DIG = digit_kind(KIND);
-    __shared__ int cE[DIG ? 2 : 1][DIG ? 128 : 1];  // digits: exponent fields of the tile's columns
+    __shared__ int cE[DIG ? (kAlt ? 4 : 2) : 1][DIG ? 128 : 1];  // digits: exponent fields of the tile's columns
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_word;
     volatile int *abort_flag = &abort_word;
@@ -593,7 +599,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&tfull[b], 1);
-            mbar_init(&tempty[b], kEpiWarps * kCtas);
+            mbar_init(&tempty[b], kGroupWarps * kCtas);
         }
         mbar_init(&drain, 1);
         *abort_flag = 0;
@@ -779,34 +785,41 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
         __syncwarp();
     } else {
         // ------------------------------------------------------- epilogue
-        const int et = threadIdx.x, quad = warp % 4, half = warp / 4;
+        constexpr int kGroup = kGroupWarps * 32;
+        const int et = threadIdx.x % kGroup, quad = warp % 4;
+        const int grp = kAlt ? warp / 4 : 0, half = kAlt ? 0 : warp / 4;
+        constexpr int kColStep = kAlt ? 32 : 64;
         const int row = quad * 32 + lane;  // accumulator row = TMEM lane
         const uint32_t lane_off = (uint32_t)(quad * 32) << 16;
         float alpha = d.alpha;
         if constexpr (KIND == GK_E4M3) alpha = d.alpha * d.qscale[0] * d.qscale[1];
         float *__restrict__ C = (float *)d.C;
         const int nch = (d.ktiles + d.chunk - 1) / d.chunk;
-        int it = 0, buf = 0;
+        int it = 0, buf = kAlt ? grp : 0;
+        int64_t seen = 0;  // tiles accumulated
         uint32_t aph = 0;  // parity: accumulator filled
         int64_t dhi[32], dlo[32];  // FP64 digits: levels 0-3 (units of 2^-36) and 4-7 (2^-60), 32 columns
         const bool plain = d.init == 2 && d.alpha64 == 1.0;
         constexpr int G = COMP ? 2 : 1;
         float hi[G][32], lo[G][32];
-        for (int64_t tile = slot0; tile < d.num_tiles; tile += nslots, ++it) {
+        for (int64_t tile = slot0; tile < d.num_tiles; tile += nslots) {
             int64_t mt, rem, ignored = 0;
             const int64_t nt = divmod(tile, d.tiles_m, mt);
             if (skip(mt, nt)) {
-                if (et == 0 && crank == 0) {
+                if (threadIdx.x == 0 && crank == 0) {
                     const unsigned long long at = atomicAdd((unsigned long long *)d.list, 1ull);
                     d.list[1 + at] = mt + d.tiles_m * (d.n_begin / d.bn + nt);
                 }
                 continue;
             }
+            if (kAlt && (int)(seen++ & 1) != grp) continue;  // the other group's
+            ++it;
             const int64_t n0 = d.n_begin + nt * d.bn, mm = (mt * kCtas + crank) * kRows + row;
             const int nval = (int)min((int64_t)d.bn, d.N - nt * d.bn);
             // one stride across the tile's columns where C has one
             int64_t lin = 0, on0 = 0, om = -1;
-            int64_t *cn = cN[it & 1];
+            const int tab = kAlt ? 2 * grp + (it & 1) : it & 1;
+            int64_t *cn = cN[tab];
             if (d.nn > 0 && d.n_chain) {
                 lin = d.n_sC[0];
                 on0 = n0 * lin;
@@ -814,7 +827,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                 decode(n0, d.nn, d.n_ext, d.n_sB, d.n_sC, ignored, on0);
                 lin = d.n_sC[0];
             } else {
-                for (int j = et; j < nval; j += kEpiThreads) {
+                for (int j = et; j < nval; j += kGroup) {
                     int64_t oc = 0;
                     decode(n0 + j, d.nn, d.n_ext, d.n_sB, d.n_sC, ignored, oc);
                     cn[j] = oc;
@@ -827,9 +840,10 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
             int rowE = 0;
             if constexpr (DIG) {
                 rowE = d.exps[0][mm];  // (padded rows have one too)
-                if (et < d.bn) cE[it & 1][et] = d.exps[1][nt * d.bn + et];
+                for (int j = et; j < d.bn; j += kGroup) cE[tab][j] = d.exps[1][nt * d.bn + j];
             }
-            if (role_sync_or<2, kEpiThreads>(*abort_flag)) break;
+            const bool quit = grp == 0 ? role_sync_or<2, kGroup>(*abort_flag) : role_sync_or<3, kGroup>(*abort_flag);
+            if (quit) break;
             bool aborted = false;
             // the old values of the first columns are on their way before
             // the accumulator is waited for, later ones before the stores
@@ -915,19 +929,19 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                 }
                 if constexpr (KIND != GK_D64 && !COMP) {
 #pragma unroll 1
-                    for (int c0 = half * 32; c0 < d.bn; c0 += 64) {
+                    for (int c0 = half * 32; c0 < d.bn; c0 += kColStep) {
                         uint32_t r[32];
                         if (split) tmem_ld32_sum(acc + (uint32_t)c0, acc + small_off + (uint32_t)c0, r);
                         else tmem_ld32(acc + (uint32_t)c0, r);
                         if constexpr (KIND == GK_D32) {  // powers of two: 2^eA of the row, 2^eB of each column
-                            const int *ce = cE[it & 1] + c0;
+                            const int *ce = cE[tab] + c0;
                             const float up = __uint_as_float((unsigned)(rowE + 1) << 23);
 #pragma unroll
                             for (int j = 0; j < 32; ++j)
                                 r[j] = __float_as_uint(__uint_as_float(r[j]) * up * __uint_as_float((unsigned)(ce[j] + 1) << 23));
                         }
                         store_row(r, old, C, om, c0, lin, on0, nval, cn, alpha, d.beta, d.init);
-                        if (d.init == 1 && c0 + 64 < d.bn) load_old(old, C, om, c0 + 64, lin, on0, nval, cn);
+                        if (d.init == 1 && c0 + kColStep < d.bn) load_old(old, C, om, c0 + kColStep, lin, on0, nval, cn);
                     }
                 }
                 tc_fence_before();
@@ -936,7 +950,8 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                     if constexpr (PAIR) mbar_arrive_remote(mapa_shared(smem_u32(&tempty[buf]), 0u));
                     else mbar_arrive(&tempty[buf]);
                 }
-                if (++buf == nbuf) buf = 0, aph ^= 1u;
+                if (kAlt) aph ^= 1u;
+                else if (++buf == nbuf) buf = 0, aph ^= 1u;
             }
             if (aborted) continue;
             if constexpr (COMP) {
@@ -953,7 +968,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
             }
             if constexpr (KIND == GK_D64) {
                 // (the next tile accumulates meanwhile)
-                const int *ce = cE[it & 1];
+                const int *ce = cE[tab];
                 if (om >= 0) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {
