@@ -1801,14 +1801,14 @@ static tc_status e4m3_scales(Plan &p, const void *A, const void *B, cudaStream_t
 // up to 11 x faster where few tiles have a long K (256^2, K = 4096, 23 / 393);
 // K = 143 301 x 19691 25 / 45, 21 / 42, 19 / 35; K = 64 300 x 200000 (ragged)
 // 91 / 120, 83 / 134, 77 / 95, but 512 x 512^2 181 / 151, 154 / 136, 145 / 153;
-// K = 16 512 x 512^2 147 / 115, 143 / 112, 142 / 110, K = 25 81 x 18190 10 /
-// 12, 12 / 12, 12 / 10.  So: from K = 128 always, from K = 48 unless TMA
-// stages both inputs of a large result, below only the split forms of a small
-// result.  (d, pk: the modes and the choice without this.)
+// K = 16 512 x 512^2 147 / 115, 143 / 112, 142 / 110, K = 32 86 x 13800 14.2 /
+// 11.9 (split-BF16), K = 25 81 x 18190 12.4 / 10.4 (BF16).  So: from K = 128
+// always, from K = 48 unless TMA stages both inputs of a large result.
+// (d, pk: the modes and the choice without this.)
 static bool images_win(const Plan &p, const GettModes &d, int pk) {
     if (p.gett_pack != 1 || d.nb != 0 || d.K > (int64_t(1) << 24)) return false;
     if (d.K >= 128) return true;
-    if (d.K < 48) return (p.dtype == TC_BF16X3 || p.dtype == TC_TF32X3) && d.M * d.N <= (int64_t(1) << 21);
+    if (d.K < 48) return false;
     if (p.dtype == TC_E4M3 || d.M * d.N < (int64_t(1) << 24)) return true;
     const int in_bytes = (p.dtype == TC_BF16 || p.dtype == TC_F16) ? 2 : 4;
     GettDesc t;
