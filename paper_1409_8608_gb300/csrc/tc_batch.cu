@@ -15,9 +15,12 @@
 // (512 >> s) for s = 0..4, and a problem's K runs in chunks of bk (8, 16 or
 // 32).  A block's sequence of (tile, K chunk) stages is software-pipelined:
 // cp.async copies of stage s+1 (16-byte pieces where the layout allows)
-// overlap the FMAs of stage s.  Each thread owns 4 rows x 4 columns; A is
-// staged k-major and B n-major with a pitch that keeps the 16-byte reads of
-// both conflict-free.  Where a tile's C is one contiguous run (one column
+// overlap the FMAs of stage s.  Each of 128 threads owns 8 rows x 4 columns
+// (FP32 multiplies row pairs with fma.rn.f32x2); A is staged k-major and B
+// n-major with a pitch that keeps the 16-byte reads of both conflict-free.
+// What bounds it on short K is issue: 4096 outputs may take 870 clocks of an
+// SM at the HBM rate, and 256 threads of 4 x 4 outputs spent 6700 warp
+// instructions on them, a quarter of those multiply-adds.  Where a tile's C is one contiguous run (one column
 // tile covers M, C dense along m) the epilogue stages it in shared memory
 // and writes it with aligned 16-byte stores.  The tile shape and K chunk
 // are chosen per problem: fixed (64 x 64, bk 16), by rule (the smallest
@@ -40,7 +43,7 @@ namespace tc {
 
 namespace {
 
-constexpr int kThreadsB = 256;
+constexpr int kThreadsB = 128;
 constexpr int kShapes = 5;           // tiles (8 << s) x (512 >> s)
 constexpr int kStageElems = 6400;    // one stage: A chunk (bk x TM) + B chunk (TN x pitch)
 constexpr int kOutElems = 4096 + 4;  // staged epilogue (in a stage buffer) + 16-byte alignment shift
@@ -98,7 +101,7 @@ __device__ __forceinline__ void lds4(const T *p, T (&v)[4]) {
 // Geometry of one pipeline stage, worked out once by the producer and read
 // by every thread from shared memory.
 struct StageMeta {
-    int q;                  // problem slot
+    int rec;                // the problem's record in shared memory
     int chunk;              // K chunk of the tile
     int m0, n0, mlim, nlim; // tile origin and valid rows / columns
     int kk;                 // K positions in this chunk
@@ -106,11 +109,10 @@ struct StageMeta {
 };
 
 // Fills the stage record for tile lt of problem P, K chunk `chunk`.
-__device__ __forceinline__ void stage_meta(const BatchProblem *__restrict__ P, int q, int lt, int chunk,
-                                           StageMeta &m) {
+__device__ __forceinline__ void stage_meta(const BatchProblem *P, int rec, int lt, int chunk, StageMeta &m) {
     const int shape = P->shape, tm = P->tiles_m, bk = P->bk;
     const int mt = tm == 1 ? 0 : lt % tm, nt = tm == 1 ? lt : lt / tm;
-    m.q = q;
+    m.rec = rec;
     m.chunk = chunk;
     m.m0 = mt * shape_rows(shape);
     m.n0 = nt * shape_cols(shape);
@@ -126,7 +128,7 @@ __device__ __forceinline__ void stage_meta(const BatchProblem *__restrict__ P, i
 // in both.  Rows past M and columns past N are left as they are: they only
 // reach outputs that are never stored.
 template <typename T>
-__device__ __forceinline__ void batch_produce(T *S, const BatchProblem *__restrict__ P, const StageMeta &g) {
+__device__ __forceinline__ void batch_produce(T *S, const BatchProblem *P, const StageMeta &g) {
     constexpr int V = 16 / sizeof(T), lgV = sizeof(T) == 4 ? 2 : 1;
     const int shape = P->shape, TM = shape_rows(shape), lgTM = 3 + shape;
     const int bk = P->bk, flags = P->flags;
@@ -185,11 +187,43 @@ __device__ __forceinline__ void batch_produce(T *S, const BatchProblem *__restri
     (void)lgV;
 }
 
-// FMAs of one staged K chunk: thread (tx, ty) owns rows 4tx..4tx+3 and
-// columns ty + j*TY, j = 0..3; K runs in increasing order.
+// two FP32 fused multiply-adds in one instruction, each rounded as fmaf
+__device__ __forceinline__ void fma_f2(float2 &c, float2 a, float b) {
+    unsigned long long &cc = reinterpret_cast<unsigned long long &>(c);
+    unsigned long long bb;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(bb) : "f"(b));
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(cc) : "l"(reinterpret_cast<unsigned long long &>(a)), "l"(bb));
+}
+
+// A thread's outputs: rows 4tx + i and 4tx + 4TX + i (i = 0..3) and columns
+// ty + j TY, j = 0..3, with TX = TM / 8.
+template <typename T>
+struct Acc {
+    T v[8][4];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[i][j] = T(0);
+    }
+    __device__ __forceinline__ T get(int i, int j) const { return v[i][j]; }
+};
+template <>
+struct Acc<float> {
+    float2 v[4][4];  // row pairs
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[i][j] = make_float2(0.0f, 0.0f);
+    }
+    __device__ __forceinline__ float get(int i, int j) const { return i % 2 ? v[i / 2][j].y : v[i / 2][j].x; }
+};
+
+// FMAs of one staged K chunk; K runs in increasing order.
 template <typename T, int SHAPE>
-__device__ __forceinline__ void batch_compute(const T *S, int bk, int kk4, int KP, T (&acc)[4][4]) {
-    constexpr int TM = shape_rows(SHAPE), TX = TM / 4, TY = kThreadsB / TX;
+__device__ __forceinline__ void batch_compute(const T *S, int bk, int kk4, int KP, Acc<T> &acc) {
+    constexpr int TM = shape_rows(SHAPE), TX = TM / 8, TY = kThreadsB / TX;
     const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
     const T *As = S + 4 * tx;
     const T *Bs = S + bk * TM + ty * KP;
@@ -199,12 +233,19 @@ __device__ __forceinline__ void batch_compute(const T *S, int bk, int kk4, int K
         for (int j = 0; j < 4; ++j) lds4(Bs + j * TY * KP + k4, b[j]);
 #pragma unroll
         for (int kq = 0; kq < 4; ++kq) {
-            T a[4];
-            lds4(As + (k4 + kq) * TM, a);
+            T a[8];
+            lds4(As + (k4 + kq) * TM, *reinterpret_cast<T(*)[4]>(&a[0]));
+            lds4(As + (k4 + kq) * TM + 4 * TX, *reinterpret_cast<T(*)[4]>(&a[4]));
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < 4; ++j) {
+                if constexpr (sizeof(T) == 4) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma_b<T>(a[i], b[j][kq], acc[i][j]);
+                    for (int i = 0; i < 4; ++i) fma_f2(acc.v[i][j], make_float2(a[2 * i], a[2 * i + 1]), b[j][kq]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) acc.v[i][j] = fma(a[i], b[j][kq], acc.v[i][j]);
+                }
+            }
         }
     }
 }
@@ -217,9 +258,9 @@ __device__ __forceinline__ T blend(T acc, T alpha, T beta, int init, const T *c)
 // C = alpha * acc (+ beta * C) for one tile.  Cs: the stage buffer just
 // consumed (free once every thread has passed the barrier below).
 template <typename T, int SHAPE>
-__device__ __forceinline__ void batch_epilogue(const BatchProblem *__restrict__ P, const StageMeta &g,
-                                               T (&acc)[4][4], T alpha, T beta, int init, T *Cs) {
-    constexpr int TM = shape_rows(SHAPE), TX = TM / 4, TY = kThreadsB / TX;
+__device__ __forceinline__ void batch_epilogue(const BatchProblem *P, const StageMeta &g,
+                                               const Acc<T> &acc, T alpha, T beta, int init, T *Cs) {
+    constexpr int TM = shape_rows(SHAPE), TX = TM / 8, TY = kThreadsB / TX;
     constexpr int V = 16 / sizeof(T);
     const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
     const int mlim = g.mlim, nlim = g.nlim;
@@ -231,13 +272,24 @@ __device__ __forceinline__ void batch_epilogue(const BatchProblem *__restrict__ 
         const int shift = (int)(((uintptr_t)Cg / sizeof(T)) & (V - 1));
         __syncthreads();  // every thread is done reading the stage
         T *cs = Cs + shift + 4 * tx;
+        const bool quads = ((M | shift) & 3) == 0;  // rows of four stay 16-byte aligned (FP32)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int n = ty + j * TY;
-            if (n < nlim) {
+            if (n >= nlim) continue;
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (4 * tx + i < M) cs[n * M + i] = acc[i][j];
+            for (int g = 0; g < 2; ++g) {
+                const int m = 4 * tx + 4 * TX * g;
+                T *c = cs + n * M + 4 * TX * g;
+                if (sizeof(T) == 4 && quads) {
+                    if (m < M)
+                        *(float4 *)c = make_float4((float)acc.get(4 * g, j), (float)acc.get(4 * g + 1, j),
+                                                   (float)acc.get(4 * g + 2, j), (float)acc.get(4 * g + 3, j));
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (m + i < M) c[i] = acc.get(4 * g + i, j);
+                }
             }
         }
         __syncthreads();
@@ -277,13 +329,13 @@ __device__ __forceinline__ void batch_epilogue(const BatchProblem *__restrict__ 
     const int sCm = (int)P->sCm, sCn = (int)P->sCn;
     T *Ct = C + g.m0 * P->sCm + g.n0 * P->sCn;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int m = 4 * tx + i, n = ty + j * TY;
+            const int m = 4 * tx + i / 4 * 4 * TX + i % 4, n = ty + j * TY;
             if (m < mlim && n < nlim) {
                 T *c = Ct + m * sCm + n * sCn;
-                *c = blend<T>(acc[i][j], alpha, beta, init, c);
+                *c = blend<T>(acc.get(i, j), alpha, beta, init, c);
             }
         }
 }
@@ -292,7 +344,7 @@ __device__ __forceinline__ void batch_epilogue(const BatchProblem *__restrict__ 
 // grid-strided; each block runs its tiles' K chunks as one pipelined
 // sequence of stages.
 template <typename T, int STAGES>
-__global__ void __launch_bounds__(kThreadsB) batch_kernel(const BatchProblem *__restrict__ probs,
+__global__ void __launch_bounds__(kThreadsB, 4) batch_kernel(const BatchProblem *__restrict__ probs,
                                                           const int32_t *__restrict__ tile_prob,
                                                           int64_t t_begin, int64_t t_end, T alpha, T beta,
                                                           int init) {
@@ -300,19 +352,45 @@ __global__ void __launch_bounds__(kThreadsB) batch_kernel(const BatchProblem *__
     extern __shared__ __align__(16) unsigned char bsm[];
     T *stages = (T *)bsm;
     __shared__ StageMeta meta[STAGES];
-    int64_t pt = t_begin + blockIdx.x;  // producer cursor: tile and K chunk
-    int pc = 0;
+    // Problem records: tile x's (x-th of this block) sits at x % kRecs, copied
+    // two tiles ahead of the producer, its problem's number read three ahead:
+    // read from global memory when a stage needed them, the two dependent
+    // loads stalled every warp for about a thousand clocks a tile.
+    constexpr int kRecs = 8;
+    static_assert(sizeof(BatchProblem) % 8 == 0 && STAGES <= 3, "record ring");
+    __shared__ __align__(16) BatchProblem recs[kRecs];
+    int64_t pt = t_begin + blockIdx.x;  // producer cursor: tile (the px-th) and K chunk
+    int px = 0, pc = 0;
+    auto prob_of = [&](int x) -> int {  // problem of tile px + x
+        const int64_t t = pt + (int64_t)x * gridDim.x;
+        return t < t_end ? tile_prob[t] : -1;
+    };
+    auto fetch = [&](int q, int slot) {
+        constexpr int kWords = sizeof(BatchProblem) / 8;
+        if (q >= 0 && threadIdx.x < kWords)
+            cp_async_elem<double>((double *)&recs[slot] + threadIdx.x, (const double *)(probs + q) + threadIdx.x);
+    };
+    fetch(prob_of(0), 0);
+    fetch(prob_of(1), 1);
+    cp_async_commit();
+    int q2 = prob_of(2);
+    cp_async_wait<0>();
+    __syncthreads();
     auto produce = [&](int slot) {
         if (pt >= t_end) return;
-        const int q = tile_prob[pt];
-        const BatchProblem *__restrict__ P = probs + q;
+        if (pc == 0) {
+            fetch(q2, (px + 2) % kRecs);
+            q2 = prob_of(3);
+        }
+        const BatchProblem *P = &recs[px % kRecs];
         StageMeta g;
-        stage_meta(P, q, (int)(pt - P->tile0), pc, g);
+        stage_meta(P, px % kRecs, (int)(pt - P->tile0), pc, g);
         batch_produce<T>(stages + slot * kStageElems, P, g);
         if (threadIdx.x == 0) meta[slot] = g;
         if (g.last) {
             pc = 0;
             pt += gridDim.x;
+            ++px;
         } else {
             ++pc;
         }
@@ -322,7 +400,7 @@ __global__ void __launch_bounds__(kThreadsB) batch_kernel(const BatchProblem *__
         produce(p);
         cp_async_commit();
     }
-    T acc[4][4];
+    Acc<T> acc;
     int s = 0;
     for (int64_t ct = t_begin + blockIdx.x; ct < t_end; ++s) {
         cp_async_wait<STAGES - 2>();
@@ -331,15 +409,10 @@ __global__ void __launch_bounds__(kThreadsB) batch_kernel(const BatchProblem *__
         cp_async_commit();
         const int slot = s % STAGES;
         const StageMeta g = meta[slot];
-        const BatchProblem *__restrict__ P = probs + g.q;
+        const BatchProblem *P = &recs[g.rec];
         const int shape = P->shape, bk = P->bk;
         const int kk4 = (g.kk + 3) & ~3, KP = b_pitch(g.kk);
-        if (g.chunk == 0) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-        }
+        if (g.chunk == 0) acc.zero();
         T *S = stages + slot * kStageElems;
         switch (shape) {
             case 0: batch_compute<T, 0>(S, bk, kk4, KP, acc); break;
