@@ -20,9 +20,11 @@
 // n-major with a pitch that keeps the 16-byte reads of both conflict-free.
 // What bounds it on short K is issue: 4096 outputs may take 870 clocks of an
 // SM at the HBM rate, and 256 threads of 4 x 4 outputs spent 6700 warp
-// instructions on them, a quarter of those multiply-adds.  Where a tile's C is one contiguous run (one column
-// tile covers M, C dense along m) the epilogue stages it in shared memory
-// and writes it with aligned 16-byte stores.  The tile shape and K chunk
+// instructions on them, a quarter of those multiply-adds (855 us for 4096
+// problems of abc=ai,ibc, a, b, c in 8..128, i in 4..32); now 4600, with the
+// problem records copied ahead 706 us, 0.37 of HBM.  Where a tile's C is one
+// contiguous run (one column tile covers M, C dense along m) the epilogue
+// stages it in shared memory and writes it with aligned 16-byte stores.  The tile shape and K chunk
 // are chosen per problem: fixed (64 x 64, bk 16), by rule (the smallest
 // tile height that covers M), or by the autotuner, which times every
 // candidate on each shape class's problems (tc_batch_autotune).

@@ -10,14 +10,13 @@
 // The persistent kernel (one CTA per SM) is warp-specialised:
 //
 //   producer warp 0      fetches the problem records of 32 tiles at a time
-//                        (one per lane, so their latency is paid once per 32
-//                        tiles) into a ring of tile records the other roles
-//                        read from shared memory; then one 1-D bulk copy of the tile's B run (128 x K
-//                        contiguous FP32) and one of the problem's A (M x K)
-//                        into a byte ring that packs tiles by their actual
-//                        size (about nine in flight: the copies take a few
-//                        microseconds to land), counted in bytes on an
-//                        mbarrier per tile;
+//                        (one per lane) into a ring of tile records the other
+//                        roles read from shared memory; then one 1-D bulk copy
+//                        of the tile's B run (128 x K contiguous FP32) and one
+//                        of the problem's A (M x K) into a byte ring that packs
+//                        tiles by their actual size (about nine in flight: the
+//                        copies take a few microseconds to land), counted in
+//                        bytes on an mbarrier per tile;
 //   converter warps 2-5  split each FP32 value into three BF16 slices
 //                        x = h0 + h1 + h2 and store both operands in the
 //                        no-swizzle K-major core-matrix layout (zeros past K);
@@ -57,7 +56,7 @@ constexpr int kMaxM = 128;                      // problem rows m (MMA N <= 128)
 constexpr int kMaxK = 32;
 constexpr int kRawSlots = 12;                   // tiles in the raw ring at most
 constexpr int kRawBytes = 94 * 1024;            // raw FP32 ring: each tile's B run and A, packed
-constexpr int kRecs = 32;                       // tile records in shared memory (the producer's lead)
+constexpr int kRecs = 64;                       // tile records in shared memory: two batches of 32
 constexpr int kConvSlots = 2;                   // converted operand ring
 constexpr int kAccs = 4;                        // TMEM accumulators of kMaxM columns
 constexpr int kMaxRawTile = kRows * kMaxK * 4 + kMaxM * kMaxK * 4;  // B run + A, at most
@@ -125,17 +124,19 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
     __shared__ __align__(8) uint64_t raw_full[kRawSlots], raw_empty[kRawSlots];
     __shared__ int raw_off[kRawSlots];  // byte offset of each raw tile in the ring
     __shared__ STile recs[kRecs];       // tile i's record at i % kRecs
-    __shared__ __align__(8) uint64_t rec_full[kRecs], rec_empty[kRecs];
+    __shared__ __align__(8) uint64_t rec_full[2], rec_empty[2];  // per half of the record ring
     __shared__ __align__(8) uint64_t conv_full[kConvSlots], conv_empty[kConvSlots];
     __shared__ __align__(8) uint64_t acc_full[kAccs], acc_empty[kAccs], drain;
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = __shfl_sync(0xffffffffu, threadIdx.x / 32, 0), lane = threadIdx.x % 32;
     if (threadIdx.x == 0) {
         for (int i = 0; i < kRawSlots; ++i) mbar_init(&raw_full[i], 1), mbar_init(&raw_empty[i], kConvWarps);
         for (int i = 0; i < kConvSlots; ++i) mbar_init(&conv_full[i], kConvWarps), mbar_init(&conv_empty[i], 1);
         for (int i = 0; i < kAccs; ++i) mbar_init(&acc_full[i], 1), mbar_init(&acc_empty[i], 4);
-        for (int i = 0; i < kRecs; ++i) mbar_init(&rec_full[i], 1), mbar_init(&rec_empty[i], 4);
+        // one arrival per epilogue warp and tile of a batch of 32 (the last,
+        // partial batch is never overwritten)
+        for (int i = 0; i < 2; ++i) mbar_init(&rec_full[i], 1), mbar_init(&rec_empty[i], 4 * 32);
         mbar_init(&drain, 1);
         abort_flag = 0;
         fence_mbar_init();
@@ -145,6 +146,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    volatile int *abort_now = &abort_flag;
     auto give_up = [&]() {
         abort_flag = 1;
         atomicExch(a.status, (int)TC_ERROR_TIMEOUT);
@@ -153,65 +155,75 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
 
     if (warp == kWProducer) {
         // ------------------------------------------------------------ producer
-        // byte ring: tiles take [pos, pos + size) in order, none wrapping the
-        // end; released in order by the converters (lane 0 keeps the books)
-        int64_t head = 0, tail = 0, oldest = 0, i = 0;
-        int64_t ends[kRawSlots];  // ring end of each tile in flight
+        // Byte ring: tiles take [pos, pos + size) in order, none wrapping the
+        // end; released in order by the converters.  Each lane prepares one
+        // tile of a batch of 32 (its record, addresses and sizes); the warp
+        // then walks the tiles together, one elected lane issuing the copies,
+        // with the bytes to release per slot held by lane `slot`: one lane
+        // alone, with 64-bit remainders and its books in local memory, took
+        // about 1900 clocks a tile and set the pace of the kernel.
+        int used = 0, pos = 0;          // bytes taken; where the next tile goes
+        int slot = 0, oldest = 0, busy = 0;  // next slot, the oldest in flight, how many
+        uint32_t ph = 0;                // parity of the oldest slot's release
+        int mine_size = 0;              // lane l: bytes that slot l's tile holds
         bool stop = false;
-        for (int64_t base = 0; !stop; base += 32) {
-            const int64_t tl = first + (base + lane) * step;  // lane l: tile base + l
-            const STile mine = tl < a.t_end ? stream_tile(a, tl) : STile{};
-            const int64_t left = (a.t_end - first + step - 1) / step - base;  // tiles of this CTA left
-            if (left <= 0) break;
-            const int nb = left < 32 ? (int)left : 32;
-            for (int jj = 0; jj < nb; ++jj, ++i) {
-                STile s;
-                s.A = (const float *)__shfl_sync(0xffffffffu, (unsigned long long)mine.A, jj);
-                s.B = (const float *)__shfl_sync(0xffffffffu, (unsigned long long)mine.B, jj);
-                s.C = (float *)__shfl_sync(0xffffffffu, (unsigned long long)mine.C, jj);
-                s.n0 = __shfl_sync(0xffffffffu, mine.n0, jj);
-                s.M = __shfl_sync(0xffffffffu, mine.M, jj);
-                s.K = __shfl_sync(0xffffffffu, mine.K, jj);
-                s.nvalid = __shfl_sync(0xffffffffu, mine.nvalid, jj);
-                if (lane == 0) {
-                    const uint32_t bytesB = (uint32_t)(s.nvalid * s.K * 4), bytesA = (uint32_t)(s.M * s.K * 4);
-                    const int64_t offA = (bytesB + 127) & ~127, size = offA + ((bytesA + 127) & ~127);
-                    int64_t pos = head % kRawBytes;
-                    if (pos + size > kRawBytes) {  // skip the ring's end
-                        head += kRawBytes - pos;
-                        pos = 0;
-                    }
-                    while (!stop && (head + size - tail > kRawBytes || i - oldest >= kRawSlots)) {
-                        const int o = (int)(oldest % kRawSlots);
-                        if (abort_flag || !mbar_wait(&raw_empty[o], (uint32_t)((oldest / kRawSlots) & 1))) stop = true;
-                        else tail = ends[o], ++oldest;
-                    }
-                    // the record slot: its previous tile's epilogue has read it
-                    const int q = (int)(i % kRecs);
-                    if (!stop && i >= kRecs && !mbar_wait(&rec_empty[q], (uint32_t)(((i / kRecs) - 1) & 1)))
-                        stop = true;
-                    if (stop || abort_flag) {
-                        stop = true;
-                        give_up();
-                    } else {
-                        recs[q] = s;
-                        mbar_arrive(&rec_full[q]);  // releases recs[q] to the epilogue
-                        const int r = (int)(i % kRawSlots);
-                        raw_off[r] = (int)pos;
-                        ends[r] = head + size;
-                        head += size;
-                        mbar_arrive_expect_tx(&raw_full[r], bytesB + bytesA);  // releases raw_off[r], recs[q]
-                        bulk_load(raw + pos, s.B + s.n0 * s.K, bytesB, &raw_full[r]);
-                        bulk_load(raw + pos + offA, s.A, bytesA, &raw_full[r]);
-                    }
+        const int64_t count = a.t_end > first ? (a.t_end - first + step - 1) / step : 0;  // tiles of this CTA
+        for (int64_t base = 0, batch = 0; base < count && !stop; base += 32, ++batch) {
+            // this half of the record ring: its last batch's epilogue is done
+            const int h = (int)(batch & 1);
+            if (batch >= 2 && !__all_sync(0xffffffffu, mbar_wait_or(&rec_empty[h], (uint32_t)(((batch >> 1) - 1) & 1), abort_now))) {
+                stop = true;
+                break;
+            }
+            const int nb = (int)min((int64_t)32, count - base);
+            unsigned long long pA = 0, pB = 0;
+            uint32_t nA = 0, nB = 0;
+            if (lane < nb) {
+                const STile s = stream_tile(a, first + (base + lane) * step);
+                recs[h * 32 + lane] = s;
+                pA = (unsigned long long)s.A;
+                pB = (unsigned long long)(s.B + s.n0 * s.K);
+                nB = (uint32_t)(s.nvalid * s.K * 4);
+                nA = (uint32_t)(s.M * s.K * 4);
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&rec_full[h]);  // releases the batch's records
+            for (int jj = 0; jj < nb && !stop; ++jj) {
+                const unsigned long long tA = __shfl_sync(0xffffffffu, pA, jj), tB = __shfl_sync(0xffffffffu, pB, jj);
+                const uint32_t bytesA = __shfl_sync(0xffffffffu, nA, jj), bytesB = __shfl_sync(0xffffffffu, nB, jj);
+                const int offA = (int)((bytesB + 127) & ~127u), size = offA + (int)((bytesA + 127) & ~127u);
+                const bool wrap = pos + size > kRawBytes;
+                const int skip = wrap ? kRawBytes - pos : 0;  // the ring's end
+                while (!stop && (used + skip + size > kRawBytes || busy == kRawSlots)) {
+                    stop = !__all_sync(0xffffffffu, mbar_wait_or(&raw_empty[oldest], ph, abort_now));
+                    used -= __shfl_sync(0xffffffffu, mine_size, oldest);
+                    --busy;
+                    if (++oldest == kRawSlots) oldest = 0, ph ^= 1u;
                 }
-                stop = __shfl_sync(0xffffffffu, stop, 0);
                 if (stop) break;
+                if (wrap) pos = 0;
+                if (lane == slot) mine_size = size + skip;
+                if (elect_one()) {
+                    raw_off[slot] = pos;
+                    mbar_arrive_expect_tx(&raw_full[slot], bytesB + bytesA);  // releases raw_off, the record
+                    bulk_load(raw + pos, (const void *)tB, bytesB, &raw_full[slot]);
+                    bulk_load(raw + pos + offA, (const void *)tA, bytesA, &raw_full[slot]);
+                }
+                __syncwarp();
+                used += size + skip;
+                pos += size;
+                ++busy;
+                if (++slot == kRawSlots) slot = 0;
             }
         }
-        // nothing may still be copying into shared memory at exit
-        if (lane == 0)
-            for (int64_t jj = oldest; jj < i; ++jj) mbar_wait(&raw_full[jj % kRawSlots], (uint32_t)((jj / kRawSlots) & 1));
+        if (stop && lane == 0) give_up();
+        // nothing may still be copying into shared memory at exit: the tiles
+        // not known released have landed
+        for (; busy > 0; --busy) {
+            mbar_wait(&raw_full[oldest], ph);
+            if (++oldest == kRawSlots) oldest = 0, ph ^= 1u;
+        }
+        __syncwarp();
     } else if (warp >= kWConv && warp < kWConv + kConvWarps) {
         // ----------------------------------------------------------- converters
         const int ct = threadIdx.x - kWConv * 32;  // 0..127: tile row n, and row m of A
@@ -335,14 +347,14 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
         const int64_t t1 = first + grp * step, gstep = kEpiGroups * step;
         for (int64_t t = t1; t < a.t_end; t += gstep, i += kEpiGroups) {
             const int b = (int)(i % kAccs), q = (int)(i % kRecs);
-            bool ok = !abort_flag && mbar_wait(&rec_full[q], (uint32_t)((i / kRecs) & 1));
+            bool ok = mbar_wait_or(&rec_full[q / 32], (uint32_t)((i / kRecs) & 1), abort_now);
             STile s{};
             if (ok) s = recs[q];
             ok = ok && mbar_wait(&acc_full[b], (uint32_t)((i / kAccs) & 1));
             // the tile's MMAs are done, so the converters and the MMA warp
             // have read the record too: its slot may take tile i + kRecs
             __syncwarp();
-            if (lane == 0 && ok) mbar_arrive(&rec_empty[q]);
+            if (lane == 0 && ok) mbar_arrive(&rec_empty[q / 32]);
             if (!__all_sync(0xffffffffu, ok)) {
                 if (lane == 0) give_up();
                 break;
