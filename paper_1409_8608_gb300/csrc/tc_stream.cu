@@ -17,19 +17,26 @@
 //                        tiles by their actual size (about nine in flight: the
 //                        copies take a few microseconds to land), counted in
 //                        bytes on an mbarrier per tile;
-//   converter warps 2-5  split each FP32 value into three BF16 slices
+//   converter warps 2-9  split each FP32 value into three BF16 slices
 //                        x = h0 + h1 + h2 and store both operands in the
 //                        no-swizzle K-major core-matrix layout (zeros past K);
-//   MMA warp 1           one thread issues the six slice products
+//                        two groups of four taking alternate tiles;
+//   MMA warp 1           one elected lane issues the six slice products
 //                        (0,0) (0,1) (1,0) (0,2) (1,1) (2,0) per 16-K step
 //                        into one of four tensor-memory accumulators;
-//   epilogue warps 6-13  two groups of four taking alternate tiles (the
-//                        epilogue is the slowest role: one group left the MMA
-//                        waiting on accumulators): tcgen05.ld 32 columns at a
-//                        time, transpose them through a per-warp buffer and
-//                        store each tile row's contiguous run of C (m
-//                        fastest) with whole-warp coalesced stores, alpha and
-//                        beta applied.
+//   epilogue warps 10-17 two groups of four taking alternate tiles: up to 32
+//                        rows m a warp's 32 columns n are one run of C, put in
+//                        order through shared memory and stored with whole
+//                        warps; above, tcgen05.ld 32 columns at a time,
+//                        transposed through the same per-warp buffer, each
+//                        tile row's contiguous run of C (m fastest), alpha and
+//                        beta applied (two rows of 16 columns a store, for
+//                        short last chunks, took 542 us).
+//
+// Each role alone, the others' work left out, on 4096 problems of abc=ai,ibc
+// (a, b, c in 8..128, i in 4..32; us): copies 146, MMAs 207, converters 231
+// (323 with one group), epilogue 395; all together 506 with one converter
+// group, 454 now.  HBM alone would take 255.
 //
 // Every mbarrier wait is bounded; on expiry the kernel records
 // TC_ERROR_TIMEOUT in the status word, stops, waits for its own copies and
@@ -64,7 +71,9 @@ constexpr int kOpA = 3 * kRows * kMaxK * 2;     // three slices of the 128 x Kpa
 constexpr int kOpB = 3 * kMaxM * kMaxK * 2;     // three slices of the Mpad x Kpad A
 constexpr int kConvSlot = kOpA + kOpB;
 constexpr int kStgFloats = 32 * 33;             // per epilogue warp: 32 x 32 transpose, pitch 33
-constexpr int kWProducer = 0, kWMma = 1, kWConv = 2, kConvWarps = 4, kWEpi = 6;
+constexpr int kWProducer = 0, kWMma = 1, kWConv = 2, kConvWarps = 4;
+constexpr int kConvGroups = 2;                  // converter groups of four warps, taking alternate tiles
+constexpr int kWEpi = kWConv + kConvGroups * kConvWarps;
 constexpr int kEpiGroups = 2;                   // epilogue groups of four warps, taking alternate tiles
 constexpr int kEpiWarps = 4 * kEpiGroups;
 constexpr int kStreamThreads = (kWEpi + kEpiWarps) * 32;
@@ -145,7 +154,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
     volatile int *abort_now = &abort_flag;
     auto give_up = [&]() {
         abort_flag = 1;
@@ -224,11 +233,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
             if (++oldest == kRawSlots) oldest = 0, ph ^= 1u;
         }
         __syncwarp();
-    } else if (warp >= kWConv && warp < kWConv + kConvWarps) {
+    } else if (warp >= kWConv && warp < kWEpi) {
         // ----------------------------------------------------------- converters
-        const int ct = threadIdx.x - kWConv * 32;  // 0..127: tile row n, and row m of A
-        int64_t i = 0;
-        for (int64_t t = first; t < a.t_end; t += step, ++i) {
+        const int ct = (threadIdx.x - kWConv * 32) % (kConvWarps * 32);  // 0..127: tile row n, and row m of A
+        const int cg = (warp - kWConv) / kConvWarps;
+        int64_t i = cg;
+        for (int64_t t = first + cg * step; t < a.t_end; t += kConvGroups * step, i += kConvGroups) {
             const int r = (int)(i % kRawSlots), c = (int)(i % kConvSlots);
             bool ok = !abort_flag && mbar_wait(&raw_full[r], (uint32_t)((i / kRawSlots) & 1));
             if (ok && i >= kConvSlots) ok = mbar_wait(&conv_empty[c], (uint32_t)(((i / kConvSlots) - 1) & 1));
@@ -287,22 +297,24 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
         }
     } else if (warp == kWMma) {
         // ------------------------------------------------------------------ MMA
-        if (lane == 0) {
+        // the whole warp runs the loop and waits; one elected lane issues
+        {
             // slice pairs in product order (0,0) (0,1) (1,0) (0,2) (1,1) (2,0)
             constexpr uint32_t kPa = 0x210100u, kPb = 0x012010u;
             bool issued = false;
             int64_t i = 0;
             for (int64_t t = first; t < a.t_end; t += step, ++i) {
                 const int c = (int)(i % kConvSlots), b = (int)(i % kAccs);
-                bool ok = !abort_flag && mbar_wait(&conv_full[c], (uint32_t)((i / kConvSlots) & 1));
-                if (ok && i >= kAccs) ok = mbar_wait(&acc_empty[b], (uint32_t)(((i / kAccs) - 1) & 1));
-                if (!ok) {
-                    give_up();
+                bool ok = mbar_wait_or(&conv_full[c], (uint32_t)((i / kConvSlots) & 1), abort_now);
+                if (ok && i >= kAccs) ok = mbar_wait_or(&acc_empty[b], (uint32_t)(((i / kAccs) - 1) & 1), abort_now);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    if (lane == 0) give_up();
                     break;
                 }
                 tc_fence_after();
-                const STile s = recs[i % kRecs];  // visible through the converters' arrival
-                const int Kp = s.K <= 16 ? 16 : 32, Mp = (s.M + 15) & ~15;
+                const STile &s = recs[i % kRecs];  // visible through the converters' arrival
+                const int Kp = __shfl_sync(0xffffffffu, s.K <= 16 ? 16 : 32, 0);
+                const int Mp = __shfl_sync(0xffffffffu, (s.M + 15) & ~15, 0);
                 const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(Mp >> 3) << 17) |
                                        ((uint32_t)(kRows >> 4) << 24);
                 const uint32_t sa = smem_u32(conv + c * kConvSlot), sb = sa + kOpA;
@@ -326,14 +338,18 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
                         }
                     }
                 };
-                if (a.nprod == 6) issue(std::integral_constant<int, 6>{});
-                else issue(std::integral_constant<int, 3>{});
-                mma_commit(&conv_empty[c]);
-                mma_commit(&acc_full[b]);
+                if (elect_one()) {
+                    if (a.nprod == 6) issue(std::integral_constant<int, 6>{});
+                    else issue(std::integral_constant<int, 3>{});
+                    mma_commit(&conv_empty[c]);
+                    mma_commit(&acc_full[b]);
+                }
+                __syncwarp();
                 issued = true;
             }
             if (issued) {  // every MMA issued is complete before the memory is freed
-                mma_commit(&drain);
+                if (elect_one()) mma_commit(&drain);
+                __syncwarp();
                 mbar_wait(&drain, 0);
             }
         }
@@ -361,6 +377,40 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
             }
             tc_fence_after();
             const int M = s.M, nbase = qd * 32;
+            const int rows = min(32, s.nvalid - nbase);
+            if (M <= 32) {
+                // the warp's 32 rows are one run of C: through shared memory
+                // with an odd pitch, then in order
+                const int P = M | 1;
+                uint32_t v[32];
+                tmem_ld32(tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(b * kMaxM), v);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&acc_empty[b]);
+#pragma unroll
+                for (int j8 = 0; j8 < 32; j8 += 8) {
+                    if (j8 >= M) break;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (j8 + j < M) stg[lane * P + j8 + j] = __uint_as_float(v[j8 + j]);
+                }
+                __syncwarp();
+                const int total = rows * M, odd = P - M;
+                float *Crun = s.C + (s.n0 + nbase) * M;
+                int row = lane / M, col = lane - row * M;
+                const int dq = 32 / M, dm = 32 - dq * M;
+#pragma unroll 4
+                for (int e = lane; e < total; e += 32) {
+                    float x = a.alpha * stg[e + row * odd];
+                    if (a.init == 1) x = fmaf(a.beta, Crun[e], x);
+                    Crun[e] = x;
+                    row += dq;
+                    col += dm;
+                    if (col >= M) col -= M, ++row;
+                }
+                __syncwarp();  // the buffer is free for the next tile
+                continue;
+            }
             for (int c0 = 0; c0 < M; c0 += 32) {
                 uint32_t v[32];
                 tmem_ld32(tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(b * kMaxM + c0), v);
@@ -378,7 +428,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
 #pragma unroll
                 for (int rr = 0; rr < 32; ++rr) x[rr] = a.alpha * stg[rr * 33 + lane];
                 __syncwarp();  // the buffer is free for the next chunk
-                const int mv = min(32, M - c0), rows = min(32, s.nvalid - nbase);
+                const int mv = min(32, M - c0);
                 if (lane < mv) {
                     float *Crow = s.C + (s.n0 + nbase) * M + c0 + lane;
                     if (a.init == 1) {
