@@ -368,6 +368,11 @@ __device__ __forceinline__ void store_cols(const uint32_t (&r)[W], float *__rest
     if (lin != 0) {
         float *p = C + om + on0 + (int64_t)c0 * lin;
         const int64_t jn = nval - c0;
+        if (init == 2 && jn >= W) {  // no test and no dependent address per column
+#pragma unroll
+            for (int j = 0; j < W; ++j) p[j * lin] = alpha * __uint_as_float(r[j]);
+            return;
+        }
 #pragma unroll
         for (int j = 0; j < W; ++j) {
             if (j < jn) {
