@@ -136,13 +136,18 @@ struct PackJob {
     char *out;
 };
 
-constexpr int kPackRows = 32, kPackK = 128, kPackThreads = 256;
+constexpr int kPackRows = 32, kPackThreads = 256;
+// K positions a block takes: enough loads in flight at two bytes each
+template <int KIND>
+__host__ __device__ constexpr int pack_k() {
+    return KIND == GK_BF16 || KIND == GK_F16 ? 256 : 128;
+}
 
 template <int KIND>
 __global__ void __launch_bounds__(kPackThreads) pack_images_kernel(const __grid_constant__ PackedDesc d,
                                                                    const PackJob ja, const PackJob jb) {
     using T = Traits<KIND>;
-    constexpr int BK = stage_k<KIND>(), CH = T::kChunk;
+    constexpr int BK = stage_k<KIND>(), CH = T::kChunk, kPackK = pack_k<KIND>();
     constexpr bool kFloatIn = float_input(KIND);
     using L = typename std::conditional<kFloatIn, float, unsigned short>::type;
     // pitches that keep both the store along K and the read along rows free
@@ -160,6 +165,7 @@ __global__ void __launch_bounds__(kPackThreads) pack_images_kernel(const __grid_
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     const L *__restrict__ src = (const L *)(J.op == 0 ? d.A : d.B);
     if (tid < kPackK) {
+        static_assert(kPackK <= kPackThreads, "one thread per K offset");
         int64_t k = k0 + tid, o = -1, u = 0;
         if (k < d.K) {
             o = 0;
@@ -170,14 +176,15 @@ __global__ void __launch_bounds__(kPackThreads) pack_images_kernel(const __grid_
             }
         }
         koff[tid] = o;
-    } else if (tid < kPackK + kPackRows) {
-        int64_t r = r0 + tid - kPackK, o = -1, u = 0;
+    }
+    if (warp == kPackThreads / 32 - 1) {
+        int64_t r = r0 + lane, o = -1, u = 0;
         if (r < (J.op == 0 ? d.M : d.N)) {
             o = 0;
             if (J.op == 0) decode(r, d.nm, d.m_ext, d.m_sA, d.m_sC, o, u);
             else decode(r + d.n_begin, d.nn, d.n_ext, d.n_sB, d.n_sC, o, u);
         }
-        roff[tid - kPackK] = o;
+        roff[lane] = o;
     }
     __syncthreads();
     constexpr int NL = kPackK * kPackRows / kPackThreads;  // elements per thread
@@ -1180,7 +1187,7 @@ tc_status run_packed(Plan &p, PackedDesc &d, bool comp, int64_t comp_k, double f
     // has the smaller stride
     ja.rfast = d.nm > 0 && (d.nk == 0 || d.m_sA[0] < d.k_sA[d.nk - 1]);
     jb.rfast = d.nn > 0 && (d.nk == 0 || d.n_sB[0] < d.k_sB[d.nk - 1]);
-    const int64_t kblocks = ((int64_t)d.ktiles * BK + kPackK - 1) / kPackK;
+    const int64_t kblocks = ((int64_t)d.ktiles * BK + pack_k<KIND>() - 1) / pack_k<KIND>();
     CUtensorMap ta, tb;
     s = image_map(ta, ja.out, bytes_a, d.img_a);
     if (s == TC_SUCCESS) s = image_map(tb, jb.out, bytes_b, d.img_b);
