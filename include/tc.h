@@ -505,9 +505,10 @@ tc_status tc_batch_destroy(tc_batch batch);
 /* Tile policy.  TC_F32 / TC_F64 tiles hold 4096 outputs, (8 << s) rows x
  * (512 >> s) columns for s = 0..4, and K runs in chunks of 8, 16 or 32:
  * 0 (fixed) 64 x 64 with chunks of 16; 1 (rule, the default) the smallest
- * tile height that covers the problem's M, with the largest chunk that
- * fits; 2 (autotuned) the choice of tc_batch_autotune for the problem's
- * shape class.  TC_BF16X3: 0 (fixed) tensor-core GETT tiles of 128 x 256;
+ * tile height that covers the problem's M (TC_F64: the shape that pads M x N
+ * least), with the largest chunk that fits; 2 (autotuned) the choice of
+ * tc_batch_autotune for the problem's shape class.  TC_BF16X3: 0 (fixed)
+ * tensor-core GETT tiles of 128 x 256;
  * 1 (rule) the split-BF16 stream kernel -- one MMA tile per 128 columns n
  * with all of M, for batches whose every problem has A, B and C dense
  * along m, k and m, K a multiple of 4 up to 32 and M up to 128 (with A

@@ -224,11 +224,12 @@ struct Acc<float> {
 
 // FMAs of one staged K chunk; K runs in increasing order.
 template <typename T, int SHAPE>
-__device__ __forceinline__ void batch_compute(const T *S, int bk, int kk4, int KP, Acc<T> &acc) {
+__device__ __forceinline__ void batch_compute(const T *S, int bk, int kk4, int KP, int nlim, Acc<T> &acc) {
     constexpr int TM = shape_rows(SHAPE), TX = TM / 8, TY = kThreadsB / TX;
     const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
     const T *As = S + 4 * tx;
     const T *Bs = S + bk * TM + ty * KP;
+    (void)nlim;
     for (int k4 = 0; k4 < kk4; k4 += 4) {
         T b[4][4];
 #pragma unroll
@@ -243,7 +244,7 @@ __device__ __forceinline__ void batch_compute(const T *S, int bk, int kk4, int K
                 if constexpr (sizeof(T) == 4) {
 #pragma unroll
                     for (int i = 0; i < 4; ++i) fma_f2(acc.v[i][j], make_float2(a[2 * i], a[2 * i + 1]), b[j][kq]);
-                } else {
+                } else if (j * TY < nlim) {  // (FP64: not on slots of columns past the tile)
 #pragma unroll
                     for (int i = 0; i < 8; ++i) acc.v[i][j] = fma(a[i], b[j][kq], acc.v[i][j]);
                 }
@@ -417,11 +418,11 @@ __global__ void __launch_bounds__(kThreadsB, 4) batch_kernel(const BatchProblem 
         if (g.chunk == 0) acc.zero();
         T *S = stages + slot * kStageElems;
         switch (shape) {
-            case 0: batch_compute<T, 0>(S, bk, kk4, KP, acc); break;
-            case 1: batch_compute<T, 1>(S, bk, kk4, KP, acc); break;
-            case 2: batch_compute<T, 2>(S, bk, kk4, KP, acc); break;
-            case 3: batch_compute<T, 3>(S, bk, kk4, KP, acc); break;
-            default: batch_compute<T, 4>(S, bk, kk4, KP, acc); break;
+            case 0: batch_compute<T, 0>(S, bk, kk4, KP, g.nlim, acc); break;
+            case 1: batch_compute<T, 1>(S, bk, kk4, KP, g.nlim, acc); break;
+            case 2: batch_compute<T, 2>(S, bk, kk4, KP, g.nlim, acc); break;
+            case 3: batch_compute<T, 3>(S, bk, kk4, KP, g.nlim, acc); break;
+            default: batch_compute<T, 4>(S, bk, kk4, KP, g.nlim, acc); break;
         }
         if (g.last) {
             switch (shape) {
@@ -526,9 +527,19 @@ std::tuple<int, int, int> class_of(const BatchProblem &P) {
 // they cut the number of chunks
 bool chunk_useful(int bk, int64_t kmax) { return bk == 8 || kmax > bk / 2; }
 
-// rule: the smallest tile height that covers M, the largest K chunk
-std::pair<int, int> rule_choice(int64_t M, int64_t kmax) {
-    const int s = std::max(0, std::min(kShapes - 1, ceil_log2(M) - 3));
+// rule: the smallest tile height that covers M, the largest K chunk.  FP64,
+// whose unit takes 16 clocks for a warp's multiply-adds, valid or padding:
+// the shape that pads M x N least (the tallest of equals).
+std::pair<int, int> rule_choice(int64_t M, int64_t N, int64_t kmax, bool f64) {
+    int s = std::max(0, std::min(kShapes - 1, ceil_log2(M) - 3));
+    if (f64) {
+        auto padded = [&](int x) {
+            const int64_t r = shape_rows(x), c = shape_cols(x);
+            return ((M + r - 1) / r * r) * ((N + c - 1) / c * c);
+        };
+        for (int x = kShapes - 1; x >= 0; --x)
+            if (padded(x) < padded(s)) s = x;
+    }
     int bk = 32;
     while (bk > 8 && (!stage_fits(s, bk) || !chunk_useful(bk, kmax))) bk /= 2;
     return {s, bk};
@@ -606,10 +617,10 @@ void assign_tiles(BatchImpl &b) {
         if (b.policy == 0) {
             c = fixed_choice(P.K);
         } else if (b.policy == 1) {
-            c = rule_choice(P.M, P.K);
+            c = rule_choice(P.M, P.N, P.K, b.dtype == TC_F64);
         } else {
             auto it = b.tuned.find(class_of(P));
-            c = it != b.tuned.end() ? it->second : rule_choice(P.M, P.K);
+            c = it != b.tuned.end() ? it->second : rule_choice(P.M, P.N, P.K, b.dtype == TC_F64);
         }
         set_tiles_of(P, c.first, c.second, t);
     }
@@ -1101,7 +1112,7 @@ tc_status tc_batch_autotune(tc_batch batch, void *stream, int32_t reps, tc_batch
                     continue;
                 }
             }
-            const std::pair<int, int> rule = rule_choice(mmax, kmax), fixed = fixed_choice(kmax);
+            const std::pair<int, int> rule = rule_choice(mmax, b.probs[g.second[0]].N, kmax, b.dtype == TC_F64), fixed = fixed_choice(kmax);
             double best = -1;
             std::pair<int, int> arg = rule;
             for (int sh = 0; sh < kShapes && s == TC_SUCCESS; ++sh) {
