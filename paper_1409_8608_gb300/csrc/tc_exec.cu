@@ -92,6 +92,19 @@ template <>
 __device__ __forceinline__ float fma_t<float>(float a, float b, float c) { return fmaf(a, b, c); }
 
 // ---------------------------------------------------------------- dot/axpy/gemv/ger
+// x = q * y + r for non-negative x, y > 0, in 32 bits when both fit (a
+// 64-bit division is a long dependent sequence on every tile's first path)
+__device__ __forceinline__ int64_t divmod_pos(int64_t x, int64_t y, int64_t &r) {
+    if (((x | y) >> 31) == 0) {
+        const uint32_t q = (uint32_t)x / (uint32_t)y;
+        r = x - (int64_t)q * y;
+        return q;
+    }
+    const int64_t q = x / y;
+    r = x - q * y;
+    return q;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) elementwise_kernel(const PhaseDesc d) {
     const T *__restrict__ A = (const T *)d.A;
@@ -103,14 +116,14 @@ __global__ void __launch_bounds__(256) elementwise_kernel(const PhaseDesc d) {
          e += (int64_t)gridDim.x * blockDim.x) {
         int64_t r = e, oA = 0, oB = 0, oC = 0;
         for (int m = 0; m < d.out.n; ++m) {
-            int64_t x = r % d.out.ext[m];
+            const int64_t x = r % d.out.ext[m];
             r /= d.out.ext[m];
             oA += x * d.out.sA[m];
             oB += x * d.out.sB[m];
             oC += x * d.out.sC[m];
         }
         for (int m = d.task.n - 1; m >= 0; --m) {
-            int64_t x = r % d.task.ext[m];
+            const int64_t x = r % d.task.ext[m];
             r /= d.task.ext[m];
             oA += x * d.task.sA[m];
             oB += x * d.task.sB[m];
@@ -138,7 +151,22 @@ __global__ void __launch_bounds__(256) elementwise_kernel(const PhaseDesc d) {
                     pa += idx[m] * d.red.sA[m];
                     pb += idx[m] * d.red.sB[m];
                 }
-                for (int64_t k = 0; k < kext; ++k) {
+                // four positions' loads in flight at a time, multiplied in
+                // order (one at a time each waited for its own loads)
+                int64_t k = 0;
+                for (; k + 4 <= kext; k += 4) {
+                    T a[4], b[4];
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        a[x] = A[pa + x * ksA];
+                        b[x] = B[pb + x * ksB];
+                    }
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) acc = fma_t<T>(d.alpha_one ? a[x] : alpha * a[x], b[x], acc);
+                    pa += 4 * ksA;
+                    pb += 4 * ksB;
+                }
+                for (; k < kext; ++k) {
                     T a = A[pa];
                     if (!d.alpha_one) a = alpha * a;
                     acc = fma_t<T>(a, B[pb], acc);
@@ -225,19 +253,6 @@ __global__ void __launch_bounds__(256) coop_reduce_kernel(const PhaseDesc d) {
 }
 
 // ---------------------------------------------------------------- gemm / SIMT GETT
-// x = q * y + r for non-negative x, y > 0, in 32 bits when both fit (a
-// 64-bit division is a long dependent sequence on every tile's first path)
-__device__ __forceinline__ int64_t divmod_pos(int64_t x, int64_t y, int64_t &r) {
-    if (((x | y) >> 31) == 0) {
-        const uint32_t q = (uint32_t)x / (uint32_t)y;
-        r = x - (int64_t)q * y;
-        return q;
-    }
-    const int64_t q = x / y;
-    r = x - q * y;
-    return q;
-}
-
 __device__ __forceinline__ uint64_t pack_f2(float lo, float hi) {
     uint64_t r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
@@ -580,8 +595,8 @@ __device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid, TileSm
 constexpr int kSimtShapes = 3;
 constexpr int simt_rows(bool f64, int shape) { return (f64 ? 64 : 128) >> shape; }
 
-// The largest shape whose tiles give each SM at least two (FP32, two
-// blocks resident) or eight (FP64), else the smallest.
+// The largest shape whose tiles give most SMs one (FP32) or each SM eight
+// (FP64), else the smallest.
 int simt_shape(bool f64, int64_t M, int64_t N, int64_t tasks);
 
 template <typename T, int SHAPE>
@@ -665,7 +680,7 @@ __global__ void __launch_bounds__(256) gather_kernel(const GatherDesc g) {
          e += (int64_t)gridDim.x * blockDim.x) {
         int64_t r = e, os = 0, od = 0;
         for (int m = 0; m < g.n; ++m) {
-            int64_t x = r % g.ext[m];
+            const int64_t x = r % g.ext[m];
             r /= g.ext[m];
             os += x * g.ss[m];
             od += x * g.sd[m];
@@ -701,7 +716,7 @@ int device_sms() {
 int simt_shape(bool f64, int64_t M, int64_t N, int64_t tasks) {
     for (int s = 0; s + 1 < kSimtShapes; ++s) {
         const int64_t b = simt_rows(f64, s);
-        if (((M + b - 1) / b) * ((N + b - 1) / b) * tasks >= (int64_t)device_sms() * (f64 ? 8 : 2)) return s;
+        if (((M + b - 1) / b) * ((N + b - 1) / b) * tasks >= (f64 ? (int64_t)device_sms() * 8 : (int64_t)device_sms() * 4 / 5)) return s;
     }
     return kSimtShapes - 1;
 }
@@ -910,7 +925,10 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
         // contracted index has unit stride in an input, a group of lanes per
         // output splits that index instead (coop_reduce_kernel, loads
         // contiguous across the group): the reduction, not the output count,
-        // then sets the parallelism.
+        // then sets the parallelism.  Each lane of a group repeats the index
+        // arithmetic of its output, which a short index does not pay for
+        // unless outputs are few: 130 k outputs of 9 x 11 positions FP32 took
+        // 91-101 us in groups, 16-21 us one thread per output.
         const int kr = pd.red.n - 1;
         if (alg.kernel == TC_KERNEL_GER && pd.out.n == 2 && pd.out.sC[1] < pd.out.sC[0]) {
             std::swap(pd.out.ext[0], pd.out.ext[1]);
@@ -919,7 +937,7 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
             std::swap(pd.out.sC[0], pd.out.sC[1]);
         }
         const bool k_unit = kr >= 0 && (pd.red.sA[kr] == 1 || pd.red.sB[kr] == 1);
-        if (k_unit && pd.red.ext[kr] > 1 && pd.total < (int64_t)device_sms() * 1024) coop_g = 1;
+        if (k_unit && pd.red.ext[kr] > 1 && pd.total < (int64_t)device_sms() * (pd.red.ext[kr] < 32 ? 64 : 1024)) coop_g = 1;
         if (coop_g) {
             const int64_t kext = pd.red.ext[kr];
             coop_g = kext <= 4 ? 4 : (kext <= 8 ? 8 : (kext <= 16 ? 16 : 32));
