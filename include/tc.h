@@ -159,11 +159,11 @@ tc_status tc_plan_select(tc_plan plan, int32_t alg_id);
 tc_status tc_plan_selected(tc_plan plan, int32_t *alg_id);
 
 /* Bytes of device workspace the algorithm needs (copy buffers; for GETT,
- * id 0, the pre-converted input of tc_plan_set_gett_pack, else 0; a large
- * TC_F64 / TC_F32 GETT needs none but uses scratch when it can have it, see
- * tc_execute).  The plan allocates it on the first tc_execute of that algorithm and keeps it
- * until tc_plan_destroy; call tc_execute once before capturing a CUDA
- * graph.  The workspace serves one execute at a time, so tc_execute
+ * id 0, the pre-converted input of tc_plan_set_gett_pack, else 0; a GETT
+ * may also use scratch that it can do without, see tc_execute and
+ * tc_plan_set_gett_pack).  The plan allocates it on the first tc_execute of
+ * that algorithm and keeps it until tc_plan_destroy; call tc_execute once
+ * before capturing a CUDA graph.  The workspace serves one execute at a time, so tc_execute
  * refuses a second stream while the plan's last execute is in flight
  * (below): give each stream its own plan. */
 tc_status tc_algorithm_workspace(tc_plan plan, int32_t alg_id, size_t *bytes);
@@ -186,8 +186,8 @@ tc_status tc_algorithm_workspace(tc_plan plan, int32_t alg_id, size_t *bytes);
  * too many small entries for that, infinities, NaN or extreme exponents run
  * as such chains, like smaller sizes.  The images of the digits take up to
  * 64 MiB for B and 256 MiB for A, allocated by the first execute outside a
- * stream capture and kept; when that fails, or inside a capture before, the
- * chains run instead. */
+ * stream capture and kept until tc_plan_destroy; when that fails, or inside
+ * a capture before, the chains run instead. */
 tc_status tc_execute(tc_plan plan, const void *alpha, const void *A,
                      const void *B, const void *beta, void *C, void *stream);
 
@@ -263,7 +263,13 @@ tc_status tc_plan_set_gett_tma(tc_plan plan, int32_t enable);
  * tc_plan_set_compensation) and wherever M and N are both at least 1024,
  * when their images fit in 2 GiB, else (FP32 inputs) the smaller input
  * when it has at most 1/8 of the larger one's elements and its images fit
- * in 64 MiB; 2: the smaller input (FP32 inputs) whenever its images fit in
+ * in 64 MiB.  Mode 1 also streams both inputs as images, without batch
+ * indices, from K = 128, and from K = 48 unless TMA stages both inputs of a
+ * result of at least 2^24 elements: in scratch of up to 512 MiB for B (in
+ * panels) and 256 MiB for A that the first execute outside a stream capture
+ * takes and the plan keeps; when it cannot be had, or inside a capture
+ * before, the form that the other rules choose runs.  2: the smaller input
+ * (FP32 inputs) whenever its images fit in
  * 64 MiB; 3: both inputs whenever their images fit in 2 GiB (else none),
  * the GETT then streams the images alone (in CTA pairs and tile widths of
  * its own choice).  Other values give
@@ -458,7 +464,8 @@ tc_status tc_chain_variants(tc_chain chain, tc_chain_variant *buf, int32_t capac
 /* Largest intermediate in bytes that tc_chain_select(-1) may choose (-1: no
  * limit).  The limit covers the intermediate only: with a tensor-core
  * dtype a step's plan may also hold the pre-converted images of its inputs
- * (tc_plan_set_gett_pack's default), allocated by its first execute. */
+ * (tc_plan_set_gett_pack's default), and with TC_F64 or TC_F32 the digits'
+ * (tc_execute), allocated by its first execute. */
 tc_status tc_chain_set_workspace_limit(tc_chain chain, int64_t bytes);
 
 /* Predicts every variant: for each step, tc_predict over every algorithm

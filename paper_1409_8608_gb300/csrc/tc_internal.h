@@ -78,6 +78,8 @@ struct Plan {
     void *gett_state = nullptr;     // owned by the GETT executor
     void *scratch = nullptr;        // GETT: images that an execute can do without (tc_packed.cu)
     size_t scratch_bytes = 0;
+    size_t scratch_refused = SIZE_MAX;  // what could not be allocated
+    std::vector<void *> scratch_old;    // outgrown, freed with the plan
     void *qbuf = nullptr;           // TC_E4M3: the inputs' maxima and scales (16 bytes)
     void *flush_buf = nullptr;      // predictor: remote regions / L2 flush
     size_t flush_bytes = 0;

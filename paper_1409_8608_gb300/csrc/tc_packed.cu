@@ -1074,12 +1074,8 @@ Tile choose_tile(int64_t M, int64_t N, double ksteps, int nprod, int slices, int
 template <int KIND, bool COMP, bool PAIR>
 tc_status launch_gett(const PackedDesc &d, const CUtensorMap &ta, const CUtensorMap &tb, cudaStream_t st) {
     auto kern = packed_gett_kernel<KIND, COMP, PAIR>;
-    static bool configured = false;
-    if (!configured) {
-        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
-        if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
-        configured = true;
-    }
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes);
+    if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kRingBytes;
@@ -1101,7 +1097,7 @@ tc_status launch_gett(const PackedDesc &d, const CUtensorMap &ta, const CUtensor
     cfg.gridDim = dim3((unsigned)grid);
     cfg.attrs = attr;
     cfg.numAttrs = na;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, d, ta, tb);
+    e = cudaLaunchKernelEx(&cfg, kern, d, ta, tb);
     if (e == cudaSuccess) e = cudaGetLastError();
     return e == cudaSuccess ? TC_SUCCESS : fail(TC_ERROR_CUDA, cudaGetErrorString(e));
 }
@@ -1116,22 +1112,30 @@ constexpr int64_t kPanelBytes = int64_t(512) << 20;
 constexpr int64_t kScratchMaxABytes = int64_t(256) << 20;
 
 // Scratch that an execute can do without: taken once, outside a capture, and
-// kept.  False: not to be had, the caller runs the form without it.
+// kept.  False: not to be had, the caller runs the form without it, and the
+// plan does not ask for as much again.  Another thread's global-mode capture
+// is not to fail for it, so the allocation runs in relaxed mode.  A larger one
+// keeps the smaller until the plan goes: graphs may hold its address.
 bool optional_scratch(Plan &p, int64_t bytes, cudaStream_t st) {
     if (p.scratch_bytes >= (size_t)bytes) return true;
+    if ((size_t)bytes >= p.scratch_refused) return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
         return false;
     }
-    if (p.scratch) cudaFree(p.scratch);
-    p.scratch = nullptr;
-    p.scratch_bytes = 0;
-    if (cudaMalloc(&p.scratch, (size_t)bytes) != cudaSuccess) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    void *mem = nullptr;
+    const cudaError_t e = cudaMalloc(&mem, (size_t)bytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
         cudaGetLastError();
-        p.scratch = nullptr;
+        p.scratch_refused = (size_t)bytes;
         return false;
     }
+    if (p.scratch) p.scratch_old.push_back(p.scratch);
+    p.scratch = mem;
     p.scratch_bytes = (size_t)bytes;
     return true;
 }
@@ -1292,9 +1296,9 @@ tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta
     constexpr int BK = stage_k<KIND>();
     DigitPlan P;
     if (!plan_digits<KIND>(d.M, d.N, d.K, P)) return TC_SUCCESS;
-    if (!optional_scratch(p, P.bytes, st)) return TC_SUCCESS;  // the SIMT tiles run
     tc_status s = ensure_device_resources(p, 0);
     if (s != TC_SUCCESS) return s;
+    if (!optional_scratch(p, P.bytes, st)) return TC_SUCCESS;  // the SIMT tiles run
     char *ws = (char *)p.scratch;
     if constexpr (D::F64) {
         d.alpha64 = *(const double *)alpha;
@@ -1327,13 +1331,9 @@ tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta
     if (s == TC_SUCCESS) s = image_map(tb, ws + P.off_b, P.image_b, d.img_b);
     if (s != TC_SUCCESS) return s;
     constexpr int kPackSmem = kDigitK * (kPackRows + 1) * (int)sizeof(typename D::In);
-    static bool configured = false;
-    if (!configured) {
-        const cudaError_t ea = cudaFuncSetAttribute(pack_digits_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPackSmem);
-        if (ea != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(ea));
-        configured = true;
-    }
-    cudaError_t e = cudaMemsetAsync(ws + P.off_small_a, 0, (size_t)P.zero_bytes, st);
+    cudaError_t e = cudaFuncSetAttribute(pack_digits_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPackSmem);
+    if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
+    e = cudaMemsetAsync(ws + P.off_small_a, 0, (size_t)P.zero_bytes, st);
     if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
     for (int64_t t0 = 0; t0 < tiles_n; t0 += P.panel_tiles) {
         d.n_begin = t0 * D::kBn;

@@ -348,6 +348,7 @@ tc_status tc_plan_destroy(tc_plan plan) {
         if (p.flush_buf) cudaFree(p.flush_buf);
         if (p.qbuf) cudaFree(p.qbuf);
         if (p.scratch) cudaFree(p.scratch);
+        for (void *old : p.scratch_old) cudaFree(old);
         if (p.busy_event) cudaEventDestroy((cudaEvent_t)p.busy_event);
         for (void *d : p.host_dev)
             if (d) cudaFree(d);

@@ -122,6 +122,9 @@ def test_left_to_simt(tcmod, dtype):
     bad[[5, 6, 7, 8, 280, 281]] = True
     bad[:, [70, N - 1]] = True
     assert np.array_equal(got[bad], simt[bad], equal_nan=True)
+    C0 = rng.uniform(-1, 1, (M, N)).astype(NP[dtype])
+    got2, simt2 = execute(tcmod, dtype, A, B, C0, 0.5, -2.0)
+    assert np.array_equal(got2[bad], simt2[bad], equal_nan=True)
     i, j = np.nonzero(~bad)
     pick = rng.integers(0, len(i), 2000)
     i, j = i[pick], j[pick]
