@@ -59,10 +59,10 @@
 // left.  Tiles where that does not hold (wide ranges or many zeros along K,
 // infinities, NaN, exponents near the ends) go to a list, and the SIMT tiles
 // compute them.  B is taken in panels whose images stay in L2.
-// abc=iaj,jbic 512^3 i=j=16: FP64 56.7 -> 3.28 ms (18 panels: pre-pass 23 us,
-// GETT 160 us each; the shared-memory port takes 1760 of its clocks per 16 K
-// positions, draining the levels, which nothing overlaps, most of the rest),
-// FP32 2.35 -> 0.62 ms (9 panels: 21 and 45 us).  Error against 80-bit and
+// abc=iaj,jbic 512^3 i=j=16: FP64 56.7 -> 3.16 ms (18 panels: pre-pass 23 us,
+// GETT 153 us each; 160 where every product reads its digit of A from shared
+// memory, not from the collector buffer; draining the levels, which nothing
+// overlaps, takes most of the rest), FP32 2.35 -> 0.59 ms (9 panels).  Error against 80-bit and
 // longer sums on uniform entries: below that of the chains (FP32 3.2e-8
 // against 2.9e-7 of the result's 2-norm).
 //
@@ -720,11 +720,16 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
 #pragma unroll
                     for (int s = 0; s < S; ++s)
 #pragma unroll
-                        for (int t = 0; t < S - s; ++t)
-                            mma_issue<KIND, PAIR>(dt + (uint32_t)(KIND == GK_D64 ? (s + t) * 64 : (s + t ? 128 : 0)),
-                                                  as + (uint64_t)((s * sliceA + ks * 2 * lboA) >> 4),
-                                                  bs + (uint64_t)((t * sliceB + ks * 2 * lboB) >> 4), idesc,
-                                                  !(first && ks == 0 && s == 0 && (KIND == GK_D64 || t < 2)));
+                        for (int t = 0; t < S - s; ++t) {
+                            const uint32_t dst = dt + (uint32_t)(KIND == GK_D64 ? (s + t) * 64 : (s + t ? 128 : 0));
+                            const uint64_t ad = as + (uint64_t)((s * sliceA + ks * 2 * lboA) >> 4);
+                            const uint64_t bd = bs + (uint64_t)((t * sliceB + ks * 2 * lboB) >> 4);
+                            const bool acc = !(first && ks == 0 && s == 0 && (KIND == GK_D64 || t < 2));
+                            if (s == S - 1) mma_issue<KIND, PAIR>(dst, ad, bd, idesc, acc);
+                            else if (t == 0) mma_issue_same_a<PAIR, 0>(dst, ad, bd, idesc, acc);
+                            else if (t == S - s - 1) mma_issue_same_a<PAIR, 2>(dst, ad, bd, idesc, acc);
+                            else mma_issue_same_a<PAIR, 1>(dst, ad, bd, idesc, acc);
+                        }
                 }
             };
             auto commit = [&](uint64_t *bar) {
