@@ -59,10 +59,10 @@
 // left.  Tiles where that does not hold (wide ranges or many zeros along K,
 // infinities, NaN, exponents near the ends) go to a list, and the SIMT tiles
 // compute them.  B is taken in panels whose images stay in L2.
-// abc=iaj,jbic 512^3 i=j=16: FP64 56.7 -> 3.16 ms (18 panels: pre-pass 23 us,
-// GETT 153 us each; 160 where every product reads its digit of A from shared
-// memory, not from the collector buffer; draining the levels, which nothing
-// overlaps, takes most of the rest), FP32 2.35 -> 0.59 ms (9 panels).  Error against 80-bit and
+// abc=iaj,jbic 512^3 i=j=16: FP64 56.7 -> 2.74 ms (18 panels: pre-pass 23 us,
+// GETT 128 us each; 135 where every product reads its digit of A from shared
+// memory, not from the collector buffer, 153 with a conversion that branches;
+// without the drains and conversions 92), FP32 2.35 -> 0.59 ms (9 panels).  Error against 80-bit and
 // longer sums on uniform entries: below that of the chains (FP32 3.2e-8
 // against 2.9e-7 of the result's 2-norm).
 //
@@ -528,33 +528,30 @@ __device__ __forceinline__ void store_row_low(const uint32_t (&r)[32], float *__
     }
 }
 
-// (hi 2^24 + lo) 2^s rounded to nearest even; the result is a normal number.
+// (hi 2^24 + lo) 2^s rounded to nearest even, |hi| < 2^58; the result is zero
+// or a normal number.  Without branches (about 50 integer instructions) and
+// without the FP64 unit, which takes 16 clocks for a warp's instruction.
 __device__ __forceinline__ double fixed_to_double(int64_t hi, int64_t lo, int s) {
-    // the 96-bit sum as (h, l), l the lowest 32 bits, unsigned
-    const uint64_t low32 = ((uint64_t)(hi & 0xff) << 24) + (uint32_t)lo;
-    int64_t h = (hi >> 8) + (lo >> 32) + (int64_t)(low32 >> 32);
-    uint32_t l = (uint32_t)low32;
-    const uint64_t sign = (uint64_t)h & 0x8000000000000000ull;
-    if (h < 0) {
-        h = l ? ~h : -h;
-        l = 0u - l;
-    }
-    if (((uint64_t)h | l) == 0) return 0.0;
-    // left-aligned: 64 bits and a sticky bit
-    uint64_t top;
-    uint32_t rest = 0;
-    const int z = h ? __clzll(h) : 64 + __clz((int)l);  // leading zeros of the 96 bits
-    if (z < 32) {
-        top = z ? ((uint64_t)h << z) | (l >> (32 - z)) : (uint64_t)h;
-        rest = l << z;
-    } else {
-        top = (((uint64_t)(uint32_t)h << 32) | l) << (z - 32);
-    }
-    uint64_t m = top >> 11;  // 53 bits, the leading one at bit 52
-    const uint32_t low = (uint32_t)top & 0x7ffu;
-    m += low > 0x400u || (low == 0x400u && (rest != 0 || (m & 1)));
-    const int field = 95 - z + s + 1023;
-    return __longlong_as_double((int64_t)(sign | (((uint64_t)(field - 1) << 52) + m)));
+    // the magnitude times 2^8 in three words
+    const int64_t h = hi + (lo >> 24);
+    const uint32_t sg = (uint32_t)((int32_t)(h >> 32) >> 31);
+    uint32_t w0 = ((uint32_t)lo << 8) ^ sg, w1 = (uint32_t)h ^ sg, w2 = (uint32_t)(h >> 32) ^ sg;
+    asm("sub.cc.u32 %0, %0, %3;\n\tsubc.cc.u32 %1, %1, %3;\n\tsubc.u32 %2, %2, %3;" : "+r"(w0), "+r"(w1), "+r"(w2) : "r"(sg));
+    // the leading one to bit 31 of w2
+    int e = s + 87 + 1022;
+    bool c = w2 == 0;
+    w2 = c ? w1 : w2, w1 = c ? w0 : w1, w0 = c ? 0 : w0, e -= c ? 32 : 0;
+    c = w2 == 0;
+    w2 = c ? w1 : w2, w1 = c ? w0 : w1, e -= c ? 32 : 0;
+    const int z = __clz((int)w2);
+    const uint32_t top = __funnelshift_l(w1, w2, z), mid = __funnelshift_l(w0, w1, z), end = w0 << z;
+    // 53 bits, the rest and a sticky bit
+    uint32_t mh = top >> 11, ml = __funnelshift_r(mid, top, 11);
+    const uint32_t rest = mid << 21 | (end != 0 ? 1u : 0u);
+    const uint32_t up = rest + (ml & 1u) > 0x80000000u ? 1u : 0u;
+    asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+r"(ml), "+r"(mh) : "r"(up));
+    mh = (mh + ((uint32_t)(e - z) << 20)) | (sg & 0x80000000u);
+    return __hiloint2double((int)(w2 == 0 ? 0u : mh), (int)ml);
 }
 
 // COMP: compensated accumulation -- units of d.chunk K stages, double-buffered
@@ -982,13 +979,13 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                 // (the next tile accumulates meanwhile)
                 const int *ce = cE[tab];
                 if (om >= 0) {
+                    double *at = (double *)d.C + om + (lin != 0 ? on0 + half * 32 * lin : 0);
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
+                    for (int j = 0; j < 32; ++j, at += lin) {
                         const int cc = half * 32 + j;
                         if (cc >= nval) break;
-                        double *q = (double *)d.C + om + (lin != 0 ? on0 + (int64_t)cc * lin : cn[cc]);
+                        double *q = lin != 0 ? at : at + cn[cc];
                         double v = fixed_to_double(dhi[j], dlo[j], rowE + ce[cc] - 2104);
-                        // (FP64 instructions cost 16 clocks a warp)
                         if (plain) *q = v;
                         else *q = d.init == 2 ? d.alpha64 * v : fma(d.alpha64, v, d.beta64 * *q);
                     }
