@@ -347,15 +347,18 @@ def measure_form(args, dtype, spec, extents, A, B, dev, stream, dist, world, tc,
     dA, dB = hA.to(dev), hB.to(dev)
     dC = torch.empty(nC, dtype=tout, device=dev)
     flops = plan.flops
-    # GETT: one kernel, plus the pre-pass when the plan pre-converts its
-    # smaller input (the only GETT workspace); nests: phases and copies
+    # GETT: one kernel, plus the pre-pass when the plan pre-converts inputs
+    # (its workspace, or scratch of tens of MiB that the first execute takes;
+    # both inputs in one launch); FP64 / FP32 from digits: also the tiles left
+    # to the SIMT kernel, and a further pair of launches per panel of the
+    # larger input, not counted here.  Nests: phases and copies
+    free0 = torch.cuda.mem_get_info()[0]
+    plan.execute(dA, dB, dC, alpha=1.0, beta=0.0, stream=stream)
+    torch.cuda.synchronize()
+    images = alg["kernel"] == "gett" and free0 - torch.cuda.mem_get_info()[0] > (16 << 20)
+    digits = images and dtype in ("f64", "f32")
     if alg["kernel"] == "gett":
-        # with a workspace: one pre-pass (the smaller input), or two (both
-        # inputs: the default of the compensated split forms, K past the
-        # 256-element chunk)
-        K = plan.flops // (2 * nC)
-        both = dtype in ("bf16x3", "tf32x3") and K > 256
-        launches_per_step = 1 + (2 if both else 1) * int(plan.workspace(alg["id"]) > 0)
+        launches_per_step = 1 + int(images or plan.workspace(alg["id"]) > 0) + int(digits)
     else:
         launches_per_step = alg["n_phases"] * (1 + sum(1 for lv in alg["copy_level"] if lv != -2))
 
@@ -454,11 +457,24 @@ def measure_form(args, dtype, spec, extents, A, B, dev, stream, dist, world, tc,
                     "frac": achieved_tf / peak_tf,
                     "traffic": captured_traffic(tkey, "paper_1409_8608_gb300/csrc/tc_gett.cu"),
                     "algorithmic_bytes": algorithmic_bytes,
-                    "kernel": "gett_tc_kernel" + (" + pack_kernel (timed together)" if launches_per_step == 2 else
-                                                  " + 2 x pack_kernel (timed together)" if launches_per_step == 3 else ""),
+                    "kernel": "packed_gett_kernel + pack_images_kernel (timed together)" if images else
+                              "gett_tc_kernel" + (" + pack_kernel (timed together)" if launches_per_step == 2 else ""),
                     "work": f"{prods} slice products x 2*prod(extents) = {work / 1e9:.1f} GFLOP per step",
                     "peak_source": "MEASURED_PEAKS bf16_tflops (burst)" +
                     (" x 0.5 (TF32 nominal ratio)" if dtype in ("tf32", "tf32x3") else "") +
+                    (" (fallback)" if peaks.get("fallback") else " (measured)")}
+    elif digits:
+        prods = 36 if dtype == "f64" else 10
+        work = flops * prods
+        achieved_tf, peak_tf = work / launch_s / 1e12, peaks["bf16_tflops"]
+        roofline = {"bound": "tensor", "achieved": achieved_tf, "peak": peak_tf, "unit": "TFLOP/s",
+                    "frac": achieved_tf / peak_tf,
+                    "traffic": captured_traffic(f"packed_gett_kernel/{dtype}/{spec}/{nkey}",
+                                                "paper_1409_8608_gb300/csrc/tc_packed.cu"),
+                    "algorithmic_bytes": algorithmic_bytes,
+                    "kernel": "packed_gett_kernel + pack_digits_kernel + tile_list_kernel (timed together)",
+                    "work": f"{prods} digit products x 2*prod(extents) = {work / 1e9:.1f} GFLOP per step",
+                    "peak_source": "MEASURED_PEAKS bf16_tflops (burst)" +
                     (" (fallback)" if peaks.get("fallback") else " (measured)")}
     else:
         achieved_tf = flops / launch_s / 1e12
@@ -562,7 +578,7 @@ PRECISION_FORMS = (
     ("tf32x3", "tf32x3", None, None),
     ("tf32", "tf32", None, None), ("bf16", "bf16", None, None), ("f16", "f16", None, None),
     ("fp8 e4m3 (power-of-two input scales)", "e4m3", None, None),
-    ("f32 (SIMT)", "f32", None, None), ("f64 (plain)", "f64", None, None),
+    ("f32", "f32", None, None), ("f64 (plain)", "f64", None, None),
 )
 
 
@@ -766,7 +782,7 @@ def run_gpu(args):
                 "steps": args.steps, "warmup": args.warmup, "ms_per_step": head["ms_per_step"],
                 "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64",
                 "data": "synthetic",
-                "config": {"workload": WORKLOAD, "algorithm": "gett (SIMT DFMA tiles)",
+                "config": {"workload": WORKLOAD, "algorithm": "gett (" + ("exact digits on tcgen05" if head["roofline"]["bound"] == "tensor" else "SIMT DFMA tiles") + ")",
                            "parallelism": f"replicas x{world}",
                            "l2": "inputs larger than L2 (no flush needed)"},
                 "roofline": head["roofline"], "e2e": head["e2e"], "gpu_launches": head["gpu_launches"],
@@ -788,7 +804,8 @@ def run_gpu(args):
         if forms:
             forms["bf16x3"]["form"] = "chosen: split-BF16 x6 slice products on tcgen05, FP32 I/O"
             forms["bf16x3"]["speedup_vs_f64"] = forms["bf16x3"]["value"] / head["value"]
-            forms["f32"]["form"] = "FP32 SIMT (FFMA tiles)"
+            forms["f32"]["form"] = "FP32 (exact digits on tcgen05)" if forms["f32"]["roofline"]["bound"] == "tensor" \
+                else "FP32 SIMT (FFMA tiles)"
             forms["tf32x3"]["form"] = "3xTF32: hi.hi + hi.lo + lo.hi on tcgen05 kind::tf32, FP32 I/O"
             forms["tf32x3"]["speedup_vs_f64"] = forms["tf32x3"]["value"] / head["value"]
             line["forms"] = forms

@@ -264,8 +264,8 @@ tc_status tc_plan_set_gett_tma(tc_plan plan, int32_t enable);
  * when their images fit in 2 GiB, else (FP32 inputs) the smaller input
  * when it has at most 1/8 of the larger one's elements and its images fit
  * in 64 MiB.  Mode 1 also streams both inputs as images, without batch
- * indices, from K = 128, and from K = 48 unless TMA stages both inputs of a
- * result of at least 2^24 elements: in scratch of up to 512 MiB for B (in
+ * indices, where that is the faster form (from a K of 48 to 257, by dtype,
+ * sizes and whether TMA can stage the inputs): in scratch of up to 512 MiB for B (in
  * panels) and 256 MiB for A that the first execute outside a stream capture
  * takes and the plan keeps; when it cannot be had, or inside a capture
  * before, the form that the other rules choose runs.  2: the smaller input

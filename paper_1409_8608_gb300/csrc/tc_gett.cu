@@ -1807,19 +1807,28 @@ static tc_status e4m3_scales(Plan &p, const void *A, const void *B, cudaStream_t
 // K = 143 301 x 19691 25 / 45, 21 / 42, 19 / 35; K = 64 300 x 200000 (ragged)
 // 91 / 120, 83 / 134, 77 / 95, but 512 x 512^2 181 / 151, 154 / 136, 145 / 153;
 // K = 16 512 x 512^2 147 / 115, 143 / 112, 142 / 110, K = 32 86 x 13800 14.2 /
-// 11.9 (split-BF16), K = 25 81 x 18190 12.4 / 10.4 (BF16).  So: from K = 128
-// always, from K = 48 unless TMA stages both inputs of a large result.
+// 11.9 (split-BF16), K = 25 81 x 18190 12.4 / 10.4 (BF16).  So: from K = 128,
+// from K = 48 unless TMA stages both inputs of a large result, but:
+// Images save nothing where one tile of M covers A and B is converted once
+// anyway, and cost a pass over B: abc=ai,ibc with 101283 columns, K = 64, M =
+// 74: FP16 27 us against 40 with images, split-BF16 33 / 38; K = 128 40 / 41
+// and 50 / 52; where TMA cannot stage B, FP16 K = 52 29 / 38, K = 100 46 / 41.
+// FP16 with two tiles of M, K = 64: 44 / 48, three 58 / 50; with 5000 columns
+// K = 64 15 / 16-18, K = 100 21 / 17 (split-BF16 17 / 17, 23 / 17).
 // (d, pk: the modes and the choice without this.)
 static bool images_win(const Plan &p, const GettModes &d, int pk) {
-    if (p.gett_pack != 1 || d.nb != 0 || d.K > (int64_t(1) << 24)) return false;
-    if (d.K >= 128) return true;
-    if (d.K < 48) return false;
-    if (p.dtype == TC_E4M3 || d.M * d.N < (int64_t(1) << 24)) return true;
-    const int in_bytes = (p.dtype == TC_BF16 || p.dtype == TC_F16) ? 2 : 4;
+    if (p.gett_pack != 1 || d.nb != 0 || d.K > (int64_t(1) << 24) || d.K < 48) return false;
+    const bool in16 = p.dtype == TC_BF16 || p.dtype == TC_F16;
+    const bool once = d.M <= kBM && d.N >= (int64_t(1) << 14);
+    if (once && (p.dtype == TC_BF16X3 || p.dtype == TC_TF32X3)) return d.K > 256;
+    if (in16 && d.K < 96 && (d.M <= 2 * kBM || d.M * d.N < (int64_t(1) << 22))) return false;
+    const bool once16 = in16 && once && d.K < 160;
+    if (!once16 && (d.K >= 128 || p.dtype == TC_E4M3 || d.M * d.N < (int64_t(1) << 24))) return true;
+    const int in_bytes = in16 ? 2 : 4;
     GettDesc t;
     std::memset(&t, 0, sizeof(t));
-    return !((pk == 1 || plan_tma_operand(p, OP_A, nullptr, in_bytes, kBM, d.nm, d.m_ext, d.m_sA, d.nk, d.k_ext, d.k_sA, t,
-                                          nullptr, kBKT)) &&
+    return !((once16 || pk == 1 ||
+              plan_tma_operand(p, OP_A, nullptr, in_bytes, kBM, d.nm, d.m_ext, d.m_sA, d.nk, d.k_ext, d.k_sA, t, nullptr, kBKT)) &&
              (pk == 2 || plan_tma_operand(p, OP_B, nullptr, in_bytes, 256, d.nn, d.n_ext, d.n_sB, d.nk, d.k_ext, d.k_sB, t,
                                           nullptr, kBKT)));
 }

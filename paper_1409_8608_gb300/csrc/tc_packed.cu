@@ -62,9 +62,9 @@
 // abc=iaj,jbic 512^3 i=j=16: FP64 56.7 -> 2.74 ms (18 panels: pre-pass 23 us,
 // GETT 128 us each; 135 where every product reads its digit of A from shared
 // memory, not from the collector buffer, 153 with a conversion that branches;
-// without the drains and conversions 92), FP32 2.35 -> 0.59 ms (9 panels).  Error against 80-bit and
-// longer sums on uniform entries: below that of the chains (FP32 3.2e-8
-// against 2.9e-7 of the result's 2-norm).
+// without the drains and conversions 92), FP32 2.35 -> 0.59 ms (9 panels).
+// Error against 80-bit and longer sums on uniform entries: below that of the
+// chains (FP32 3.2e-8 against 2.9e-7 of the result's 2-norm).
 //
 // Every wait on an mbarrier is bounded; on expiry the kernel records
 // TC_ERROR_TIMEOUT, stops issuing, drains, frees its tensor memory, returns.

@@ -48,6 +48,8 @@ IMAGES = [
     ("bca=iaj,jbic", {"a": 70, "b": 33, "c": 9, "i": 20, "j": 8}),
     ("cab=ija,bjic", {"a": 131, "b": 5, "c": 30, "i": 13, "j": 11}),
     ("dacb=aijd,cjbi", {"a": 17, "b": 6, "c": 40, "d": 9, "i": 30, "j": 9}),  # K = 270: past a chunk
+    ("abc=ai,ibc", {"a": 74, "b": 371, "c": 50, "i": 52}),   # one tile of M, many columns
+    ("abc=ai,ibc", {"a": 74, "b": 371, "c": 50, "i": 128}),
     ("ab=ai,ib", {"a": 4200, "b": 4100, "i": 50}),  # a result of more than 2^24
 ]
 
