@@ -349,14 +349,14 @@ def measure_form(args, dtype, spec, extents, A, B, dev, stream, dist, world, tc,
     flops = plan.flops
     # GETT: one kernel, plus the pre-pass when the plan pre-converts inputs
     # (its workspace, or scratch of tens of MiB that the first execute takes;
-    # both inputs in one launch); FP64 / FP32 from digits: also the tiles left
+    # both inputs in one launch); FP64 from digits: also the tiles left
     # to the SIMT kernel, and a further pair of launches per panel of the
     # larger input, not counted here.  Nests: phases and copies
     free0 = torch.cuda.mem_get_info()[0]
     plan.execute(dA, dB, dC, alpha=1.0, beta=0.0, stream=stream)
     torch.cuda.synchronize()
     images = alg["kernel"] == "gett" and free0 - torch.cuda.mem_get_info()[0] > (16 << 20)
-    digits = images and dtype in ("f64", "f32")
+    digits = images and dtype == "f64"
     if alg["kernel"] == "gett":
         launches_per_step = 1 + int(images or plan.workspace(alg["id"]) > 0) + int(digits)
     else:
@@ -464,7 +464,7 @@ def measure_form(args, dtype, spec, extents, A, B, dev, stream, dist, world, tc,
                     (" x 0.5 (TF32 nominal ratio)" if dtype in ("tf32", "tf32x3") else "") +
                     (" (fallback)" if peaks.get("fallback") else " (measured)")}
     elif digits:
-        prods = 36 if dtype == "f64" else 10
+        prods = 36
         work = flops * prods
         achieved_tf, peak_tf = work / launch_s / 1e12, peaks["bf16_tflops"]
         roofline = {"bound": "tensor", "achieved": achieved_tf, "peak": peak_tf, "unit": "TFLOP/s",
@@ -804,8 +804,7 @@ def run_gpu(args):
         if forms:
             forms["bf16x3"]["form"] = "chosen: split-BF16 x6 slice products on tcgen05, FP32 I/O"
             forms["bf16x3"]["speedup_vs_f64"] = forms["bf16x3"]["value"] / head["value"]
-            forms["f32"]["form"] = "FP32 (exact digits on tcgen05)" if forms["f32"]["roofline"]["bound"] == "tensor" \
-                else "FP32 SIMT (FFMA tiles)"
+            forms["f32"]["form"] = "FP32 SIMT (FFMA tiles)"
             forms["tf32x3"]["form"] = "3xTF32: hi.hi + hi.lo + lo.hi on tcgen05 kind::tf32, FP32 I/O"
             forms["tf32x3"]["speedup_vs_f64"] = forms["tf32x3"]["value"] / head["value"]
             line["forms"] = forms

@@ -177,12 +177,11 @@ tc_status tc_algorithm_workspace(tc_plan plan, int32_t alg_id, size_t *bytes);
  * another as usual.  While `stream` is capturing a CUDA graph the check is
  * skipped and nothing is recorded.
  *
- * TC_F64 and TC_F32 with GETT selected: where the size makes it the faster
- * form (K from 32 to 2^20, TC_F32 to 4096; no batch indices), the tensor
- * cores compute the contraction from exact 8-bit digits of the inputs, FP64
- * from 62 and FP32 from 30 bits below the largest magnitude of a row of A
- * and a column of B, rounded once: at least as close to the exact result as
- * a chain of K fused multiply-adds.  Parts of C whose rows or columns hold
+ * TC_F64 with GETT selected: where the size makes it the faster form (K from
+ * 32 to 2^20; no batch indices), the tensor cores compute the contraction
+ * from exact 8-bit digits of the inputs, 62 bits below the largest magnitude
+ * of a row of A and a column of B, rounded once: at least as close to the
+ * exact result as a chain of K fused multiply-adds.  Parts of C whose rows or columns hold
  * too many small entries for that, infinities, NaN or extreme exponents run
  * as such chains, like smaller sizes.  The images of the digits take up to
  * 64 MiB for B and 256 MiB for A, allocated by the first execute outside a
@@ -464,7 +463,7 @@ tc_status tc_chain_variants(tc_chain chain, tc_chain_variant *buf, int32_t capac
 /* Largest intermediate in bytes that tc_chain_select(-1) may choose (-1: no
  * limit).  The limit covers the intermediate only: with a tensor-core
  * dtype a step's plan may also hold the pre-converted images of its inputs
- * (tc_plan_set_gett_pack's default), and with TC_F64 or TC_F32 the digits'
+ * (tc_plan_set_gett_pack's default), and with TC_F64 the digits'
  * (tc_execute), allocated by its first execute. */
 tc_status tc_chain_set_workspace_limit(tc_chain chain, int64_t bytes);
 

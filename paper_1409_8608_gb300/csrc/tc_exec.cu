@@ -654,12 +654,11 @@ tile_batch_kernel(const TileDesc *__restrict__ descs, const int32_t *__restrict_
     else TileOf<T, 2>::run(sd, bid, buf);
 }
 
-// Tiles of a device list: item m + tiles_m * n stands for sub_m x sub_n tiles
-// of the largest shape.
-template <typename T>
+// FP64 tiles of a device list: item m + tiles_m * n stands for sub_m x sub_n
+// tiles of the largest shape.
 __global__ void __launch_bounds__(256, 2) tile_list_kernel(const TileDesc d, const int64_t *__restrict__ list,
                                                            int64_t tiles_m, int sub_m, int sub_n) {
-    __shared__ __align__(16) unsigned char buf[sizeof(typename TileOf<T, 0>::Smem)];
+    __shared__ __align__(16) unsigned char buf[sizeof(TileOf<double, 0>::Smem)];
     const int64_t count = list[0] * sub_m * sub_n;
     for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
         const int64_t item = list[1 + q / (sub_m * sub_n)];
@@ -667,7 +666,7 @@ __global__ void __launch_bounds__(256, 2) tile_list_kernel(const TileDesc d, con
         const int64_t tm = item % tiles_m * sub_m + sub % sub_m, tn = item / tiles_m * sub_n + sub / sub_m;
         if (tm >= d.tiles_m || tn >= d.tiles_n) continue;
         __syncthreads();  // the last tile's tables have been read
-        TileOf<T, 0>::run(d, tm + d.tiles_m * tn, buf);
+        TileOf<double, 0>::run(d, tm + d.tiles_m * tn, buf);
     }
 }
 
@@ -1157,16 +1156,13 @@ tc_status simt_run_list(Plan &p, const void *alpha, const void *A, const void *B
                         const int64_t *list, int64_t tiles_m, int rows, int cols, void *stream) {
     TileDesc td;
     cudaStream_t st = (cudaStream_t)stream;
-    const bool f64 = p.dtype == TC_F64;
-    const int b = simt_rows(f64, 0);
-    if (f64) describe_gett_simt<double>(p, *(const double *)alpha, (const double *)A, (const double *)B, *(const double *)beta, (double *)C, td);
-    else describe_gett_simt<float>(p, *(const float *)alpha, (const float *)A, (const float *)B, *(const float *)beta, (float *)C, td);
+    const int b = simt_rows(true, 0);
+    describe_gett_simt<double>(p, *(const double *)alpha, (const double *)A, (const double *)B, *(const double *)beta, (double *)C, td);
     td.shape = 0;
     td.tiles_m = (td.M + b - 1) / b;
     td.tiles_n = (td.N + b - 1) / b;
-    const unsigned grid = (unsigned)device_sms() * (f64 ? 4 : 2);
-    if (f64) tile_list_kernel<double><<<grid, 256, 0, st>>>(td, list, tiles_m, rows / b, cols / b);
-    else tile_list_kernel<float><<<grid, 256, 0, st>>>(td, list, tiles_m, rows / b, cols / b);
+    const unsigned grid = (unsigned)device_sms() * 4;
+    tile_list_kernel<<<grid, 256, 0, st>>>(td, list, tiles_m, rows / b, cols / b);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? TC_SUCCESS : fail(TC_ERROR_CUDA, cudaGetErrorString(e));
 }

@@ -17,9 +17,8 @@
 namespace tc {
 namespace dev {
 
-// (GK_D64, GK_D32: FP64 and FP32 inputs as exact BF16 digits, tc_packed.cu)
-enum GettKind { GK_BF16X3 = 0, GK_BF16 = 1, GK_F16 = 2, GK_TF32 = 3, GK_TF32X3 = 4, GK_E4M3 = 5, GK_D64 = 6, GK_D32 = 7 };
-__host__ __device__ constexpr bool digit_kind(int k) { return k == GK_D64 || k == GK_D32; }
+// (GK_D64: FP64 inputs as exact BF16 digits, tc_packed.cu)
+enum GettKind { GK_BF16X3 = 0, GK_BF16 = 1, GK_F16 = 2, GK_TF32 = 3, GK_TF32X3 = 4, GK_E4M3 = 5, GK_D64 = 6 };
 
 // MMA on TF32 words (kind::tf32, 4-byte operand elements)
 __host__ __device__ constexpr bool tf32_kind(int k) { return k == GK_TF32 || k == GK_TF32X3; }
@@ -300,7 +299,7 @@ __device__ __forceinline__ uint32_t f32_to_tf32(float x) {
 template <int KIND, int BK>
 struct KindTraits {
     static constexpr int kElemBytes = tf32_kind(KIND) ? 4 : (KIND == GK_E4M3 ? 1 : 2);  // smem operand element
-    static constexpr int kSlices = KIND == GK_BF16X3 ? 3 : (KIND == GK_TF32X3 ? 2 : (KIND == GK_D64 ? 8 : (KIND == GK_D32 ? 4 : 1)));
+    static constexpr int kSlices = KIND == GK_BF16X3 ? 3 : (KIND == GK_TF32X3 ? 2 : (KIND == GK_D64 ? 8 : 1));
     static constexpr int kChunk = 16 / kElemBytes;              // K elements per 16-byte row
     static constexpr int kKc = BK / kChunk;                     // core matrices along K per stage
     static constexpr int kKsteps = BK * kElemBytes / 32;        // MMA instructions along K per stage

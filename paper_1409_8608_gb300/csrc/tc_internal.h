@@ -153,11 +153,11 @@ int64_t packed_bytes(tc_dtype dt, int64_t M, int64_t N, int64_t K);
 tc_status exec_packed(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
                       void *stream, double fraction, int64_t comp_k, bool split, const float *qscale, bool *done);
 
-// A large FP64 / FP32 GETT as exact digits on the tensor cores (tc_packed.cu);
+// A large FP64 GETT as exact digits on the tensor cores (tc_packed.cu);
 // *done = false, with nothing enqueued, where the SIMT tiles are to run.
 tc_status exec_digits(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C, void *stream,
                       double fraction, bool *done);
-// The SIMT GETT over the tiles of a device list (list[0] of them, each
+// The FP64 SIMT GETT over the tiles of a device list (list[0] of them, each
 // m + tiles_m * n of tiles of rows x cols, whole SIMT tiles).
 tc_status simt_run_list(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
                         const int64_t *list, int64_t tiles_m, int rows, int cols, void *stream);

@@ -31,40 +31,41 @@
 // number the same tiles took 178 and 918 us (elect_one).  The compensated
 // sums' (hi, lo) in registers leave the tensor memory to two accumulators.
 //
-// FP64 and FP32 (GK_D64, GK_D32): digits.  The FP64 unit runs two
-// multiply-adds per SM and clock (1.26 TFLOP/s), so a large FP64 or FP32 GETT
-// is computed from integers on the tensor cores (the digit splitting of
-// Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix
-// multiplication by using fast routines of matrix multiplication", 2012):
+// FP64 (GK_D64): digits.  The FP64 unit runs two multiply-adds per SM and
+// clock (1.26 TFLOP/s), so a large FP64 GETT is computed from integers on the
+// tensor cores (the digit splitting of Ozaki, Ogita, Oishi and Rump,
+// "Error-free transformations of matrix multiplication by using fast routines
+// of matrix multiplication", 2012):
 //   * a row of A (column of B) is scaled by the power of two 2^e just above
-//     its largest magnitude and cut into S balanced base-256 digits d_s,
-//     |d| <= 128 (64 for s = 0), x = 2^e sum_s d_s 2^(-6-8s), S = 8 (FP64) or
-//     4 (FP32): 62 or 30 bits below 2^e, exact as BF16 values;
-//   * FP64: the products d_s d_t with s + t = l < 8 add up in accumulator l.
-//     A sum over 128 K positions stays within 2^24 in magnitude, so every
-//     FP32 accumulation is exact, in any order; the epilogue adds the levels
-//     as 64-bit integers (0-3 and 4-7 apart) and rounds the total once;
-//   * FP32: level 0 has its own accumulator, exact up to K = 4096, levels 1
-//     to 3 (weights 2^-8 and less) share a second one; the two are added and
-//     rounded once.
-// What is left out is at most 2^-59 (FP64) or 2^-28 (FP32) of 2^(eA + eB) per
-// term: the products of level S and past it, and the bits under the last
-// digit.  That is small against |A||B| only where the row and the column
-// hold enough large entries, so the pre-pass counts per row the entries
-// below 2^(e-5) (FP64) or 2^(e-3) (FP32): where those of a row of A and of a
-// column of B are together at most K / 2, at least K / 2 terms of the sum
-// are at least 2^(eA+eB-10) (2^-6), and the error left out is at most
-// 2^-48 |A||B| (2^-21), under the K 2^-53 (K 2^-24) of a chain of fused
-// multiply-adds for K >= 32; on uniform entries only the last rounding is
-// left.  Tiles where that does not hold (wide ranges or many zeros along K,
-// infinities, NaN, exponents near the ends) go to a list, and the SIMT tiles
-// compute them.  B is taken in panels whose images stay in L2.
-// abc=iaj,jbic 512^3 i=j=16: FP64 56.7 -> 2.74 ms (18 panels: pre-pass 23 us,
-// GETT 128 us each; 135 where every product reads its digit of A from shared
+//     its largest magnitude and cut into 8 balanced base-256 digits d_s,
+//     |d| <= 128 (64 for s = 0), x = 2^e sum_s d_s 2^(-6-8s): 62 bits below
+//     2^e, exact as BF16 values;
+//   * the products d_s d_t with s + t = l < 8 add up in accumulator l.  A sum
+//     over 128 K positions stays within 2^24 in magnitude, so every FP32
+//     accumulation is exact, in any order; the epilogue adds the levels as
+//     64-bit integers (0-3 and 4-7 apart) and rounds the total once.
+// What is left out is at most 2^-59 of 2^(eA + eB) per term: the products of
+// level 8 and past it, and the bits under the last digit.  That is small
+// against |A||B| only where the row and the column hold enough large entries,
+// so the pre-pass counts per row the entries below 2^(e-5): where those of a
+// row of A and of a column of B are together at most K / 2, at least K / 2
+// terms of the sum are at least 2^(eA+eB-10), and the error left out is at
+// most 2^-48 |A||B|, under the K 2^-53 of a chain of fused multiply-adds for
+// K >= 32; on uniform entries only the last rounding is left.  Tiles where
+// that does not hold (wide ranges or many zeros along K, infinities, NaN,
+// exponents near the ends) go to a list, and the SIMT tiles compute them.  B
+// is taken in panels whose images stay in L2.
+// abc=iaj,jbic 512^3 i=j=16: 56.7 -> 2.74 ms (18 panels: pre-pass 23 us, GETT
+// 128 us each; 135 where every product reads its digit of A from shared
 // memory, not from the collector buffer, 153 with a conversion that branches;
-// without the drains and conversions 92), FP32 2.35 -> 0.59 ms (9 panels).
-// Error against 80-bit and longer sums on uniform entries: below that of the
-// chains (FP32 3.2e-8 against 2.9e-7 of the result's 2-norm).
+// without the drains and conversions 92).
+//
+// FP32 stays on the SIMT tiles.  Four digits (10 products, 0.59 ms against
+// 1.83 on the same contraction with uniform entries) hold 30 bits below the
+// largest entry of a row, six more than an entry has: where large terms
+// cancel, small ones that a chain keeps are lost (7e-5 of the result against
+// 2e-7), and the check of every result that would refuse such sums refuses
+// about 1 % of ordinary ones.
 //
 // Every wait on an mbarrier is bounded; on expiry the kernel records
 // TC_ERROR_TIMEOUT, stops issuing, drains, frees its tensor memory, returns.
@@ -240,30 +241,21 @@ __global__ void __launch_bounds__(kPackThreads) pack_images_kernel(const __grid_
 }
 
 // ---- digits
-template <int KIND>
-struct Digits {
-    static constexpr bool F64 = KIND == GK_D64;
-    using In = typename std::conditional<F64, double, float>::type;
-    static constexpr int kLow = F64 ? 623 : 77, kHigh = F64 ? 1423 : 177;  // exponent fields taken
-    static constexpr int kChunkK = F64 ? 128 : 1 << 12;  // K positions per accumulation
-    static constexpr int kBn = F64 ? 64 : 128;        // columns per tile: 8 levels, or two double-buffered accumulators
-    static constexpr int64_t kMaxK = F64 ? 1 << 20 : 1 << 12;  // the summed levels stay below 2^62; level 0 exact
-};
+constexpr int kDigitLow = 623, kDigitHigh = 1423;  // exponent fields taken
+constexpr int kDigitChunkK = 128;         // K positions per accumulation
+constexpr int kDigitBn = 64;              // columns per tile: eight levels fill the tensor memory
+constexpr int64_t kDigitMaxK = 1 << 20;   // the summed levels stay below 2^62
 constexpr int kRowBad = 1 << 29;
 constexpr int kDigitK = 256;  // K positions a block holds at a time
 
 // One input as digit images: a block takes 32 rows; K positions stay in
 // registers between the search for the largest magnitudes and the digits (a
 // longer K is read twice, the second time mostly from L2).
-template <int KIND>
-__global__ void __launch_bounds__(kPackThreads, Digits<KIND>::F64 ? 2 : 4) pack_digits_kernel(const __grid_constant__ PackedDesc d,
-                                                                   const PackJob ja, const PackJob jb) {
-    using D = Digits<KIND>;
-    using T = Traits<KIND>;
-    using In = typename D::In;
-    constexpr int BK = stage_k<KIND>(), S = T::kSlices, P = kPackRows + 1;
+__global__ void __launch_bounds__(kPackThreads, 2) pack_digits_kernel(const __grid_constant__ PackedDesc d,
+                                                                      const PackJob ja, const PackJob jb) {
+    constexpr int BK = stage_k<GK_D64>(), S = Traits<GK_D64>::kSlices, P = kPackRows + 1;
     extern __shared__ __align__(16) unsigned char dsm[];
-    In *tile = (In *)dsm;  // [kDigitK][P]
+    double *tile = (double *)dsm;  // [kDigitK][P]
     __shared__ int64_t koff[kDigitK], roff[kPackRows];
     __shared__ unsigned emax[kPackRows];
     __shared__ int nlarge[kPackRows];
@@ -272,7 +264,7 @@ __global__ void __launch_bounds__(kPackThreads, Digits<KIND>::F64 ? 2 : 4) pack_
     const PackJob &J = second ? jb : ja;
     const int64_t r0 = (second ? (int64_t)blockIdx.x - ja.blocks : (int64_t)blockIdx.x) * kPackRows;
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const In *__restrict__ src = (const In *)(J.op == 0 ? d.A : d.B);
+    const double *__restrict__ src = (const double *)(J.op == 0 ? d.A : d.B);
     if (tid < kPackRows) {
         int64_t r = r0 + tid, o = -1, u = 0;
         if (r < (J.op == 0 ? d.M : d.N)) {
@@ -285,7 +277,7 @@ __global__ void __launch_bounds__(kPackThreads, Digits<KIND>::F64 ? 2 : 4) pack_
         nlarge[tid] = 0;
     }
     constexpr int NL = kDigitK * kPackRows / kPackThreads, KJ = kDigitK / 32;
-    In x[NL];
+    double x[NL];
     auto load = [&](int64_t k0) {  // (a barrier on both sides of the offset table)
         __syncthreads();
         static_assert(kDigitK == kPackThreads, "one thread per K offset");
@@ -304,18 +296,14 @@ __global__ void __launch_bounds__(kPackThreads, Digits<KIND>::F64 ? 2 : 4) pack_
         for (int j = 0; j < NL; ++j) {
             const int64_t ro = roff[J.rfast ? lane : warp * 4 + j / KJ];
             const int64_t ko = koff[J.rfast ? warp + 8 * j : lane + 32 * (j % KJ)];
-            x[j] = ro >= 0 && ko >= 0 ? __ldg(src + ro + ko) : In(0);
+            x[j] = ro >= 0 && ko >= 0 ? __ldg(src + ro + ko) : 0.0;
         }
     };
-    // largest magnitude: the high word of |x| (for FP64 with a bit for a
-    // nonzero low word), ordered as integers
-    auto mag = [](In v) -> unsigned {
-        if constexpr (D::F64) {
-            const unsigned long long b = __double_as_longlong(v);
-            return ((unsigned)(b >> 32) & 0x7fffffffu) | ((unsigned)b != 0 ? 1u : 0u);
-        } else {
-            return __float_as_uint(v) & 0x7fffffffu;
-        }
+    // largest magnitude: the high word of |x| with a bit for a nonzero low
+    // word, ordered as integers
+    auto mag = [](double v) -> unsigned {
+        const unsigned long long b = __double_as_longlong(v);
+        return ((unsigned)(b >> 32) & 0x7fffffffu) | ((unsigned)b != 0 ? 1u : 0u);
     };
     unsigned mx[4] = {0, 0, 0, 0};
     for (int64_t k0 = 0; k0 < d.K; k0 += kDigitK) {
@@ -334,15 +322,13 @@ __global__ void __launch_bounds__(kPackThreads, Digits<KIND>::F64 ? 2 : 4) pack_
     }
     __syncthreads();
     const unsigned top = emax[lane];
-    const int E = (int)(top >> (D::F64 ? 20 : 23));
+    const int E = (int)(top >> 20);
     const int64_t R = r0 + lane;
     int64_t rr;
     const int64_t rt = divmod(R, J.rows, rr);
     const int slice = J.rows * BK * 2;
     char *out = J.out + rt * d.ktiles * (int64_t)(S * slice) + (rr / 8) * 128 + (rr % 8) * 16;
     int large = 0;
-    // FP32: 2^-e (rows whose exponent is not taken get zeros)
-    const float down = D::F64 || E < D::kLow || E > D::kHigh ? 0.0f : __uint_as_float((unsigned)(253 - E) << 23);
     const bool once = d.K <= kDigitK;
     for (int64_t k0 = 0; k0 < (int64_t)d.ktiles * BK; k0 += kDigitK) {
         if (!once) load(k0);
@@ -357,66 +343,42 @@ __global__ void __launch_bounds__(kPackThreads, Digits<KIND>::F64 ? 2 : 4) pack_
             const int64_t k = k0 + c * 8;
             if (R >= J.total_rows || k >= (int64_t)d.ktiles * BK) break;
             char *dst = out + (k / BK) * (int64_t)(S * slice) + (int)((k % BK) / 8) * (J.rows / 8) * 128;
-            if constexpr (D::F64) {
-                constexpr int kLarge = 4;  // large: exponent field at least the row's minus this
-                unsigned long long y[8];
+            constexpr int kLarge = 4;  // large: exponent field at least the row's minus this
+            unsigned long long y[8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const unsigned long long b = __double_as_longlong(tile[(c * 8 + e) * P + lane]);
-                    const unsigned long long frac = b & ((1ull << 52) - 1);
-                    const int ex = (int)(b >> 52) & 2047;
-                    const unsigned long long m = ex ? frac | (1ull << 52) : frac;
-                    const int sh = E - (ex ? ex : 1);
-                    large += m != 0 && sh <= kLarge;
-                    // x 2^-e 2^62 = m 2^(9 - sh), rounded where bits fall
-                    // under the last digit
-                    unsigned long long w;
-                    if (sh <= 9) w = m << (9 - sh);
-                    else w = sh <= 62 ? (m + (1ull << (sh - 10))) >> (sh - 9) : 0ull;
-                    if (b >> 63) w = 0ull - w;
-                    y[e] = w + 0x8080808080808080ull;  // bytes: digit + 128
-                }
+            for (int e = 0; e < 8; ++e) {
+                const unsigned long long b = __double_as_longlong(tile[(c * 8 + e) * P + lane]);
+                const unsigned long long frac = b & ((1ull << 52) - 1);
+                const int ex = (int)(b >> 52) & 2047;
+                const unsigned long long m = ex ? frac | (1ull << 52) : frac;
+                const int sh = E - (ex ? ex : 1);
+                large += m != 0 && sh <= kLarge;
+                // x 2^-e 2^62 = m 2^(9 - sh), rounded where bits fall
+                // under the last digit
+                unsigned long long w;
+                if (sh <= 9) w = m << (9 - sh);
+                else w = sh <= 62 ? (m + (1ull << (sh - 10))) >> (sh - 9) : 0ull;
+                if (b >> 63) w = 0ull - w;
+                y[e] = w + 0x8080808080808080ull;  // bytes: digit + 128
+            }
 #pragma unroll
-                for (int s = 0; s < S; ++s) {
-                    // 2^23 + byte as FP32 less 2^23 + 128: the digit, whose
-                    // upper half is its BF16 value
-                    constexpr unsigned kMagic = 0x4B000000u;
-                    const int byte = S - 1 - s;
-                    unsigned q[4];
+            for (int s = 0; s < S; ++s) {
+                // 2^23 + byte as FP32 less 2^23 + 128: the digit, whose
+                // upper half is its BF16 value
+                constexpr unsigned kMagic = 0x4B000000u;
+                const int byte = S - 1 - s;
+                unsigned q[4];
 #pragma unroll
-                    for (int e = 0; e < 8; e += 2) {
-                        float f[2];
+                for (int e = 0; e < 8; e += 2) {
+                    float f[2];
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const unsigned word = (unsigned)(y[e + h] >> (byte >= 4 ? 32 : 0));
-                            f[h] = __uint_as_float(__byte_perm(word, kMagic, 0x7440 | (byte & 3))) - 8388736.0f;
-                        }
-                        q[e / 2] = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632);
+                    for (int h = 0; h < 2; ++h) {
+                        const unsigned word = (unsigned)(y[e + h] >> (byte >= 4 ? 32 : 0));
+                        f[h] = __uint_as_float(__byte_perm(word, kMagic, 0x7440 | (byte & 3))) - 8388736.0f;
                     }
-                    *(uint4 *)(dst + (int64_t)s * slice) = make_uint4(q[0], q[1], q[2], q[3]);
+                    q[e / 2] = __byte_perm(__float_as_uint(f[0]), __float_as_uint(f[1]), 0x7632);
                 }
-            } else {
-                // z = x 2^-e, |z| < 1: rounding to a multiple of 2^(-6-8s) by
-                // adding 1.5 2^(17-8s) leaves d_s 2^(-6-8s), a BF16 value
-                float z[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    z[e] = tile[(c * 8 + e) * P + lane] * down;
-                    large += fabsf(z[e]) >= 0.125f;
-                }
-#pragma unroll
-                for (int s = 0; s < S; ++s) {
-                    const float add = __uint_as_float(((unsigned)(127 + 17 - 8 * s) << 23) | 0x400000u);
-                    unsigned q[4];
-#pragma unroll
-                    for (int e = 0; e < 8; e += 2) {
-                        const float w0 = __fsub_rn(__fadd_rn(z[e], add), add), w1 = __fsub_rn(__fadd_rn(z[e + 1], add), add);
-                        z[e] = __fsub_rn(z[e], w0);
-                        z[e + 1] = __fsub_rn(z[e + 1], w1);
-                        q[e / 2] = __byte_perm(__float_as_uint(w0), __float_as_uint(w1), 0x7632);
-                    }
-                    *(uint4 *)(dst + (int64_t)s * slice) = make_uint4(q[0], q[1], q[2], q[3]);
-                }
+                *(uint4 *)(dst + (int64_t)s * slice) = make_uint4(q[0], q[1], q[2], q[3]);
             }
         }
     }
@@ -425,8 +387,8 @@ __global__ void __launch_bounds__(kPackThreads, Digits<KIND>::F64 ? 2 : 4) pack_
     if (tid < kPackRows && R < J.total_rows) {  // warp 0: lane = row
         int few = (int)min(d.K, (int64_t)kRowBad) - nlarge[lane];
         if (top == 0) few = 0;  // a row of zeros (or past the extent): exact
-        else if (E < D::kLow || E > D::kHigh) few = kRowBad;
-        d.exps[J.op][R] = top == 0 ? D::kLow : E;
+        else if (E < kDigitLow || E > kDigitHigh) few = kRowBad;
+        d.exps[J.op][R] = top == 0 ? kDigitLow : E;
         if (few > 0) atomicMax(&d.small[J.op][(J.op == 0 ? 0 : d.n_begin / J.rows) + rt], few);
     }
 }
@@ -575,8 +537,8 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
     constexpr bool kAlt = !COMP && KIND != GK_D64;
     constexpr int kGroupWarps = kAlt ? kEpiWarps / 2 : kEpiWarps;
     __shared__ int64_t cN[kAlt ? 4 : 2][kMaxBn];
-    constexpr bool DIG = digit_kind(KIND);
-    __shared__ int cE[DIG ? (kAlt ? 4 : 2) : 1][DIG ? 128 : 1];  // digits: exponent fields of the tile's columns
+    constexpr bool DIG = KIND == GK_D64;
+    __shared__ int cE[DIG ? 2 : 1][DIG ? kDigitBn : 1];  // digits: exponent fields of the tile's columns
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_word;
     volatile int *abort_flag = &abort_word;
@@ -593,7 +555,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
         *abort_flag = 1;
         atomicExch(d.status, (int)TC_ERROR_TIMEOUT);
     };
-    const bool split = KIND == GK_D32 || (!COMP && d.split != 0);
+    const bool split = !COMP && d.split != 0;
     const int nbuf = KIND == GK_D64 ? 1 : 2;
     const uint32_t small_off = split ? 128u : 0u;  // the smaller products' accumulator (bn <= 128)
     if (threadIdx.x == 0) {
@@ -707,8 +669,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                     }
                 }
             };
-            // digits: product d_s d_t into accumulator s + t (FP64), or into the
-            // second one unless s = t = 0 (FP32)
+            // digits: product d_s d_t into accumulator s + t
             auto issue_digits = [&](uint64_t as, uint64_t bs, uint32_t dt, bool first, int nks) {
                 constexpr int S = T::kSlices;
 #pragma unroll
@@ -718,10 +679,10 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                     for (int s = 0; s < S; ++s)
 #pragma unroll
                         for (int t = 0; t < S - s; ++t) {
-                            const uint32_t dst = dt + (uint32_t)(KIND == GK_D64 ? (s + t) * 64 : (s + t ? 128 : 0));
+                            const uint32_t dst = dt + (uint32_t)((s + t) * kDigitBn);
                             const uint64_t ad = as + (uint64_t)((s * sliceA + ks * 2 * lboA) >> 4);
                             const uint64_t bd = bs + (uint64_t)((t * sliceB + ks * 2 * lboB) >> 4);
-                            const bool acc = !(first && ks == 0 && s == 0 && (KIND == GK_D64 || t < 2));
+                            const bool acc = !(first && ks == 0 && s == 0);
                             if (s == S - 1) mma_issue<KIND, PAIR>(dst, ad, bd, idesc, acc);
                             else if (t == 0) mma_issue_same_a<PAIR, 0>(dst, ad, bd, idesc, acc);
                             else if (t == S - s - 1) mma_issue_same_a<PAIR, 2>(dst, ad, bd, idesc, acc);
@@ -922,7 +883,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
 #pragma unroll
                     for (int g4 = 0; g4 < 8; ++g4) {  // four columns of every level at a time
                         uint32_t r[32];
-                        tmem_ld8x4(tmem + lane_off + (uint32_t)(half * 32 + g4 * 4), 64, r);
+                        tmem_ld8x4(tmem + lane_off + (uint32_t)(half * 32 + g4 * 4), kDigitBn, r);
                         auto lev = [&](int n, int j) { return __uint_as_float(r[n * 4 + j]); };
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
@@ -942,13 +903,6 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                         uint32_t r[32];
                         if (split) tmem_ld32_sum(acc + (uint32_t)c0, acc + small_off + (uint32_t)c0, r);
                         else tmem_ld32(acc + (uint32_t)c0, r);
-                        if constexpr (KIND == GK_D32) {  // powers of two: 2^eA of the row, 2^eB of each column
-                            const int *ce = cE[tab] + c0;
-                            const float up = __uint_as_float((unsigned)(rowE + 1) << 23);
-#pragma unroll
-                            for (int j = 0; j < 32; ++j)
-                                r[j] = __float_as_uint(__uint_as_float(r[j]) * up * __uint_as_float((unsigned)(ce[j] + 1) << 23));
-                        }
                         store_row(r, old, C, om, c0, lin, on0, nval, cn, alpha, d.beta, d.init);
                         if (d.init == 1 && c0 + kColStep < d.bn) load_old(old, C, om, c0 + kColStep, lin, on0, nval, cn);
                     }
@@ -1238,13 +1192,10 @@ struct DigitPlan {
 // The digit form of an M x N x K product, or false where SIMT is the faster
 // estimate or the form does not apply.  Clocks per 16 K positions as
 // choose_tile counts them (the shared-memory port), plus what draining the
-// levels of a unit costs; SIMT at its measured rates.
-template <int KIND>
+// levels of a unit costs; SIMT at its measured rate.
 bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
-    using D = Digits<KIND>;
-    using T = Traits<KIND>;
-    constexpr int BK = stage_k<KIND>(), S = T::kSlices;
-    if (K < kDigitMinK || K > D::kMaxK) return false;
+    constexpr int BK = stage_k<GK_D64>(), S = Traits<GK_D64>::kSlices;
+    if (K < kDigitMinK || K > kDigitMaxK) return false;
     const int64_t Kp = (K + BK - 1) / BK * BK;
     double best = -1;
     for (int pair = 1; pair >= 0; --pair) {
@@ -1253,21 +1204,21 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
         DigitPlan q;
         q.pair = pair != 0;
         q.tiles_m = (M + rows - 1) / rows;
-        q.tiles_n = (N + D::kBn - 1) / D::kBn;
+        q.tiles_n = (N + kDigitBn - 1) / kDigitBn;
         if (q.tiles_n > kDigitMaxTiles / q.tiles_m) continue;
         q.rows_a = q.tiles_m * rows;
         q.image_a = q.rows_a * Kp * S * 2;
         if (q.image_a > kScratchMaxABytes) continue;
-        q.panel_tiles = panel_tiles_for(kDigitPanelBytes, q.tiles_n, q.tiles_m, Kp * S * 2 * D::kBn, slots);
-        q.image_b = q.panel_tiles * D::kBn * Kp * S * 2;
+        q.panel_tiles = panel_tiles_for(kDigitPanelBytes, q.tiles_n, q.tiles_m, Kp * S * 2 * kDigitBn, slots);
+        q.image_b = q.panel_tiles * kDigitBn * Kp * S * 2;
         const int64_t panels = (q.tiles_n + q.panel_tiles - 1) / q.panel_tiles;
-        const int brows = pair ? D::kBn / 2 : D::kBn, nprod = S * (S + 1) / 2;
+        const int brows = pair ? kDigitBn / 2 : kDigitBn, nprod = S * (S + 1) / 2;
         const double port = ((4096.0 + 32.0 * brows) * nprod + 32.0 * (kRows + brows) * S) / 128.0;
-        const double tile = (Kp / 16) * std::max(D::kBn / 2.0 * nprod, port) +
-                            (D::F64 ? (K + D::kChunkK - 1) / D::kChunkK * 6000.0 : 0.0) + 3000.0;
+        const double tile = (Kp / 16) * std::max(kDigitBn / 2.0 * nprod, port) +
+                            (K + kDigitChunkK - 1) / kDigitChunkK * 6000.0 + 3000.0;
         const int64_t waves = (panels - 1) * ((q.panel_tiles * q.tiles_m + slots - 1) / slots) +
                               ((q.tiles_n - (panels - 1) * q.panel_tiles) * q.tiles_m + slots - 1) / slots;
-        const double pack = (double)(q.rows_a + q.tiles_n * D::kBn) * Kp * (sizeof(typename D::In) + S * 2) / 3e12;
+        const double pack = (double)(q.rows_a + q.tiles_n * kDigitBn) * Kp * (8 + S * 2) / 3e12;
         const double sec = waves * tile / 1.9e9 + pack + 12e-6 + panels * 6e-6;
         if (best < 0 || sec < best) {
             best = sec;
@@ -1275,14 +1226,14 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
         }
     }
     if (best < 0) return false;
-    const double simt = 2.0 * (double)M * (double)N * (double)K / (D::F64 ? 1.24e12 : 37e12);
+    const double simt = 2.0 * (double)M * (double)N * (double)K / 1.24e12;
     if (best > 0.8 * simt) return false;
     auto up = [](int64_t x) { return (x + 511) / 512 * 512; };
     P.off_b = P.image_a;
     P.off_exp_a = P.off_b + P.image_b;
     P.off_exp_b = P.off_exp_a + up(P.rows_a * 4);
     // zeroed before each execute: the row tiles' counts and the list's length
-    P.off_small_a = P.off_exp_b + up(P.panel_tiles * D::kBn * 4);
+    P.off_small_a = P.off_exp_b + up(P.panel_tiles * kDigitBn * 4);
     P.off_small_b = P.off_small_a + up(P.rows_a / kRows * 4);
     P.off_list = P.off_small_b + up(P.tiles_n * 2 * 4);
     P.zero_bytes = P.off_list + 8 - P.off_small_a;
@@ -1290,38 +1241,29 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
     return true;
 }
 
-template <int KIND>
 tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta, double fraction, cudaStream_t st,
                      bool *done) {
-    using D = Digits<KIND>;
-    using T = Traits<KIND>;
-    constexpr int BK = stage_k<KIND>();
+    constexpr int KIND = GK_D64, BK = stage_k<KIND>(), S = Traits<KIND>::kSlices;
     DigitPlan P;
-    if (!plan_digits<KIND>(d.M, d.N, d.K, P)) return TC_SUCCESS;
+    if (!plan_digits(d.M, d.N, d.K, P)) return TC_SUCCESS;
     tc_status s = ensure_device_resources(p, 0);
     if (s != TC_SUCCESS) return s;
     if (!optional_scratch(p, P.bytes, st)) return TC_SUCCESS;  // the SIMT tiles run
     char *ws = (char *)p.scratch;
-    if constexpr (D::F64) {
-        d.alpha64 = *(const double *)alpha;
-        d.beta64 = *(const double *)beta;
-        d.init = d.beta64 == 0.0 ? 2 : 1;
-    } else {
-        d.alpha = *(const float *)alpha;
-        d.beta = *(const float *)beta;
-        d.init = d.beta == 0.0f ? 2 : 1;
-    }
+    d.alpha64 = *(const double *)alpha;
+    d.beta64 = *(const double *)beta;
+    d.init = d.beta64 == 0.0 ? 2 : 1;
     int64_t tiles_n = P.tiles_n;
-    const int64_t N = fraction < 1.0 ? std::min<int64_t>(d.N, std::max<int64_t>(D::kBn, (int64_t)(d.N * fraction))) : d.N;
-    tiles_n = (N + D::kBn - 1) / D::kBn;
+    const int64_t N = fraction < 1.0 ? std::min<int64_t>(d.N, std::max<int64_t>(kDigitBn, (int64_t)(d.N * fraction))) : d.N;
+    tiles_n = (N + kDigitBn - 1) / kDigitBn;
     d.status = p.dev_status;
-    d.bn = D::kBn;
-    d.brows = P.pair ? D::kBn / 2 : D::kBn;
+    d.bn = kDigitBn;
+    d.brows = P.pair ? kDigitBn / 2 : kDigitBn;
     d.tiles_m = P.tiles_m;
     d.ktiles = (int)((d.K + BK - 1) / BK);
-    d.chunk = std::min(d.ktiles, D::kChunkK / BK);
-    d.img_a = (uint32_t)(T::kSlices * kRows * BK * 2);
-    d.img_b = (uint32_t)(T::kSlices * d.brows * BK * 2);
+    d.chunk = std::min(d.ktiles, kDigitChunkK / BK);
+    d.img_a = (uint32_t)(S * kRows * BK * 2);
+    d.img_b = (uint32_t)(S * d.brows * BK * 2);
     d.stages = std::min<int>(kMaxStages, kRingBytes / (int)(d.img_a + d.img_b));
     d.exps[0] = (int *)(ws + P.off_exp_a);
     d.exps[1] = (int *)(ws + P.off_exp_b);
@@ -1332,15 +1274,15 @@ tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta
     s = image_map(ta, ws, P.image_a, d.img_a);
     if (s == TC_SUCCESS) s = image_map(tb, ws + P.off_b, P.image_b, d.img_b);
     if (s != TC_SUCCESS) return s;
-    constexpr int kPackSmem = kDigitK * (kPackRows + 1) * (int)sizeof(typename D::In);
-    cudaError_t e = cudaFuncSetAttribute(pack_digits_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPackSmem);
+    constexpr int kPackSmem = kDigitK * (kPackRows + 1) * (int)sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(pack_digits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPackSmem);
     if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
     e = cudaMemsetAsync(ws + P.off_small_a, 0, (size_t)P.zero_bytes, st);
     if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
     for (int64_t t0 = 0; t0 < tiles_n; t0 += P.panel_tiles) {
-        d.n_begin = t0 * D::kBn;
+        d.n_begin = t0 * kDigitBn;
         d.tiles_n = std::min(P.panel_tiles, tiles_n - t0);
-        d.N = std::min<int64_t>(N - d.n_begin, d.tiles_n * D::kBn);
+        d.N = std::min<int64_t>(N - d.n_begin, d.tiles_n * kDigitBn);
         d.num_tiles = d.tiles_m * d.tiles_n;
         PackJob ja = {}, jb = {};
         ja.op = 0;
@@ -1351,17 +1293,17 @@ tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta
         ja.blocks = t0 == 0 ? (ja.total_rows + kPackRows - 1) / kPackRows : 0;  // A's with the first panel
         jb.op = 1;
         jb.rows = d.brows;
-        jb.total_rows = d.tiles_n * D::kBn;
+        jb.total_rows = d.tiles_n * kDigitBn;
         jb.rfast = d.nn > 0 && d.n_sB[0] < d.k_sB[d.nk - 1];
         jb.out = ws + P.off_b;
         jb.blocks = (jb.total_rows + kPackRows - 1) / kPackRows;
-        pack_digits_kernel<KIND><<<(unsigned)(ja.blocks + jb.blocks), kPackThreads, kPackSmem, st>>>(d, ja, jb);
+        pack_digits_kernel<<<(unsigned)(ja.blocks + jb.blocks), kPackThreads, kPackSmem, st>>>(d, ja, jb);
         e = cudaGetLastError();
         if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
         s = P.pair ? launch_gett<KIND, false, true>(d, ta, tb, st) : launch_gett<KIND, false, false>(d, ta, tb, st);
         if (s != TC_SUCCESS) return s;
     }
-    s = simt_run_list(p, alpha, d.A, d.B, beta, d.C, d.list, P.tiles_m, P.pair ? 2 * kRows : kRows, D::kBn, st);
+    s = simt_run_list(p, alpha, d.A, d.B, beta, d.C, d.list, P.tiles_m, P.pair ? 2 * kRows : kRows, kDigitBn, st);
     if (s == TC_SUCCESS) *done = true;
     return s;
 }
@@ -1371,7 +1313,7 @@ tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta
 tc_status exec_digits(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C, void *stream,
                       double fraction, bool *done) {
     *done = false;
-    if (!p.batch.empty() || p.contracted.empty()) return TC_SUCCESS;
+    if (p.dtype != TC_F64 || !p.batch.empty() || p.contracted.empty()) return TC_SUCCESS;
     PackedDesc d;
     std::memset(&d, 0, sizeof(d));
     tc_status s = describe_modes(p, 3, d);
@@ -1379,8 +1321,7 @@ tc_status exec_digits(Plan &p, const void *alpha, const void *A, const void *B, 
     d.A = A;
     d.B = B;
     d.C = C;
-    if (p.dtype == TC_F64) return run_digits<GK_D64>(p, d, alpha, beta, fraction, (cudaStream_t)stream, done);
-    return run_digits<GK_D32>(p, d, alpha, beta, fraction, (cudaStream_t)stream, done);
+    return run_digits(p, d, alpha, beta, fraction, (cudaStream_t)stream, done);
 }
 
 int64_t packed_bytes(tc_dtype dt, int64_t M, int64_t N, int64_t K) {
