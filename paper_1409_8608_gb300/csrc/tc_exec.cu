@@ -654,19 +654,145 @@ tile_batch_kernel(const TileDesc *__restrict__ descs, const int32_t *__restrict_
     else TileOf<T, 2>::run(sd, bid, buf);
 }
 
-// FP64 tiles of a device list: item m + tiles_m * n stands for sub_m x sub_n
-// tiles of the largest shape.
-__global__ void __launch_bounds__(256, 2) tile_list_kernel(const TileDesc d, const int64_t *__restrict__ list,
-                                                           int64_t tiles_m, int sub_m, int sub_n) {
-    __shared__ __align__(16) unsigned char buf[sizeof(TileOf<double, 0>::Smem)];
-    const int64_t count = list[0] * sub_m * sub_n;
+// What an FP64 GETT on digits leaves to the chain of fused multiply-adds, with
+// the bits that the SIMT GETT gives: single outputs marked in `weak`, one
+// thread each; patches of 32 x 32 that are marked as a whole, as tiles; and
+// the tiles of a list (item m + list_m * n: sub_m x sub_n tiles of 64 x 64).
+// (512^3 i=j=16: 76 us for the marks of 4.2 M rows of 32 columns and about 20000
+// single outputs; a list of every tile takes what tile_kernel takes, 56.3 ms;
+// in tiles of 32 x 32 57.6, and 958 instead of 820 us for 300 x 4000 x 257.)
+// A block gathers the marks of its patches (32 at a time, all blocks in turn,
+// so that a weak region of C is spread over them) before it computes any: the
+// single outputs are bound by one chain's K dependent multiply-adds and reads
+// where they are few, by a 32-byte sector per element of A and B where many.
+struct LeftSingles {
+    static constexpr int kCap = 8192, kStep = 32 * kWeakMax;  // places, and the most that one step adds
+    uint32_t list[kCap];
+    int64_t kA[256], kB[256];
+};
+
+__global__ void __launch_bounds__(256, 2)
+left_kernel(const TileDesc d, const TileDesc patch, const uint32_t *__restrict__ weak, int64_t rows, int64_t g0, int64_t g1,
+            const int64_t *__restrict__ list, int64_t list_m, int sub_m, int sub_n) {
+    using Tile = TileOf<double, 0>;
+    using Patch = TileOf<double, 1>;
+    constexpr int kPatches = 32, kWhole = 256, kAhead = 16;
+    constexpr size_t kBytes = sizeof(LeftSingles) > sizeof(Tile::Smem) ? sizeof(LeftSingles) : sizeof(Tile::Smem);
+    static_assert(Patch::B == 32, "a patch is a tile");
+    __shared__ __align__(16) unsigned char buf[kBytes];
+    LeftSingles &sm = *reinterpret_cast<LeftSingles *>(buf);
+    __shared__ uint32_t whole[kWhole];
+    __shared__ int nlist, nwhole;
+    const double *__restrict__ A = (const double *)d.A;
+    const double *__restrict__ B = (const double *)d.B;
+    double *__restrict__ C = (double *)d.C;
+    const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
+    const int64_t rp = rows / 32, patches = rp * (g1 - g0), stride = (int64_t)gridDim.x * kPatches;
+    // the patch at place x of this block's: rows 32 pm .., columns 32 (g0 + pn) ..
+    auto patch_at = [&](int64_t x, int64_t &pm) -> int64_t {
+        return divmod_pos((int64_t)blockIdx.x * kPatches + x / kPatches * stride + x % kPatches, rp, pm);
+    };
+    auto singles = [&](int count) {
+        for (int e0 = 0; e0 < count; e0 += 256) {
+            const bool live = e0 + tid < count;
+            int64_t oA = 0, oB = 0, oC = 0;
+            if (live) {
+                const uint32_t at = sm.list[e0 + tid];
+                int64_t x, mm, nn = g0 + patch_at(at >> 10, mm);
+                mm = mm * 32 + (at >> 5 & 31);
+                nn = nn * 32 + (at & 31);
+                for (int m = 0; m < d.m.n; ++m) {
+                    mm = divmod_pos(mm, d.m.ext[m], x);
+                    oA += x * d.m.sA[m];
+                    oC += x * d.m.sC[m];
+                }
+                for (int m = 0; m < d.n.n; ++m) {
+                    nn = divmod_pos(nn, d.n.ext[m], x);
+                    oB += x * d.n.sB[m];
+                    oC += x * d.n.sC[m];
+                }
+            }
+            double acc = 0.0;
+            if (live && d.init != 2) acc = d.init == 1 ? d.beta * C[oC] : C[oC];
+            for (int64_t k0 = 0; k0 < d.K; k0 += 256) {
+                __syncthreads();  // the last offsets have been read
+                int64_t k = k0 + tid, x, a = 0, b = 0;
+                if (k < d.K) {
+                    for (int m = d.red.n - 1; m >= 0; --m) {
+                        k = divmod_pos(k, d.red.ext[m], x);
+                        a += x * d.red.sA[m];
+                        b += x * d.red.sB[m];
+                    }
+                }
+                sm.kA[tid] = a;
+                sm.kB[tid] = b;
+                __syncthreads();
+                if (!live) continue;
+                const int len = (int)min((int64_t)256, d.K - k0);
+                int kk = 0;
+                for (; kk + kAhead <= len; kk += kAhead) {
+                    double u[kAhead], v[kAhead];
+#pragma unroll
+                    for (int i = 0; i < kAhead; ++i) {
+                        u[i] = A[oA + sm.kA[kk + i]];
+                        v[i] = B[oB + sm.kB[kk + i]];
+                    }
+#pragma unroll
+                    for (int i = 0; i < kAhead; ++i) acc = fma(d.alpha_one ? u[i] : d.alpha * u[i], v[i], acc);
+                }
+                for (; kk < len; ++kk) {
+                    const double u = A[oA + sm.kA[kk]];
+                    acc = fma(d.alpha_one ? u : d.alpha * u, B[oB + sm.kB[kk]], acc);
+                }
+            }
+            if (live) C[oC] = acc;
+        }
+    };
+    if (tid == 0) nlist = nwhole = 0;
+    __syncthreads();
+    int64_t x0 = 0;
+    for (int64_t c = (int64_t)blockIdx.x * kPatches; c < patches; c += stride, x0 += kPatches) {
+        uint32_t w[kPatches / 8];
+#pragma unroll
+        for (int i = 0; i < kPatches / 8; ++i) {
+            int64_t pm;
+            const int64_t pn = divmod_pos(c + warp + 8 * i, rp, pm);
+            w[i] = c + warp + 8 * i < patches ? weak[pn * rows + pm * 32 + lane] : 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < kPatches / 8; ++i) {
+            const uint32_t x = (uint32_t)x0 + warp + 8 * i;
+            if (__all_sync(0xffffffffu, w[i] == ~0u)) {
+                if (lane == 0) whole[atomicAdd(&nwhole, 1)] = x;
+                continue;
+            }
+            for (uint32_t b = w[i]; b != 0; b &= b - 1) {
+                const int at = atomicAdd(&nlist, 1);
+                if (at < sm.kCap) sm.list[at] = x << 10 | lane << 5 | (__ffs((int)b) - 1);
+            }
+        }
+        __syncthreads();
+        const int count = min(nlist, sm.kCap), tiles = nwhole;
+        if (c + stride < patches && count <= sm.kCap - sm.kStep && tiles <= kWhole - kPatches) continue;
+        singles(count);
+        __syncthreads();
+        for (int i = 0; i < tiles; ++i) {
+            int64_t pm;
+            const int64_t pn = g0 + patch_at(whole[i], pm);
+            if (pm < patch.tiles_m && pn < patch.tiles_n) Patch::run(patch, pm + patch.tiles_m * pn, buf);
+            __syncthreads();
+        }
+        if (tid == 0) nlist = nwhole = 0;
+        __syncthreads();
+    }
+    const int64_t count = list ? list[0] * sub_m * sub_n : 0;
     for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
         const int64_t item = list[1 + q / (sub_m * sub_n)];
         const int sub = (int)(q % (sub_m * sub_n));
-        const int64_t tm = item % tiles_m * sub_m + sub % sub_m, tn = item / tiles_m * sub_n + sub / sub_m;
+        const int64_t tm = item % list_m * sub_m + sub % sub_m, tn = item / list_m * sub_n + sub / sub_m;
         if (tm >= d.tiles_m || tn >= d.tiles_n) continue;
         __syncthreads();  // the last tile's tables have been read
-        TileOf<double, 0>::run(d, tm + d.tiles_m * tn, buf);
+        Tile::run(d, tm + d.tiles_m * tn, buf);
     }
 }
 
@@ -1152,17 +1278,23 @@ tc_status run_gett_simt(Plan &p, T alpha, const T *A, const T *B, T beta, T *C,
 
 }  // namespace
 
-tc_status simt_run_list(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
-                        const int64_t *list, int64_t tiles_m, int rows, int cols, void *stream) {
+tc_status simt_run_left(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
+                        const uint32_t *weak, int64_t rows, int64_t g0, int64_t g1, const int64_t *list, int64_t list_m,
+                        int item_rows, int item_cols, void *stream) {
     TileDesc td;
-    cudaStream_t st = (cudaStream_t)stream;
-    const int b = simt_rows(true, 0);
     describe_gett_simt<double>(p, *(const double *)alpha, (const double *)A, (const double *)B, *(const double *)beta, (double *)C, td);
-    td.shape = 0;
-    td.tiles_m = (td.M + b - 1) / b;
-    td.tiles_n = (td.N + b - 1) / b;
+    auto shaped = [&](int shape) {
+        TileDesc t = td;
+        const int b = simt_rows(true, shape);
+        t.shape = shape;
+        t.tiles_m = (t.M + b - 1) / b;
+        t.tiles_n = (t.N + b - 1) / b;
+        return t;
+    };
+    const int b = simt_rows(true, 0);
     const unsigned grid = (unsigned)device_sms() * 4;
-    tile_list_kernel<<<grid, 256, 0, st>>>(td, list, tiles_m, rows / b, cols / b);
+    left_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(shaped(0), shaped(1), weak, rows, g0, g1, list, list_m, item_rows / b,
+                                                         item_cols / b);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? TC_SUCCESS : fail(TC_ERROR_CUDA, cudaGetErrorString(e));
 }

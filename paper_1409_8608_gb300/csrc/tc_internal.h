@@ -157,10 +157,15 @@ tc_status exec_packed(Plan &p, const void *alpha, const void *A, const void *B, 
 // *done = false, with nothing enqueued, where the SIMT tiles are to run.
 tc_status exec_digits(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C, void *stream,
                       double fraction, bool *done);
-// The FP64 SIMT GETT over the tiles of a device list (list[0] of them, each
-// m + tiles_m * n of tiles of rows x cols, whole SIMT tiles).
-tc_status simt_run_list(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
-                        const int64_t *list, int64_t tiles_m, int rows, int cols, void *stream);
+// What such a GETT leaves to the chain of fused multiply-adds.  Word
+// (g - g0) * rows + m of `weak` has a bit for each of the columns 32 g ..
+// 32 g + 31 of row m, g0 <= g < g1; a patch of 32 rows with more than
+// kWeakMax of them has them all set.  list (may be null): list[0] items
+// m + list_m * n of item_rows x item_cols, whole SIMT tiles.
+constexpr int kWeakMax = 128;
+tc_status simt_run_left(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
+                        const uint32_t *weak, int64_t rows, int64_t g0, int64_t g1, const int64_t *list, int64_t list_m,
+                        int item_rows, int item_cols, void *stream);
 
 // One phase of a gemm loop nest on the tensor cores (tensor dtypes): the
 // kernel's free index of A (m: sA, sC) and of B (n: sB, sC), its K modes

@@ -44,21 +44,30 @@
 //     over 128 K positions stays within 2^24 in magnitude, so every FP32
 //     accumulation is exact, in any order; the epilogue adds the levels as
 //     64-bit integers (0-3 and 4-7 apart) and rounds the total once.
-// What is left out is at most 2^-59 of 2^(eA + eB) per term: the products of
-// level 8 and past it, and the bits under the last digit.  That is small
-// against |A||B| only where the row and the column hold enough large entries,
-// so the pre-pass counts per row the entries below 2^(e-5): where those of a
-// row of A and of a column of B are together at most K / 2, at least K / 2
-// terms of the sum are at least 2^(eA+eB-10), and the error left out is at
-// most 2^-48 |A||B|, under the K 2^-53 of a chain of fused multiply-adds for
-// K >= 32; on uniform entries only the last rounding is left.  Tiles where
-// that does not hold (wide ranges or many zeros along K, infinities, NaN,
-// exponents near the ends) go to a list, and the SIMT tiles compute them.  B
-// is taken in panels whose images stay in L2.
-// abc=iaj,jbic 512^3 i=j=16: 56.7 -> 2.74 ms (18 panels: pre-pass 23 us, GETT
-// 128 us each; 135 where every product reads its digit of A from shared
-// memory, not from the collector buffer, 153 with a conversion that branches;
-// without the drains and conversions 92).
+// What is left out of a term is at most 8.2 x 2^-62 of 2^(eA + eB): 7 products
+// of level 8 (2^-62 each) and past it, an entry's rounding to 62 bits (2^-63 of
+// either input) and that of level 7 (0.1 x 2^-62 at K = 32).  Two checks keep
+// that small:
+//   * the pre-pass counts per row the entries below 2^(e-5): where those of a
+//     row of A and of a column of B are together at most K / 2, at least K / 2
+//     terms of the sum are at least 2^(eA+eB-10), and what is left out is at
+//     most 2^-47.9 |A||B|, under the K 2^-53 of a chain of fused multiply-adds
+//     from K = 34 on.  Tiles where that does not hold (wide ranges or many
+//     zeros along K, infinities, NaN, exponents near the ends) go to a list.
+//   * where large terms cancel, |A||B| says little about the result: a chain may
+//     be exact where small terms are left beside them.  So a result v is stored
+//     only where it is at least 2^-10 2^(eA + eB), the error then at most
+//     K 2^-48.9 |v| whatever the terms, and marked otherwise: one of 7000 on
+//     uniform entries at K = 256, one of 1700 on normal ones.
+// Both are left to the chain (tc_exec.cu, left_kernel).  On uniform and normal
+// entries little but the last rounding is lost (5e-17 of the result, 6e-16 in
+// the chain).
+// B is taken in panels whose images stay in L2.
+// abc=iaj,jbic 512^3 i=j=16: 56.7 -> 2.95 ms (18 panels: pre-pass 23 us, GETT
+// 137 us each, 128 without the check of the results; left_kernel 76 us.  Of
+// the 128, 92 without the drains and conversions; 135 where every product
+// reads its digit of A from shared memory, not from the collector buffer, 153
+// with a conversion that branches).
 //
 // FP32 stays on the SIMT tiles.  Four digits (10 products, 0.59 ms against
 // 1.83 on the same contraction with uniform entries) hold 30 bits below the
@@ -119,12 +128,16 @@ struct PackedDesc : GettModes {
     int *status;
     const float *qscale;        // E4M3: the inputs' scales
     int64_t n_begin;            // first column of the panel (N then counts the panel's)
-    // digits: scalars in FP64, per row the exponent field of its largest magnitude, per
-    // image row tile the most small entries of a row, and the tiles left to
-    // SIMT (list[0]: how many)
+    // digits: scalars in FP64, per row the exponent field of its largest
+    // magnitude (0: a row of zeros), per image row tile the most small entries
+    // of a row, and the tiles left to SIMT (list[0]: how many)
     double alpha64, beta64;
     int *exps[2], *small[2];
     int64_t *list;
+    // results left to the chain: a bit per column of 32 for each row of A's
+    // images, the columns from weak_n0 on
+    uint32_t *weak;
+    int64_t weak_n0, rows_a, weak_below;
 };
 
 // One input's share of the pre-pass.
@@ -388,7 +401,7 @@ __global__ void __launch_bounds__(kPackThreads, 2) pack_digits_kernel(const __gr
         int few = (int)min(d.K, (int64_t)kRowBad) - nlarge[lane];
         if (top == 0) few = 0;  // a row of zeros (or past the extent): exact
         else if (E < kDigitLow || E > kDigitHigh) few = kRowBad;
-        d.exps[J.op][R] = top == 0 ? kDigitLow : E;
+        d.exps[J.op][R] = E;  // (0: zeros, of a row that is taken)
         if (few > 0) atomicMax(&d.small[J.op][(J.op == 0 ? 0 : d.n_begin / J.rows) + rt], few);
     }
 }
@@ -932,6 +945,15 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
             if constexpr (KIND == GK_D64) {
                 // (the next tile accumulates meanwhile)
                 const int *ce = cE[tab];
+                uint32_t weak = 0;
+                if (om >= 0 && rowE != 0) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if ((uint64_t)(dhi[j] + d.weak_below) < (uint64_t)(2 * d.weak_below) && ce[half * 32 + j] != 0) weak |= 1u << j;
+                }
+                // a patch of 32 x 32 with many of them is left as a whole
+                if (__reduce_add_sync(0xffffffffu, __popc(weak)) > kWeakMax) weak = ~0u;
+                d.weak[((n0 - d.weak_n0) / 32 + half) * d.rows_a + mm] = weak;
                 if (om >= 0) {
                     double *at = (double *)d.C + om + (lin != 0 ? on0 + half * 32 * lin : 0);
 #pragma unroll
@@ -939,9 +961,10 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                         const int cc = half * 32 + j;
                         if (cc >= nval) break;
                         double *q = lin != 0 ? at : at + cn[cc];
-                        double v = fixed_to_double(dhi[j], dlo[j], rowE + ce[cc] - 2104);
+                        const double v = fixed_to_double(dhi[j], dlo[j], rowE + ce[cc] - 2104);
                         if (plain) *q = v;
-                        else *q = d.init == 2 ? d.alpha64 * v : fma(d.alpha64, v, d.beta64 * *q);
+                        else if (d.init == 2) *q = d.alpha64 * v;
+                        else if (!(weak & 1u << j)) *q = fma(d.alpha64, v, d.beta64 * *q);  // (the chain needs the old value)
                     }
                 }
             }
@@ -1181,12 +1204,14 @@ tc_status run_packed(Plan &p, PackedDesc &d, bool comp, int64_t comp_k, double f
 // ---- digits, host side
 constexpr int64_t kDigitMinK = 32;       // where the bound of the digits meets the chain's
 constexpr int64_t kDigitMaxTiles = int64_t(1) << 22;
+constexpr int64_t kWeakBytes = int64_t(32) << 20;
 
 struct DigitPlan {
     bool pair;
     int64_t tiles_m, tiles_n, panel_tiles;  // panel_tiles: columns of tiles per panel of B
     int64_t rows_a, image_a, image_b;       // padded rows of A; bytes of A's images and of a panel's
-    int64_t off_b, off_exp_a, off_exp_b, off_small_a, off_small_b, off_list, zero_bytes, bytes;
+    int64_t weak_tiles;                     // columns of tiles whose weak results are kept before the chain runs
+    int64_t off_b, off_exp_a, off_exp_b, off_weak, off_small_a, off_small_b, off_list, zero_bytes, bytes;
 };
 
 // The digit form of an M x N x K product, or false where SIMT is the faster
@@ -1210,6 +1235,9 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
         q.image_a = q.rows_a * Kp * S * 2;
         if (q.image_a > kScratchMaxABytes) continue;
         q.panel_tiles = panel_tiles_for(kDigitPanelBytes, q.tiles_n, q.tiles_m, Kp * S * 2 * kDigitBn, slots);
+        const int64_t weak_max = std::max<int64_t>(1, kWeakBytes / (q.rows_a * kDigitBn / 8));
+        q.panel_tiles = std::min(q.panel_tiles, weak_max);
+        q.weak_tiles = std::min(q.tiles_n, weak_max);
         q.image_b = q.panel_tiles * kDigitBn * Kp * S * 2;
         const int64_t panels = (q.tiles_n + q.panel_tiles - 1) / q.panel_tiles;
         const int brows = pair ? kDigitBn / 2 : kDigitBn, nprod = S * (S + 1) / 2;
@@ -1219,7 +1247,8 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
         const int64_t waves = (panels - 1) * ((q.panel_tiles * q.tiles_m + slots - 1) / slots) +
                               ((q.tiles_n - (panels - 1) * q.panel_tiles) * q.tiles_m + slots - 1) / slots;
         const double pack = (double)(q.rows_a + q.tiles_n * kDigitBn) * Kp * (8 + S * 2) / 3e12;
-        const double sec = waves * tile / 1.9e9 + pack + 12e-6 + panels * 6e-6;
+        // (left_kernel: a launch and, nearly always, some output's chain)
+        const double sec = waves * tile / 1.9e9 + pack + 20e-6 + K * 30e-9 + panels * 6e-6;
         if (best < 0 || sec < best) {
             best = sec;
             P = q;
@@ -1232,11 +1261,13 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
     P.off_b = P.image_a;
     P.off_exp_a = P.off_b + P.image_b;
     P.off_exp_b = P.off_exp_a + up(P.rows_a * 4);
-    // zeroed before each execute: the row tiles' counts and the list's length
-    P.off_small_a = P.off_exp_b + up(P.panel_tiles * kDigitBn * 4);
+    // zeroed before each execute: the weak results, the row tiles' counts and
+    // the list's length
+    P.off_weak = P.off_exp_b + up(P.panel_tiles * kDigitBn * 4);
+    P.off_small_a = P.off_weak + up(P.weak_tiles * P.rows_a * kDigitBn / 8);
     P.off_small_b = P.off_small_a + up(P.rows_a / kRows * 4);
     P.off_list = P.off_small_b + up(P.tiles_n * 2 * 4);
-    P.zero_bytes = P.off_list + 8 - P.off_small_a;
+    P.zero_bytes = P.off_list + 8 - P.off_weak;
     P.bytes = P.off_list + up((P.tiles_m * P.tiles_n + 1) * 8);
     return true;
 }
@@ -1277,11 +1308,29 @@ tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta
     constexpr int kPackSmem = kDigitK * (kPackRows + 1) * (int)sizeof(double);
     cudaError_t e = cudaFuncSetAttribute(pack_digits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPackSmem);
     if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
-    e = cudaMemsetAsync(ws + P.off_small_a, 0, (size_t)P.zero_bytes, st);
+    d.weak = (uint32_t *)(ws + P.off_weak);
+    d.rows_a = P.rows_a;
+    // 2^-10 in the units of levels 0-3, 2^-36; levels 4-7 add at most 2^8.1 of
+    // them per K position
+    d.weak_below = (int64_t(1) << 26) + d.K * 512;
+    e = cudaMemsetAsync(ws + P.off_weak, 0, (size_t)P.zero_bytes, st);
     if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
+    int64_t weak0 = 0;  // first column of tiles of those in d.weak
+    auto run_left = [&](int64_t end, const int64_t *list) {
+        return simt_run_left(p, alpha, d.A, d.B, beta, d.C, d.weak, P.rows_a, weak0 * kDigitBn / 32, end * kDigitBn / 32, list,
+                             P.tiles_m, P.pair ? 2 * kRows : kRows, kDigitBn, st);
+    };
     for (int64_t t0 = 0; t0 < tiles_n; t0 += P.panel_tiles) {
         d.n_begin = t0 * kDigitBn;
         d.tiles_n = std::min(P.panel_tiles, tiles_n - t0);
+        if (t0 + d.tiles_n - weak0 > P.weak_tiles) {
+            s = run_left(t0, nullptr);
+            if (s != TC_SUCCESS) return s;
+            weak0 = t0;
+            e = cudaMemsetAsync(d.weak, 0, (size_t)(P.weak_tiles * P.rows_a * kDigitBn / 8), st);
+            if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
+        }
+        d.weak_n0 = weak0 * kDigitBn;
         d.N = std::min<int64_t>(N - d.n_begin, d.tiles_n * kDigitBn);
         d.num_tiles = d.tiles_m * d.tiles_n;
         PackJob ja = {}, jb = {};
@@ -1303,7 +1352,7 @@ tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta
         s = P.pair ? launch_gett<KIND, false, true>(d, ta, tb, st) : launch_gett<KIND, false, false>(d, ta, tb, st);
         if (s != TC_SUCCESS) return s;
     }
-    s = simt_run_list(p, alpha, d.A, d.B, beta, d.C, d.list, P.tiles_m, P.pair ? 2 * kRows : kRows, kDigitBn, st);
+    s = run_left(tiles_n, d.list);
     if (s == TC_SUCCESS) *done = true;
     return s;
 }

@@ -127,7 +127,7 @@ def test_left_to_simt(tcmod, dtype):
     assert np.all(np.abs(got[i, j] - want) <= K * U[dtype] * np.abs(want))
 
 
-@pytest.mark.parametrize("dtype,small", [("f32", 2.0 ** -26)])
+@pytest.mark.parametrize("dtype,small", [("f32", 2.0 ** -26), ("f64", 2.0 ** -56)])
 def test_large_terms_cancel(tcmod, dtype, small):
     # pairs of terms that cancel exactly, beside entries far below them: a
     # chain keeps the small terms to their last bit, K roundings at most
@@ -142,3 +142,41 @@ def test_large_terms_cancel(tcmod, dtype, small):
     i, j = rng.integers(0, M, 2000), rng.integers(0, N, 2000)
     want = (A[i, 128:].astype(np.longdouble) * B[128:, j].T.astype(np.longdouble)).sum(1)
     assert np.all(np.abs(got[i, j] - want) <= K * U[dtype] * np.abs(want))
+
+
+@pytest.mark.parametrize("alpha,beta", [(1.0, 0.0), (0.5, -2.0)])
+@pytest.mark.parametrize("spec", ["ab=ai,ib", "ab=ia,bi"])
+def test_small_results_by_the_chain(tcmod, spec, alpha, beta):
+    """Results below 2^-10 of the scales of their row and column come from the
+    chain bit for bit -- single ones, a row of a patch of 32 x 32, patches with
+    more than an eighth of them --, all others within half a unit in the last
+    place and K 2^-48.9 of the result."""
+    M, N, K = 300, 4000, 258
+    rng = np.random.default_rng(10)
+    A, B = rng.uniform(-1, 1, (M, K)), rng.uniform(-1, 1, (K, N))
+    for rows in (slice(32, 75), slice(200, 201)):
+        A[rows, 0::2], A[rows, 1::2] = 1, -1
+    B[1::2, 100:300] = B[0::2, 100:300]
+    A[250] = 0
+    C0 = rng.uniform(-1, 1, (M, N)) if beta else None
+    got, simt = execute(tcmod, "f64", A, B, C0, alpha, beta, spec=spec)
+    want = A @ B
+    scale = np.exp2(np.frexp(np.abs(A).max(1))[1])[:, None] * np.exp2(np.frexp(np.abs(B).max(0))[1])
+    v = np.abs(want) / scale
+    few = v < 2.0 ** -10.1
+    few[250] = False
+    assert few[:32].sum() > 5 and few[32:75, 100:300].all() and few[200, 100:300].all()
+    assert np.array_equal(got[few], simt[few])
+    assert not np.array_equal(got, simt)  # the digits ran
+    strong = v > 2.0 ** -9.9
+    strong[32:96, 96:320] = False  # patches there are left as a whole
+    i, j = np.nonzero(strong)
+    pick = rng.integers(0, len(i), 3000)
+    i, j = i[pick], j[pick]
+    v = (A[i].astype(np.longdouble) * B[:, j].T.astype(np.longdouble)).sum(1)
+    want = alpha * v + (beta * C0[i, j].astype(np.longdouble) if beta else 0)
+    u = U["f64"] * 1.01
+    bound = abs(alpha) * (K * 2.0 ** -48.9 + u) * np.abs(v) + u * np.abs(want)
+    if beta:
+        bound += u * np.abs(beta * C0[i, j])
+    assert np.all(np.abs(got[i, j] - want) <= bound)
