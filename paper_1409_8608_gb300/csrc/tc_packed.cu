@@ -83,6 +83,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <type_traits>
 
@@ -963,7 +964,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                         double *q = lin != 0 ? at : at + cn[cc];
                         const double v = fixed_to_double(dhi[j], dlo[j], rowE + ce[cc] - 2104);
                         if (plain) *q = v;
-                        else if (d.init == 2) *q = d.alpha64 * v;
+                        else if (d.init == 2) *q = fma(d.alpha64, v, 0.0);  // (+0 where the chain has it)
                         else if (!(weak & 1u << j)) *q = fma(d.alpha64, v, d.beta64 * *q);  // (the chain needs the old value)
                     }
                 }
@@ -1363,6 +1364,9 @@ tc_status exec_digits(Plan &p, const void *alpha, const void *A, const void *B, 
                       double fraction, bool *done) {
     *done = false;
     if (p.dtype != TC_F64 || !p.batch.empty() || p.contracted.empty()) return TC_SUCCESS;
+    // the chain multiplies A by alpha entry by entry: an infinite one gives NaN
+    // beside a zero or opposite signs, which the digits' one product would not
+    if (!std::isfinite(*(const double *)alpha)) return TC_SUCCESS;
     PackedDesc d;
     std::memset(&d, 0, sizeof(d));
     tc_status s = describe_modes(p, 3, d);

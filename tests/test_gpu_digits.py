@@ -180,3 +180,15 @@ def test_small_results_by_the_chain(tcmod, spec, alpha, beta):
     if beta:
         bound += u * np.abs(beta * C0[i, j])
     assert np.all(np.abs(got[i, j] - want) <= bound)
+
+
+@pytest.mark.parametrize("alpha", [float("inf"), float("-inf"), float("nan"), 0.0, -0.0])
+def test_special_alpha(tcmod, alpha):
+    M, N, K = SIZES["f64"][0]
+    rng = np.random.default_rng(11)
+    A, B = rng.uniform(-1, 1, (M, K)), rng.uniform(-1, 1, (K, N))
+    A[17], A[18] = np.abs(A[17]), 0
+    B[:, 40] = np.abs(B[:, 40])
+    got, simt = execute(tcmod, "f64", A, B, None, alpha, 0.0)
+    assert np.array_equal(got, simt, equal_nan=True)
+    assert np.array_equal(np.signbit(got), np.signbit(simt)) or np.isnan(simt).any()
