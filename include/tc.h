@@ -189,7 +189,8 @@ tc_status tc_algorithm_workspace(tc_plan plan, int32_t alg_id, size_t *bytes);
  * like smaller sizes.  The images of the digits take up to 64 MiB for B and 256
  * MiB for A, the marks of single results 32 MiB, allocated by the first execute
  * outside a stream capture and kept until tc_plan_destroy; when that fails, or
- * inside a capture before, the chains run instead. */
+ * inside a capture before, the chains run instead.  tc_plan_set_gett_pack(plan,
+ * 0) keeps the chains, which take no memory. */
 tc_status tc_execute(tc_plan plan, const void *alpha, const void *A,
                      const void *B, const void *beta, void *C, void *stream);
 
@@ -260,7 +261,8 @@ tc_status tc_plan_set_gett_tma(tc_plan plan, int32_t enable);
  * 16-bit values or the scaled E4M3 bytes in the MMA's core-matrix layout,
  * zeros past the extents), and the GETT copies
  * them instead of loading and converting the input per tile; the K order
- * then follows the larger input alone.  mode 0: never; 1 (default): both
+ * then follows the larger input alone.  mode 0: never (TC_F64: the chains of
+ * fused multiply-adds at every size, no scratch); 1 (default): both
  * inputs for the compensated split form (K past the chunk of
  * tc_plan_set_compensation) and wherever M and N are both at least 1024,
  * when their images fit in 2 GiB, else (FP32 inputs) the smaller input

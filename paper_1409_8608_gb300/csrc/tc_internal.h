@@ -62,7 +62,7 @@ struct Plan {
     int split_products = 6;         // TC_BF16X3: 3, 6 or 9 slice products
     int gett_bn = 0;                // tensor-core GETT tile width (0: by N)
     int gett_tma = 1;               // tensor-core GETT: TMA staging where legal
-    int gett_pack = 1;              // tensor-core GETT: pre-convert the small input (0 never, 1 auto, 2 always)
+    int gett_pack = 1;              // pre-convert inputs (0 never, 1 auto, 2 the small one, 3 both); FP64: 0 no digits
     int comp_chunk = -1;            // TC_BF16X3: compensated K chunk (-1 default, 0 off)
     int gett_pair = 0;              // tensor-core GETT: CTA pairs (cta_group::2) where legal
     int gett_split = -1;            // TC_BF16X3: (0,0) products in their own accumulator (-1 auto)

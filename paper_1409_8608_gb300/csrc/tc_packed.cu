@@ -1363,7 +1363,7 @@ tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta
 tc_status exec_digits(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C, void *stream,
                       double fraction, bool *done) {
     *done = false;
-    if (p.dtype != TC_F64 || !p.batch.empty() || p.contracted.empty()) return TC_SUCCESS;
+    if (p.dtype != TC_F64 || p.gett_pack == 0 || !p.batch.empty() || p.contracted.empty()) return TC_SUCCESS;
     // the chain multiplies A by alpha entry by entry: an infinite one gives NaN
     // beside a zero or opposite signs, which the digits' one product would not
     if (!std::isfinite(*(const double *)alpha)) return TC_SUCCESS;

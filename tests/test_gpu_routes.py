@@ -179,6 +179,31 @@ def test_digits_and_capture(tcmod, dtype):
     plan.close()
 
 
+def test_pack_mode_0_keeps_the_chain(tcmod):
+    """FP64 with tc_plan_set_gett_pack(0): the SIMT tiles' bits, no scratch."""
+    spec, e = DIGITS[0]
+    strides, C0, A, B, _ = digit_operands("f64", spec, e, 0, False)
+    simt = simt_plan(tcmod, spec, e, strides, "f64")
+    want = torch.zeros_like(C0)
+    simt.execute(A, B, want)
+    simt.close()
+    plan = tcmod.Plan(spec, [e[c] for c in synth.index_order(spec)], strides=strides, dtype="f64")
+    plan.set_gett_pack(0)
+    plan.execute(A, B, C0)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    assert torch.equal(C0, want)
+    plan.set_gett_pack(1)
+    plan.execute(A, B, C0)
+    torch.cuda.synchronize()
+    assert not torch.equal(C0, want) and torch.cuda.mem_get_info()[0] < free
+    plan.set_gett_pack(0)
+    plan.execute(A, B, C0)
+    torch.cuda.synchronize()
+    assert torch.equal(C0, want)
+    plan.close()
+
+
 @pytest.mark.parametrize("dtype", ["f64", "f32"])
 @pytest.mark.parametrize("K", [1, 3, 4, 5, 31, 32, 33])
 @pytest.mark.parametrize("a", [97, 100])  # either side of 64 outputs per SM
