@@ -252,6 +252,81 @@ __global__ void __launch_bounds__(256) coop_reduce_kernel(const PhaseDesc d) {
     }
 }
 
+// The same sums, one thread per output: where the index is short and outputs
+// are many, the lanes of a group mostly repeat one another's index arithmetic
+// (130 k outputs of 9 x 11 positions, FP32: 93-111 us in groups, 24-28 so).
+// A thread keeps the G partial sums of a group (kext <= G) and adds them in the
+// butterfly's order, so the results are the same bits.
+template <typename T, int G>
+__global__ void __launch_bounds__(256) lane_sums_kernel(const PhaseDesc d) {
+    const T *__restrict__ A = (const T *)d.A;
+    const T *__restrict__ B = (const T *)d.B;
+    T *__restrict__ C = (T *)d.C;
+    const int nr = d.red.n;
+    const int kext = (int)d.red.ext[nr - 1];
+    const int64_t ksA = d.red.sA[nr - 1], ksB = d.red.sB[nr - 1];
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < d.total;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        int64_t r = e, oA = 0, oB = 0, oC = 0;
+        for (int m = 0; m < d.out.n; ++m) {
+            const int64_t x = r % d.out.ext[m];
+            r /= d.out.ext[m];
+            oA += x * d.out.sA[m];
+            oB += x * d.out.sB[m];
+            oC += x * d.out.sC[m];
+        }
+        for (int m = d.task.n - 1; m >= 0; --m) {
+            const int64_t x = r % d.task.ext[m];
+            r /= d.task.ext[m];
+            oA += x * d.task.sA[m];
+            oB += x * d.task.sB[m];
+            oC += x * d.task.sC[m];
+        }
+        T acc[G];
+#pragma unroll
+        for (int l = 0; l < G; ++l) acc[l] = T(0);
+        int64_t idx[kMaxModes];
+        for (int m = 0; m < nr - 1; ++m) idx[m] = 0;
+        for (;;) {
+            int64_t pa = oA, pb = oB;
+            for (int m = 0; m < nr - 1; ++m) {
+                pa += idx[m] * d.red.sA[m];
+                pb += idx[m] * d.red.sB[m];
+            }
+            constexpr int V = 4;  // positions whose loads are in flight together
+#pragma unroll
+            for (int l0 = 0; l0 < G; l0 += V) {
+                if (l0 >= kext) break;
+                T a[V], b[V];
+#pragma unroll
+                for (int l = 0; l < V; ++l) {
+                    const bool in = l0 + l < kext;
+                    a[l] = in ? A[pa + (l0 + l) * ksA] : T(0);
+                    b[l] = in ? B[pb + (l0 + l) * ksB] : T(0);
+                }
+#pragma unroll
+                for (int l = 0; l < V; ++l)
+                    if (l0 + l < kext) acc[l0 + l] = fma_t<T>(a[l], b[l], acc[l0 + l]);
+            }
+            int m = nr - 2;
+            while (m >= 0) {
+                if (++idx[m] < d.red.ext[m]) break;
+                idx[m] = 0;
+                --m;
+            }
+            if (m < 0) break;
+        }
+#pragma unroll
+        for (int off = G / 2; off > 0; off /= 2)
+#pragma unroll
+            for (int l = 0; l < off; ++l) acc[l] += acc[l + off];
+        T v = d.alpha_one ? acc[0] : (T)d.alpha * acc[0];
+        if (d.init == 0) v += C[oC];
+        else if (d.init == 1) v = fma_t<T>((T)d.beta, C[oC], v);
+        C[oC] = v;
+    }
+}
+
 // ---------------------------------------------------------------- gemm / SIMT GETT
 __device__ __forceinline__ uint64_t pack_f2(float lo, float hi) {
     uint64_t r;
@@ -1007,6 +1082,7 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
     PhaseDesc pd;
     TileDesc td;
     int coop_g = 0;  // lanes per output of coop_reduce_kernel (0: elementwise_kernel)
+    bool coop_thread = false;  // its sums in one thread
     std::memset(&pd, 0, sizeof(pd));
     std::memset(&td, 0, sizeof(td));
     int64_t ntasks = 1;
@@ -1050,10 +1126,8 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
         // contracted index has unit stride in an input, a group of lanes per
         // output splits that index instead (coop_reduce_kernel, loads
         // contiguous across the group): the reduction, not the output count,
-        // then sets the parallelism.  Each lane of a group repeats the index
-        // arithmetic of its output, which a short index does not pay for
-        // unless outputs are few: 130 k outputs of 9 x 11 positions FP32 took
-        // 91-101 us in groups, 16-21 us one thread per output.
+        // then sets the parallelism.  Where that index is short and outputs
+        // are not few, one thread computes a group's sums (lane_sums_kernel).
         const int kr = pd.red.n - 1;
         if (alg.kernel == TC_KERNEL_GER && pd.out.n == 2 && pd.out.sC[1] < pd.out.sC[0]) {
             std::swap(pd.out.ext[0], pd.out.ext[1]);
@@ -1062,8 +1136,9 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
             std::swap(pd.out.sC[0], pd.out.sC[1]);
         }
         const bool k_unit = kr >= 0 && (pd.red.sA[kr] == 1 || pd.red.sB[kr] == 1);
-        if (k_unit && pd.red.ext[kr] > 1 && pd.total < (int64_t)device_sms() * (pd.red.ext[kr] < 32 ? 64 : 1024)) coop_g = 1;
+        if (k_unit && pd.red.ext[kr] > 1 && pd.total < (int64_t)device_sms() * 1024) coop_g = 1;
         if (coop_g) {
+            coop_thread = pd.red.ext[kr] < 32 && pd.total >= (int64_t)device_sms() * 64;
             const int64_t kext = pd.red.ext[kr];
             coop_g = kext <= 4 ? 4 : (kext <= 8 ? 8 : (kext <= 16 ? 16 : 32));
         }
@@ -1149,7 +1224,15 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
             q.C = Cptr;
             q.init = init;
             q.total = cut(pd.total);
-            if (coop_g) {
+            if (coop_thread) {
+                const unsigned grid = (unsigned)grid_for(q.total, 256);
+                switch (coop_g) {
+                    case 4: lane_sums_kernel<T, 4><<<grid, 256, 0, st>>>(q); break;
+                    case 8: lane_sums_kernel<T, 8><<<grid, 256, 0, st>>>(q); break;
+                    case 16: lane_sums_kernel<T, 16><<<grid, 256, 0, st>>>(q); break;
+                    default: lane_sums_kernel<T, 32><<<grid, 256, 0, st>>>(q); break;
+                }
+            } else if (coop_g) {
                 const int64_t grid = grid_for(q.total * coop_g, 256);
                 switch (coop_g) {
                     case 4: coop_reduce_kernel<T, 4><<<(unsigned)grid, 256, 0, st>>>(q); break;

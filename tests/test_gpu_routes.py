@@ -229,6 +229,38 @@ def test_nests_short_contracted(tcmod, a, K, dtype):
     plan.close()
 
 
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("K", [2, 4, 5, 11, 16, 17, 31])
+@pytest.mark.parametrize("alpha,beta", [(1.0, 0.0), (0.7, 1.0), (1.0, -0.3)])
+def test_nests_sum_in_the_same_order(tcmod, alpha, beta, K, dtype):
+    """Few outputs go to groups of lanes, a hundred per SM to a thread each:
+    the same sums, so a slice of the larger contraction has the same bits."""
+    spec = "ab=ija,ijb"
+    N = 128
+    rng = np.random.default_rng(K)
+    A, B, C0 = (torch.from_numpy(rng.uniform(-1, 1, n).astype(NP[dtype])).cuda()
+                for n in (K * 9 * N, K * 9 * N, N * N))
+    out = []
+    for b in (N, 64):  # 16384 outputs, and 8192: fewer than 64 per SM
+        plan = tcmod.Plan(spec, [N, b, K, 9], dtype=dtype)
+        ids = {}
+        for alg in plan.algorithms():
+            if alg["kernel"] not in ("gemm", "gett") and alg["n_phases"] == 1:
+                ids[alg["name"]] = alg["id"]
+        res = {}
+        for name, i in ids.items():
+            plan.select(i)
+            dC = C0[:N * b].clone()
+            plan.execute(A, B[:K * 9 * b], dC, alpha=alpha, beta=beta)
+            torch.cuda.synchronize()
+            res[name] = dC.cpu().numpy()
+        plan.close()
+        out.append(res)
+    assert out[0].keys() == out[1].keys() and len(out[0]) >= 2
+    for name, c in out[1].items():
+        assert np.array_equal(out[0][name][:N * 64], c), name
+
+
 @pytest.mark.parametrize("K", [1, 15, 17])
 def test_batch_f64_tiles(tcmod, K):
     spec = "abc=ai,ibc"
