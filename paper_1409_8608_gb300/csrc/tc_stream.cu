@@ -50,6 +50,7 @@
 #include <type_traits>
 
 #include "tc_internal.h"
+#include "tc_ring.h"
 #include "tc_tcgen05.cuh"
 
 namespace tc {
@@ -171,9 +172,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
         // with the bytes to release per slot held by lane `slot`: one lane
         // alone, with 64-bit remainders and its books in local memory, took
         // about 1900 clocks a tile and set the pace of the kernel.
-        int used = 0, pos = 0;          // bytes taken; where the next tile goes
-        int slot = 0, oldest = 0, busy = 0;  // next slot, the oldest in flight, how many
-        uint32_t ph = 0;                // parity of the oldest slot's release
+        ByteRing<kRawBytes, kRawSlots> ring;
         int mine_size = 0;              // lane l: bytes that slot l's tile holds
         bool stop = false;
         const int64_t count = a.t_end > first ? (a.t_end - first + step - 1) / step : 0;  // tiles of this CTA
@@ -201,16 +200,13 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
                 const unsigned long long tA = __shfl_sync(0xffffffffu, pA, jj), tB = __shfl_sync(0xffffffffu, pB, jj);
                 const uint32_t bytesA = __shfl_sync(0xffffffffu, nA, jj), bytesB = __shfl_sync(0xffffffffu, nB, jj);
                 const int offA = (int)((bytesB + 127) & ~127u), size = offA + (int)((bytesA + 127) & ~127u);
-                const bool wrap = pos + size > kRawBytes;
-                const int skip = wrap ? kRawBytes - pos : 0;  // the ring's end
-                while (!stop && (used + skip + size > kRawBytes || busy == kRawSlots)) {
-                    stop = !__all_sync(0xffffffffu, mbar_wait_or(&raw_empty[oldest], ph, abort_now));
-                    used -= __shfl_sync(0xffffffffu, mine_size, oldest);
-                    --busy;
-                    if (++oldest == kRawSlots) oldest = 0, ph ^= 1u;
-                }
+                int skip;
+                stop = !ring.make_room(
+                    size, skip,
+                    [&](int s, uint32_t ph) { return __all_sync(0xffffffffu, mbar_wait_or(&raw_empty[s], ph, abort_now)) != 0; },
+                    [&](int s) { return __shfl_sync(0xffffffffu, mine_size, s); });
                 if (stop) break;
-                if (wrap) pos = 0;
+                const int slot = ring.slot, pos = ring.take(size, skip);
                 if (lane == slot) mine_size = size + skip;
                 if (elect_one()) {
                     raw_off[slot] = pos;
@@ -219,19 +215,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const StreamA
                     bulk_load(raw + pos + offA, (const void *)tA, bytesA, &raw_full[slot]);
                 }
                 __syncwarp();
-                used += size + skip;
-                pos += size;
-                ++busy;
-                if (++slot == kRawSlots) slot = 0;
             }
         }
         if (stop && lane == 0) give_up();
         // nothing may still be copying into shared memory at exit: the tiles
         // not known released have landed
-        for (; busy > 0; --busy) {
-            mbar_wait(&raw_full[oldest], ph);
-            if (++oldest == kRawSlots) oldest = 0, ph ^= 1u;
-        }
+        ring.drain([&](int s, uint32_t ph) { mbar_wait(&raw_full[s], ph); });
         __syncwarp();
     } else if (warp >= kWConv && warp < kWEpi) {
         // ----------------------------------------------------------- converters
