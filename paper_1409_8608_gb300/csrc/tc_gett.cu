@@ -52,6 +52,7 @@
 
 #include "tc_gett.cuh"
 #include "tc_internal.h"
+#include "tc_ring.h"
 
 namespace tc {
 
@@ -886,6 +887,8 @@ gett_tc_kernel(const GettDesc d, const __grid_constant__ CUtensorMap tmA, const 
                 *abort_flag = 1;
                 atomicExch(d.status, (int)TC_ERROR_TIMEOUT);
             }
+            // the last boxes have landed before the CTA may leave
+            last_filled(g, NSL, [&](int s, uint32_t parity) { mbar_wait(&sfull[s], parity); });
         }
         __syncwarp();
     } else if (warp == kMmaWarp) {

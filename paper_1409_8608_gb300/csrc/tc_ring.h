@@ -1,6 +1,8 @@
-// Books of a byte ring into which a producer copies tiles of their own sizes,
-// released by their readers in order (tc_stream.cu); plain C++, so that they
-// can be run on the host too.
+// Books of the rings into which a producer copies tiles: one of bytes, tiles of
+// their own sizes released by their readers in order (tc_stream.cu), and what
+// a producer of any ring waits for before its block may leave, since another
+// role may have given up with copies on their way.  Plain C++, so that they can
+// be run on the host too.
 #pragma once
 
 #include <cstdint>
@@ -62,5 +64,13 @@ struct ByteRing {
         }
     }
 };
+
+// f(slot, parity) for the last fillings of a ring's slots that nothing may have
+// read: filling q goes to slot q % slots and completes phase q / slots of its
+// barrier.
+template <class F>
+TC_RING_FN void last_filled(int64_t filled, int slots, F f) {
+    for (int64_t q = filled > slots ? filled - slots : 0; q < filled; ++q) f((int)(q % slots), (uint32_t)((q / slots) & 1));
+}
 
 }  // namespace tc

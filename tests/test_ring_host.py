@@ -52,6 +52,20 @@ int main() {
             CHECK(waited[i].slot == flight[i].slot && waited[i].ph == flight[i].ph);
         CHECK(ring.busy == 0);
     }
+    // the fillings of a ring's slots that a producer waits for at the end: each
+    // slot's last one, with the parity of the phase that it completes
+    for (int slots = 1; slots <= 8; ++slots)
+        for (int filled = 0; filled < 40; ++filled) {
+            std::vector<int> last(slots, -1);
+            for (int q = 0; q < filled; ++q) last[q % slots] = q;
+            int n = 0, ok = 0;
+            tc::last_filled(filled, slots, [&](int s, unsigned parity) {
+                ++n;
+                ok += last[s] >= 0 && parity == (unsigned)(last[s] / slots % 2);
+                last[s] = -1;
+            });
+            CHECK(n == (filled < slots ? filled : slots) && ok == n);
+        }
     return 0;
 }
 """
