@@ -89,6 +89,7 @@
 
 #include "tc_gett.cuh"
 #include "tc_internal.h"
+#include "tc_ring.h"
 
 namespace tc {
 
@@ -105,6 +106,7 @@ constexpr int kMmaWarp = kEpiWarps, kCopyWarp = kEpiWarps + 1;
 constexpr int kThreads = (kCopyWarp + 1) * 32;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMapRow = 512;               // bytes per row of an image tensor map
+constexpr unsigned long long kLandNs = 2000000;  // copies on their way land within this (microseconds)
 
 // K positions per stage: about 32-48 KB of images per CTA
 template <int KIND>
@@ -618,6 +620,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
         const int32_t rows_a = (int32_t)(d.img_a / kMapRow), rows_b = (int32_t)(d.img_b / kMapRow);
         int s = 0;
         uint32_t ph = 1;  // parity of the slot's last release (the first round finds it free)
+        int64_t filled = 0;
         bool stop = false;
         for (int64_t tile = slot0; tile < d.num_tiles && !stop; tile += nslots) {
             int64_t mt;
@@ -639,14 +642,19 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
                     image_load<PAIR>(dst + d.img_a, &tmB, bar, rb);
                 }
                 __syncwarp();
+                ++filled;
                 if (++s == d.stages) s = 0, ph ^= 1u;
             }
         }
-        if (stop) {
-            if (lane == 0) give_up();
-            // copies in flight land (microseconds) before the CTA leaves
+        if (stop && lane == 0) give_up();
+        // the last copies have landed before the CTA may leave (a pair's arrive
+        // on the first CTA's barriers, and neither leaves before both are done)
+        if (crank == 0) last_filled(filled, d.stages, [&](int i, uint32_t parity) { mbar_wait(&full[i], parity, kLandNs); });
+        // a pair: the first CTA may have stopped before it counted a copy of the
+        // second's
+        if (PAIR && stop) {
             const uint64_t t0 = globaltimer();
-            while (globaltimer() - t0 < 2000000ull) {
+            while (globaltimer() - t0 < kLandNs) {
             }
         }
         __syncwarp();
