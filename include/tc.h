@@ -385,7 +385,8 @@ tc_status tc_setup_list(tc_plan plan, int32_t alg_id, int32_t granularity, int32
  * touch kernels and L2-sized remote reads, then one representative phase
  * runs over a few waves of its work, timed ten times with CUDA events; the
  * median, scaled to the whole phase and weighted by the case's count, sums
- * to the prediction.  The GETT runs a few waves of its real tiles.
+ * to the prediction.  The GETT runs a few waves of its real tiles and twice
+ * as many, and the line through both times gives the prediction.
  * alg_ids: n ids, or NULL for every algorithm (seconds then holds
  * tc_algorithm_count entries).  A, B, C: device buffers laid out as the plan
  * describes, or NULL for zero-filled scratch the call allocates and frees.

@@ -13,7 +13,8 @@
 //     at 5/4 of the L2 size queried from the device;
 //   * the timed part is one representative phase -- its copies and its
 //     kernel -- over a fraction of its work of a few waves, scaled back up
-//     (the GETT runs a few waves of its real tiles);
+//     (the GETT runs a few waves of its real tiles, and twice as many: its
+//     cost beside them is not scaled);
 //   * each case is timed ten times with CUDA events; the median counts.
 #include <cuda_runtime.h>
 
@@ -227,10 +228,18 @@ tc_status predict_one(Plan &p, int alg_id, const Operands &ops, unsigned *sink, 
         NestView v;
         v.kernel.assign(p.nidx, true);
         std::vector<SetupItem> none;
-        double t = 0;
-        tc_status s = time_case(p, alg_id, v, none, pr, ops, sink, st, &t);
-        if (s != TC_SUCCESS) return s;
-        *out = t / pr.fraction;
+        // Part of a GETT does not shrink with the fraction (a pre-pass over all
+        // of A, launches, what the digits leave to the chain): times over one
+        // and two such fractions, extrapolated along the line through them.
+        const double f = pr.fraction;
+        double t[2] = {0, 0};
+        const int n = 2 * f < 1.0 ? 2 : 1;
+        for (int i = 0; i < n; ++i) {
+            pr.fraction = n == 1 ? 1.0 : f * (i + 1);
+            tc_status s = time_case(p, alg_id, v, none, pr, ops, sink, st, &t[i]);
+            if (s != TC_SUCCESS) return s;
+        }
+        *out = n == 1 ? t[0] : t[1] + std::max(0.0, t[1] - t[0]) / f * (1.0 - 2 * f);
         return TC_SUCCESS;
     }
     tc_status s = ensure_device_resources(p, nest_workspace_bytes(p, alg));

@@ -52,6 +52,32 @@ def test_permuted_workload_ranking(tcmod):
     assert r["spearman"] > 0.6, {k: v for k, v in r.items() if k != "algorithms"}
 
 
+@pytest.mark.parametrize("dtype,ext", [("f64", [2048, 30000, 512]), ("bf16x3", [2048, 60000, 512]),
+                                       ("f32", [700, 16001, 301])])
+def test_gett_prediction_scales_what_shrinks(tcmod, dtype, ext):
+    """The GETT's probe cuts the columns, not the pre-pass over A nor the
+    launches: prediction within a fifth of the time of the whole."""
+    plan = tcmod.Plan("ab=ai,ib", ext, dtype=dtype)
+    dt = torch.float64 if dtype == "f64" else torch.float32
+    M, N, K = ext
+    gen = torch.Generator(device="cuda").manual_seed(0)
+    A, B = (torch.empty(n, dtype=dt, device="cuda").uniform_(-1, 1, generator=gen) for n in (M * K, K * N))
+    C = torch.empty(M * N, dtype=dt, device="cuda")
+    st = torch.cuda.current_stream()
+    times = []
+    for _ in range(12):
+        e0, e1 = torch.cuda.Event(True), torch.cuda.Event(True)
+        e0.record(st)
+        plan.execute(A, B, C, stream=st)
+        e1.record(st)
+        torch.cuda.synchronize()
+        times.append(e0.elapsed_time(e1) * 1e-3)
+    want = sorted(times)[5]
+    got = plan.predict([0])[0]
+    plan.close()
+    assert 0.8 * want < got < 1.2 * want, (got, want)
+
+
 def test_tensor_dtype_ranks_gemm_nests_and_gett(tcmod):
     # at tensor-core dtypes the gemm nests and the GETT are predicted (the
     # other kernels cannot run there), and the best prediction is one of them
