@@ -389,7 +389,11 @@ tc_status tc_setup_list(tc_plan plan, int32_t alg_id, int32_t granularity, int32
  * as many, and the line through both times gives the prediction.
  * alg_ids: n ids, or NULL for every algorithm (seconds then holds
  * tc_algorithm_count entries).  A, B, C: device buffers laid out as the plan
- * describes, or NULL for zero-filled scratch the call allocates and frees.
+ * describes, or NULL for scratch that the call allocates and frees, A and B
+ * with entries uniform in [-1, 1).  The time of a large TC_F64 GETT depends on
+ * the entries (tc_execute): up to that of the chains, 20 times as long, where
+ * every row or column has wide ranges or many zeros.  For such data give the
+ * operands; tc_chain_predict has uniform ones.
  * seconds[i] < 0 marks an algorithm that cannot run with the plan's dtype
  * (the loop nests run in FP64 and FP32 only).  Synchronises the stream.
  * The results stay in the plan for tc_plan_select_best. */

@@ -16,6 +16,8 @@
 //     (the GETT runs a few waves of its real tiles, and twice as many: its
 //     cost beside them is not scaled);
 //   * each case is timed ten times with CUDA events; the median counts.
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -69,6 +71,18 @@ __global__ void __launch_bounds__(256) remote_kernel(const uint4 *buf, int64_t n
         acc ^= v.x ^ v.w;
     }
     if (acc == 0x9E3779B9u) sink[0] = acc;
+}
+
+// Entries uniform in [-1, 1) on a grid of 2^-23 (BF16 and FP16: rounded), from
+// their places by Knuth's multiplicative hashing, twice.
+template <typename T>
+__global__ void __launch_bounds__(256) uniform_kernel(T *p, int64_t n) {
+    constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ull;  // 2^64 over the golden ratio
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        uint64_t x = (uint64_t)(e + 1) * kGolden;
+        x = (x ^ x >> 32) * kGolden;
+        p[e] = T((float)(int32_t)(x >> 40) * 0x1p-23f - 1.0f);
+    }
 }
 
 int g_sms = 0;
@@ -331,7 +345,10 @@ tc_status tc_predict(tc_plan plan, const int32_t *alg_ids, int32_t n, const void
     s = ensure_flush(p);
     if (s != TC_SUCCESS) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    // operands: the caller's, or zero-filled scratch of the operands' spans
+    // operands: the caller's, or scratch of the operands' spans, A and B with
+    // uniform entries: the time of a GETT may depend on them (on zeros the
+    // digits of FP64 leave nothing to the chain, and the tensor cores draw
+    // less power)
     Operands ops{A, B, C};
     void *own[3] = {nullptr, nullptr, nullptr};
     for (int o = 0; o < 3; ++o) {
@@ -344,7 +361,13 @@ tc_status tc_predict(tc_plan plan, const int32_t *alg_ids, int32_t n, const void
                 if (own[x]) cudaFree(own[x]);
             return fail(TC_ERROR_OUT_OF_MEMORY, cudaGetErrorString(e));
         }
-        cudaMemsetAsync(own[o], 0, bytes + 16, st);
+        const int64_t elems = span_elems(p, o);
+        const unsigned grid = (unsigned)blocks_for(elems);
+        if (o == OP_C) cudaMemsetAsync(own[o], 0, bytes + 16, st);
+        else if (p.dtype == TC_F64) uniform_kernel<<<grid, 256, 0, st>>>((double *)own[o], elems);
+        else if (p.dtype == TC_BF16) uniform_kernel<<<grid, 256, 0, st>>>((__nv_bfloat16 *)own[o], elems);
+        else if (p.dtype == TC_F16) uniform_kernel<<<grid, 256, 0, st>>>((__half *)own[o], elems);
+        else uniform_kernel<<<grid, 256, 0, st>>>((float *)own[o], elems);
         if (o == OP_A) ops.A = own[o];
         else if (o == OP_B) ops.B = own[o];
         else ops.C = own[o];

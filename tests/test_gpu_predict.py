@@ -31,7 +31,7 @@ def test_rank_statistics_helpers():
 
 def test_predictions_are_positive_and_selection_uses_them(tcmod):
     plan = tcmod.Plan("abc=ai,ibc", [64, 64, 64, 8])
-    pred = plan.predict()  # zero-filled scratch operands
+    pred = plan.predict()  # scratch operands
     assert len(pred) == 37 and all(p > 0 for p in pred)
     best = plan.select_best()
     assert best == int(np.argmin(pred)) and plan.selected == best
@@ -76,6 +76,21 @@ def test_gett_prediction_scales_what_shrinks(tcmod, dtype, ext):
     got = plan.predict([0])[0]
     plan.close()
     assert 0.8 * want < got < 1.2 * want, (got, want)
+
+
+def test_prediction_without_operands_has_entries(tcmod):
+    """Scratch operands hold uniform entries, not zeros, which the digits of an
+    FP64 GETT never leave to the chain: the prediction is that on uniform ones."""
+    plan = tcmod.Plan("ab=ai,ib", [300, 4000, 257], dtype="f64")
+    gen = torch.Generator(device="cuda").manual_seed(0)
+    A, B = (torch.empty(n, dtype=torch.float64, device="cuda").uniform_(-1, 1, generator=gen)
+            for n in (300 * 257, 257 * 4000))
+    C = torch.empty(300 * 4000, dtype=torch.float64, device="cuda")
+    zero = plan.predict([0], torch.zeros_like(A), torch.zeros_like(B), C)[0]
+    uniform = plan.predict([0], A, B, C)[0]
+    own = plan.predict([0])[0]
+    plan.close()
+    assert zero < 0.95 * uniform and abs(own - uniform) < abs(own - zero), (zero, uniform, own)
 
 
 def test_tensor_dtype_ranks_gemm_nests_and_gett(tcmod):
