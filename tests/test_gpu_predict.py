@@ -121,3 +121,30 @@ def test_autotune_and_cache(tcmod, tmp_path):
     assert plan2.autotune() == (width, tma)  # answered from the cache
     plan.close()
     plan2.close()
+
+
+def test_autotuned_is_no_slower_than_the_default(tcmod):
+    # 16-bit inputs, both as images by default: among the candidates too
+    spec, ext = "ab=aij,jib", [700, 900, 16, 40]
+    M, N, K = 700, 900, 640
+    A, B = (torch.ones(n, dtype=torch.bfloat16, device="cuda") for n in (M * K, K * N))
+    C = torch.empty(M * N, device="cuda")
+    st = torch.cuda.current_stream()
+
+    def time(plan):
+        ts = []
+        for _ in range(20):
+            e0, e1 = torch.cuda.Event(True), torch.cuda.Event(True)
+            e0.record(st)
+            plan.execute(A, B, C, stream=st)
+            e1.record(st)
+            torch.cuda.synchronize()
+            ts.append(e0.elapsed_time(e1))
+        return sorted(ts)[5]
+
+    plan = tcmod.Plan(spec, ext, dtype="bf16")
+    default = time(plan)
+    plan.autotune()
+    tuned = time(plan)
+    plan.close()
+    assert tuned < 1.3 * default, (tuned, default)
