@@ -178,19 +178,20 @@ tc_status tc_algorithm_workspace(tc_plan plan, int32_t alg_id, size_t *bytes);
  * skipped and nothing is recorded.
  *
  * TC_F64 with GETT selected: where the size makes it the faster form (K from
- * 32 to 2^20; no batch indices), the tensor cores compute the contraction
- * from exact 8-bit digits of the inputs, 62 bits below the largest magnitude
- * of a row of A and a column of B, rounded once.  A result v of A times B
- * computed so is off by at most half a unit in its last place, K 2^-48.9 |v|
- * and 2^-47.9 of the sum of its terms' magnitudes (on uniform and normal
- * entries little but the rounding).  Parts of C for which that does not hold --
- * single results that nearly cancel, rows or columns with many small entries,
- * infinities, NaN, extreme exponents -- run as chains of K fused multiply-adds,
- * like smaller sizes.  The images of the digits take up to 64 MiB for B and 256
- * MiB for A, the marks of single results 32 MiB, allocated by the first execute
- * outside a stream capture and kept until tc_plan_destroy; when that fails, or
- * inside a capture before, the chains run instead.  tc_plan_set_gett_pack(plan,
- * 0) keeps the chains, which take no memory. */
+ * 32 to 2^15, M up to 2^24 / K; no batch indices), the tensor cores compute
+ * the contraction from exact 8-bit digits of the inputs, 62 bits below the
+ * largest magnitude of a row of A and a column of B, rounded once.  A result v
+ * of A times B computed so is off by at most half a unit in its last place, K
+ * 2^-48.9 |v| and 2^-47.9 of the sum of its terms' magnitudes (on uniform and
+ * normal entries little but the rounding).  Parts of C for which that does not
+ * hold -- single results that nearly cancel, rows or columns with many small
+ * entries, infinities, NaN, extreme exponents -- run as chains of K fused
+ * multiply-adds, like smaller sizes.  The images of the digits take up to 64
+ * MiB for B and 256 MiB for A, the marks of results left to the chain up to 64
+ * MiB, allocated by the first execute outside a stream capture and kept until
+ * tc_plan_destroy; when that fails, or inside a capture before, the chains run
+ * instead.  tc_plan_set_gett_pack(plan, 0) keeps the chains, which take no
+ * memory. */
 tc_status tc_execute(tc_plan plan, const void *alpha, const void *A,
                      const void *B, const void *beta, void *C, void *stream);
 

@@ -260,7 +260,9 @@ __global__ void __launch_bounds__(kPackThreads) pack_images_kernel(const __grid_
 constexpr int kDigitLow = 623, kDigitHigh = 1423;  // exponent fields taken
 constexpr int kDigitChunkK = 128;         // K positions per accumulation
 constexpr int kDigitBn = 64;              // columns per tile: eight levels fill the tensor memory
-constexpr int64_t kDigitMaxK = 1 << 20;   // the summed levels stay below 2^62
+// Past it the images of A and of a panel of B hold fewer tiles than SMs, and no
+// size is estimated faster than SIMT (the summed levels stay below 2^52).
+constexpr int64_t kDigitMaxK = 1 << 15;
 constexpr int kRowBad = 1 << 29;
 constexpr int kDigitK = 256;  // K positions a block holds at a time
 
@@ -1095,7 +1097,7 @@ tc_status launch_gett(const PackedDesc &d, const CUtensorMap &ta, const CUtensor
 // launches cost more than reading the images from HBM (split-BF16 512^3
 // iaj,jbic: 7 panels of 64 MiB 122 us of pre-pass and 290 us of GETT, one of
 // 402 MB 102 and 257 us).
-constexpr int64_t kDigitPanelBytes = int64_t(64) << 20;
+constexpr int64_t kDigitPanelBytes = int64_t(64) << 20;  // (a tile takes 32 MiB at most)
 constexpr int64_t kPanelBytes = int64_t(512) << 20;
 constexpr int64_t kScratchMaxABytes = int64_t(256) << 20;
 

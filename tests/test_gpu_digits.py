@@ -192,3 +192,59 @@ def test_special_alpha(tcmod, alpha):
     got, simt = execute(tcmod, "f64", A, B, None, alpha, 0.0)
     assert np.array_equal(got, simt, equal_nan=True)
     assert np.array_equal(np.signbit(got), np.signbit(simt)) or np.isnan(simt).any()
+
+
+def test_panels(tcmod):
+    """Three panels of B, the last one ragged: exact on integers in all of them;
+    with rows and columns that the digits refuse in the later ones, listed and
+    digit tiles side by side."""
+    M, N, K = 600, 64 * 484 + 17, 257
+    rng = np.random.default_rng(12)
+    A, B = rng.integers(-(2 ** 22), 2 ** 22, (M, K)), rng.integers(-(2 ** 22), 2 ** 22, (K, N))
+    want = (torch.from_numpy(A).double().cuda() @ torch.from_numpy(B).double().cuda()).cpu().numpy()
+    got, _ = execute(tcmod, "f64", A.astype(np.float64), B.astype(np.float64))
+    assert np.array_equal(got, want)
+    A, B = rng.uniform(-1, 1, (M, K)), rng.uniform(-1, 1, (K, N))
+    A[530] *= 2.0 ** -np.arange(K)        # the third row tile: listed in every panel
+    B[0, 16000] = np.inf                  # second panel
+    B[:, 25000] = 1e300
+    B[: K // 2 + 9, N - 1] = 0            # the last, ragged tile
+    B[1:256:2, 30000:30040] = B[0:256:2, 30000:30040]  # third panel: results that cancel
+    A[10, 0:256:2], A[10, 1:256:2], A[10, 256] = 1, -1, 2.0 ** -50
+    listed = np.zeros((M, N), bool)
+    listed[512:] = True
+    for n in (16000, 25000, N - 1):
+        listed[:, n // 64 * 64: n // 64 * 64 + 64] = True
+    got, simt = execute(tcmod, "f64", A, B)
+    assert np.array_equal(got[listed], simt[listed], equal_nan=True)
+    assert np.array_equal(got[10, 30000:30040], simt[10, 30000:30040])
+    for m0 in (0, 256):  # every other tile by the digits
+        for n0 in range(0, N, 64):
+            if not listed[m0, n0]:
+                assert not np.array_equal(got[m0:m0 + 256, n0:n0 + 64], simt[m0:m0 + 256, n0:n0 + 64]), (m0, n0)
+    i, j = np.nonzero(~listed)
+    pick = rng.integers(0, len(i), 4000)
+    i, j = i[pick], j[pick]
+    terms = A[i].astype(np.longdouble) * B[:, j].T.astype(np.longdouble)
+    v = terms.sum(1)
+    small = np.abs(v) < 2.0 ** -9  # some of these by the chain
+    bound = (K * 2.0 ** -48.9 + 1.01 * U["f64"]) * np.abs(v) + np.where(small, K * U["f64"] * np.abs(terms).sum(1), 0)
+    assert np.all(np.abs(got[i, j] - v) <= bound)
+
+
+def test_long_k(tcmod):
+    # few tiles of B to a panel, many accumulations to a tile
+    M, N, K = 500, 600, 10001
+    gen = torch.Generator().manual_seed(13)
+    A, B = (torch.randint(-(2 ** 15), 2 ** 15, s, generator=gen).double() for s in ((M, K), (K, N)))
+    want = (A.cuda() @ B.cuda()).cpu().numpy()  # exact: sums below 2^44
+    got, _ = execute(tcmod, "f64", A.numpy(), B.numpy())
+    assert np.array_equal(got, want)
+    A, B = (torch.empty(s, dtype=torch.float64).uniform_(-1, 1, generator=gen) for s in ((M, K), (K, N)))
+    got, simt = execute(tcmod, "f64", A.numpy(), B.numpy())
+    assert not np.array_equal(got, simt)
+    i, j = torch.arange(0, 500, 5), torch.arange(0, 600, 6)
+    terms = A[i].numpy().astype(np.longdouble) * B[:, j].T.numpy().astype(np.longdouble)
+    v = terms.sum(1)
+    assert np.all(np.abs(got[i, j] - v) <= 1.01 * U["f64"] * np.abs(v) + K * 2.0 ** -58.9)
+    assert np.linalg.norm(got[i, j] - v) < np.linalg.norm(simt[i, j] - v)

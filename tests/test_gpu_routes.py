@@ -79,6 +79,30 @@ def test_images_by_default(tcmod, spec, e, pad, dtype):
         assert np.array_equal(out[0], oc.contract(spec, ext, A, B, C=C0.copy(), alpha=2.0, beta=-0.5, strides=strides))
 
 
+def test_image_panels(tcmod):
+    """Images of B past 512 MiB: two panels, the second one ragged, against the
+    inputs as they are; integers, so exact in every form."""
+    M, N, K = 200, 600011, 160
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    A, B = (torch.randint(-8, 9, (n,), device="cuda", generator=gen).float() for n in (M * K, K * N))
+    out = []
+    for mode in (1, 0):
+        plan = tcmod.Plan("ab=ai,ib", [M, N, K], dtype="bf16x3")
+        plan.set_gett_pack(mode)
+        C = torch.full((M * N,), float("nan"), device="cuda")
+        free = torch.cuda.mem_get_info()[0]
+        plan.execute(A, B, C)
+        torch.cuda.synchronize()
+        scratch = free - torch.cuda.mem_get_info()[0]
+        assert (scratch > 256 << 20) == (mode == 1), scratch  # the images ran
+        plan.device_status()
+        plan.close()
+        out.append(C)
+    assert torch.equal(out[0], out[1])
+    want = B.view(N, K).double() @ A.view(K, M).double()
+    assert torch.equal(out[0].double().view(N, M), want)
+
+
 DIGITS = [
     ("cab=iaj,jbic", {"a": 300, "b": 40, "c": 100, "i": 17, "j": 16}),
     ("bac=jai,cibj", {"a": 300, "b": 80, "c": 60, "i": 30, "j": 9}),
