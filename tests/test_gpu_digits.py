@@ -248,3 +248,19 @@ def test_long_k(tcmod):
     v = terms.sum(1)
     assert np.all(np.abs(got[i, j] - v) <= 1.01 * U["f64"] * np.abs(v) + K * 2.0 ** -58.9)
     assert np.linalg.norm(got[i, j] - v) < np.linalg.norm(simt[i, j] - v)
+
+
+def test_marks_in_groups(tcmod):
+    """More results than marks are kept for at a time: the chain runs between
+    the panels too (beta = 1, so results left to it would keep the old C)."""
+    M, N, K = 33000, 8300, 40
+    gen = torch.Generator(device="cuda").manual_seed(14)
+    A, B, C = (torch.randint(-(2 ** 20), 2 ** 20, (n,), device="cuda", generator=gen).double()
+               for n in (M * K, K * N, M * N))
+    want = C.view(N, M) + B.view(N, K) @ A.view(K, M)  # exact: sums below 2^46
+    plan = tcmod.Plan("ab=ai,ib", [M, N, K], dtype="f64")
+    plan.execute(A, B, C, alpha=1.0, beta=1.0)
+    torch.cuda.synchronize()
+    plan.device_status()
+    plan.close()
+    assert torch.equal(C.view(N, M), want)
