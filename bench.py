@@ -27,6 +27,7 @@ oracle runs only in the CPU leg below (timing it, and computing expected
 values for sampled outputs); the GPU numbers come from libtc.so alone.
 """
 import argparse
+import ctypes
 import hashlib
 import json
 import math
@@ -87,6 +88,34 @@ def captured_traffic(key, source):
     if not entry or entry.get("source_sha256") != source_sha(source):
         return None
     return entry.get("bytes_per_launch")
+
+
+def kernels_of(call, stream):
+    """Kernels that `call` launches on `stream`: those of a CUDA graph of it,
+    captured after a first call and thrown away."""
+    try:
+        rt = ctypes.CDLL("libcudart.so.13")  # PyTorch's
+    except OSError:
+        rt = ctypes.CDLL("/usr/local/cuda/lib64/libcudart.so")
+    handle, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+
+    def ok(status):
+        if status != 0:
+            raise RuntimeError(f"CUDA error {status} while counting launches")
+
+    ok(rt.cudaStreamBeginCapture(handle, 2))  # relaxed
+    call()
+    ok(rt.cudaStreamEndCapture(handle, ctypes.byref(graph)))
+    ok(rt.cudaGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    ok(rt.cudaGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    kernels = 0
+    for node in nodes:
+        kind = ctypes.c_int()
+        ok(rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        kernels += kind.value == 0
+    ok(rt.cudaGraphDestroy(graph))
+    return kernels
 
 
 def measured_peaks():
@@ -347,23 +376,18 @@ def measure_form(args, dtype, spec, extents, A, B, dev, stream, dist, world, tc,
     dA, dB = hA.to(dev), hB.to(dev)
     dC = torch.empty(nC, dtype=tout, device=dev)
     flops = plan.flops
-    # GETT: one kernel, plus the pre-pass when the plan pre-converts inputs
-    # (its workspace, or scratch of tens of MiB that the first execute takes;
-    # both inputs in one launch); FP64 from digits: also the tiles left
-    # to the SIMT kernel, and a further pair of launches per panel of the
-    # larger input, not counted here.  Nests: phases and copies
     free0 = torch.cuda.mem_get_info()[0]
     plan.execute(dA, dB, dC, alpha=1.0, beta=0.0, stream=stream)
     torch.cuda.synchronize()
+    # a GETT on images (of both inputs, or of FP64 digits) takes tens of MiB
+    # with its first execute
     images = alg["kernel"] == "gett" and free0 - torch.cuda.mem_get_info()[0] > (16 << 20)
     digits = images and dtype == "f64"
-    if alg["kernel"] == "gett":
-        launches_per_step = 1 + int(images or plan.workspace(alg["id"]) > 0) + int(digits)
-    else:
-        launches_per_step = alg["n_phases"] * (1 + sum(1 for lv in alg["copy_level"] if lv != -2))
 
     def step():
         plan.execute(dA, dB, dC, alpha=1.0, beta=0.0, stream=stream)
+
+    launches_per_step = kernels_of(step, stream)
 
     for _ in range(args.warmup):
         step()
@@ -452,10 +476,11 @@ def measure_form(args, dtype, spec, extents, A, B, dev, stream, dist, world, tc,
         work = flops * prods
         peak_tf = peaks["bf16_tflops"] * (0.5 if dtype in ("tf32", "tf32x3") else 1.0)
         achieved_tf = work / launch_s / 1e12
-        tkey = f"gett_tc_kernel/{dtype}/{spec}/{nkey}" + (f"/p{prods}" if dtype == "bf16x3" else "")
+        kern, source = ("packed_gett_kernel", "tc_packed.cu") if images else ("gett_tc_kernel", "tc_gett.cu")
+        tkey = f"{kern}/{dtype}/{spec}/{nkey}" + (f"/p{prods}" if dtype == "bf16x3" else "")
         roofline = {"bound": "tensor", "achieved": achieved_tf, "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": achieved_tf / peak_tf,
-                    "traffic": captured_traffic(tkey, "paper_1409_8608_gb300/csrc/tc_gett.cu"),
+                    "traffic": captured_traffic(tkey, "paper_1409_8608_gb300/csrc/" + source),
                     "algorithmic_bytes": algorithmic_bytes,
                     "kernel": "packed_gett_kernel + pack_images_kernel (timed together)" if images else
                               "gett_tc_kernel" + (" + pack_kernel (timed together)" if launches_per_step == 2 else ""),
@@ -472,7 +497,7 @@ def measure_form(args, dtype, spec, extents, A, B, dev, stream, dist, world, tc,
                     "traffic": captured_traffic(f"packed_gett_kernel/{dtype}/{spec}/{nkey}",
                                                 "paper_1409_8608_gb300/csrc/tc_packed.cu"),
                     "algorithmic_bytes": algorithmic_bytes,
-                    "kernel": "packed_gett_kernel + pack_digits_kernel + tile_list_kernel (timed together)",
+                    "kernel": "packed_gett_kernel + pack_digits_kernel + left_kernel (timed together)",
                     "work": f"{prods} digit products x 2*prod(extents) = {work / 1e9:.1f} GFLOP per step",
                     "peak_source": "MEASURED_PEAKS bf16_tflops (burst)" +
                     (" (fallback)" if peaks.get("fallback") else " (measured)")}

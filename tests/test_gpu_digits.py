@@ -264,3 +264,18 @@ def test_marks_in_groups(tcmod):
     plan.device_status()
     plan.close()
     assert torch.equal(C.view(N, M), want)
+
+
+def test_benchmark_counts_every_launch(tcmod):
+    from bench import kernels_of
+    stream = torch.cuda.Stream()
+    for N, panels in ((4000, 1), (64 * 484 + 17, 3)):
+        M, K = 600, 257
+        A, B, C = (torch.ones(n, dtype=torch.float64, device="cuda") for n in (M * K, K * N, M * N))
+        torch.cuda.synchronize()
+        plan = tcmod.Plan("ab=ai,ib", [M, N, K], dtype="f64")
+        plan.execute(A, B, C, stream=stream)
+        torch.cuda.synchronize()
+        # a pre-pass and a GETT per panel, and one launch for what they leave
+        assert kernels_of(lambda: plan.execute(A, B, C, stream=stream), stream) == 2 * panels + 1
+        plan.close()
