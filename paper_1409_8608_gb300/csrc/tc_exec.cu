@@ -732,10 +732,12 @@ tile_batch_kernel(const TileDesc *__restrict__ descs, const int32_t *__restrict_
 // What an FP64 GETT on digits leaves to the chain of fused multiply-adds, with
 // the bits that the SIMT GETT gives: single outputs marked in `weak`, one
 // thread each; patches of 32 x 32 that are marked as a whole, as tiles; and
-// the tiles of a list (item m + list_m * n: sub_m x sub_n tiles of 64 x 64).
-// (512^3 i=j=16: 76 us for the marks of 4.2 M rows of 32 columns and about 20000
-// single outputs; a list of every tile takes what tile_kernel takes, 56.3 ms;
-// in tiles of 32 x 32 57.6, and 958 instead of 820 us for 300 x 4000 x 257.)
+// the tiles of a list (list[0] items m + list_m * n from list[2] on, each
+// sub_m x sub_n tiles of 64 x 64; list[1] counts the tiles taken).
+// 512^3 i=j=16: 60 us for the marks of 4.2 M rows of 32 columns and about 20000
+// single outputs.  Tiles refused as a whole: 55.7 ms there; 2148 x 218 x 2150,
+// 36 items, 2.28 ms, 4.45 where blocks take fixed tiles of 64 x 64, two on
+// some SMs and none on others (the SIMT GETT alone 2.29).
 // A block gathers the marks of its patches (32 at a time, all blocks in turn,
 // so that a weak region of C is spread over them) before it computes any: the
 // single outputs are bound by one chain's K dependent multiply-adds and reads
@@ -746,9 +748,9 @@ struct LeftSingles {
     int64_t kA[256], kB[256];
 };
 
-__global__ void __launch_bounds__(256, 2)
-left_kernel(const TileDesc d, const TileDesc patch, const uint32_t *__restrict__ weak, int64_t rows, int64_t g0, int64_t g1,
-            const int64_t *__restrict__ list, int64_t list_m, int sub_m, int sub_n) {
+__global__ void __launch_bounds__(256, 4)
+left_kernel(const TileDesc d, const TileDesc patch, const TileDesc small, const uint32_t *__restrict__ weak, int64_t rows, int64_t g0, int64_t g1,
+            int64_t *list, int64_t list_m, int sub_m, int sub_n) {
     using Tile = TileOf<double, 0>;
     using Patch = TileOf<double, 1>;
     constexpr int kPatches = 32, kWhole = 256, kAhead = 16;
@@ -758,6 +760,7 @@ left_kernel(const TileDesc d, const TileDesc patch, const uint32_t *__restrict__
     LeftSingles &sm = *reinterpret_cast<LeftSingles *>(buf);
     __shared__ uint32_t whole[kWhole];
     __shared__ int nlist, nwhole;
+    __shared__ int64_t taken;
     const double *__restrict__ A = (const double *)d.A;
     const double *__restrict__ B = (const double *)d.B;
     double *__restrict__ C = (double *)d.C;
@@ -860,14 +863,28 @@ left_kernel(const TileDesc d, const TileDesc patch, const uint32_t *__restrict__
         if (tid == 0) nlist = nwhole = 0;
         __syncthreads();
     }
-    const int64_t count = list ? list[0] * sub_m * sub_n : 0;
-    for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
-        const int64_t item = list[1 + q / (sub_m * sub_n)];
-        const int sub = (int)(q % (sub_m * sub_n));
-        const int64_t tm = item % list_m * sub_m + sub % sub_m, tn = item / list_m * sub_n + sub / sub_m;
-        if (tm >= d.tiles_m || tn >= d.tiles_n) continue;
-        __syncthreads();  // the last tile's tables have been read
-        Tile::run(d, tm + d.tiles_m * tn, buf);
+    // the listed tiles, taken in turn: 64 x 64 where every SM gets eight, 32 x 32
+    // where it gets four (with the four blocks that fit here 16 x 16 are slower
+    // per output: 1024^2, K = 256, 534 against 490 us)
+    const int64_t items = list ? list[0] : 0, tiles = items * sub_m * sub_n;
+    const int shape = tiles >= 2 * (int64_t)gridDim.x ? 0 : (4 * tiles >= (int64_t)gridDim.x ? 1 : 2);
+    const int rows_n = sub_m << shape, per = rows_n * (sub_n << shape);
+    while (items > 0) {
+        __syncthreads();  // the last tile's tables and number have been read
+        if (tid == 0) taken = (int64_t)atomicAdd((unsigned long long *)list + 1, 1ull);
+        __syncthreads();
+        const int64_t q = taken;
+        if (q >= items * per) break;
+        const int64_t item = list[2 + q / per];
+        const int sub = (int)(q % per);
+        const int64_t tm = item % list_m * rows_n + sub % rows_n, tn = item / list_m * (per / rows_n) + sub / rows_n;
+        if (shape == 0) {
+            if (tm < d.tiles_m && tn < d.tiles_n) Tile::run(d, tm + d.tiles_m * tn, buf);
+        } else if (shape == 1) {
+            if (tm < patch.tiles_m && tn < patch.tiles_n) Patch::run(patch, tm + patch.tiles_m * tn, buf);
+        } else if (tm < small.tiles_m && tn < small.tiles_n) {
+            TileOf<double, 2>::run(small, tm + small.tiles_m * tn, buf);
+        }
     }
 }
 
@@ -1362,7 +1379,7 @@ tc_status run_gett_simt(Plan &p, T alpha, const T *A, const T *B, T beta, T *C,
 }  // namespace
 
 tc_status simt_run_left(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
-                        const uint32_t *weak, int64_t rows, int64_t g0, int64_t g1, const int64_t *list, int64_t list_m,
+                        const uint32_t *weak, int64_t rows, int64_t g0, int64_t g1, int64_t *list, int64_t list_m,
                         int item_rows, int item_cols, void *stream) {
     TileDesc td;
     describe_gett_simt<double>(p, *(const double *)alpha, (const double *)A, (const double *)B, *(const double *)beta, (double *)C, td);
@@ -1376,8 +1393,8 @@ tc_status simt_run_left(Plan &p, const void *alpha, const void *A, const void *B
     };
     const int b = simt_rows(true, 0);
     const unsigned grid = (unsigned)device_sms() * 4;
-    left_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(shaped(0), shaped(1), weak, rows, g0, g1, list, list_m, item_rows / b,
-                                                         item_cols / b);
+    left_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(shaped(0), shaped(1), shaped(2), weak, rows, g0, g1, list, list_m,
+                                                         item_rows / b, item_cols / b);
     const cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? TC_SUCCESS : fail(TC_ERROR_CUDA, cudaGetErrorString(e));
 }

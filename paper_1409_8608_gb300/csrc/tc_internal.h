@@ -161,10 +161,11 @@ tc_status exec_digits(Plan &p, const void *alpha, const void *A, const void *B, 
 // (g - g0) * rows + m of `weak` has a bit for each of the columns 32 g ..
 // 32 g + 31 of row m, g0 <= g < g1; a patch of 32 rows with more than
 // kWeakMax of them has them all set.  list (may be null): list[0] items
-// m + list_m * n of item_rows x item_cols, whole SIMT tiles.
+// m + list_m * n of item_rows x item_cols, whole SIMT tiles, from list[2] on;
+// list[1] is 0.
 constexpr int kWeakMax = 128;
 tc_status simt_run_left(Plan &p, const void *alpha, const void *A, const void *B, const void *beta, void *C,
-                        const uint32_t *weak, int64_t rows, int64_t g0, int64_t g1, const int64_t *list, int64_t list_m,
+                        const uint32_t *weak, int64_t rows, int64_t g0, int64_t g1, int64_t *list, int64_t list_m,
                         int item_rows, int item_cols, void *stream);
 
 // One phase of a gemm loop nest on the tensor cores (tensor dtypes): the

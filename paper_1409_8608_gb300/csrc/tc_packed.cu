@@ -133,7 +133,7 @@ struct PackedDesc : GettModes {
     int64_t n_begin;            // first column of the panel (N then counts the panel's)
     // digits: scalars in FP64, per row the exponent field of its largest
     // magnitude (0: a row of zeros), per image row tile the most small entries
-    // of a row, and the tiles left to SIMT (list[0]: how many)
+    // of a row, and the tiles left to SIMT (list[0]: how many, from list[2] on)
     double alpha64, beta64;
     int *exps[2], *small[2];
     int64_t *list;
@@ -802,7 +802,7 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
             if (skip(mt, nt)) {
                 if (threadIdx.x == 0 && crank == 0) {
                     const unsigned long long at = atomicAdd((unsigned long long *)d.list, 1ull);
-                    d.list[1 + at] = mt + d.tiles_m * (d.n_begin / d.bn + nt);
+                    d.list[2 + at] = mt + d.tiles_m * (d.n_begin / d.bn + nt);
                 }
                 continue;
             }
@@ -1233,7 +1233,7 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
     constexpr int BK = stage_k<GK_D64>(), S = Traits<GK_D64>::kSlices;
     if (K < kDigitMinK || K > kDigitMaxK) return false;
     const int64_t Kp = (K + BK - 1) / BK * BK;
-    double best = -1;
+    double best = -1, best_pack = 0;
     for (int pair = 1; pair >= 0; --pair) {
         const int64_t rows = pair ? 2 * kRows : kRows, slots = pair ? sm_count() / 2 : sm_count();
         if (slots < 1) continue;
@@ -1262,12 +1262,17 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
         const double sec = waves * tile / 1.9e9 + pack + 20e-6 + K * 30e-9 + panels * 6e-6;
         if (best < 0 || sec < best) {
             best = sec;
+            best_pack = pack;
             P = q;
         }
     }
     if (best < 0) return false;
     const double simt = 2.0 * (double)M * (double)N * (double)K / 1.24e12;
     if (best > 0.8 * simt) return false;
+    // Values that the digits refuse cost the pre-pass and three launches for
+    // nothing: where that is much of a small GETT, only for twice the speed
+    // (414 x 2622, K = 32, all refused: 99 us, 82 with 64 x 64 SIMT tiles).
+    if (best > 0.5 * simt && best_pack + 30e-6 > 0.15 * simt) return false;
     auto up = [](int64_t x) { return (x + 511) / 512 * 512; };
     P.off_b = P.image_a;
     P.off_exp_a = P.off_b + P.image_b;
@@ -1278,8 +1283,8 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
     P.off_small_a = P.off_weak + up(P.weak_tiles * P.rows_a * kDigitBn / 8);
     P.off_small_b = P.off_small_a + up(P.rows_a / kRows * 4);
     P.off_list = P.off_small_b + up(P.tiles_n * 2 * 4);
-    P.zero_bytes = P.off_list + 8 - P.off_weak;
-    P.bytes = P.off_list + up((P.tiles_m * P.tiles_n + 1) * 8);
+    P.zero_bytes = P.off_list + 16 - P.off_weak;
+    P.bytes = P.off_list + up((P.tiles_m * P.tiles_n + 2) * 8);
     return true;
 }
 
@@ -1327,7 +1332,7 @@ tc_status run_digits(Plan &p, PackedDesc &d, const void *alpha, const void *beta
     e = cudaMemsetAsync(ws + P.off_weak, 0, (size_t)P.zero_bytes, st);
     if (e != cudaSuccess) return fail(TC_ERROR_CUDA, cudaGetErrorString(e));
     int64_t weak0 = 0;  // first column of tiles of those in d.weak
-    auto run_left = [&](int64_t end, const int64_t *list) {
+    auto run_left = [&](int64_t end, int64_t *list) {
         return simt_run_left(p, alpha, d.A, d.B, beta, d.C, d.weak, P.rows_a, weak0 * kDigitBn / 32, end * kDigitBn / 32, list,
                              P.tiles_m, P.pair ? 2 * kRows : kRows, kDigitBn, st);
     };

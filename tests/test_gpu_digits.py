@@ -279,3 +279,30 @@ def test_benchmark_counts_every_launch(tcmod):
         # a pre-pass and a GETT per panel, and one launch for what they leave
         assert kernels_of(lambda: plan.execute(A, B, C, stream=stream), stream) == 2 * panels + 1
         plan.close()
+
+
+@pytest.mark.parametrize("size", [(2148, 218, 2150), (300, 4000, 257)])
+def test_refused_tiles_spread_over_the_sms(tcmod, size):
+    # everything left to the chain: little more than the SIMT GETT takes
+    M, N, K = size
+    gen = torch.Generator(device="cuda").manual_seed(15)
+    A, B = (torch.empty(n, dtype=torch.float64, device="cuda").uniform_(-1, 1, generator=gen) for n in (M * K, K * N))
+    A.view(K, M)[: K // 2 + 9] = 0
+    C = torch.empty(M * N, dtype=torch.float64, device="cuda")
+    st, times, out = torch.cuda.current_stream(), [], []
+    for mode in (1, 0):
+        plan = tcmod.Plan("ab=ai,ib", [M, N, K], dtype="f64")
+        plan.set_gett_pack(mode)
+        ts = []
+        for _ in range(7):
+            e0, e1 = torch.cuda.Event(True), torch.cuda.Event(True)
+            e0.record(st)
+            plan.execute(A, B, C, stream=st)
+            e1.record(st)
+            torch.cuda.synchronize()
+            ts.append(e0.elapsed_time(e1))
+        plan.close()
+        times.append(sorted(ts)[3])
+        out.append(C.clone())
+    assert torch.equal(out[0], out[1])
+    assert times[0] < 1.5 * times[1], times
