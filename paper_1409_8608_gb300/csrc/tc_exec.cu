@@ -68,6 +68,7 @@ struct TileDesc {
     double alpha, beta;
     int init, alpha_one;
     int a_m_fast, b_n_fast;  // load mapping: M (N) contiguous in memory
+    int swapped, unused;     // M and N, A and B exchanged (orient): alpha scales B's side
     int64_t tile0;           // batched form: the problem's first tile in the list
     int64_t shape;           // tile shape (simt_rows)
 };
@@ -546,15 +547,23 @@ __device__ __forceinline__ void tile_body(const TileDesc &d, int64_t bid, TileSm
         else side(No{}, std::integral_constant<int, BN>{}, std::integral_constant<int, LB>{}, std::integral_constant<int, QB>{}, B, roB, sm.kB[b], rB0, kB0, &sm.Bs[b][0][0], BN + sm.PAD);
     };
     // the stage's copies have landed; with alpha != 1 each thread scales the
-    // elements of A that it copied itself
+    // elements of A (of B where they are exchanged) that it copied itself
     auto land_stage = [&](int b) {
         asm volatile("cp.async.wait_all;" ::: "memory");
         if (d.alpha_one) return;
+        int q, r, kk;
+        if (!d.swapped) {
 #pragma unroll
-        for (int l = 0; l < LA; ++l) {
-            int q, r, kk;
-            at(fa, BM, QA, l, rA0, kA0, q, r, kk);
-            sm.As[b][kk][r] = alpha * sm.As[b][kk][r];
+            for (int l = 0; l < LA; ++l) {
+                at(fa, BM, QA, l, rA0, kA0, q, r, kk);
+                sm.As[b][kk][r] = alpha * sm.As[b][kk][r];
+            }
+        } else {
+#pragma unroll
+            for (int l = 0; l < LB; ++l) {
+                at(fb, BN, QB, l, rB0, kB0, q, r, kk);
+                sm.Bs[b][kk][r] = alpha * sm.Bs[b][kk][r];
+            }
         }
     };
     auto step = [&](int sb, int kk) {
@@ -938,6 +947,19 @@ int simt_shape(bool f64, int64_t M, int64_t N, int64_t tasks) {
     return kSimtShapes - 1;
 }
 
+// A warp stores C along M: where C runs along N faster, M and N are exchanged
+// (FP32 bca=iaj,jbic, 403 x 18018, K = 12: 44 us along the slower index, 26
+// so).  Every product and sum stays the same.
+void orient(TileDesc &t) {
+    if (t.n.n == 0 || (t.m.n > 0 && t.m.sC[0] <= t.n.sC[0])) return;
+    std::swap(t.m, t.n);
+    std::swap(t.M, t.N);
+    std::swap(t.A, t.B);
+    std::swap(t.a_m_fast, t.b_n_fast);
+    for (Dims *x : {&t.m, &t.n, &t.red, &t.task}) std::swap(x->sA, x->sB);
+    t.swapped = 1;
+}
+
 // one launch over the first `tiles` tiles of d's shape
 template <typename T>
 void launch_tiles(const TileDesc &d, int64_t tiles, cudaStream_t st) {
@@ -1123,6 +1145,7 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
         int64_t kinB = td.red.n ? td.red.sB[td.red.n - 1] : 0;
         td.a_m_fast = td.m.sA[0] <= kinA || kinA == 0;
         td.b_n_fast = td.n.sB[0] <= kinB || kinB == 0;
+        if (!tensor) orient(td);
     } else {
         fill(pd.out, L.out_ids);
         fill(pd.task, L.task_ids);
@@ -1226,8 +1249,8 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
             g.beta = init == 1 ? (float)beta : 1.0f;
             return gett_launch_nest(p, g, frac, st);
         } else if (tiled) {
-            td.A = Aeff;
-            td.B = Beff;
+            td.A = td.swapped ? Beff : Aeff;
+            td.B = td.swapped ? Aeff : Beff;
             td.C = Cptr;
             td.init = init;
             const int64_t b = simt_rows(sizeof(T) == 8, (int)td.shape);
@@ -1301,9 +1324,10 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
 // of A, N = free indices of B, K = contracted indices.
 // The SIMT GETT's descriptor: M = free indices of A, N = free indices of B
 // (each sorted by their C stride), K = contracted indices with the one
-// contiguous in A (or else in B) innermost; the tile shape by simt_shape.
+// contiguous in A (or else in B) innermost; the tile shape by simt_shape; with
+// `oriented` A's and B's sides exchanged where orient would.
 template <typename T>
-void describe_gett_simt(const Plan &p, T alpha, const T *A, const T *B, T beta, T *C, TileDesc &td) {
+void describe_gett_simt(const Plan &p, T alpha, const T *A, const T *B, T beta, T *C, TileDesc &td, bool oriented = true) {
     std::memset(&td, 0, sizeof(td));
     auto by_c_stride = [&](std::vector<int> ids) {
         std::stable_sort(ids.begin(), ids.end(), [&](int x, int y) {
@@ -1346,6 +1370,7 @@ void describe_gett_simt(const Plan &p, T alpha, const T *A, const T *B, T beta, 
     td.b_n_fast = td.n.n ? (td.n.sB[0] <= kinB || kinB == 0) : 0;
     int64_t tasks = 1;
     for (int id : p.batch) tasks *= p.ext[id];
+    if (oriented) orient(td);
     td.shape = simt_shape(sizeof(T) == 8, td.M, td.N, tasks);
     const int64_t bm = simt_rows(sizeof(T) == 8, (int)td.shape);
     td.tiles_m = (td.M + bm - 1) / bm;
@@ -1382,7 +1407,7 @@ tc_status simt_run_left(Plan &p, const void *alpha, const void *A, const void *B
                         const uint32_t *weak, int64_t rows, int64_t g0, int64_t g1, int64_t *list, int64_t list_m,
                         int item_rows, int item_cols, void *stream) {
     TileDesc td;
-    describe_gett_simt<double>(p, *(const double *)alpha, (const double *)A, (const double *)B, *(const double *)beta, (double *)C, td);
+    describe_gett_simt<double>(p, *(const double *)alpha, (const double *)A, (const double *)B, *(const double *)beta, (double *)C, td, false);
     auto shaped = [&](int shape) {
         TileDesc t = td;
         const int b = simt_rows(true, shape);

@@ -48,3 +48,28 @@ def test_tile_shapes_exact_on_integers(tcmod, spec, dtype, size, K):
         torch.cuda.synchronize()
         plan.close()
         assert np.array_equal(dC.double().cpu().numpy(), alpha * S + beta * 2 * C0), (alpha, beta)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("size", [(129, 300, 37), (40, 1000, 7), (1, 500, 20), (500, 1, 20)])
+def test_order_of_c_does_not_change_the_sums(tcmod, dtype, size):
+    """Tiles store C along its fastest index, A's or B's: the same bits either
+    way, alpha multiplying A's entries (uniform values, alpha and beta inexact)."""
+    M, N, K = size
+    np_t = {"f64": np.float64, "f32": np.float32}[dtype]
+    rng = np.random.default_rng(1)
+    A, B, C0 = (torch.from_numpy(rng.uniform(-1, 1, n).astype(np_t)).cuda() for n in (M * K, K * N, M * N))
+    out = []
+    for spec in ("ab=ai,ib", "ba=ai,ib"):
+        e = {"a": M, "b": N, "i": K}
+        plan = tcmod.Plan(spec, [e[c] for c in synth.index_order(spec)], dtype=dtype)
+        first = spec[0] == "a"
+        gemm = next(a["id"] for a in plan.algorithms() if a["kernel"] == "gemm" and not a["loops"])
+        for alg in (0, gemm):
+            plan.select(alg)
+            C = (C0.view(N, M) if first else C0.view(N, M).T.contiguous()).clone().reshape(-1)
+            plan.execute(A, B, C, alpha=0.7, beta=0.3)
+            torch.cuda.synchronize()
+            out.append(C.view(N, M) if first else C.view(M, N).T)
+        plan.close()
+    assert torch.equal(out[0], out[2]) and torch.equal(out[1], out[3])
