@@ -106,7 +106,10 @@ __device__ __forceinline__ int64_t divmod_pos(int64_t x, int64_t y, int64_t &r) 
     return q;
 }
 
-template <typename T>
+// AHEAD: four positions' loads in flight at a time, multiplied in order, where
+// the innermost index is long (gemv n = 128: 2.03 -> 0.90 ms; on 4 to 32
+// positions it costs 4 to 10 %).
+template <typename T, bool AHEAD>
 __global__ void __launch_bounds__(256) elementwise_kernel(const PhaseDesc d) {
     const T *__restrict__ A = (const T *)d.A;
     const T *__restrict__ B = (const T *)d.B;
@@ -152,10 +155,8 @@ __global__ void __launch_bounds__(256) elementwise_kernel(const PhaseDesc d) {
                     pa += idx[m] * d.red.sA[m];
                     pb += idx[m] * d.red.sB[m];
                 }
-                // four positions' loads in flight at a time, multiplied in
-                // order (one at a time each waited for its own loads)
                 int64_t k = 0;
-                for (; k + 4 <= kext; k += 4) {
+                for (; AHEAD && k + 4 <= kext; k += 4) {
                     T a[4], b[4];
 #pragma unroll
                     for (int x = 0; x < 4; ++x) {
@@ -1169,7 +1170,10 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
         // output splits that index instead (coop_reduce_kernel, loads
         // contiguous across the group): the reduction, not the output count,
         // then sets the parallelism.  Where that index is short and outputs
-        // are not few, one thread computes a group's sums (lane_sums_kernel).
+        // are not few, one thread computes a group's sums (lane_sums_kernel);
+        // a thread's positions follow one another, so with many of them more
+        // outputs are needed (FP64, 19200 outputs of 5 x 23: 27 us in groups,
+        // 34 so; 9802 of 15 x 10 23 and 30; 27000 of 5 x 4 17 and 14).
         const int kr = pd.red.n - 1;
         if (alg.kernel == TC_KERNEL_GER && pd.out.n == 2 && pd.out.sC[1] < pd.out.sC[0]) {
             std::swap(pd.out.ext[0], pd.out.ext[1]);
@@ -1180,7 +1184,9 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
         const bool k_unit = kr >= 0 && (pd.red.sA[kr] == 1 || pd.red.sB[kr] == 1);
         if (k_unit && pd.red.ext[kr] > 1 && pd.total < (int64_t)device_sms() * 1024) coop_g = 1;
         if (coop_g) {
-            coop_thread = pd.red.ext[kr] < 32 && pd.total >= (int64_t)device_sms() * 64;
+            int64_t positions = 1;
+            for (int m = 0; m < pd.red.n; ++m) positions *= pd.red.ext[m];
+            coop_thread = pd.red.ext[kr] < 32 && pd.total >= (int64_t)device_sms() * (positions <= 64 ? 64 : 256);
             const int64_t kext = pd.red.ext[kr];
             coop_g = kext <= 4 ? 4 : (kext <= 8 ? 8 : (kext <= 16 ? 16 : 32));
         }
@@ -1283,8 +1289,9 @@ tc_status run_nest(Plan &p, const Algorithm &alg, T alpha, const T *A, const T *
                     default: coop_reduce_kernel<T, 32><<<(unsigned)grid, 256, 0, st>>>(q); break;
                 }
             } else {
-                int64_t grid = grid_for(q.total, 256);
-                elementwise_kernel<T><<<(unsigned)grid, 256, 0, st>>>(q);
+                const unsigned grid = (unsigned)grid_for(q.total, 256);
+                if (pd.red.n && pd.red.ext[pd.red.n - 1] >= 64) elementwise_kernel<T, true><<<grid, 256, 0, st>>>(q);
+                else elementwise_kernel<T, false><<<grid, 256, 0, st>>>(q);
             }
         }
         cudaError_t e = cudaGetLastError();
