@@ -175,7 +175,8 @@ tc_status tc_algorithm_workspace(tc_plan plan, int32_t alg_id, size_t *bytes);
  * TC_ERROR_INVALID_ARGUMENT is returned: concurrent executes of one plan
  * would share its workspace.  Executes on the same stream queue behind one
  * another as usual.  While `stream` is capturing a CUDA graph the check is
- * skipped and nothing is recorded.
+ * skipped and nothing is recorded.  Graphs captured from one plan share its
+ * workspace and scratch: replay them one after another.
  *
  * TC_F64 with GETT selected: where the size makes it the faster form (K from
  * 32 to 2^15, M up to 2^24 / K; no batch indices), the tensor cores compute

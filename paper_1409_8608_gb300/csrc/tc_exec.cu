@@ -750,15 +750,24 @@ tile_batch_kernel(const TileDesc *__restrict__ descs, const int32_t *__restrict_
 // single outputs.  Tiles refused as a whole: 55.7 ms there; 2148 x 218 x 2150,
 // 36 items, 2.28 ms, 4.45 where blocks take fixed tiles of 64 x 64, two on
 // some SMs and none on others (the SIMT GETT alone 2.29).
-// A block gathers the marks of its patches (32 at a time, all blocks in turn,
-// so that a weak region of C is spread over them) before it computes any: the
-// single outputs are bound by one chain's K dependent multiply-adds and reads
-// where they are few, by a 32-byte sector per element of A and B where many.
+// A block gathers the marks of its patches (8 or 32 at a time, all blocks in
+// turn, so that a weak region of C is spread over them) before it computes any.
+// Many single outputs are bound by a 32-byte sector per element of A and B; few
+// by the chain's K dependent multiply-adds, to which every read of 16 positions
+// added its latency: up to kFew of them have their operands brought to shared
+// memory by the whole block (500 x 1500, K = 8000: 3.31 -> 2.82 ms; 2000^3 903
+// -> 804 us; in two rounds of kFew no faster than a thread each).
 struct LeftSingles {
     static constexpr int kCap = 8192, kStep = 32 * kWeakMax;  // places, and the most that one step adds
+    static constexpr int kFew = 15;       // outputs computed so, at most,
+    static constexpr int kFewK = 128, kFewPitch = 2 * kFewK + 1;  // by so many K positions; their operands
+    static constexpr int kFewAt = 64;     // lie in the list from here on
     uint32_t list[kCap];
     int64_t kA[256], kB[256];
 };
+static_assert((LeftSingles::kCap - LeftSingles::kFewAt) * 4 >= LeftSingles::kFew * LeftSingles::kFewPitch * 8 &&
+                  LeftSingles::kFewAt >= LeftSingles::kFew,
+              "operands fit");
 
 __global__ void __launch_bounds__(256, 4)
 left_kernel(const TileDesc d, const TileDesc patch, const TileDesc small, const uint32_t *__restrict__ weak, int64_t rows, int64_t g0, int64_t g1,
@@ -777,43 +786,88 @@ left_kernel(const TileDesc d, const TileDesc patch, const TileDesc small, const 
     const double *__restrict__ B = (const double *)d.B;
     double *__restrict__ C = (double *)d.C;
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
-    const int64_t rp = rows / 32, patches = rp * (g1 - g0), stride = (int64_t)gridDim.x * kPatches;
+    const int64_t rp = rows / 32, patches = rp * (g1 - g0);
+    // patches that a block looks at together: eight where that spreads them
+    // over more blocks
+    const int group = patches >= (int64_t)gridDim.x * kPatches ? kPatches : 8;
+    const int64_t stride = (int64_t)gridDim.x * group;
     // the patch at place x of this block's: rows 32 pm .., columns 32 (g0 + pn) ..
     auto patch_at = [&](int64_t x, int64_t &pm) -> int64_t {
-        return divmod_pos((int64_t)blockIdx.x * kPatches + x / kPatches * stride + x % kPatches, rp, pm);
+        return divmod_pos((int64_t)blockIdx.x * group + x / group * stride + x % group, rp, pm);
+    };
+    // operand offsets and C of a listed output
+    auto place = [&](uint32_t at, int64_t &oA, int64_t &oB, int64_t &oC) {
+        int64_t x, mm, nn = g0 + patch_at(at >> 10, mm);
+        mm = mm * 32 + (at >> 5 & 31);
+        nn = nn * 32 + (at & 31);
+        oA = oB = oC = 0;
+        for (int m = 0; m < d.m.n; ++m) {
+            mm = divmod_pos(mm, d.m.ext[m], x);
+            oA += x * d.m.sA[m];
+            oC += x * d.m.sC[m];
+        }
+        for (int m = 0; m < d.n.n; ++m) {
+            nn = divmod_pos(nn, d.n.ext[m], x);
+            oB += x * d.n.sB[m];
+            oC += x * d.n.sC[m];
+        }
+    };
+    auto k_place = [&](int64_t k, int64_t &a, int64_t &b) {
+        int64_t x;
+        a = b = 0;
+        if (k >= d.K) return;
+        for (int m = d.red.n - 1; m >= 0; --m) {
+            k = divmod_pos(k, d.red.ext[m], x);
+            a += x * d.red.sA[m];
+            b += x * d.red.sB[m];
+        }
+    };
+    auto few_singles = [&](int count) {
+        constexpr int F = LeftSingles::kFew, K = LeftSingles::kFewK, P = LeftSingles::kFewPitch;
+        double *ops = reinterpret_cast<double *>(sm.list + sm.kFewAt);  // output o: K of A, K of B from o P on
+        const int pos = tid % K;
+        const bool side = tid >= K;
+        const bool live = tid < count;  // lanes of one warp: a multiply-add takes the unit as long for one lane
+        int64_t oA, oB, oC = 0;
+        double acc = 0.0;
+        if (live) {
+            place(sm.list[tid], oA, oB, oC);
+            sm.kA[tid] = oA;
+            sm.kB[tid] = oB;
+            if (d.init != 2) acc = d.init == 1 ? d.beta * C[oC] : C[oC];
+        }
+        for (int64_t k0 = 0; k0 < d.K && count > 0; k0 += K) {
+            __syncthreads();  // the places are there, the last operands have been read
+            int64_t a, b;
+            k_place(k0 + pos, a, b);
+            const double *src = side ? B + b : A + a;
+            const int64_t *at = side ? sm.kB : sm.kA;
+            double v[F];
+#pragma unroll
+            for (int o = 0; o < F; ++o) v[o] = o < count && k0 + pos < d.K ? src[at[o]] : 0.0;
+#pragma unroll
+            for (int o = 0; o < F; ++o)
+                if (o < count) ops[o * P + tid] = side || d.alpha_one ? v[o] : d.alpha * v[o];
+            __syncthreads();
+            if (!live) continue;
+            const int len = (int)min((int64_t)K, d.K - k0);
+            const double *q = ops + tid * P;
+#pragma unroll 8
+            for (int kk = 0; kk < len; ++kk) acc = fma(q[kk], q[K + kk], acc);
+        }
+        if (live) C[oC] = acc;
     };
     auto singles = [&](int count) {
         for (int e0 = 0; e0 < count; e0 += 256) {
             const bool live = e0 + tid < count;
             int64_t oA = 0, oB = 0, oC = 0;
-            if (live) {
-                const uint32_t at = sm.list[e0 + tid];
-                int64_t x, mm, nn = g0 + patch_at(at >> 10, mm);
-                mm = mm * 32 + (at >> 5 & 31);
-                nn = nn * 32 + (at & 31);
-                for (int m = 0; m < d.m.n; ++m) {
-                    mm = divmod_pos(mm, d.m.ext[m], x);
-                    oA += x * d.m.sA[m];
-                    oC += x * d.m.sC[m];
-                }
-                for (int m = 0; m < d.n.n; ++m) {
-                    nn = divmod_pos(nn, d.n.ext[m], x);
-                    oB += x * d.n.sB[m];
-                    oC += x * d.n.sC[m];
-                }
-            }
+            if (live) place(sm.list[e0 + tid], oA, oB, oC);
             double acc = 0.0;
             if (live && d.init != 2) acc = d.init == 1 ? d.beta * C[oC] : C[oC];
             for (int64_t k0 = 0; k0 < d.K; k0 += 256) {
                 __syncthreads();  // the last offsets have been read
-                int64_t k = k0 + tid, x, a = 0, b = 0;
-                if (k < d.K) {
-                    for (int m = d.red.n - 1; m >= 0; --m) {
-                        k = divmod_pos(k, d.red.ext[m], x);
-                        a += x * d.red.sA[m];
-                        b += x * d.red.sB[m];
-                    }
-                }
+                int64_t a, b;
+                k_place(k0 + tid, a, b);
                 sm.kA[tid] = a;
                 sm.kB[tid] = b;
                 __syncthreads();
@@ -841,13 +895,13 @@ left_kernel(const TileDesc d, const TileDesc patch, const TileDesc small, const 
     if (tid == 0) nlist = nwhole = 0;
     __syncthreads();
     int64_t x0 = 0;
-    for (int64_t c = (int64_t)blockIdx.x * kPatches; c < patches; c += stride, x0 += kPatches) {
+    for (int64_t c = (int64_t)blockIdx.x * group; c < patches; c += stride, x0 += group) {
         uint32_t w[kPatches / 8];
 #pragma unroll
         for (int i = 0; i < kPatches / 8; ++i) {
             int64_t pm;
             const int64_t pn = divmod_pos(c + warp + 8 * i, rp, pm);
-            w[i] = c + warp + 8 * i < patches ? weak[pn * rows + pm * 32 + lane] : 0u;
+            w[i] = 8 * i < group && c + warp + 8 * i < patches ? weak[pn * rows + pm * 32 + lane] : 0u;
         }
 #pragma unroll
         for (int i = 0; i < kPatches / 8; ++i) {
@@ -864,7 +918,8 @@ left_kernel(const TileDesc d, const TileDesc patch, const TileDesc small, const 
         __syncthreads();
         const int count = min(nlist, sm.kCap), tiles = nwhole;
         if (c + stride < patches && count <= sm.kCap - sm.kStep && tiles <= kWhole - kPatches) continue;
-        singles(count);
+        if (count <= sm.kFew) few_singles(count);
+        else singles(count);
         __syncthreads();
         for (int i = 0; i < tiles; ++i) {
             int64_t pm;

@@ -5,18 +5,19 @@
 // GETT copies them: no input is converted more than once, however many tiles
 // of the other input it meets, and any strides cost the GETT nothing.
 //
-// pack_images_kernel: a block takes 32 rows x 128 K positions through shared
-// memory, so that its loads run along the operand's contiguous index (rows or
-// K) and its stores are 512-byte runs of an image; one launch for both inputs
-// (4096 x 4096 each: BF16 39 us, split-BF16 53 us; one 16-byte chunk per
-// thread straight from global memory took 67 and 77 us in two launches).
+// pack_images_kernel: a block takes 32 rows x 128 K positions (256 of 16-bit
+// inputs) through shared memory, so that its loads run along the operand's
+// contiguous index (rows or K) and its stores are 512-byte runs of an image;
+// one launch for both inputs (4096 x 4096 each: BF16 36 us, split-BF16 53 us;
+// one 16-byte chunk per thread straight from global memory took 67 and 77 us
+// in two launches).
 //
 // packed_gett_kernel: persistent and warp-specialised, one CTA per SM or a
 // pair of CTAs sharing each MMA (cta_group::2):
-//   copy warp 9      one lane streams each stage's two images with
+//   copy warp 9      an elected lane streams each stage's two images with
 //                    cp.async.bulk.tensor into a ring (both CTAs of a pair
 //                    count their bytes on the issuing CTA's barrier);
-//   MMA warp 8       one lane issues the stage's slice products;
+//   MMA warp 8       an elected lane issues the stage's slice products;
 //   epilogue warps 0-7  drain the accumulators and store C (two groups of
 //                    four, alternate tiles or alternate 32 columns).
 // Why pairs and these widths: an MMA of N columns takes N / 2 clocks and reads
@@ -26,8 +27,8 @@
 // half of B each, 128.  The tile width follows the number of waves
 // (choose_tile).  ab=aij,jib 4096^2 i=j=64: BF16 78 us on pairs of 256 x 224
 // (lone 128 x 256 98 us, pairs of 256 x 256 in four uneven waves 86 us), split-
-// BF16 with compensation 462 us on pairs of 256 x 128 (lone 543 us): tensor
-// pipe 78-80 % active.  With the MMAs issued under a branch on the lane
+// BF16 with compensation 462 us on pairs of 256 x 128 (lone 543 us); BF16
+// keeps the tensor pipe active 82 % of the SMs' active cycles.  With the MMAs issued under a branch on the lane
 // number the same tiles took 178 and 918 us (elect_one).  The compensated
 // sums' (hi, lo) in registers leave the tensor memory to two accumulators.
 //
@@ -840,9 +841,10 @@ packed_gett_kernel(const __grid_constant__ PackedDesc d, const __grid_constant__
             if (quit) break;
             bool aborted = false;
             // the old values of the first columns are on their way before
-            // the accumulator is waited for, later ones before the stores
-            // ahead of them (a column at a time each cost a memory latency:
-            // 46 us for 24 MB of C; the compensated form has no registers for it)
+            // the accumulator is waited for, those of the next ones once the
+            // stores have used the last (a column at a time each cost a memory
+            // latency: 46 us for 24 MB of C; the compensated form has no
+            // registers for it)
             float old[32];
             if (!COMP && KIND != GK_D64 && d.init == 1) load_old(old, C, om, half * 32, lin, on0, nval, cn);
             for (int c = 0; c < nch; ++c) {
