@@ -1260,8 +1260,9 @@ bool plan_digits(int64_t M, int64_t N, int64_t K, DigitPlan &P) {
         const int64_t waves = (panels - 1) * ((q.panel_tiles * q.tiles_m + slots - 1) / slots) +
                               ((q.tiles_n - (panels - 1) * q.panel_tiles) * q.tiles_m + slots - 1) / slots;
         const double pack = (double)(q.rows_a + q.tiles_n * kDigitBn) * Kp * (8 + S * 2) / 3e12;
-        // (left_kernel: a launch and, nearly always, some output's chain)
-        const double sec = waves * tile / 1.9e9 + pack + 20e-6 + K * 30e-9 + panels * 6e-6;
+        // (left_kernel: a launch and, nearly always, some output's chain, 65 to
+        // 105 ns per position)
+        const double sec = waves * tile / 1.9e9 + pack + 15e-6 + K * 80e-9 + panels * 6e-6;
         if (best < 0 || sec < best) {
             best = sec;
             best_pack = pack;

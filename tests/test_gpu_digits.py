@@ -1,9 +1,9 @@
 """Large FP64 GETTs as exact digits on the tensor cores (FP32: by SIMT): exact on
-integers, within the stated bound of |A||B| on uniform entries (and closer
-than one rounding per term), rows and columns at the edges of tiles and of
-panels, and the tiles that the digits may not compute -- wide ranges and
-zeros along K, infinities and NaN, exponents near the ends -- left to the
-SIMT tiles bit for bit."""
+integers, within the stated bound of |A||B| on uniform entries (and closer than
+one rounding per term), one panel of B and several, and what the digits leave
+to the SIMT chains bit for bit: single results and patches of C where large
+terms cancel, tiles with wide ranges and zeros along K, infinities and NaN,
+exponents near the ends."""
 import numpy as np
 import pytest
 
