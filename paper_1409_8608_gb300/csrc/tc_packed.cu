@@ -59,13 +59,13 @@
 //     be exact where small terms are left beside them.  So a result v is stored
 //     only where it is at least 2^-10 2^(eA + eB), the error then at most
 //     K 2^-48.9 |v| whatever the terms, and marked otherwise: one of 7000 on
-//     uniform entries at K = 256, one of 1700 on normal ones.
+//     uniform entries at K = 256, one of 1300 on normal ones.
 // Both are left to the chain (tc_exec.cu, left_kernel).  On uniform and normal
 // entries little but the last rounding is lost (5e-17 of the result, 6e-16 in
 // the chain).
 // B is taken in panels whose images stay in L2.
 // abc=iaj,jbic 512^3 i=j=16: 56.7 -> 2.95 ms (18 panels: pre-pass 23 us, GETT
-// 137 us each, 128 without the check of the results; left_kernel 76 us.  Of
+// 137 us each, 128 without the check of the results; left_kernel 60 us.  Of
 // the 128, 92 without the drains and conversions; 135 where every product
 // reads its digit of A from shared memory, not from the collector buffer, 153
 // with a conversion that branches).
